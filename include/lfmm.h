@@ -98,12 +98,13 @@ enum {
     LFMM_PROFILE_STAGES = 1 /* time every stage of lfmm_matvec with CUDA events on the call's
                                stream (adds one stream synchronisation per call); read the
                                totals with lfmm_geometry_query("stage_times") */,
-    LFMM_AUTOTUNE = 2       /* choose the schedule of the M2L work items (cap on the work of
-                               one item, one row per narrow box or not) by timing the
-                               candidates on this geometry at set-up (some 40 M2L launches);
-                               read the choice with lfmm_geometry_query("tuning").  Results
-                               differ from the default schedule only in the order in which
-                               the parts of a split sum are added */,
+    LFMM_AUTOTUNE = 2       /* choose the schedule of the M2L (cap on the work of one unit of
+                               the FP64 form and of one item of the precision form) by timing
+                               the candidates' FP64 M2L on this geometry at set-up (some 10
+                               launches); read the choice with lfmm_geometry_query("tuning").
+                               FP64 results do not depend on the schedule; the precision form's
+                               differ only in the order in which the parts of a split sum are
+                               added */,
     LFMM_COMBINED_FIELD = 4 /* combined-field operator instead of the paper's single layer
                                (needs the normals): 1/2 I + D - i k S with D the double
                                layer of the layered Green's function (normal derivative at

@@ -486,6 +486,7 @@ lfmm_status lfmm_matvec(lfmm_geometry g, int32_t nrhs, const void* x, void* y, i
         if (!dev) {
             cuda_check(cudaMemcpyAsync(y, g->d_hostbuf_y, esz * elems, cudaMemcpyDeviceToHost, s), "y d2h");
             cuda_check(cudaStreamSynchronize(s), "matvec sync");
+            split_check_waits(g);
             mixed_check_waits(g);
         }
         return LFMM_OK;

@@ -18,6 +18,7 @@
 
 #include "fmm_kernels.cuh"
 #include "geometry.h"
+#include "split.cuh"
 
 namespace lfmm {
 
@@ -192,6 +193,187 @@ static void build_m2l_work(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, c
     make_m2l_items(g, M2L_ITEM_WORK, 1);
 }
 
+// The split M2L's matrices, pairs and destinations (split.cuh).  Matrices, and with them
+// units and workspace rows, in level order, so that the levels above the precision form's
+// first FP32 level are a prefix.
+static size_t split_col_bytes(const lfmm_geometry_s* g) {   // workspace of one column
+    return sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) +
+           (size_t)g->sp_nvec * (SP_ND * SP_POS * sizeof(uint32_t) + sizeof(int)) + 16;
+}
+static void split_alloc(lfmm_geometry_s* g, int cols) {   // products, then digits, then exponents
+    unsigned char* p = (unsigned char*)dev_alloc_ready(split_col_bytes(g) * cols, "split M2L workspace");
+    const size_t rows = sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) * cols;
+    g->d_sp_ws = (double*)p;
+    g->d_sp_vdig = (uint32_t*)(p + ((rows + 15) & ~(size_t)15));
+    g->d_sp_vexp = (int*)(g->d_sp_vdig + (size_t)g->sp_nvec * cols * SP_ND * SP_POS);
+    g->sp_ws_cols = cols;
+}
+// Units: a matrix's pairs in groups of up to cap, of nearly equal size, by row tiles of up
+// to 64 complex rows.  Replaces the geometry's units.
+static void make_split_units(lfmm_geometry_s* g, int cap) {
+    std::vector<SplitUnit> units;
+    const int nlev = g->tree.D + 1;
+    g->sp_unit_start.assign(nlev + 2, -1);
+    g->sp_max_cnt = 0;
+    for (const SplitTab& s : g->sp_tabs_host) {
+        if (g->sp_unit_start[s.level] < 0) g->sp_unit_start[s.level] = (int)units.size();
+        const int nco = 2 * s.pT + 1, nu = (s.npairs + cap - 1) / cap;
+        for (int u = 0; u < nu; ++u) {
+            const int q0 = (int)((int64_t)s.npairs * u / nu), q1 = (int)((int64_t)s.npairs * (u + 1) / nu);
+            g->sp_max_cnt = std::max(g->sp_max_cnt, q1 - q0);
+            for (int k = 0; k * split_tile(nco) < nco; ++k)
+                units.push_back(SplitUnit{s.base, s.out0 + (int64_t)q0 * 2 * nco, s.sr, s.sc, s.pT, s.pS, s.rexp, s.dexp, s.react,
+                                          s.pair0 + q0, q1 - q0, k});
+        }
+    }
+    for (int l = nlev + 1, next = (int)units.size(); l >= 0; --l) {
+        if (g->sp_unit_start[l] < 0) g->sp_unit_start[l] = next;
+        next = g->sp_unit_start[l];
+    }
+    auto it = std::find(g->allocs.begin(), g->allocs.end(), (void*)g->d_sp_unit);
+    if (g->d_sp_unit && it != g->allocs.end()) { g->allocs.erase(it); dev_release(g->d_sp_unit); }   // units being replaced
+    g->d_sp_unit = dupload(g, units);
+}
+static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, const std::vector<int>& vr_src,
+                        const std::vector<int>& vr_key, const std::vector<int>& vr_comp,
+                        const std::vector<int>& vr_flip, const std::vector<ReactKey>& keys) {
+    TreeHost& t = g->tree;
+    const int D = t.D, l0 = t.l0, nlev = D + 1, nl = g->m.nl;
+    const int nF = (int)g->ftab_lay.size(), nR = (int)keys.size();
+    // source scales per (layer, level): d_n = -floor(log2 max_{m >= |n|} |J_m(k R)|), R the
+    // half diagonal of a cell (one order lower for the combined field's dipole basis)
+    std::vector<int> dexp, dexp_off(nl * nlev, 0);
+    for (int lay = 0; lay < nl; ++lay)
+        for (int l = l0; l <= D; ++l) {
+            const int p = t.p_level[l];
+            std::vector<double> J(p + 1);
+            bessel_j_seq(g->m.k[lay] * t.width(l) * std::sqrt(0.5), p, J.data());
+            dexp_off[lay * nlev + l] = (int)dexp.size();
+            std::vector<int> d(p + 1);
+            double env = 0.0;
+            for (int n = p; n >= 0; --n) {
+                env = std::max(env, std::fabs(J[std::max(0, n - (g->combined ? 1 : 0))]));
+                d[n] = env > 1e-300 ? -std::ilogb(env) : 997;
+            }
+            dexp.insert(dexp.end(), d.begin(), d.end());
+        }
+    // pairs per matrix: free-space canonical tables, then reaction keys
+    std::vector<int> cnt(nF + nR, 0);
+    for (int v : g->vf_tab_host) ++cnt[g->ftab_canon[v]];
+    for (int v : vr_key) ++cnt[nF + v];
+    std::vector<std::vector<int>> by_level(nlev);
+    for (int i = 0; i < nF; ++i) if (cnt[i]) by_level[g->ftab_lev[i]].push_back(i);
+    for (int i = 0; i < nR; ++i) if (cnt[nF + i]) by_level[keys[i].level].push_back(nF + i);
+    std::vector<SplitTab> tabs;
+    std::vector<int> tab_of(nF + nR, -1), fill(nF + nR, 0);
+    int np = 0, nrexp = 0;
+    int64_t rows = 0;
+    for (int l = 0; l < nlev; ++l) {
+        for (int i : by_level[l]) {
+            SplitTab s{};
+            const int p = t.p_level[l], nco = 2 * p + 1;
+            s.pT = s.pS = p;
+            if (i < nF) {   // A[n][m] = T[m - n]
+                s.base = g->ftab_off_host[i] + 2 * p;
+                s.sr = -1; s.sc = 1; s.react = 0;
+                s.dexp = dexp_off[g->ftab_lay[i] * nlev + l];
+            } else {        // column-major
+                s.base = keys[i - nF].off;
+                s.sr = 1; s.sc = nco; s.react = 1;
+                s.dexp = dexp_off[g->rkey_lay_s[i - nF] * nlev + l];
+            }
+            s.rexp = nrexp; nrexp += nco * split_nseg(p);
+            s.pair0 = np; s.npairs = cnt[i]; np += cnt[i];
+            s.out0 = rows; rows += (int64_t)cnt[i] * 2 * nco;
+            tab_of[i] = (int)tabs.size();
+            s.level = l;
+            tabs.push_back(s);
+        }
+    }
+    // source vectors: every cell's and reaction centre's multipole, by segments
+    std::vector<SplitVec> vecs;
+    std::vector<int> vec_of(t.nbox, -1), vec_of_slot(g->n_slots, -1);
+    g->sp_vec_start.assign(nlev + 2, 0);
+    for (int l = 0; l < nlev; ++l) {
+        g->sp_vec_start[l] = (int)vecs.size();
+        if (l < l0) continue;
+        const int p = t.p_level[l];
+        auto add = [&](int64_t off, int lay, int slot) {
+            const int v = (int)vecs.size();
+            for (int s = 0; s < split_nseg(p); ++s) vecs.push_back(SplitVec{off, p, s, dexp_off[lay * nlev + l], slot});
+            return v;
+        };
+        for (int b = t.level_start[l]; b < t.level_start[l + 1]; ++b) {
+            vec_of[b] = add(g->box_coef_off_host[b], t.box_layer[b], 0);
+            for (int side = 0; side < 2; ++side) {
+                const int q = g->slot_of_host[2 * b + side];
+                if (q >= 0) vec_of_slot[q] = add(g->slot_coef_host[q], t.box_layer[b], 1);
+            }
+        }
+    }
+    for (int l = nlev; l <= nlev + 1; ++l) g->sp_vec_start[l] = (int)vecs.size();
+    std::vector<SplitPair> pairs(np);
+    std::vector<SplitRow> rowv[3];
+    std::vector<SplitRow> rlist;
+    rlist.reserve(np);
+    std::vector<SplitDst> dst;
+    g->sp_dst_start.assign(nlev + 2, 0);
+    for (int l = 0; l < nlev; ++l) {
+        g->sp_dst_start[l] = (int)dst.size();
+        if (l < l0) continue;
+        const int p = t.p_level[l], nco = 2 * p + 1;
+        auto add = [&](int i, int vec, int fin, int fout, int d) {
+            const SplitTab& s = tabs[tab_of[i]];
+            const int q = fill[i]++;
+            pairs[s.pair0 + q] = SplitPair{vec, fin};
+            rowv[d].push_back(SplitRow{s.out0 + (int64_t)q * 2 * nco, fout, 0});
+        };
+        for (int T = t.level_start[l]; T < t.level_start[l + 1]; ++T) {
+            for (int e = g->vf_ptr_host[T]; e < g->vf_ptr_host[T + 1]; ++e) {
+                const int tab = g->vf_tab_host[e], turn = g->ftab_turn[tab];
+                const int mir = turn >> 2, q = (turn + 2 * mir) & 3;
+                add(g->ftab_canon[tab], vec_of[g->vf_src_host[e]], (mir ? SP_REV : 0) | (q << SP_Q_SHIFT),
+                    (mir ? SP_REV : 0) | (((4 - q) & 3) << SP_Q_SHIFT), 0);
+            }
+            for (int e = vr_ptr[T]; e < vr_ptr[T + 1]; ++e) {
+                const int S = vr_src[e];
+                const Component& C = t.comps[vr_comp[e]];
+                const int ssl = g->slot_of_host[2 * S + (C.a == 0 ? 0 : 1)];
+                const int side = (C.b == 0) ? 1 : 0;
+                const int d = (g->slot_of_host[2 * T + side] >= 0) ? 1 + side : 0;
+                const int rin = (C.a ? 0 : 1) ^ vr_flip[e], rout = (C.b ? 0 : 1) ^ vr_flip[e];
+                add(nF + vr_key[e], ssl >= 0 ? vec_of_slot[ssl] : vec_of[S],
+                    (rin ? SP_REV : 0) | ((C.a ? 0 : 2) << SP_Q_SHIFT),
+                    (rout ? SP_REV : 0) | ((C.b ? 0 : 2) << SP_Q_SHIFT), d);
+            }
+            for (int d = 0; d < 3; ++d) {
+                const int ts = d == 0 ? -1 : g->slot_of_host[2 * T + d - 1];
+                if (d > 0 && ts < 0) continue;
+                const int r0 = (int)rlist.size();
+                rlist.insert(rlist.end(), rowv[d].begin(), rowv[d].end());
+                rowv[d].clear();
+                dst.push_back(SplitDst{d == 0 ? g->box_coef_off_host[T] : g->slot_coef_host[ts], p, d > 0 ? 1 : 0, r0,
+                                       (int)rlist.size()});
+            }
+        }
+    }
+    for (int l = nlev; l <= nlev + 1; ++l) g->sp_dst_start[l] = (int)dst.size();
+    g->d_sp_tab = dupload(g, tabs);
+    g->d_sp_vec = dupload(g, vecs);
+    g->sp_nvec = (int)vecs.size();
+    g->d_sp_pair = dupload(g, pairs);
+    g->d_sp_row = dupload(g, rlist);
+    g->d_sp_dst = dupload(g, dst);
+    g->d_sp_dexp = dupload(g, dexp);
+    g->d_sp_rexp = dalloc<int>(g, (size_t)std::max(nrexp, 1));
+    g->sp_ntab = (int)tabs.size();
+    g->sp_tabs_host = tabs;
+    make_split_units(g, SP_COLS);
+    g->sp_rows = rows;
+    split_alloc(g, 1);
+    cuda_check(cudaHostAlloc((void**)&g->wait_err, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable), "wait status");
+    *g->wait_err = 0;
+}
 
 void fmm_build(lfmm_geometry_s* g) {
     TreeHost& t = g->tree;
@@ -457,6 +639,35 @@ void fmm_build(lfmm_geometry_s* g) {
             }
             vf_ptr[T + 1] = (int)vf_src.size();
         }
+        // each offset's equivalent in the first octant (quarter turns and mirror images of
+        // one offset share a matrix of the split M2L)
+        const int nlisted = (int)tl.size();
+        g->ftab_canon.resize(nlisted);
+        g->ftab_turn.resize(nlisted);
+        for (int i = 0; i < nlisted; ++i) {
+            int bx = tdx[i], by = tdy[i], q = 0;
+            while (!(bx > 0 && by >= 0 && by < bx) && !(bx > 0 && by == bx) && !(bx >= 0 && by > bx)) {
+                const int u = bx;   // turn back by a quarter until the offset is in the first quadrant
+                bx = by; by = -u; ++q;
+            }
+            // (dx, dy) = the offset (bx, by), bx > 0 or (0, by), turned by q quarters; a steep
+            // one is the mirror image of a flat one turned by one quarter more
+            int mir = 0;
+            if (by > bx) { std::swap(bx, by); mir = 1; q += 1; }
+            auto key = std::make_tuple(tl[i], tlev[i], bx, by);
+            auto it = id.find(key);
+            if (it == id.end()) {
+                it = id.emplace(key, (int)tl.size()).first;
+                tl.push_back(tl[i]); tlev.push_back(tlev[i]); tdx.push_back(bx); tdy.push_back(by);
+                tp.push_back(tp[i]); tw.push_back(tw[i]);
+                toff.push_back(tot);
+                tot += 4 * tp[i] + 1;
+            }
+            g->ftab_canon[i] = it->second;
+            g->ftab_turn[i] = (q & 3) | (mir << 2);
+        }
+        g->ftab_off_host = toff;
+        g->ftab_p = tp;
         g->d_m2lf = dalloc<cd>(g, (size_t)std::max<int64_t>(tot, 1));
         g->m2lf_len = tot;
         g->d_m2lf_off = dupload(g, toff);
@@ -528,6 +739,7 @@ void fmm_build(lfmm_geometry_s* g) {
         g->d_vr_key = dupload(g, vr_key);
         g->d_vr_comp = dupload(g, vr_comp);
         build_m2l_work(g, vr_ptr, vr_src, vr_key, vr_comp, vr_flip, keys);
+        build_split(g, vr_ptr, vr_src, vr_key, vr_comp, vr_flip, keys);
         g->d_rkeys = dupload(g, keys);
         g->rkeys_host = keys;
         g->d_m2lr = dalloc<cd>(g, (size_t)std::max<int64_t>(tot, 1));
@@ -578,6 +790,10 @@ void fmm_build(lfmm_geometry_s* g) {
                 cuda_check(cudaGetLastError(), "k_react_tables_same");
             }
         }
+        if (g->sp_ntab > 0) {
+            k_split_rexp<<<g->sp_ntab, 128>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_sp_dexp, g->d_sp_rexp);
+            cuda_check(cudaGetLastError(), "k_split_rexp");
+        }
     }
     cuda_check(cudaStreamSynchronize(cudaStreamPerThread), "fmm_build");
 }
@@ -599,7 +815,6 @@ static void set_smem_limits() {
     const size_t lim = 200 * 1024;
     raise_smem_limit((const void*)k_p2m, lim, "smem p2m");
     raise_smem_limit((const void*)k_l2p, lim, "smem l2p");
-    raise_smem_limit((const void*)k_m2l, lim, "smem m2l");
 }
 
 static void ensure_coef(lfmm_geometry_s* g, int nrhs) {
@@ -618,14 +833,18 @@ void fmm_free(lfmm_geometry_s* g) {
     dev_release(g->d_m2l_part);
     g->d_m2l_part = nullptr;
     g->m2l_part_cols = 0;
+    dev_release(g->d_sp_ws);
+    g->d_sp_ws = nullptr;
+    g->sp_ws_cols = 0;
+    if (g->wait_err) cudaFreeHost(g->wait_err);
+    g->wait_err = nullptr;
     dev_release(g->d_M); dev_release(g->d_L);
     dev_release(g->d_Mp); dev_release(g->d_Lp);
     g->d_M = g->d_L = g->d_Mp = g->d_Lp = nullptr;
     g->coef_cols = 0;
 }
 
-// FP64 M2L over the first n64 work items and the first r64 reductions of split
-// items (the levels below the precision form's first FP32 level, or all levels).
+// partial sums of the precision form's double-float M2L
 static void ensure_m2l_part(lfmm_geometry_s* g, int nrhs) {
     if (g->n_m2l_parts > 0 && g->m2l_part_cols < nrhs) {
         dev_release_now(g->d_m2l_part);
@@ -635,27 +854,62 @@ static void ensure_m2l_part(lfmm_geometry_s* g, int nrhs) {
         g->m2l_part_cols = nrhs;
     }
 }
-// FP64 M2L of the work items [i0, i1) and the reductions [r0, r1) (a range of levels)
-static void launch_m2l_range(lfmm_geometry_s* g, int nrhs, int i0, int i1, int r0, int r1, cudaStream_t s) {
-    if (i1 > i0) {
-        k_m2l<<<i1 - i0, 128, 0, s>>>(g->d_m2l_items + i0, g->d_m2l_ents, g->d_box_level, g->d_p_level,
-                                      g->d_coef_off, g->d_slot_of, g->d_slot_coef, g->d_m2lf, g->d_m2lf_off,
-                                      g->d_m2lr, nrhs, g->ncoef, g->nslotcoef, g->n_m2l_parts, g->d_M, g->d_Mp,
-                                      g->d_L, g->d_Lp, g->d_m2l_part);
-        cuda_check(cudaGetLastError(), "k_m2l");
-        ++g->n_launches;
-    }
-    if (r1 > r0) {
-        k_m2l_reduce<<<r1 - r0, 64, 0, s>>>(g->d_m2l_reds + r0, g->d_box_level, g->d_p_level, g->d_coef_off,
-                                            g->d_slot_of, g->d_slot_coef, nrhs, g->ncoef, g->nslotcoef,
-                                            g->n_m2l_parts, g->d_m2l_part, g->d_L, g->d_Lp);
-        cuda_check(cudaGetLastError(), "k_m2l_reduce");
-        ++g->n_launches;
-    }
+// reductions [0, r1) of the double-float M2L's split items
+static void launch_m2l_reduce(lfmm_geometry_s* g, int nrhs, int r1, cudaStream_t s) {
+    if (r1 <= 0) return;
+    k_m2l_reduce<<<r1, 64, 0, s>>>(g->d_m2l_reds, g->d_box_level, g->d_p_level, g->d_coef_off, g->d_slot_of,
+                                   g->d_slot_coef, nrhs, g->ncoef, g->nslotcoef, g->n_m2l_parts, g->d_m2l_part, g->d_L,
+                                   g->d_Lp);
+    cuda_check(cudaGetLastError(), "k_m2l_reduce");
+    ++g->n_launches;
 }
-static void launch_m2l64(lfmm_geometry_s* g, int nrhs, int n64, int r64, cudaStream_t s) {
-    ensure_m2l_part(g, nrhs);
-    launch_m2l_range(g, nrhs, 0, n64, 0, r64, s);
+
+// The split M2L's workspace: one row of products per (pair, column), for as many columns
+// at once as fit SP_WS_BYTES (at least one); a wider block takes several rounds.
+#define SP_WS_BYTES (2ll << 30)
+static int split_round(const lfmm_geometry_s* g, int nrhs) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(nrhs, SP_WS_BYTES / (int64_t)split_col_bytes(g)));
+}
+static void ensure_split(lfmm_geometry_s* g, int nrhs) {
+    const int want = split_round(g, nrhs);
+    if (g->sp_ws_cols >= want) return;
+    dev_release_now(g->d_sp_ws);
+    g->d_sp_ws = nullptr;
+    g->sp_ws_cols = 0;
+    split_alloc(g, want);
+}
+void split_check_waits(lfmm_geometry_s* g) {
+    if (!g->wait_err || *(volatile int*)g->wait_err == 0) return;
+    *(volatile int*)g->wait_err = 0;
+    throw TimeoutError{"split M2L: an mbarrier wait gave up; that product's M2L contributions were zeroed"};
+}
+static SplitArgs split_args(lfmm_geometry_s* g, int col0, int ncols) {
+    return SplitArgs{g->d_sp_vec, g->d_sp_pair, g->d_sp_unit, g->d_sp_row, g->d_sp_dst, g->d_sp_rexp, g->d_sp_dexp,
+                     g->d_m2lf, g->d_m2lr, g->d_M, g->d_Mp, g->d_L, g->d_Lp, g->ncoef, g->nslotcoef,
+                     g->d_sp_vdig, g->d_sp_vexp, g->sp_nvec, g->d_sp_ws, col0, ncols, g->wait_err};
+}
+static int split_chunks(const lfmm_geometry_s* g, int ncols) { return (g->sp_max_cnt * ncols + SP_COLS - 1) / SP_COLS; }
+// FP64 M2L of the levels below lm
+static void launch_split(lfmm_geometry_s* g, int nrhs, int lm, cudaStream_t s) {
+    split_check_waits(g);
+    ensure_split(g, nrhs);
+    const int nu = g->sp_unit_start[lm], nd = g->sp_dst_start[lm];
+    raise_smem_limit((const void*)k_split, SP_SMEM, "split M2L smem");
+    for (int c0 = 0; c0 < nrhs && nd > 0; c0 += g->sp_ws_cols) {
+        const SplitArgs a = split_args(g, c0, std::min(nrhs - c0, g->sp_ws_cols));
+        if (nu > 0) {
+            const int nv = g->sp_vec_start[lm];
+            k_split_vec<<<dim3((nv + 3) / 4, a.ncols), 128, 0, s>>>(a, 0, nv);
+            cuda_check(cudaGetLastError(), "k_split_vec");
+            ++g->n_launches;
+            k_split<<<dim3(nu, split_chunks(g, a.ncols)), 256, SP_SMEM, s>>>(a);
+            cuda_check(cudaGetLastError(), "k_split");
+            ++g->n_launches;
+        }
+        k_split_reduce<<<dim3(nd, a.ncols), 192, 0, s>>>(a, 0);
+        cuda_check(cudaGetLastError(), "k_split_reduce");
+        ++g->n_launches;
+    }
 }
 
 // one level's M2M (into parents at level - 1: down = 0) or L2L (into children at level:
@@ -749,9 +1003,9 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
             // precision form: the coarse (wide-band) levels in double-float, the rest in FP32
             ensure_m2l_part(g, nrhs);
             mixed_m2l_coarse(g, nrhs, n64, s);
-            launch_m2l_range(g, nrhs, 0, 0, 0, r64, s);
+            launch_m2l_reduce(g, nrhs, r64, s);
         } else {
-            launch_m2l64(g, nrhs, n64, r64, s);
+            launch_split(g, nrhs, lm, s);
         }
         if (lm <= D) mixed_m2l(g, nrhs, lm, s);
         prof_end(g, ST_M2L, s);
@@ -821,17 +1075,10 @@ struct XJob {
     XPass P;
     int nrhs;
 };
-struct M2LJob {
-    const M2LItem* items;
-    const M2LReduce* reds;
-    const M2LEnt* ents;
-    const int *box_level, *p_level, *slot_of;
-    const int64_t *coef_off, *slot_coef, *m2lf_off;
-    const cd *m2lf, *m2lr;
-    int nrhs, nparts;
-    int64_t ncoef, nslotcoef;
-    const cd *M, *Mp;
-    cd *L, *Lp, *part;
+struct SplitJob {
+    SplitArgs a;
+    int chunks;   // column chunks per unit
+    int vblocks;  // blocks of k_split_vec per column
 };
 
 __device__ __forceinline__ int job_of(const int* __restrict__ prefix, int njobs, int b) {
@@ -863,19 +1110,23 @@ __global__ void __launch_bounds__(128) k_translate_multi(const XJob* __restrict_
     const XPass P = jobs[j].P;
     translate_item(blockIdx.x - prefix[j], P, 0, jobs[j].nrhs, xsm);
 }
-__global__ void __launch_bounds__(128) k_m2l_multi(const M2LJob* __restrict__ jobs, const int* __restrict__ prefix,
-                                                   int njobs) {
-    const int j = job_of(prefix, njobs, blockIdx.x);
-    const M2LJob& J = jobs[j];
-    m2l_item(blockIdx.x - prefix[j], J.items, J.ents, J.box_level, J.p_level, J.coef_off, J.slot_of, J.slot_coef,
-             J.m2lf, J.m2lf_off, J.m2lr, J.nrhs, J.ncoef, J.nslotcoef, J.nparts, J.M, J.Mp, J.L, J.Lp, J.part);
-}
-__global__ void __launch_bounds__(64) k_m2l_reduce_multi(const M2LJob* __restrict__ jobs,
+__global__ void __launch_bounds__(128) k_split_vec_multi(const SplitJob* __restrict__ jobs,
                                                          const int* __restrict__ prefix, int njobs) {
     const int j = job_of(prefix, njobs, blockIdx.x);
-    const M2LJob& J = jobs[j];
-    m2l_reduce_one(blockIdx.x - prefix[j], J.reds, J.box_level, J.p_level, J.coef_off, J.slot_of, J.slot_coef,
-                   J.nrhs, J.ncoef, J.nslotcoef, J.nparts, J.part, J.L, J.Lp);
+    const int b = blockIdx.x - prefix[j], vb = jobs[j].vblocks;
+    split_vec(jobs[j].a, b % vb, b / vb, 0, (int)jobs[j].a.nvec);
+}
+__global__ void __launch_bounds__(256, 2) k_split_multi(const SplitJob* __restrict__ jobs,
+                                                        const int* __restrict__ prefix, int njobs) {
+    const int j = job_of(prefix, njobs, blockIdx.x);
+    const int b = blockIdx.x - prefix[j], ch = jobs[j].chunks;
+    split_unit(jobs[j].a, b / ch, b % ch);
+}
+__global__ void __launch_bounds__(192) k_split_reduce_multi(const SplitJob* __restrict__ jobs,
+                                                            const int* __restrict__ prefix, int njobs) {
+    const int j = job_of(prefix, njobs, blockIdx.x);
+    const int b = blockIdx.x - prefix[j], nc = jobs[j].a.ncols;
+    split_reduce(jobs[j].a, b / nc, b % nc);
 }
 
 void JobTables::upload(cudaStream_t s) {
@@ -918,13 +1169,8 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
         if (t.l0 > t.D) continue;
         far.push_back(&op);
         ensure_coef(g, op.nrhs);
-        if (g->n_m2l_parts > 0 && g->m2l_part_cols < op.nrhs) {
-            dev_release_now(g->d_m2l_part);
-            g->d_m2l_part = nullptr;
-            g->d_m2l_part = (cd*)dev_alloc_ready(sizeof(cd) * (size_t)g->n_m2l_parts * 3 * XT_W * op.nrhs,
-                                                 "M2L partial sums");
-            g->m2l_part_cols = op.nrhs;
-        }
+        split_check_waits(g);
+        ensure_split(g, op.nrhs);
         const int pD = t.p_level[t.D], gp = g->group_max_pts, ge = g->group_max_ent;
         const int rs = 2 * (g->combined ? pD + 1 : pD) + 1;
         smem_p2m = std::max(smem_p2m, (size_t)gp * rs * sizeof(cd) + (size_t)gp * sizeof(cd) + (size_t)(gp + 1) * sizeof(int));
@@ -970,21 +1216,27 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
         raise_smem_limit((const void*)k_translate_multi, smem, "translate smem");
         launch_jobs(jobs, blocks, k_translate_multi, 128, smem, s, "k_translate_multi (M2M)");
     }
-    {   // M2L of every level, then the reductions of split items
-        std::vector<M2LJob> jobs;
-        std::vector<int> blocks, rblocks;
+    // M2L of every level: products, then each destination's sum; a block too wide for its
+    // workspace takes several rounds
+    raise_smem_limit((const void*)k_split_multi, SP_SMEM, "split M2L smem");
+    for (int round = 0;; ++round) {
+        std::vector<SplitJob> jobs;
+        std::vector<int> blocks, rblocks, vblocks;
         for (const BatchOp* op : far) {
             lfmm_geometry_s* g = op->g;
-            const int D = g->tree.D;
-            jobs.push_back(M2LJob{g->d_m2l_items, g->d_m2l_reds, g->d_m2l_ents, g->d_box_level, g->d_p_level,
-                                  g->d_slot_of, g->d_coef_off, g->d_slot_coef, g->d_m2lf_off, g->d_m2lf, g->d_m2lr,
-                                  op->nrhs, g->n_m2l_parts, g->ncoef, g->nslotcoef, g->d_M, g->d_Mp, g->d_L, g->d_Lp,
-                                  g->d_m2l_part});
-            blocks.push_back(g->m2l_item_level_start[D + 1]);
-            rblocks.push_back(g->m2l_red_level_start[D + 1]);
+            const int c0 = round * g->sp_ws_cols, D = g->tree.D;
+            if (c0 >= op->nrhs) continue;
+            const int nc = std::min(op->nrhs - c0, g->sp_ws_cols);
+            const int vb = (g->sp_nvec + 3) / 4;
+            jobs.push_back(SplitJob{split_args(g, c0, nc), split_chunks(g, nc), vb});
+            vblocks.push_back(vb * nc);
+            blocks.push_back(g->sp_unit_start[D + 1] * split_chunks(g, nc));
+            rblocks.push_back(g->sp_dst_start[D + 1] * nc);
         }
-        launch_jobs(jobs, blocks, k_m2l_multi, 128, 0, s, "k_m2l_multi");
-        launch_jobs(jobs, rblocks, k_m2l_reduce_multi, 64, 0, s, "k_m2l_reduce_multi");
+        if (jobs.empty()) break;
+        launch_jobs(jobs, vblocks, k_split_vec_multi, 128, 0, s, "k_split_vec_multi");
+        launch_jobs(jobs, blocks, k_split_multi, 256, SP_SMEM, s, "k_split_multi");
+        launch_jobs(jobs, rblocks, k_split_reduce_multi, 192, 0, s, "k_split_reduce_multi");
     }
     // L2L: pass k takes each geometry's children at level l0 + 1 + k
     for (int k = 0; k < max_dn; ++k) {
@@ -1027,17 +1279,15 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
     }
 }
 
-// Schedule of the M2L work items chosen by measurement on this geometry: the cap
-// on the work of one item (entries x output coefficients; heavier (box, chunk)s
-// are split and their parts reduced) and whether an unsplit box with a narrow
-// coefficient row gets one item for all of its coefficients.  Each candidate's
-// FP64 M2L (items plus reductions) runs twice untimed and three times timed with
-// CUDA events on the calling thread's stream, on zeroed expansions (the time of
-// the FP64 pipe does not depend on the values), and the fastest is kept.  The
-// schedule changes only the order in which the parts of a split sum are added.
+// Schedule of the M2L chosen by measurement on this geometry: the cap on the work of one
+// unit of the FP64 M2L (item_work / 64 box pairs, at most SP_COLS of them) and of one item
+// of the precision form's.  Each candidate's FP64 M2L runs twice untimed and three times
+// timed with CUDA events on the calling thread's stream, on zeroed expansions (the time
+// does not depend on the values), and the fastest is kept.  The FP64 results do not depend
+// on the schedule; the precision form's differ in the order in which parts are added.
 void fmm_autotune(lfmm_geometry_s* g) {
     TreeHost& t = g->tree;
-    if (t.l0 > t.D || g->n_m2l_items == 0) return;
+    if (t.l0 > t.D || g->sp_tabs_host.empty()) return;
     set_smem_limits();
     cudaStream_t s = cudaStreamPerThread;
     ensure_coef(g, 1);
@@ -1047,28 +1297,25 @@ void fmm_autotune(lfmm_geometry_s* g) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cuda_check(cudaEventCreate(&e0), "event");
     cuda_check(cudaEventCreate(&e1), "event");
-    const int works[] = {1024, 2048, 4096, 8192};
-    int best_work = g->m2l_item_work, best_wide = g->m2l_wide;
+    int best_work = M2L_ITEM_WORK;
     double best = 1e300, dflt = 0.0;
-    for (int wide = 1; wide >= 0; --wide) {
-        for (int work : works) {
-            make_m2l_items(g, work, wide);
-            const int n64 = g->n_m2l_items, r64 = g->m2l_red_level_start[t.D + 2];
-            for (int r = 0; r < 2; ++r) launch_m2l64(g, 1, n64, r64, s);
-            cuda_check(cudaEventRecord(e0, s), "event");
-            for (int r = 0; r < 3; ++r) launch_m2l64(g, 1, n64, r64, s);
-            cuda_check(cudaEventRecord(e1, s), "event");
-            cuda_check(cudaEventSynchronize(e1), "tune sync");
-            float ms = 0.f;
-            cuda_check(cudaEventElapsedTime(&ms, e0, e1), "event");
-            const double per = ms / 3.0;
-            if (work == M2L_ITEM_WORK && wide == 1) dflt = per;
-            if (per < best) { best = per; best_work = work; best_wide = wide; }
-        }
+    for (int work : {1024, M2L_ITEM_WORK}) {   // 16 and 32 pairs
+        make_split_units(g, std::min(SP_COLS, work / 64));
+        for (int r = 0; r < 2; ++r) launch_split(g, 1, t.D + 1, s);
+        cuda_check(cudaEventRecord(e0, s), "event");
+        for (int r = 0; r < 3; ++r) launch_split(g, 1, t.D + 1, s);
+        cuda_check(cudaEventRecord(e1, s), "event");
+        cuda_check(cudaEventSynchronize(e1), "tune sync");
+        float ms = 0.f;
+        cuda_check(cudaEventElapsedTime(&ms, e0, e1), "event");
+        const double per = ms / 3.0;
+        if (work == M2L_ITEM_WORK) dflt = per;
+        if (per < best) { best = per; best_work = work; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    make_m2l_items(g, best_work, best_wide);
+    make_split_units(g, std::min(SP_COLS, best_work / 64));
+    make_m2l_items(g, best_work, 1);
     cuda_check(cudaStreamSynchronize(s), "tune");
     g->n_launches = launches;
     g->tune_ms_default = dflt;

@@ -150,113 +150,14 @@ __global__ void __launch_bounds__(128) k_basis(const ExpGroup* __restrict__ grou
     }
 }
 
-// M2L into the target boxes of levels >= l0 (free space and reaction components).
-// A CTA of 128 threads takes one work item: W output lanes (W = XT_W, or every
-// coefficient, see lane_width) x 128 / W slices of the sum over the source
-// index, over the item's range of list entries, whose descriptors are staged in
-// shared memory 64 at a time; the slices are reduced
-// in a fixed order at the end.  Free space (Graf): L_n += sum_m M_m T[m - n]
-// (Toeplitz vector per table).  Reaction (eq. generalintegral): beta_m =
-// sum_n I[m][n] alpha_n with the arrival and departure index flips; moment
-// tables are column-major (entry (m, n) at n (2p+1) + m).
-#define M2L_STAGE 64
-
-__device__ __forceinline__ void m2l_item(int ii, const M2LItem* __restrict__ items, const M2LEnt* __restrict__ ents,
-                      const int* __restrict__ box_level, const int* __restrict__ p_level,
-                      const int64_t* __restrict__ coef_off, const int* __restrict__ slot_of,
-                      const int64_t* __restrict__ slot_coef, const cd* __restrict__ m2lf,
-                      const int64_t* __restrict__ m2lf_off, const cd* __restrict__ m2lr, int nrhs, int64_t ncoef,
-                      int64_t nslotcoef, int nparts, const cd* __restrict__ Min, const cd* __restrict__ Mp,
-                      cd* __restrict__ Lout, cd* __restrict__ Lp, cd* __restrict__ part) {
-    __shared__ cd red[3 * 128];
-    __shared__ M2LEnt se[M2L_STAGE];
-    const M2LItem it = items[ii];
-    const int T = it.box;
-    const int p = p_level[box_level[T]];
-    const int nco = 2 * p + 1;
-    const int W = it.w, NS = 128 / W;
-    const int lane = threadIdx.x % W, sl = threadIdx.x / W;
-    const int idx = it.chunk * W + lane;
-    const bool live = sl < NS && idx < nco;
-    const int nn = idx - p;
-    for (int col = 0; col < nrhs; ++col) {
-        const cd* Mc = Min + (int64_t)col * ncoef;
-        const cd* Mpc = Mp + (int64_t)col * nslotcoef;
-        cd acc0 = mk(0, 0), acc1 = mk(0, 0), acc2 = mk(0, 0);   // L, side-0 / side-1 reaction centre
-        for (int eb = it.e0; eb < it.e1; eb += M2L_STAGE) {
-            const int cnt = min(M2L_STAGE, it.e1 - eb);
-            __syncthreads();
-            if (threadIdx.x < cnt) se[threadIdx.x] = ents[eb + threadIdx.x];
-            __syncthreads();
-            if (!live) continue;
-            for (int q = 0; q < cnt; ++q) {
-                const M2LEnt E = se[q];
-                if (!(E.flags & M2L_REACT)) {
-                    const cd* src = Mc + E.src;
-                    const cd* tb = m2lf + m2lf_off[E.tab] + p - nn;   // T[m - n] at (mi - p) - nn + 2p
-                    for (int mi = sl; mi < nco; mi += NS) cfma(acc0, src[mi], tb[mi]);
-                } else {
-                    const cd* src = ((E.flags & M2L_SRC_SLOT) ? Mpc : Mc) + E.src;
-                    const bool bdown = (E.flags & M2L_B_DOWN) != 0;
-                    // departure down: L_n += beta_n;  departure up: L_{-n} += (-1)^n beta_n
-                    const int mrow = bdown ? nn : -nn;
-                    // column of row mrow; a mirrored table is read at (-mrow, -n)
-                    const bool flip = (E.flags & M2L_FLIP) != 0;
-                    const cd* col_m = m2lr + E.tab + (flip ? (p - mrow) + (int64_t)2 * p * nco : (mrow + p));
-                    const int64_t cs = flip ? -(int64_t)nco : (int64_t)nco;
-                    cd bsum = mk(0, 0);
-                    if (E.flags & M2L_A_DOWN) {   // alpha_i = M_i
-                        for (int mi = sl; mi < nco; mi += NS) cfma(bsum, col_m[mi * cs], src[mi]);
-                    } else {                      // alpha_i = (-1)^(i-p) M_{2p-i}
-                        for (int mi = sl; mi < nco; mi += NS) cfma(bsum, col_m[mi * cs], csign(src[2 * p - mi], mi - p));
-                    }
-                    bsum = csign(bsum, (!bdown) & mrow);
-                    const int dst = (E.flags >> M2L_DST_SHIFT) & 3;
-                    if (dst == 0) acc0 += bsum;
-                    else if (dst == 1) acc1 += bsum;
-                    else acc2 += bsum;
-                }
-            }
-        }
-        if (sl < NS) {
-            red[(0 * NS + sl) * W + lane] = acc0;
-            red[(1 * NS + sl) * W + lane] = acc1;
-            red[(2 * NS + sl) * W + lane] = acc2;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < 3 * W; i += blockDim.x) {
-            const int k = i / W, ln = i - k * W, ix = it.chunk * W + ln;
-            if (ix >= nco) continue;
-            cd t = red[(k * NS) * W + ln];
-            for (int q = 1; q < NS; ++q) t += red[(k * NS + q) * W + ln];
-            if (it.part >= 0) {   // split items are always XT_W lanes wide
-                part[(((int64_t)col * nparts + it.part) * 3 + k) * XT_W + ln] = t;
-            } else {
-                const int ts = (k == 0) ? -1 : slot_of[2 * T + k - 1];
-                if (k == 0) Lout[(int64_t)col * ncoef + coef_off[T] + ix] = t;
-                else if (ts >= 0) Lp[(int64_t)col * nslotcoef + slot_coef[ts] + ix] = t;
-            }
-        }
-        __syncthreads();
-    }
-}
-__global__ void __launch_bounds__(128) k_m2l(const M2LItem* __restrict__ items, const M2LEnt* __restrict__ ents,
-                      const int* __restrict__ box_level, const int* __restrict__ p_level,
-                      const int64_t* __restrict__ coef_off, const int* __restrict__ slot_of,
-                      const int64_t* __restrict__ slot_coef, const cd* __restrict__ m2lf,
-                      const int64_t* __restrict__ m2lf_off, const cd* __restrict__ m2lr, int nrhs, int64_t ncoef,
-                      int64_t nslotcoef, int nparts, const cd* __restrict__ Min, const cd* __restrict__ Mp,
-                      cd* __restrict__ Lout, cd* __restrict__ Lp, cd* __restrict__ part) {
-    m2l_item(blockIdx.x, items, ents, box_level, p_level, coef_off, slot_of, slot_coef, m2lf, m2lf_off, m2lr, nrhs,
-             ncoef, nslotcoef, nparts, Min, Mp, Lout, Lp, part);
-}
-// Sum the partial results of split (box, chunk)s in part order and write them.
-__device__ __forceinline__ void m2l_reduce_one(int ri, const M2LReduce* __restrict__ reds,
+// Sum the partial results of split (box, chunk)s in part order and write them (the
+// precision form's double-float M2L).
+__global__ void __launch_bounds__(64) k_m2l_reduce(const M2LReduce* __restrict__ reds,
                       const int* __restrict__ box_level, const int* __restrict__ p_level,
                       const int64_t* __restrict__ coef_off, const int* __restrict__ slot_of,
                       const int64_t* __restrict__ slot_coef, int nrhs, int64_t ncoef, int64_t nslotcoef, int nparts,
                       const cd* __restrict__ part, cd* __restrict__ Lout, cd* __restrict__ Lp) {
-    const M2LReduce r = reds[ri];
+    const M2LReduce r = reds[blockIdx.x];
     const int p = p_level[box_level[r.box]];
     const int lane = threadIdx.x % XT_W, k = threadIdx.x / XT_W;   // k < 4; 3 used
     const int idx = r.chunk * XT_W + lane;
@@ -270,15 +171,6 @@ __device__ __forceinline__ void m2l_reduce_one(int ri, const M2LReduce* __restri
         else Lp[(int64_t)col * nslotcoef + slot_coef[ts] + idx] = t;
     }
 }
-__global__ void __launch_bounds__(64) k_m2l_reduce(const M2LReduce* __restrict__ reds,
-                      const int* __restrict__ box_level, const int* __restrict__ p_level,
-                      const int64_t* __restrict__ coef_off, const int* __restrict__ slot_of,
-                      const int64_t* __restrict__ slot_coef, int nrhs, int64_t ncoef, int64_t nslotcoef, int nparts,
-                      const cd* __restrict__ part, cd* __restrict__ Lout, cd* __restrict__ Lp) {
-    m2l_reduce_one(blockIdx.x, reds, box_level, p_level, coef_off, slot_of, slot_coef, nrhs, ncoef, nslotcoef, nparts,
-                   part, Lout, Lp);
-}
-
 // L2P over a list of point ranges: y_i += sum_n L_n J_n(k rho_i) e^{i n theta_i}
 // about (cx, cy).  Leaves (cell centres) and straddling leaves (reaction centres).
 __device__ __forceinline__ void l2p_group(int gi, const ExpGroup* __restrict__ groups,

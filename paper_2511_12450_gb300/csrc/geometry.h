@@ -136,6 +136,63 @@ struct M2LEnt {
 struct M2LReduce {
     int box, chunk, part0, nparts;
 };
+// FP64 M2L as split integer products (split.cuh).  A matrix: element (r, c) at
+// base + r sr + c sc of the free-space Toeplitz vectors or the reaction tables.
+struct SplitTab {
+    int64_t base;
+    int64_t out0;      // first workspace row of its pairs (doubles, one column)
+    int sr, sc;
+    int pT, pS;        // orders of the result and of the source
+    int rexp, dexp;    // offsets of its row exponents and of its source scales (by |n|)
+    int pair0, npairs;
+    int react;         // 0: Toeplitz vectors, 1: reaction tables
+    int level;
+};
+// Its pairs: the source vector enters as v_c = i^(q m) M_m with m = c - p, or p - c with
+// SP_REV, and the result leaves as L_n = i^(q n) y_n, or y_-n with SP_REV (SplitRow); the
+// symmetries of the tables (quarter turns and mirror images of a free-space offset, the
+// directions and mirror images of a reaction pair) are exact in these forms.
+enum { SP_REV = 1, SP_Q_SHIFT = 2 };
+struct SplitPair {
+    int vec;           // source vector (index of its first segment)
+    int flags;
+};
+struct SplitVec {      // one segment of a source vector
+    int64_t src;       // coefficient offset (M, or Mp with slot)
+    int p, seg, dexp, slot;
+};
+struct SplitRow {
+    int64_t row;       // the pair's workspace row (doubles, one column)
+    int flags, pad;
+};
+struct SplitUnit {     // up to SP_COLS pairs of one matrix, one row tile
+    int64_t base, out0;         // as the matrix's; out0 of the first pair
+    int sr, sc, pT, pS, rexp, dexp, react;
+    int pair0, cnt, tile;
+};
+struct SplitDst {
+    int64_t off;       // coefficient offset of the local expansion (L, or Lp with slot)
+    int p, slot;
+    int r0, r1;        // its rows
+};
+struct SplitArgs {
+    const SplitVec* vec;
+    const SplitPair* pair;
+    const SplitUnit* unit;
+    const SplitRow* row;
+    const SplitDst* dst;
+    const int *rexp, *dexp;
+    const cd *tf, *tr;            // Toeplitz vectors, reaction tables
+    const cd *M, *Mp;
+    cd *L, *Lp;
+    int64_t ncoef, nslotcoef;
+    uint32_t* vdig;               // the vectors' digits and exponents
+    int* vexp;
+    int64_t nvec;
+    double* ws;
+    int col0, ncols;              // columns of this launch
+    int* err;                     // host-mapped: a bounded wait gave up
+};
 struct MixedState;
 
 // reaction M2L table key (built on the host, evaluated on the device)
@@ -262,6 +319,26 @@ struct lfmm_geometry_s {
     std::vector<int> m2l_red_level_start;   // same for the reductions
     cd* d_m2l_part = nullptr;               // partial sums [cols][n_m2l_parts][3][XT_W]
     int m2l_part_cols = 0;
+    // FP64 M2L as split integer products: matrices, pairs, units and destinations, coarse
+    // levels first
+    std::vector<lfmm::SplitTab> sp_tabs_host;
+    lfmm::SplitTab* d_sp_tab = nullptr;
+    lfmm::SplitVec* d_sp_vec = nullptr;
+    lfmm::SplitPair* d_sp_pair = nullptr;
+    lfmm::SplitUnit* d_sp_unit = nullptr;
+    lfmm::SplitRow* d_sp_row = nullptr;
+    lfmm::SplitDst* d_sp_dst = nullptr;
+    int *d_sp_rexp = nullptr, *d_sp_dexp = nullptr;
+    std::vector<int> sp_unit_start, sp_dst_start, sp_vec_start;   // [nlev + 2]: first unit / destination / vector of each level
+    uint32_t* d_sp_vdig = nullptr;                  // digits and exponents of the vectors, sp_ws_cols columns
+    int* d_sp_vexp = nullptr;
+    int sp_nvec = 0;
+    int sp_ntab = 0;
+    int sp_max_cnt = 0;                             // largest pair count of a unit
+    int64_t sp_rows = 0;                            // workspace doubles per column
+    double* d_sp_ws = nullptr;
+    int sp_ws_cols = 0;                             // columns it holds
+    int* wait_err = nullptr;                        // pinned, written by the device: a bounded wait gave up
     std::vector<int> vf_ptr_host, vf_src_host, vf_tab_host, slot_of_host;
     std::vector<int> m2l_ent_ptr_host;      // entry range per target box
     int m2l_item_work = 0, m2l_wide = 1;    // schedule of the items (see make_m2l_items)
@@ -273,6 +350,9 @@ struct lfmm_geometry_s {
     std::vector<lfmm::ReactKey> rkeys_host;
     std::vector<int> rkey_lay_s, rkey_lay_t;       // layers of the source / target boxes of each key
     std::vector<int> ftab_lay, ftab_lev;           // layer and level of each free-space M2L table
+    std::vector<int> ftab_p;                       // order and offset of each
+    std::vector<int64_t> ftab_off_host;
+    std::vector<int> ftab_canon, ftab_turn;        // per listed offset: its first-octant table; quarter turns | mirrored << 2
     std::vector<int> slot_box_host;
     std::vector<int64_t> box_coef_off_host;
     std::vector<int64_t> slot_coef_host;
@@ -433,6 +513,8 @@ void mixed_destroy(lfmm_geometry_s* g);
 // this geometry's host copy of the status has seen (copied after every launch; current
 // once the launching stream has been synchronised).  Clears the status.
 void mixed_check_waits(lfmm_geometry_s* g);
+// the same for the FP64 form's split M2L
+void split_check_waits(lfmm_geometry_s* g);
 void fmm_free(lfmm_geometry_s* g);   // per-nrhs coefficient buffers
 // permutation helpers and the full operator (solver.cu)
 void gather_sorted(lfmm_geometry_s* g, const cd* x_in, cd* x_sorted, int nrhs, cudaStream_t s);

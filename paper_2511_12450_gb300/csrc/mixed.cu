@@ -177,9 +177,12 @@ __global__ void k_react32_tables(const cd* __restrict__ m2lr, const ReactKey* __
 }
 
 // ---------------------------------------------------------------------------
-// M2L in FP32 on the scaled expansions: the same work items, entry descriptors,
-// lane/slice split, index flips and partial-sum reduction as the FP64 kernel,
-// with dense tables for the free-space part too.
+// M2L in FP32 on the scaled expansions.  A CTA of 128 threads takes one work item: W
+// output lanes (W = XT_W, or every coefficient, see lane_width) x 128 / W slices of the sum
+// over the source index, over the item's range of list entries, whose descriptors are
+// staged in shared memory 64 at a time; the slices are reduced in a fixed order at the end.
+// Free space (Graf) and reaction (eq. generalintegral, beta_m = sum_n I[m][n] alpha_n with
+// the arrival and departure index flips) both use dense column-major tables.
 #define M2L_STAGE32 64
 // v or -v by flipping the sign bits with integer instructions (a conditional
 // negation otherwise takes a floating-point instruction in the inner loop)
@@ -796,7 +799,7 @@ __global__ void k_m_to_df(const cd* __restrict__ in, int64_t ld_in, const double
 }
 
 // M2L of the coarse levels in double-float: the work items, entry descriptors, index flips
-// and partial-sum slots of the FP64 k_m2l (fmm_kernels.cuh).  Multipoles: Ms (scaled) and Mu
+// and partial-sum slots of the FP32 k_m2l32.  Multipoles: Ms (scaled) and Mu
 // (unscaled) of the boxes from coefficient c0, Mps (scaled) of the reaction centres from s0.
 // Each thread turns its sums to unscaled FP64 before the slices are added in a fixed order;
 // the outputs (L, reaction-centre locals, or partial sums for k_m2l_reduce) are FP64.
