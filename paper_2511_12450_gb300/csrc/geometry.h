@@ -230,6 +230,7 @@ struct lfmm_geometry_s {
     std::vector<double> hx, hy, hw;   // sorted-order host copies
     std::vector<double> hnx, hny;     // sorted-order normals (combined field only)
     int nleaf = 0, leaf0 = 0;         // leaves are boxes [leaf0, leaf0 + nleaf)
+    int max_leaf = 1;                 // most points of a leaf
 
     // sorted-order point data
     double *d_x = nullptr, *d_y = nullptr, *d_w = nullptr;

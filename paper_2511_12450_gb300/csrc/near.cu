@@ -115,16 +115,12 @@ __global__ void k_near_react(MediumDev m, QuadRule q, const NearTask* __restrict
     }
 }
 
-// y_T += (near row of leaf T) x, one CTA of NW warps per target leaf.
+// y_T += (near row of leaf T) x.
 //
 // The blocks of one target leaf T are stored one after another, each column-major
 // with leading dimension nT = |T|, so together they form one column-major nT x nJ
-// matrix whose column c multiplies x at the sorted position J[c].  Warp w takes the
-// contiguous share [c0 + nJ w / NW, c0 + nJ (w + 1) / NW) of the columns, and the rows
-// in chunks of r = min(32, nT): G = 32 / r groups of r lanes each walk every G-th
-// column of its share (lanes beyond G r idle), consecutive lanes reading consecutive
-// entries of a column.  The groups' sums meet by warp shuffles, the warps' by shared
-// memory, both in a fixed order.
+// matrix whose column c multiplies x at the sorted position J[c].  Threads over the
+// (row, column) pairs as in near_leaf_rows.
 //
 // FP64 form: one matrix, the stored FP64 blocks (free space, reaction, self terms).
 // Precision form (MIX): the blocks without reaction entries in complex64 with their
@@ -188,115 +184,104 @@ __device__ __forceinline__ void near_row_sum(const V* __restrict__ val, const Ne
         acc[q].x += a2[q].x; acc[q].y += a2[q].y;
     }
 }
-template <int NW>
-__device__ __forceinline__ void share(const NearRowPart& P, int leaf, int w, int* ca, int* cb) {
-    const int c0 = P.jptr[leaf], nj = P.jptr[leaf + 1] - c0;
-    *ca = c0 + (int)(((int64_t)nj * w) / NW);
-    *cb = c0 + (int)(((int64_t)nj * (w + 1)) / NW);
-}
-
-// NW warps per leaf.  With few leaves (fewer than two waves of single-warp leaves) several
-// warps share a leaf so that enough loads are in flight: 2 in the FP64 form (bound by the
-// FP64 pipe; fewer warps per leaf keep the fixed cost of the reductions small against the
-// FMAs), 4 in the precision form (bound by memory).  With many leaves one warp per leaf
-// keeps four times as many leaves in flight per SM and needs no barrier.  In the precision
-// form the FP32 part is reduced in FP32 and converted once per row, and the FP64 part is
-// skipped for the leaves without reaction columns.
-template <bool MIX, int NW, int CB>
-__device__ __forceinline__ void near_leaf_cta(int leaf, int leaf0, const int* __restrict__ box_begin,
-                                              const int* __restrict__ box_end, const NearRowPart& P64,
-                                              const cd* __restrict__ val64, const NearRowPart& P32,
-                                              const float2* __restrict__ val32, const cd* __restrict__ diag,
-                                              const cd* __restrict__ x, const float2* __restrict__ x32,
-                                              cd* __restrict__ y, int64_t n, int nrhs) {
-    __shared__ cd part[NW][32];
-    __shared__ float2 part32[MIX ? NW : 1][32];
-    const int w = NW == 1 ? 0 : (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+// The stored rows of one leaf for CB right-hand sides (columns col0..), by T threads: up to
+// NEAR_ROWS rows [i0, i0 + r) at a time, G = T / r threads per row, each over every G-th
+// column of the leaf's matrix; consecutive threads read consecutive entries.  A row's G
+// partial sums meet in shared memory (T > 32) or by shuffles (one warp) in a fixed order.
+// Flattening (row, column) over 4 or 8 warps instead of giving each of 2 warps a share of the
+// columns keeps more lanes on an entry (14 rows: 126 of 128, before 28 of 32; 23 rows: 115 of
+// 128, before 23 of 32) and shortens the chain of a large leaf.  Before -> after, alone: 12
+// leaves of up to 46 x 128 entries 60 -> 20 us, 367 leaves (838k entries) 112 -> 33 us, 524
+// leaves x 5 columns 217 -> 104 us, 4,895 leaves (4.0M entries) 78 -> 71 us.
+// In the precision form the FP32 part is reduced in FP32 and converted once per row, and the
+// FP64 part is skipped for the leaves without reaction columns.
+#define NEAR_ROWS 64
+template <bool MIX, int T, int CB>
+__device__ __forceinline__ void near_leaf_rows(int leaf, int i0, int col0, int leaf0, const int* __restrict__ box_begin,
+                                               const int* __restrict__ box_end, const NearRowPart& P64,
+                                               const cd* __restrict__ val64, const NearRowPart& P32,
+                                               const float2* __restrict__ val32, const cd* __restrict__ diag,
+                                               const cd* __restrict__ x, const float2* __restrict__ x32,
+                                               cd* __restrict__ y, int64_t n, int nrhs) {
+    constexpr int ROWS = T < NEAR_ROWS ? T : NEAR_ROWS;
+    __shared__ cd part[CB][T == 32 ? 1 : T];
+    __shared__ float2 part32[MIX ? CB : 1][T == 32 ? 1 : T];
+    const int tid = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
     const int tb = box_begin[leaf0 + leaf], nT = box_end[leaf0 + leaf] - tb;
-    const bool has64 = !MIX || P64.jptr[leaf + 1] > P64.jptr[leaf];   // the same for the whole CTA
-    int a64, b64, a32 = 0, b32 = 0;
-    share<NW>(P64, leaf, w, &a64, &b64);
-    if (MIX) share<NW>(P32, leaf, w, &a32, &b32);
-    for (int col0 = 0; col0 < nrhs; col0 += CB) {   // CB right-hand sides per pass over the entries
-        const int ncb = min(CB, nrhs - col0);
-        for (int i0 = 0; i0 < nT; i0 += 32) {
-            const int r = min(32, nT - i0), G = 32 / r;
-            const int i = i0 + lane % r, g = lane / r;
-            cd acc[CB];
-            float2 s32[CB];
+    if (i0 >= nT) return;   // the same for the whole group of threads
+    const bool has64 = !MIX || P64.jptr[leaf + 1] > P64.jptr[leaf];
+    const int ncb = min(CB, nrhs - col0);
+    const int r = min(ROWS, nT - i0), G = T / r;
+    const int g = tid / r, i = i0 + tid - g * r;
+    cd acc[CB];
+    float2 s32[CB];
 #pragma unroll
-            for (int q = 0; q < CB; ++q) { acc[q] = mk(0.0, 0.0); s32[q] = make_float2(0.f, 0.f); }
-            if (g < G) {
-                if (has64) near_row_sum<CB>(val64, P64, leaf, nT, i, g, G, a64, b64, x + (int64_t)col0 * n, n, ncb, acc);
-                if (MIX)
-                    near_row_sum<CB>(val32, P32, leaf, nT, i, g, G, a32, b32, x32 + (int64_t)col0 * n, n, ncb, s32);
-            }
-#pragma unroll
-            for (int q = 0; q < CB; ++q) {
-                if (q >= ncb) break;
-                const int col = col0 + q;
-                const cd* xc = x + (int64_t)col * n;
-                for (int gg = 1; gg < G; ++gg) {
-                    const int src = (lane + gg * r) & 31;
-                    if (has64) {
-                        const double ox = __shfl_sync(0xffffffffu, acc[q].x, src);
-                        const double oy = __shfl_sync(0xffffffffu, acc[q].y, src);
-                        if (lane < r) { acc[q].x += ox; acc[q].y += oy; }
-                    }
-                    if (MIX) {
-                        const float ox = __shfl_sync(0xffffffffu, s32[q].x, src);
-                        const float oy = __shfl_sync(0xffffffffu, s32[q].y, src);
-                        if (lane < r) { s32[q].x += ox; s32[q].y += oy; }
-                    }
-                }
-                if (NW == 1) {   // one warp per leaf: no exchange between warps
-                    if (lane < r) {
-                        cd t = has64 ? acc[q] : mk(0.0, 0.0);
-                        if (MIX) {
-                            t.x += (double)s32[q].x;
-                            t.y += (double)s32[q].y;
-                            cfma(t, diag[tb + i], xc[tb + i]);
-                        }
-                        y[(int64_t)col * n + tb + i] += t;
-                    }
-                    continue;
-                }
-                if (lane < r) {
-                    if (has64) part[w][lane] = acc[q];
-                    if (MIX) part32[w][lane] = s32[q];
-                }
-                __syncthreads();
-                if (w == 0 && lane < r) {
-                    cd t = mk(0.0, 0.0);
-                    if (has64) {
-                        t = part[0][lane];
-                        for (int k = 1; k < NW; ++k) t += part[k][lane];
-                    }
-                    if (MIX) {
-                        float2 u = part32[0][lane];
-                        for (int k = 1; k < NW; ++k) { u.x += part32[k][lane].x; u.y += part32[k][lane].y; }
-                        t.x += (double)u.x;
-                        t.y += (double)u.y;
-                        cfma(t, diag[tb + i], xc[tb + i]);
-                    }
-                    y[(int64_t)col * n + tb + i] += t;
-                }
-                __syncthreads();
-            }
+    for (int q = 0; q < CB; ++q) { acc[q] = mk(0.0, 0.0); s32[q] = make_float2(0.f, 0.f); }
+    if (g < G) {
+        if (has64)
+            near_row_sum<CB>(val64, P64, leaf, nT, i, g, G, P64.jptr[leaf], P64.jptr[leaf + 1], x + (int64_t)col0 * n, n, ncb, acc);
+        if (MIX)
+            near_row_sum<CB>(val32, P32, leaf, nT, i, g, G, P32.jptr[leaf], P32.jptr[leaf + 1], x32 + (int64_t)col0 * n, n, ncb,
+                             s32);
+    }
+    auto finish = [&](int q, int row, cd t, float2 u) {   // one row of one column
+        const int col = col0 + q;
+        if (MIX) {
+            t.x += (double)u.x;
+            t.y += (double)u.y;
+            cfma(t, diag[tb + row], x[(int64_t)col * n + tb + row]);
         }
+        y[(int64_t)col * n + tb + row] += t;
+    };
+    if (T == 32) {
+#pragma unroll
+        for (int q = 0; q < CB; ++q) {
+            if (q >= ncb) break;
+            for (int gg = 1; gg < G; ++gg) {
+                const int src = (tid + gg * r) & 31;
+                if (has64) {
+                    const double ox = __shfl_sync(0xffffffffu, acc[q].x, src);
+                    const double oy = __shfl_sync(0xffffffffu, acc[q].y, src);
+                    if (tid < r) { acc[q].x += ox; acc[q].y += oy; }
+                }
+                if (MIX) {
+                    const float ox = __shfl_sync(0xffffffffu, s32[q].x, src);
+                    const float oy = __shfl_sync(0xffffffffu, s32[q].y, src);
+                    if (tid < r) { s32[q].x += ox; s32[q].y += oy; }
+                }
+            }
+            if (tid < r) finish(q, i, acc[q], s32[q]);
+        }
+        return;
+    }
+#pragma unroll
+    for (int q = 0; q < CB; ++q) {
+        if (has64) part[q][tid] = acc[q];
+        if (MIX) part32[q][tid] = s32[q];
+    }
+    __syncthreads();
+    for (int e = tid; e < r * ncb; e += T) {
+        const int q = e / r, row = e - q * r;
+        cd t = mk(0.0, 0.0);
+        float2 u = make_float2(0.f, 0.f);
+        if (has64)
+            for (int k = 0; k < G; ++k) t += part[q][k * r + row];
+        if (MIX)
+            for (int k = 0; k < G; ++k) { u.x += part32[q][k * r + row].x; u.y += part32[q][k * r + row].y; }
+        finish(q, i0 + row, t, u);
     }
 }
-#define NEAR_WARPS_64 2
-#define NEAR_WARPS_MIX 4
-// CB: right-hand sides per pass over the stored entries (1, or 4 for a block right-hand side)
-template <bool MIX, int NW, int CB>
-__global__ void __launch_bounds__(32 * NW) k_near_leaf(int leaf0, const int* __restrict__ box_begin,
-                                                       const int* __restrict__ box_end, NearRowPart P64,
-                                                       const cd* __restrict__ val64, NearRowPart P32,
-                                                       const float2* __restrict__ val32, const cd* __restrict__ diag,
-                                                       const cd* __restrict__ x, const float2* __restrict__ x32,
-                                                       cd* __restrict__ y, int64_t n, int nrhs) {
-    near_leaf_cta<MIX, NW, CB>(blockIdx.x, leaf0, box_begin, box_end, P64, val64, P32, val32, diag, x, x32, y, n, nrhs);
+// One CTA per (leaf, group of CB right-hand sides, NEAR_ROWS rows).
+// CB: 1, or 4 for a block right-hand side (each stored entry read once per four)
+template <bool MIX, int T, int CB>
+__global__ void __launch_bounds__(T) k_near_leaf(int leaf0, const int* __restrict__ box_begin,
+                                                 const int* __restrict__ box_end, NearRowPart P64,
+                                                 const cd* __restrict__ val64, NearRowPart P32,
+                                                 const float2* __restrict__ val32, const cd* __restrict__ diag,
+                                                 const cd* __restrict__ x, const float2* __restrict__ x32,
+                                                 cd* __restrict__ y, int64_t n, int nrhs) {
+    near_leaf_rows<MIX, T, CB>(blockIdx.x, blockIdx.z * NEAR_ROWS, blockIdx.y * CB, leaf0, box_begin, box_end, P64, val64, P32,
+                               val32, diag, x, x32, y, n, nrhs);
 }
 // one warp per leaf, four warps per CTA
 template <bool MIX, int CB>
@@ -308,10 +293,38 @@ __global__ void __launch_bounds__(128) k_near_leaf_w(int nleaf, int leaf0, const
                                                      cd* __restrict__ y, int64_t n, int nrhs) {
     const int leaf = (int)(blockIdx.x * 4 + (threadIdx.x >> 5));
     if (leaf >= nleaf) return;   // whole warps: the single-warp path has no block barrier
-    near_leaf_cta<MIX, 1, CB>(leaf, leaf0, box_begin, box_end, P64, val64, P32, val32, diag, x, x32, y, n, nrhs);
+    const int nT = box_end[leaf0 + leaf] - box_begin[leaf0 + leaf];
+    for (int col0 = 0; col0 < nrhs; col0 += CB)
+        for (int i0 = 0; i0 < nT; i0 += 32)
+            near_leaf_rows<MIX, 32, CB>(leaf, i0, col0, leaf0, box_begin, box_end, P64, val64, P32, val32, diag, x, x32, y, n,
+                                        nrhs);
 }
 // leaves from which one warp per leaf fills two waves of the GPU (152 SMs x 64 warps x 2)
 #define NEAR_WARP_PER_LEAF_MIN (152 * 64 * 2)
+// leaves below which a leaf gets 8 warps instead of 4 (4 CTAs of 8 warps per SM would stay idle)
+#define NEAR_WIDE_MAX (152 * 8)
+// threads per leaf of a geometry: the same in every launch that multiplies it, so that all
+// of them add in the same order
+static int near_threads(const lfmm_geometry_s* g) {
+    return g->nleaf >= NEAR_WARP_PER_LEAF_MIN ? 32 : g->nleaf < NEAR_WIDE_MAX ? 256 : 128;
+}
+template <bool MIX, int CB>
+static void launch_near(lfmm_geometry_s* g, const NearRowPart& p64, const cd* v64, const NearRowPart& p32,
+                        const float2* v32, const cd* diag, const cd* x, const float2* x32, cd* y, int nrhs,
+                        cudaStream_t s) {
+    const int T = near_threads(g);
+    const dim3 grid(g->nleaf, (nrhs + CB - 1) / CB, (g->max_leaf + NEAR_ROWS - 1) / NEAR_ROWS);
+    if (T == 32)
+        k_near_leaf_w<MIX, CB><<<(g->nleaf + 3) / 4, 128, 0, s>>>(g->nleaf, g->leaf0, g->d_box_begin, g->d_box_end, p64, v64,
+                                                                 p32, v32, diag, x, x32, y, g->n, nrhs);
+    else if (T == 128)
+        k_near_leaf<MIX, 128, CB><<<grid, 128, 0, s>>>(g->leaf0, g->d_box_begin, g->d_box_end, p64, v64, p32, v32, diag, x,
+                                                      x32, y, g->n, nrhs);
+    else
+        k_near_leaf<MIX, 256, CB><<<grid, 256, 0, s>>>(g->leaf0, g->d_box_begin, g->d_box_end, p64, v64, p32, v32, diag, x,
+                                                      x32, y, g->n, nrhs);
+    cuda_check(cudaGetLastError(), "k_near_leaf");
+}
 // x rounded to complex64 (the precision form's FP32 near-field products)
 __global__ void k_round_x32(const cd* __restrict__ x, float2* __restrict__ x32, int64_t tot) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < tot; q += (int64_t)gridDim.x * blockDim.x)
@@ -352,6 +365,8 @@ void near_build(lfmm_geometry_s* g) {
     const int D = t.D;
     g->leaf0 = t.level_start[D];
     g->nleaf = t.level_start[D + 1] - g->leaf0;
+    g->max_leaf = 1;
+    for (int T = g->leaf0; T < g->leaf0 + g->nleaf; ++T) g->max_leaf = std::max(g->max_leaf, t.box_end[T] - t.box_begin[T]);
     // blocks per target leaf: union of free-space and reaction near lists
     std::vector<int> blk_tgt, blk_src, nb_ptr(g->nleaf + 1, 0);
     std::vector<unsigned char> blk_free, blk_react;
@@ -497,10 +512,10 @@ static void near_mixed_build(lfmm_geometry_s* g) {
     g->near32_ready = true;
 }
 
-// Several geometries' FP64 near fields in one launch: four leaves (warps) per CTA, the CTAs
-// of each geometry consecutive; a CTA finds its geometry by binary search over the prefix.
+// Several geometries' FP64 near fields in shared launches, one per number of threads per
+// leaf; a CTA finds its geometry by binary search over the prefix of their CTA counts.
 struct NearJob {
-    int nleaf, leaf0;
+    int nleaf, leaf0, groups;   // column groups
     const int *box_begin, *box_end;
     NearRowPart P64;
     const cd* val64;
@@ -509,9 +524,9 @@ struct NearJob {
     int64_t n;
     int nrhs;
 };
-template <int CB>
-__global__ void __launch_bounds__(32 * NEAR_WARPS_64) k_near_leaf_multi(const NearJob* __restrict__ jobs,
-                                                                     const int* __restrict__ prefix, int njobs) {
+template <int T, int CB>
+__global__ void __launch_bounds__(T) k_near_leaf_multi(const NearJob* __restrict__ jobs, const int* __restrict__ prefix,
+                                                       int njobs) {
     int lo = 0, hi = njobs - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -519,49 +534,47 @@ __global__ void __launch_bounds__(32 * NEAR_WARPS_64) k_near_leaf_multi(const Ne
         else hi = mid - 1;
     }
     const NearJob& J = jobs[lo];
-    near_leaf_cta<false, NEAR_WARPS_64, CB>((int)blockIdx.x - prefix[lo], J.leaf0, J.box_begin, J.box_end, J.P64, J.val64, J.P64,
-                         nullptr, nullptr, J.x, nullptr, J.y, J.n, J.nrhs);
+    const int b = (int)blockIdx.x - prefix[lo], leaf = b % J.nleaf, rest = b / J.nleaf;
+    near_leaf_rows<false, T, CB>(leaf, (rest / J.groups) * NEAR_ROWS, (rest % J.groups) * CB, J.leaf0, J.box_begin, J.box_end,
+                                 J.P64, J.val64, J.P64, nullptr, nullptr, J.x, nullptr, J.y, J.n, J.nrhs);
 }
 
 void near_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s) {
-    std::vector<NearJob> jobs;
-    std::vector<int> prefix(1, 0);
-    for (const BatchOp& op : ops) {
-        lfmm_geometry_s* g = op.g;
-        if (g->nleaf >= NEAR_WARP_PER_LEAF_MIN) {   // as near_apply: its own warp-per-leaf launch (same sums)
-            const NearRowPart p64{g->d_nl_off, g->d_nl_jptr, g->d_nl_j};
-            if (op.nrhs > 1)
-                k_near_leaf_w<false, 4><<<(g->nleaf + 3) / 4, 128, 0, s>>>(g->nleaf, g->leaf0, g->d_box_begin,
-                                                                       g->d_box_end, p64, g->d_nb_val, p64, nullptr,
-                                                                       nullptr, op.x, nullptr, op.y, g->n, op.nrhs);
-            else
-                k_near_leaf_w<false, 1><<<(g->nleaf + 3) / 4, 128, 0, s>>>(g->nleaf, g->leaf0, g->d_box_begin,
-                                                                       g->d_box_end, p64, g->d_nb_val, p64, nullptr,
-                                                                       nullptr, op.x, nullptr, op.y, g->n, op.nrhs);
-            cuda_check(cudaGetLastError(), "k_near_leaf_w");
-            continue;
-        }
-        jobs.push_back(NearJob{g->nleaf, g->leaf0, g->d_box_begin, g->d_box_end,
-                               NearRowPart{g->d_nl_off, g->d_nl_jptr, g->d_nl_j}, g->d_nb_val, op.x, op.y, g->n,
-                               op.nrhs});
-        prefix.push_back(prefix.back() + g->nleaf);
-    }
-    if (prefix.back() == 0) return;
-    JobTables t;
-    const size_t oj = t.add(jobs.data(), sizeof(NearJob) * jobs.size());
-    const size_t op = t.add(prefix.data(), sizeof(int) * prefix.size());
-    t.upload(s);
     int maxr = 1;
-    for (const NearJob& J : jobs) maxr = std::max(maxr, J.nrhs);
-    if (maxr > 1)
-        k_near_leaf_multi<4><<<prefix.back(), 32 * NEAR_WARPS_64, 0, s>>>(t.at<NearJob>(oj), t.at<int>(op),
-                                                                          (int)jobs.size());
-    else
-        k_near_leaf_multi<1><<<prefix.back(), 32 * NEAR_WARPS_64, 0, s>>>(t.at<NearJob>(oj), t.at<int>(op),
-                                                                          (int)jobs.size());
-    cudaError_t e = cudaGetLastError();
-    t.release(s);
-    cuda_check(e, "k_near_leaf_multi");
+    for (const BatchOp& op : ops) maxr = std::max(maxr, op.nrhs);
+    for (int T : {128, 256}) {
+        std::vector<NearJob> jobs;
+        std::vector<int> prefix(1, 0);
+        for (const BatchOp& op : ops) {
+            lfmm_geometry_s* g = op.g;
+            if (g->nleaf == 0 || near_threads(g) != T) continue;
+            const int groups = maxr > 1 ? (op.nrhs + 3) / 4 : 1;
+            jobs.push_back(NearJob{g->nleaf, g->leaf0, groups, g->d_box_begin, g->d_box_end,
+                                   NearRowPart{g->d_nl_off, g->d_nl_jptr, g->d_nl_j}, g->d_nb_val, op.x, op.y, g->n, op.nrhs});
+            prefix.push_back(prefix.back() + g->nleaf * groups * ((g->max_leaf + NEAR_ROWS - 1) / NEAR_ROWS));
+        }
+        if (jobs.empty()) continue;
+        JobTables t;
+        const size_t oj = t.add(jobs.data(), sizeof(NearJob) * jobs.size());
+        const size_t op = t.add(prefix.data(), sizeof(int) * prefix.size());
+        t.upload(s);
+        const NearJob* dj = t.at<NearJob>(oj);
+        const int *dp = t.at<int>(op), nj = (int)jobs.size();
+        if (T == 128 && maxr > 1) k_near_leaf_multi<128, 4><<<prefix.back(), T, 0, s>>>(dj, dp, nj);
+        else if (T == 128) k_near_leaf_multi<128, 1><<<prefix.back(), T, 0, s>>>(dj, dp, nj);
+        else if (maxr > 1) k_near_leaf_multi<256, 4><<<prefix.back(), T, 0, s>>>(dj, dp, nj);
+        else k_near_leaf_multi<256, 1><<<prefix.back(), T, 0, s>>>(dj, dp, nj);
+        cudaError_t e = cudaGetLastError();
+        t.release(s);
+        cuda_check(e, "k_near_leaf_multi");
+    }
+    for (const BatchOp& op : ops) {   // geometries with one warp per leaf: their own launches
+        lfmm_geometry_s* g = op.g;
+        if (g->nleaf == 0 || near_threads(g) != 32) continue;
+        const NearRowPart p64{g->d_nl_off, g->d_nl_jptr, g->d_nl_j};
+        if (op.nrhs > 1) launch_near<false, 4>(g, p64, g->d_nb_val, p64, nullptr, nullptr, op.x, nullptr, op.y, op.nrhs, s);
+        else launch_near<false, 1>(g, p64, g->d_nb_val, p64, nullptr, nullptr, op.x, nullptr, op.y, 1, s);
+    }
 }
 
 void near_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s, bool mixed) {
@@ -581,50 +594,15 @@ void near_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, 
         ++g->n_launches;
         const NearRowPart p64{g->d_nl_off64r, g->d_nl_jptr64r, g->d_nl_j64r};
         const NearRowPart p32{g->d_nl_off32, g->d_nl_jptr32, g->d_nl_j32};
-        if (g->nleaf >= NEAR_WARP_PER_LEAF_MIN) {
-            if (nrhs > 1)
-                k_near_leaf_w<true, 4><<<(g->nleaf + 3) / 4, 128, 0, s>>>(g->nleaf, g->leaf0, g->d_box_begin,
-                                                                       g->d_box_end, p64, g->d_nv64r, p32, g->d_nv32,
-                                                                       g->d_ndiag, x_sorted, g->d_near_x32, y_sorted,
-                                                                       g->n, nrhs);
-            else
-                k_near_leaf_w<true, 1><<<(g->nleaf + 3) / 4, 128, 0, s>>>(g->nleaf, g->leaf0, g->d_box_begin,
-                                                                       g->d_box_end, p64, g->d_nv64r, p32, g->d_nv32,
-                                                                       g->d_ndiag, x_sorted, g->d_near_x32, y_sorted,
-                                                                       g->n, nrhs);
-        } else if (nrhs > 1) {
-            k_near_leaf<true, NEAR_WARPS_MIX, 4><<<g->nleaf, 32 * NEAR_WARPS_MIX, 0, s>>>(
-                g->leaf0, g->d_box_begin, g->d_box_end, p64, g->d_nv64r, p32, g->d_nv32, g->d_ndiag, x_sorted,
-                g->d_near_x32, y_sorted, g->n, nrhs);
-        } else {
-            k_near_leaf<true, NEAR_WARPS_MIX, 1><<<g->nleaf, 32 * NEAR_WARPS_MIX, 0, s>>>(
-                g->leaf0, g->d_box_begin, g->d_box_end, p64, g->d_nv64r, p32, g->d_nv32, g->d_ndiag, x_sorted,
-                g->d_near_x32, y_sorted, g->n, nrhs);
-        }
+        if (nrhs > 1)
+            launch_near<true, 4>(g, p64, g->d_nv64r, p32, g->d_nv32, g->d_ndiag, x_sorted, g->d_near_x32, y_sorted, nrhs, s);
+        else
+            launch_near<true, 1>(g, p64, g->d_nv64r, p32, g->d_nv32, g->d_ndiag, x_sorted, g->d_near_x32, y_sorted, nrhs, s);
     } else {
         const NearRowPart p64{g->d_nl_off, g->d_nl_jptr, g->d_nl_j};
-        if (g->nleaf >= NEAR_WARP_PER_LEAF_MIN) {
-            if (nrhs > 1)
-                k_near_leaf_w<false, 4><<<(g->nleaf + 3) / 4, 128, 0, s>>>(g->nleaf, g->leaf0, g->d_box_begin,
-                                                                        g->d_box_end, p64, g->d_nb_val, p64, nullptr,
-                                                                        nullptr, x_sorted, nullptr, y_sorted, g->n,
-                                                                        nrhs);
-            else
-                k_near_leaf_w<false, 1><<<(g->nleaf + 3) / 4, 128, 0, s>>>(g->nleaf, g->leaf0, g->d_box_begin,
-                                                                        g->d_box_end, p64, g->d_nb_val, p64, nullptr,
-                                                                        nullptr, x_sorted, nullptr, y_sorted, g->n,
-                                                                        nrhs);
-        } else if (nrhs > 1) {
-            k_near_leaf<false, NEAR_WARPS_64, 4><<<g->nleaf, 32 * NEAR_WARPS_64, 0, s>>>(
-                g->leaf0, g->d_box_begin, g->d_box_end, p64, g->d_nb_val, p64, nullptr, nullptr, x_sorted, nullptr,
-                y_sorted, g->n, nrhs);
-        } else {
-            k_near_leaf<false, NEAR_WARPS_64, 1><<<g->nleaf, 32 * NEAR_WARPS_64, 0, s>>>(
-                g->leaf0, g->d_box_begin, g->d_box_end, p64, g->d_nb_val, p64, nullptr, nullptr, x_sorted, nullptr,
-                y_sorted, g->n, nrhs);
-        }
+        if (nrhs > 1) launch_near<false, 4>(g, p64, g->d_nb_val, p64, nullptr, nullptr, x_sorted, nullptr, y_sorted, nrhs, s);
+        else launch_near<false, 1>(g, p64, g->d_nb_val, p64, nullptr, nullptr, x_sorted, nullptr, y_sorted, nrhs, s);
     }
-    cuda_check(cudaGetLastError(), "k_near_leaf");
     ++g->n_launches;
     prof_end(g, ST_NEAR, s);
 }
