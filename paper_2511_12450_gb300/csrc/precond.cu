@@ -21,93 +21,207 @@
 
 namespace lfmm {
 
-// one CTA per leaf: assemble A = P_B^T, factor, solve A X = E_own, store W (column-major: W[b * s + i])
+// Set-up of one leaf's rows: A = P_B^T is assembled beside the identity columns of the own
+// points, [A | E] (column-major, q rows), eliminated by a blocked right-looking LU with partial
+// pivoting that carries the E columns along, and solved backwards: A X = E, W[b s + t] = X[b][t].
+// The FP64 pipe bounds it (8/3 q^3 + 8 q^2 s flops a leaf), and leaves are uneven: one of 229
+// points holds 57 MFLOP, 7 ms on one SM, where the 367 leaves of an 8,199-point geometry
+// average 5.  So a cluster of CTAs shares a leaf: blocks of nb columns go round the CTAs; the
+// owner of a block factors it in shared memory once its own updates have reached it, one
+// cluster barrier hands the block over, and every CTA updates its own columns.  The E columns
+// need no exchange backwards.  8,199 points: 5.6 ms; one CTA a leaf with column-by-column
+// elimination in global memory took 19.3 ms.
+#define PC_NB 16
+struct PcLeaf {
+    int leaf, q, s;          // leaf, points of the neighbourhood, own points
+    int64_t aoff;            // (q + s) q scratch values
+};
+__device__ __forceinline__ void pc_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ double pc_abs2(cd v) { return v.x * v.x + v.y * v.y; }
+
 __global__ void __launch_bounds__(256) k_pc_setup(MediumDev m, const int* __restrict__ pc_ptr,
                                                   const int* __restrict__ pc_idx, const int* __restrict__ own_pos,
-                                                  const int* __restrict__ own_cnt, const int64_t* __restrict__ aoff,
+                                                  const PcLeaf* __restrict__ leaves, int cs, int nb,
                                                   const int64_t* __restrict__ woff, const int* __restrict__ layer_of_leaf,
                                                   const double* __restrict__ px, const double* __restrict__ py,
                                                   const double* __restrict__ pw, const double* __restrict__ nx,
-                                                  const double* __restrict__ ny, cd* __restrict__ Ascr,
-                                                  int* __restrict__ pivscr, cd* __restrict__ W) {
-    const int B = blockIdx.x;
-    const int jb = pc_ptr[B], q = pc_ptr[B + 1] - jb;
-    const int s = own_cnt[B], o0 = own_pos[B];
+                                                  const double* __restrict__ ny, cd* Ascr, int* pivscr,
+                                                  cd* __restrict__ W) {
+    extern __shared__ cd pc_sm[];          // the panel [nb][q]
+    __shared__ cd U[PC_NB][PC_NB];         // a block's rows of U, then of X
+    __shared__ cd D[PC_NB][PC_NB];         // diagonal block
+    __shared__ double rv[8];
+    __shared__ int ri[8];
+    __shared__ cd sinv;
+    const PcLeaf lf = leaves[blockIdx.x / cs];
+    const int rank = blockIdx.x % cs, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int B = lf.leaf, jb = pc_ptr[B], q = lf.q, s = lf.s, o0 = own_pos[B];
     const double k = m.k[layer_of_leaf[B]];
-    cd* A = Ascr + aoff[B];            // row-major q x q
+    cd* A = Ascr + lf.aoff;
     int* piv = pivscr + jb;
-    __shared__ double red_v[256];
-    __shared__ int red_i[256];
-    // A[a][b] = P[b][a]: P[i][j] = w_j G(c_j, c_i) (i != j), I^s_i (i == j)
-    for (int e = threadIdx.x; e < q * q; e += blockDim.x) {
-        int a = e / q, b = e % q;
-        int i = pc_idx[jb + b], j = pc_idx[jb + a];   // P[i=b][j=a]
-        const bool cf = nx != nullptr;
-        A[e] = (a == b) ? self_entry(k, pw[i], cf)
-                        : pw[j] * free_kernel(k, px[j] - px[i], py[j] - py[i], cf, cf ? nx[j] : 0.0, cf ? ny[j] : 0.0);
+    cd* P = pc_sm;
+    const int nA = (q + nb - 1) / nb, nR = (s + nb - 1) / nb;   // column blocks of A and of E
+    // A[a][b] = P[b][a]: P[i][j] = w_j G(c_j, c_i) (i != j), I^s_i (i == j); own columns only
+    const bool cf = nx != nullptr;
+    for (int blk = rank; blk < nA + nR; blk += cs) {
+        const bool rhs = blk >= nA;
+        const int b0 = rhs ? (blk - nA) * nb : blk * nb, w = min(nb, (rhs ? s : q) - b0);
+        for (int e = tid; e < w * q; e += 256) {
+            const int b = b0 + e / q, a = e % q;
+            if (rhs) {
+                A[(int64_t)(q + b) * q + a] = mk(a == o0 + b ? 1.0 : 0.0, 0.0);
+            } else {
+                const int i = pc_idx[jb + b], j = pc_idx[jb + a];   // P[i=b][j=a]
+                A[(int64_t)b * q + a] = (a == b) ? self_entry(k, pw[i], cf)
+                                                 : pw[j] * free_kernel(k, px[j] - px[i], py[j] - py[i], cf,
+                                                                       cf ? nx[j] : 0.0, cf ? ny[j] : 0.0);
+            }
+        }
     }
     __syncthreads();
-    // LU with partial pivoting
-    for (int c = 0; c < q; ++c) {
-        double best = -1.0;
-        int bi = c;
-        for (int r = c + threadIdx.x; r < q; r += blockDim.x) {
-            double v = absc(A[(int64_t)r * q + c]);
-            if (v > best) { best = v; bi = r; }
-        }
-        red_v[threadIdx.x] = best;
-        red_i[threadIdx.x] = bi;
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o && red_v[threadIdx.x + o] > red_v[threadIdx.x]) {
-                red_v[threadIdx.x] = red_v[threadIdx.x + o];
-                red_i[threadIdx.x] = red_i[threadIdx.x + o];
+    for (int pb = 0; pb < nA; ++pb) {
+        const int c0 = pb * nb, w = min(nb, q - c0), rows = q - c0;
+        if (pb % cs == rank) {   // factor the block
+            for (int e = tid; e < w * rows; e += 256) {
+                const int j = e / rows, r = e - j * rows;
+                P[j * q + r] = A[(int64_t)(c0 + j) * q + c0 + r];
             }
             __syncthreads();
-        }
-        const int pr = red_i[0];
-        __syncthreads();
-        if (threadIdx.x == 0) piv[c] = pr;
-        if (pr != c)
-            for (int jj = threadIdx.x; jj < q; jj += blockDim.x) {
-                cd t = A[(int64_t)c * q + jj];
-                A[(int64_t)c * q + jj] = A[(int64_t)pr * q + jj];
-                A[(int64_t)pr * q + jj] = t;
+            for (int j = 0; j < w; ++j) {
+                double best = -1.0;
+                int bi = j;
+                for (int r = j + tid; r < rows; r += 256) {
+                    const double v = pc_abs2(P[j * q + r]);
+                    if (v > best) { best = v; bi = r; }
+                }
+                for (int o = 16; o > 0; o >>= 1) {
+                    const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+                    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                    if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+                }
+                if (lane == 0) { rv[warp] = best; ri[warp] = bi; }
+                __syncthreads();
+                best = rv[0];
+                bi = ri[0];
+                for (int i = 1; i < 8; ++i)
+                    if (rv[i] > best || (rv[i] == best && ri[i] < bi)) { best = rv[i]; bi = ri[i]; }
+                if (tid < w) {
+                    const cd a = P[tid * q + j], b = P[tid * q + bi];
+                    P[tid * q + j] = b;
+                    P[tid * q + bi] = a;
+                    if (tid == j) { sinv = cinv(b); piv[c0 + j] = c0 + bi; }
+                }
+                __syncthreads();
+                const cd inv = sinv;
+                for (int r = j + 1 + tid; r < rows; r += 256) {
+                    const cd l = P[j * q + r] * inv;
+                    P[j * q + r] = l;
+                    for (int c = j + 1; c < w; ++c) {
+                        cd v = P[c * q + r];
+                        cfma(v, -l, P[c * q + j]);
+                        P[c * q + r] = v;
+                    }
+                }
+                __syncthreads();
             }
-        __syncthreads();
-        const cd inv = cinv(A[(int64_t)c * q + c]);
-        for (int r = c + 1 + threadIdx.x; r < q; r += blockDim.x) A[(int64_t)r * q + c] = A[(int64_t)r * q + c] * inv;
-        __syncthreads();
-        const int rem = q - c - 1;
-        for (int e = threadIdx.x; e < rem * rem; e += blockDim.x) {
-            int r = c + 1 + e / rem, jj = c + 1 + e % rem;
-            cfma(A[(int64_t)r * q + jj], -A[(int64_t)r * q + c], A[(int64_t)c * q + jj]);
+            for (int e = tid; e < w * rows; e += 256) {
+                const int j = e / rows, r = e - j * rows;
+                A[(int64_t)(c0 + j) * q + c0 + r] = P[j * q + r];
+            }
+        }
+        pc_cluster_sync();
+        if (pb % cs != rank) {
+            for (int e = tid; e < w * rows; e += 256) {
+                const int j = e / rows, r = e - j * rows;
+                P[j * q + r] = A[(int64_t)(c0 + j) * q + c0 + r];
+            }
+        }
+        // own columns: row exchanges, U = L11^-1 of the block's rows, then the rows below
+        for (int blk = rank; blk < nA + nR; blk += cs) {
+            if (blk <= pb) continue;
+            const bool rhs = blk >= nA;
+            const int b0 = rhs ? q + (blk - nA) * nb : blk * nb, bw = min(nb, (rhs ? q + s : q) - b0);
+            __syncthreads();
+            if (tid < bw) {
+                cd* col = A + (int64_t)(b0 + tid) * q;
+                for (int j = 0; j < w; ++j) {
+                    const int pr = piv[c0 + j];
+                    if (pr != c0 + j) {
+                        const cd t = col[c0 + j];
+                        col[c0 + j] = col[pr];
+                        col[pr] = t;
+                    }
+                }
+                for (int j = 0; j < w; ++j) {
+                    cd v = col[c0 + j];
+                    for (int c = 0; c < j; ++c) cfma(v, -P[c * q + j], U[c][tid]);
+                    U[j][tid] = v;
+                    col[c0 + j] = v;
+                }
+            }
+            __syncthreads();
+            const int below = rows - w, quads = (bw + 3) >> 2;
+            for (int e = tid; e < below * quads; e += 256) {
+                const int h = e / below, r = w + (e - h * below), cc = 4 * h;
+                cd* col = A + (int64_t)(b0 + cc) * q + c0 + r;
+                cd v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = cc + i < bw ? col[(int64_t)i * q] : mk(0, 0);
+                for (int j = 0; j < w; ++j) {
+                    const cd l = -P[j * q + r];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) cfma(v[i], l, U[j][min(cc + i, bw - 1)]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (cc + i < bw) col[(int64_t)i * q] = v[i];
+            }
         }
         __syncthreads();
     }
-    // solve A X = E for the own columns; thread t handles own column t
+    pc_cluster_sync();
+    // backwards over the own E columns: X of a block of rows, then the rows above
     cd* Wb = W + woff[B];
-    for (int t = threadIdx.x; t < s; t += blockDim.x) {
-        // X column stored in W as W[b * s + t]
-        for (int b = 0; b < q; ++b) Wb[(int64_t)b * s + t] = mk(0.0, 0.0);
-        Wb[(int64_t)(o0 + t) * s + t] = mk(1.0, 0.0);
-        for (int c = 0; c < q; ++c) {   // apply row swaps
-            int pr = piv[c];
-            if (pr != c) {
-                cd tmp = Wb[(int64_t)c * s + t];
-                Wb[(int64_t)c * s + t] = Wb[(int64_t)pr * s + t];
-                Wb[(int64_t)pr * s + t] = tmp;
+    for (int blk = nA + (rank + cs - nA % cs) % cs; blk < nA + nR; blk += cs) {
+        const int t0 = (blk - nA) * nb, bw = min(nb, s - t0);
+        for (int pb = nA - 1; pb >= 0; --pb) {
+            const int c0 = pb * nb, w = min(nb, q - c0);
+            __syncthreads();
+            for (int e = tid; e < w * w; e += 256) {
+                const int j = e / w, r = e - j * w;
+                const cd v = A[(int64_t)(c0 + j) * q + c0 + r];
+                D[r][j] = r == j ? cinv(v) : v;
             }
-        }
-        for (int r = 0; r < q; ++r) {   // L y = P e (unit lower)
-            cd acc = Wb[(int64_t)r * s + t];
-            for (int c = 0; c < r; ++c) cfma(acc, -A[(int64_t)r * q + c], Wb[(int64_t)c * s + t]);
-            Wb[(int64_t)r * s + t] = acc;
-        }
-        for (int r = q - 1; r >= 0; --r) {   // U x = y
-            cd acc = Wb[(int64_t)r * s + t];
-            for (int c = r + 1; c < q; ++c) cfma(acc, -A[(int64_t)r * q + c], Wb[(int64_t)c * s + t]);
-            Wb[(int64_t)r * s + t] = cdiv(acc, A[(int64_t)r * q + r]);
+            __syncthreads();
+            if (tid < bw) {
+                const cd* col = A + (int64_t)(q + t0 + tid) * q + c0;
+                for (int j = w - 1; j >= 0; --j) {
+                    cd v = col[j];
+                    for (int c = j + 1; c < w; ++c) cfma(v, -D[j][c], U[c][tid]);
+                    v = v * D[j][j];
+                    U[j][tid] = v;
+                    Wb[(int64_t)(c0 + j) * s + t0 + tid] = v;
+                }
+            }
+            __syncthreads();
+            const int quads = (bw + 3) >> 2;
+            for (int e = tid; e < c0 * quads; e += 256) {
+                const int h = e / c0, r = e - h * c0, cc = 4 * h;
+                cd* col = A + (int64_t)(q + t0 + cc) * q + r;
+                cd v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = cc + i < bw ? col[(int64_t)i * q] : mk(0, 0);
+                for (int j = 0; j < w; ++j) {
+                    const cd u = -A[(int64_t)(c0 + j) * q + r];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) cfma(v[i], u, U[j][min(cc + i, bw - 1)]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (cc + i < bw) col[(int64_t)i * q] = v[i];
+            }
         }
     }
 }
@@ -153,7 +267,9 @@ void precond_build(lfmm_geometry_s* g) {
     TreeHost& t = g->tree;
     const int nleaf = g->nleaf;
     std::vector<int> ptr(nleaf + 1, 0), idx, own_pos(nleaf), own_cnt(nleaf), own_first(nleaf), lay(nleaf);
-    std::vector<int64_t> aoff(nleaf), woff(nleaf);
+    std::vector<int64_t> woff(nleaf);
+    std::vector<PcLeaf> leaves;
+    double flops = 0.0, flops_max = 0.0;
     int64_t at = 0, wt = 0;
     for (int li = 0; li < nleaf; ++li) {
         const int B = g->leaf0 + li;
@@ -168,8 +284,11 @@ void precond_build(lfmm_geometry_s* g) {
         own_cnt[li] = t.box_end[B] - t.box_begin[B];
         own_first[li] = t.box_begin[B];
         lay[li] = t.box_layer[B];
-        aoff[li] = at;
-        at += (int64_t)q * q;
+        leaves.push_back(PcLeaf{li, q, own_cnt[li], at});
+        at += (int64_t)q * (q + own_cnt[li]);
+        const double fl = 8.0 / 3.0 * q * (double)q * q + 8.0 * q * (double)q * own_cnt[li];
+        flops += fl;
+        flops_max = std::max(flops_max, fl);
         woff[li] = wt;
         wt += (int64_t)q * own_cnt[li];
     }
@@ -187,7 +306,16 @@ void precond_build(lfmm_geometry_s* g) {
     int* d_own_cnt = dupload(g, own_cnt);
     int* d_own_first = dupload(g, own_first);
     int* d_lay = dupload(g, lay);
-    int64_t* d_aoff = dupload(g, aoff);
+    // largest leaves first; CTAs per leaf: until the largest takes no longer on its SMs than
+    // all of them on the whole GPU
+    std::stable_sort(leaves.begin(), leaves.end(), [](const PcLeaf& a, const PcLeaf& b) { return a.q > b.q; });
+    int cs = 1;
+    while (cs < 8 && flops_max / cs > flops / 152.0) cs *= 2;
+    // columns per block: the panel (nb q values) stays within 200 KB
+    const int nb = std::max(1, std::min<int>(PC_NB, (int)(200 * 1024 / (sizeof(cd) * std::max(qmax, 1)))));
+    const size_t smem_setup = sizeof(cd) * (size_t)nb * qmax;
+    raise_smem_limit((const void*)k_pc_setup, smem_setup, "pc set-up smem");
+    PcLeaf* d_leaves = dupload(g, leaves);
     g->d_pc_W = dalloc<cd>(g, (size_t)wt);
     g->pc_w_len = wt;
     cd* Ascr = nullptr;
@@ -196,9 +324,23 @@ void precond_build(lfmm_geometry_s* g) {
                "malloc pc scratch");
     cuda_check(cudaMallocAsync((void**)&piv, sizeof(int) * std::max<size_t>(idx.size(), 1), cudaStreamPerThread),
                "malloc pc piv");
-    k_pc_setup<<<nleaf, 256>>>(g->m, g->d_pc_ptr, g->d_pc_idx, d_own_pos, d_own_cnt, d_aoff, g->d_pc_woff, d_lay,
-                               g->d_x, g->d_y, g->d_w, g->d_nx, g->d_ny, Ascr, piv, g->d_pc_W);
-    cudaError_t e1 = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nleaf * cs));
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem_setup;
+    cfg.stream = cudaStreamPerThread;
+    cudaLaunchAttribute att = {};
+    att.id = cudaLaunchAttributeClusterDimension;
+    att.val.clusterDim.x = (unsigned)cs;
+    att.val.clusterDim.y = att.val.clusterDim.z = 1;
+    cfg.attrs = &att;
+    cfg.numAttrs = 1;
+    cudaError_t e1 = cudaLaunchKernelEx(&cfg, k_pc_setup, g->m, (const int*)g->d_pc_ptr, (const int*)g->d_pc_idx,
+                                        (const int*)d_own_pos, (const PcLeaf*)d_leaves, cs, nb,
+                                        (const int64_t*)g->d_pc_woff, (const int*)d_lay, (const double*)g->d_x,
+                                        (const double*)g->d_y, (const double*)g->d_w, (const double*)g->d_nx,
+                                        (const double*)g->d_ny, Ascr, piv, g->d_pc_W);
+    if (e1 == cudaSuccess) e1 = cudaGetLastError();
     cudaError_t e2 = cudaStreamSynchronize(cudaStreamPerThread);
     dev_release(Ascr);
     dev_release(piv);
