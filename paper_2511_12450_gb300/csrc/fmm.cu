@@ -442,6 +442,7 @@ void fmm_build(lfmm_geometry_s* g) {
             ExpEntry e{t.box_begin[b], t.box_end[b], t.box_layer[b], t.p_level[t.box_level[b]], t.cx(b), slot_cy[q],
                        slot_coef[q], brows};
             if (t.box_level[b] == D) {
+                leaf_e[b - t.level_start[D]].slot[slot_side[q]] = (int)slot_e.size();
                 slot_e.push_back(e);
                 slot_leaf_e.push_back(e);
                 brows += t.box_end[b] - t.box_begin[b];
@@ -468,15 +469,16 @@ void fmm_build(lfmm_geometry_s* g) {
         // leaf order (one more for the combined field's dipole basis)
         g->basis_ord = t.p_level[D] + (g->combined ? 1 : 0);
         g->d_basis = dalloc<cd>(g, (size_t)brows * (g->basis_ord + 1));
+        if (g->combined) g->d_gbasis = dalloc<cd>(g, (size_t)brows * (g->basis_ord + 1));
         {
             const size_t smem = (size_t)g->group_max_pts * (g->basis_ord + 1) * sizeof(double);
             raise_smem_limit((const void*)k_basis, smem, "basis smem");
             if (g->n_leaf_groups > 0)
                 k_basis<<<g->n_leaf_groups, 128, smem>>>(g->d_leaf_groups, g->d_leaf_entries, g->m, g->d_x, g->d_y,
-                                                         g->basis_ord, g->d_basis);
+                                                         g->d_nx, g->d_ny, g->basis_ord, g->d_basis, g->d_gbasis);
             if (g->n_slot_groups > 0)
                 k_basis<<<g->n_slot_groups, 128, smem>>>(g->d_slot_groups, g->d_slot_entries, g->m, g->d_x, g->d_y,
-                                                         g->basis_ord, g->d_basis);
+                                                         g->d_nx, g->d_ny, g->basis_ord, g->d_basis, g->d_gbasis);
             cuda_check(cudaGetLastError(), "k_basis");
         }
         // Upward (M2M) and downward (L2L) passes.  Cells translate as families (a
@@ -799,7 +801,7 @@ void fmm_build(lfmm_geometry_s* g) {
 }
 
 void raise_smem_limit(const void* func, size_t bytes, const char* what) {
-    if (bytes <= 48 * 1024) return;   // no opt-in needed
+    if (bytes <= 32 * 1024) return;   // no opt-in needed (48 KB, less what a kernel declares statically)
     static std::mutex mu;
     static std::map<std::pair<const void*, int>, size_t> granted;
     int dev = 0;
@@ -809,12 +811,6 @@ void raise_smem_limit(const void* func, size_t bytes, const char* what) {
     if (bytes <= cur) return;
     cuda_check(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), what);
     cur = bytes;
-}
-
-static void set_smem_limits() {
-    const size_t lim = 200 * 1024;
-    raise_smem_limit((const void*)k_p2m, lim, "smem p2m");
-    raise_smem_limit((const void*)k_l2p, lim, "smem l2p");
 }
 
 static void ensure_coef(lfmm_geometry_s* g, int nrhs) {
@@ -868,7 +864,7 @@ static void launch_m2l_reduce(lfmm_geometry_s* g, int nrhs, int r1, cudaStream_t
 // at once as fit SP_WS_BYTES (at least one); a wider block takes several rounds.
 #define SP_WS_BYTES (2ll << 30)
 static int split_round(const lfmm_geometry_s* g, int nrhs) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(nrhs, SP_WS_BYTES / (int64_t)split_col_bytes(g)));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(nrhs, 2048), SP_WS_BYTES / (int64_t)split_col_bytes(g)));
 }
 static void ensure_split(lfmm_geometry_s* g, int nrhs) {
     const int want = split_round(g, nrhs);
@@ -948,23 +944,23 @@ static void launch_pass(lfmm_geometry_s* g, const XPass& P, int nrhs, cudaStream
     ++g->n_launches;
 }
 
+static P2MArgs p2m_args(lfmm_geometry_s* g, const cd* x, int nrhs) {
+    return P2MArgs{g->d_leaf_groups, g->d_slot_groups, g->d_leaf_entries, g->d_slot_entries, g->n_leaf_groups, g->m, g->d_w,
+                   g->d_basis, g->d_gbasis, g->basis_ord + 1, x, g->n, g->ncoef, g->nslotcoef, nrhs, g->d_M, g->d_Mp};
+}
+static L2PArgs l2p_args(lfmm_geometry_s* g, cd* y, int nrhs) {
+    return L2PArgs{g->d_leaf_groups, g->d_leaf_entries, g->d_slot_entries, g->d_basis, g->basis_ord + 1, g->n, g->ncoef,
+                   g->nslotcoef, nrhs, g->d_L, g->d_Lp, y};
+}
+// right-hand sides per CTA of the L2P: four where their P, Q fit beside the basis rows
+static int l2p_cols(const lfmm_geometry_s* g, int nrhs) { return nrhs > 1 && g->tree.p_level[g->tree.D] <= 40 ? 4 : 1; }
+
 void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s, bool mixed,
                cudaEvent_t before_l2p) {
-    set_smem_limits();
     TreeHost& t = g->tree;
     const int D = t.D, l0 = t.l0;
     if (l0 > D) return;
     ensure_coef(g, nrhs);
-    const int pD = t.p_level[D];
-    int pmax = 0;
-    for (int l = l0; l <= D; ++l) pmax = std::max(pmax, t.p_level[l]);
-    // shared memory of the grouped P2M / L2P kernels (same order p = p_D for every entry)
-    const int gp = g->group_max_pts, ge = g->group_max_ent;
-    const int rs_p2m = 2 * (g->combined ? pD + 1 : pD) + 1;   // basis row length (k_p2m)
-    const size_t smem_p2m = (size_t)gp * rs_p2m * sizeof(cd) + (size_t)gp * sizeof(cd) + (size_t)(gp + 1) * sizeof(int);
-    const size_t smem_l2p = (size_t)ge * 2 * (pD + 1) * sizeof(cd);
-    raise_smem_limit((const void*)k_p2m, smem_p2m, "p2m smem");
-    raise_smem_limit((const void*)k_l2p, smem_l2p, "l2p smem");
     // precision form: the levels >= lm run in FP32 on scaled expansions (lm > D: none)
     const int lm = mixed ? std::max(l0, std::min(mixed_level(g), D + 1)) : D + 1;
     if (lm <= D) mixed_setup(g, nrhs);
@@ -973,18 +969,12 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
         if (lm <= D) {
             mixed_p2m(g, x_sorted, nrhs, s);
         } else {
-            k_p2m<<<g->n_leaf_groups, 128, smem_p2m, s>>>(g->d_leaf_groups, g->d_leaf_entries, g->m, g->d_w, g->d_nx,
-                                                          g->d_ny, g->d_basis, g->basis_ord + 1, x_sorted, g->n, nrhs,
-                                                          g->ncoef, g->d_M);
+            const P2MArgs a = p2m_args(g, x_sorted, nrhs);
+            const int nb = g->n_leaf_groups + g->n_slot_groups;
+            if (nrhs > 1) k_p2m<4><<<dim3(nb, (nrhs + 3) / 4), 128, 0, s>>>(a);
+            else k_p2m<1><<<nb, 128, 0, s>>>(a);
             cuda_check(cudaGetLastError(), "k_p2m");
             ++g->n_launches;
-            if (g->n_slot_groups > 0) {
-                k_p2m<<<g->n_slot_groups, 128, smem_p2m, s>>>(g->d_slot_groups, g->d_slot_entries, g->m, g->d_w,
-                                                              g->d_nx, g->d_ny, g->d_basis, g->basis_ord + 1, x_sorted,
-                                                              g->n, nrhs, g->nslotcoef, g->d_Mp);
-                cuda_check(cudaGetLastError(), "k_p2m slots");
-                ++g->n_launches;
-            }
         }
         prof_end(g, ST_P2M, s);
     }
@@ -1027,17 +1017,14 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
         if (lm <= D) {
             mixed_l2p(g, y_sorted, nrhs, s);
         } else {
-            k_l2p<<<g->n_leaf_groups, 128, smem_l2p, s>>>(g->d_leaf_groups, g->d_leaf_entries, g->d_basis,
-                                                          g->basis_ord + 1, g->n, nrhs, g->ncoef, g->d_L, y_sorted);
+            const L2PArgs a = l2p_args(g, y_sorted, nrhs);
+            const int cb = l2p_cols(g, nrhs);
+            const size_t smem = l2p_smem(cb, g->group_max_ent, t.p_level[D]);
+            raise_smem_limit(cb > 1 ? (const void*)k_l2p<4> : (const void*)k_l2p<1>, smem, "l2p smem");
+            if (cb > 1) k_l2p<4><<<dim3(g->n_leaf_groups, (nrhs + 3) / 4), 128, smem, s>>>(a);
+            else k_l2p<1><<<dim3(g->n_leaf_groups, nrhs), 128, smem, s>>>(a);
             cuda_check(cudaGetLastError(), "k_l2p");
             ++g->n_launches;
-            if (g->n_slot_groups > 0) {
-                k_l2p<<<g->n_slot_groups, 128, smem_l2p, s>>>(g->d_slot_groups, g->d_slot_leaf_entries, g->d_basis,
-                                                              g->basis_ord + 1, g->n, nrhs, g->nslotcoef, g->d_Lp,
-                                                              y_sorted);
-                cuda_check(cudaGetLastError(), "k_l2p slots");
-                ++g->n_launches;
-            }
         }
         prof_end(g, ST_L2P, s);
     }
@@ -1050,26 +1037,12 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
 // single-geometry kernel with its block index within the job, so every geometry's
 // result is the one its own launches give, bit for bit.
 struct P2MJob {
-    const ExpGroup* groups;
-    const ExpEntry* ent;
-    MediumDev m;
-    const double *pw, *nx, *ny;
-    const cd* basis;
-    int bstride;
-    const cd* phi;
-    int64_t n, stride;
-    int nrhs;
-    cd* M;
+    P2MArgs a;
+    int blocks;   // per column group
 };
 struct L2PJob {
-    const ExpGroup* groups;
-    const ExpEntry* ent;
-    const cd* basis;
-    int bstride;
-    int64_t n, stride;
-    int nrhs;
-    const cd* L;
-    cd* y;
+    L2PArgs a;
+    int blocks;
 };
 struct XJob {
     XPass P;
@@ -1090,18 +1063,19 @@ __device__ __forceinline__ int job_of(const int* __restrict__ prefix, int njobs,
     }
     return lo;
 }
+template <int CB>
 __global__ void __launch_bounds__(128) k_p2m_multi(const P2MJob* __restrict__ jobs, const int* __restrict__ prefix,
                                                    int njobs) {
     const int j = job_of(prefix, njobs, blockIdx.x);
-    const P2MJob& J = jobs[j];
-    p2m_group(blockIdx.x - prefix[j], J.groups, J.ent, J.m, J.pw, J.nx, J.ny, J.basis, J.bstride, J.phi, J.n, J.nrhs,
-              J.stride, J.M);
+    const int b = blockIdx.x - prefix[j], nb = jobs[j].blocks;
+    p2m_block<CB>(jobs[j].a, b % nb, (b / nb) * CB);
 }
+template <int CB>
 __global__ void __launch_bounds__(128) k_l2p_multi(const L2PJob* __restrict__ jobs, const int* __restrict__ prefix,
                                                    int njobs) {
     const int j = job_of(prefix, njobs, blockIdx.x);
-    const L2PJob& J = jobs[j];
-    l2p_group(blockIdx.x - prefix[j], J.groups, J.ent, J.basis, J.bstride, J.n, J.nrhs, J.stride, J.L, J.y);
+    const int b = blockIdx.x - prefix[j], nb = jobs[j].blocks;
+    l2p_group<CB>(jobs[j].a, b % nb, (b / nb) * CB);
 }
 __global__ void __launch_bounds__(128) k_translate_multi(const XJob* __restrict__ jobs, const int* __restrict__ prefix,
                                                          int njobs) {
@@ -1159,9 +1133,9 @@ static void launch_jobs(const std::vector<J>& jobs, const std::vector<int>& bloc
 }
 
 void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_t before_l2p) {
-    set_smem_limits();
     std::vector<const BatchOp*> far;
-    size_t smem_p2m = 0, smem_l2p = 0;
+    size_t smem_l2p = 0;
+    int max_nrhs = 1, cb_l2p = 4;
     int max_up = 0, max_dn = 0;
     for (const BatchOp& op : ops) {
         lfmm_geometry_s* g = op.g;
@@ -1171,10 +1145,8 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
         ensure_coef(g, op.nrhs);
         split_check_waits(g);
         ensure_split(g, op.nrhs);
-        const int pD = t.p_level[t.D], gp = g->group_max_pts, ge = g->group_max_ent;
-        const int rs = 2 * (g->combined ? pD + 1 : pD) + 1;
-        smem_p2m = std::max(smem_p2m, (size_t)gp * rs * sizeof(cd) + (size_t)gp * sizeof(cd) + (size_t)(gp + 1) * sizeof(int));
-        smem_l2p = std::max(smem_l2p, (size_t)ge * 2 * (pD + 1) * sizeof(cd));
+        max_nrhs = std::max(max_nrhs, op.nrhs);
+        cb_l2p = std::min(cb_l2p, t.p_level[t.D] <= 40 ? 4 : 1);
         max_up = std::max(max_up, t.D - t.l0);
         max_dn = std::max(max_dn, t.D - t.l0);
     }
@@ -1182,21 +1154,20 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
         if (before_l2p) cuda_check(cudaStreamWaitEvent(s, before_l2p, 0), "wait for the near field");
         return;
     }
-    raise_smem_limit((const void*)k_p2m_multi, smem_p2m, "p2m smem");
-    raise_smem_limit((const void*)k_l2p_multi, smem_l2p, "l2p smem");
+    if (max_nrhs == 1) cb_l2p = 1;
+    for (const BatchOp* op : far)
+        smem_l2p = std::max(smem_l2p, l2p_smem(cb_l2p, op->g->group_max_ent, op->g->tree.p_level[op->g->tree.D]));
     {   // P2M: leaves about cell centres, straddling leaves about reaction centres
         std::vector<P2MJob> jobs;
         std::vector<int> blocks;
+        const int cb = max_nrhs > 1 ? 4 : 1;
         for (const BatchOp* op : far) {
-            lfmm_geometry_s* g = op->g;
-            jobs.push_back(P2MJob{g->d_leaf_groups, g->d_leaf_entries, g->m, g->d_w, g->d_nx, g->d_ny, g->d_basis,
-                                  g->basis_ord + 1, op->x, g->n, g->ncoef, op->nrhs, g->d_M});
-            blocks.push_back(g->n_leaf_groups);
-            jobs.push_back(P2MJob{g->d_slot_groups, g->d_slot_entries, g->m, g->d_w, g->d_nx, g->d_ny, g->d_basis,
-                                  g->basis_ord + 1, op->x, g->n, g->nslotcoef, op->nrhs, g->d_Mp});
-            blocks.push_back(g->n_slot_groups);
+            const int nb = op->g->n_leaf_groups + op->g->n_slot_groups;
+            jobs.push_back(P2MJob{p2m_args(op->g, op->x, op->nrhs), nb});
+            blocks.push_back(nb * ((op->nrhs + cb - 1) / cb));
         }
-        launch_jobs(jobs, blocks, k_p2m_multi, 128, smem_p2m, s, "k_p2m_multi");
+        if (cb > 1) launch_jobs(jobs, blocks, k_p2m_multi<4>, 128, 0, s, "k_p2m_multi");
+        else launch_jobs(jobs, blocks, k_p2m_multi<1>, 128, 0, s, "k_p2m_multi");
     }
     // M2M: pass k takes each geometry's parents at level D - 1 - k (down to its l0)
     for (int k = 0; k < max_up; ++k) {
@@ -1258,25 +1229,15 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
     }
     // L2P after the near field, which adds into the same y
     if (before_l2p) cuda_check(cudaStreamWaitEvent(s, before_l2p, 0), "wait for the near field");
-    // the leaves about cell centres, then (a second launch: both add into the same points
-    // of y) the straddling leaves about their reaction centres, as each geometry's own launches
-    for (int slots = 0; slots < 2; ++slots) {
-        std::vector<L2PJob> jobs;
-        std::vector<int> blocks;
-        for (const BatchOp* op : far) {
-            lfmm_geometry_s* g = op->g;
-            if (slots == 0) {
-                jobs.push_back(L2PJob{g->d_leaf_groups, g->d_leaf_entries, g->d_basis, g->basis_ord + 1, g->n,
-                                      g->ncoef, op->nrhs, g->d_L, op->y});
-                blocks.push_back(g->n_leaf_groups);
-            } else {
-                jobs.push_back(L2PJob{g->d_slot_groups, g->d_slot_leaf_entries, g->d_basis, g->basis_ord + 1, g->n,
-                                      g->nslotcoef, op->nrhs, g->d_Lp, op->y});
-                blocks.push_back(g->n_slot_groups);
-            }
-        }
-        launch_jobs(jobs, blocks, k_l2p_multi, 128, smem_l2p, s, "k_l2p_multi");
+    std::vector<L2PJob> jobs;
+    std::vector<int> blocks;
+    for (const BatchOp* op : far) {
+        jobs.push_back(L2PJob{l2p_args(op->g, op->y, op->nrhs), op->g->n_leaf_groups});
+        blocks.push_back(op->g->n_leaf_groups * ((op->nrhs + cb_l2p - 1) / cb_l2p));
     }
+    raise_smem_limit(cb_l2p > 1 ? (const void*)k_l2p_multi<4> : (const void*)k_l2p_multi<1>, smem_l2p, "l2p smem");
+    if (cb_l2p > 1) launch_jobs(jobs, blocks, k_l2p_multi<4>, 128, smem_l2p, s, "k_l2p_multi");
+    else launch_jobs(jobs, blocks, k_l2p_multi<1>, 128, smem_l2p, s, "k_l2p_multi");
 }
 
 // Schedule of the M2L chosen by measurement on this geometry: the cap on the work of one
@@ -1288,7 +1249,6 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
 void fmm_autotune(lfmm_geometry_s* g) {
     TreeHost& t = g->tree;
     if (t.l0 > t.D || g->sp_tabs_host.empty()) return;
-    set_smem_limits();
     cudaStream_t s = cudaStreamPerThread;
     ensure_coef(g, 1);
     cuda_check(cudaMemsetAsync(g->d_M, 0, sizeof(cd) * std::max<int64_t>(g->ncoef, 1), s), "tune memset");

@@ -42,92 +42,151 @@ __device__ __forceinline__ void group_point(const ExpEntry* __restrict__ ent, in
 
 // P2M about the entries' centres (leaves about cell centres, straddling leaves
 // about their reaction centres): M_n = sum_j q_j J_n(k rho_j) e^{-i n theta_j},
-// q_j = |Gamma_j| phi_j.  Phase 1, one thread per point of the group: its basis
-// row u_{j,n} = J_n(k rho_j) e^{-i n theta_j} for n = -p..p (J_{-n} = (-1)^n J_n,
-// e^{+i n theta} = conj) into shared memory.  Phase 2, one thread per (entry,
-// coefficient): the sum over the entry's points, pure complex FMAs.
-// Combined field (normals given): the row is the basis of a dipole along n_j
-// plus -i k times the charge's, E_n = n_j . grad u_n - i k u_n, with
-// n . grad u_n = (k/2)(conj(nu) u_{n-1} - nu u_{n+1}), nu = n_x + i n_y (from
-// (d_x +- i d_y) J_m e^{i m theta} = -+k J_{m+-1} e^{i (m+-1) theta}); the
-// translations are linear and carry it unchanged.
-__device__ __forceinline__ void p2m_group(int gi, const ExpGroup* __restrict__ groups,
-                                          const ExpEntry* __restrict__ ent, const MediumDev& m,
-                                          const double* __restrict__ pw, const double* __restrict__ nx,
-                                          const double* __restrict__ ny, const cd* __restrict__ basis,
-                                          int bstride, const cd* __restrict__ phi, int64_t n,
-                                          int nrhs, int64_t stride, cd* __restrict__ M) {
-    extern __shared__ cd su[];   // [npts][rs] basis rows, then [npts] q, then [nent + 1] point offsets (ints)
-    const ExpGroup G = groups[gi];
-    const int p = ent[G.e0].p, nco = 2 * p + 1;
-    const bool cf = nx != nullptr;
-    const int pb = cf ? p + 1 : p, rs = 2 * pb + 1;   // order and length of the plain basis rows
-    const int ne = G.e1 - G.e0;
-    cd* sq = su + (size_t)G.npts * rs;
-    int* soff = (int*)(sq + G.npts);
+// q_j = |Gamma_j| phi_j, from the stored basis b_n = J_n e^{i n theta}, n = 0..p.  With
+//   S1 = sum qx bx, S2 = sum qy by, S3 = sum qy bx, S4 = sum qx by,
+//   M_n = (S1 + S2) + i (S3 - S4),  M_{-n} = (-1)^n ((S1 - S2) + i (S3 + S4)),
+// so a point costs 4 FMAs for both of +-n (8 when each is summed by itself).  Combined field
+// (gbasis given): the dipole along n_j less i k times the charge, E_n = n_j . grad u_n - i k u_n,
+// u_n = conj(b_n); gbasis holds conj(n_j . grad u_n), summed the same way.
+// A CTA takes one group: threads over (entry, n, slice of the points), consecutive threads
+// reading consecutive basis values; charges staged for P2M_PTS points at a time (a group of
+// several entries has at most that many); slices added in a fixed order.  CB right-hand sides
+// per basis value read.  N = 65,536: 28 us for the 22 MB basis; staging every point's 2p + 1
+// row in shared memory and 8 FMAs per output took 56 us, and the few reaction-centre groups
+// another 17 us in a launch of their own.
+#define P2M_PTS 64
+template <int CB>
+__device__ __forceinline__ void p2m_group(const ExpGroup& G, const ExpEntry* __restrict__ ent, const MediumDev& m,
+                                          const double* __restrict__ pw, const cd* __restrict__ basis,
+                                          const cd* __restrict__ gbasis, int bstride, const cd* __restrict__ phi,
+                                          int64_t n, int col0, int nrhs, int64_t stride, cd* __restrict__ M) {
+    __shared__ cd sq[CB][P2M_PTS];
+    __shared__ int soff[EXP_GROUP_ENTRIES + 1];
+    __shared__ double red[CB][8][128];
+    const int p = ent[G.e0].p, np1 = p + 1, ne = G.e1 - G.e0, tasks = ne * np1;
+    const int ncb = min(CB, nrhs - col0);
     if (threadIdx.x == 0) {
         int o = 0;
         for (int e = 0; e < ne; ++e) { soff[e] = o; o += ent[G.e0 + e].end - ent[G.e0 + e].beg; }
         soff[ne] = o;
     }
-    for (int t = threadIdx.x; t < G.npts; t += blockDim.x) {
-        int er, j;
-        group_point(ent, G.e0, G.e1, t, &er, &j);
-        const ExpEntry& E = ent[G.e0 + er];
-        cd* u = su + (size_t)t * rs;
-        // u_n = J_n(k rho) e^{-i n theta} = conj of the stored basis, n = 0..pb, into slots pb..2pb
-        const cd* b = basis + (E.brow + (j - E.beg)) * (int64_t)bstride;
-        for (int k2 = 0; k2 <= pb; ++k2) {
-            const cd v = b[k2];
-            u[pb + k2] = mk(v.x, -v.y);
-        }
-        // u_{-n} = (-1)^n conj(u_n) into slots pb-1..0; the signs by integer bit flips
-        // (no FP64 instruction)
-        for (int k2 = 1; k2 <= pb; ++k2) {
-            const cd v = u[pb + k2];
-            u[pb - k2] = mk(dsign(v.x, k2), dsign(v.y, k2 + 1));
-        }
-        if (cf) {   // E_n into slot n + p from u_{n-1}, u_n, u_{n+1} (slots n+p, n+p+1, n+p+2);
-                    // ascending n overwrites only u_{n-1}, which later n do not read
-            const double k = m.k[E.lay];
-            const cd nu = mk(nx[j], ny[j]), nub = conjc(nu);
-            for (int s2 = 0; s2 < nco; ++s2) {
-                const cd um = u[s2], u0 = u[s2 + 1], up = u[s2 + 2];
-                const cd d = 0.5 * (nub * um - nu * up);
-                u[s2] = k * mk(d.x + u0.y, d.y - u0.x);   // k (d - i u_n)
-            }
-        }
-    }
-    for (int col = 0; col < nrhs; ++col) {
+    const int NS = max(1, min(4, 128 / tasks));
+    double a[CB][4], d[CB][4];
+#pragma unroll
+    for (int c = 0; c < CB; ++c)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { a[c][i] = 0.0; d[c][i] = 0.0; }
+    for (int p0 = 0; p0 < G.npts; p0 += P2M_PTS) {   // more than one round only for a single entry
+        const int np = min(P2M_PTS, G.npts - p0);
+        const bool last = p0 + P2M_PTS >= G.npts;
         __syncthreads();
-        for (int t = threadIdx.x; t < G.npts; t += blockDim.x) {
+        for (int t = threadIdx.x; t < np * ncb; t += blockDim.x) {
+            const int c = t / np, i = t - c * np;
             int er, j;
-            group_point(ent, G.e0, G.e1, t, &er, &j);
-            sq[t] = pw[j] * phi[(int64_t)col * n + j];
+            group_point(ent, G.e0, G.e1, p0 + i, &er, &j);
+            sq[c][i] = pw[j] * phi[(int64_t)(col0 + c) * n + j];
         }
         __syncthreads();
-        for (int task = threadIdx.x; task < ne * nco; task += blockDim.x) {
-            const int er = task / nco, idx = task - er * nco;
-            cd a = mk(0, 0);
-            for (int t = soff[er]; t < soff[er + 1]; ++t) cfma(a, sq[t], su[(size_t)t * rs + idx]);
-            M[(int64_t)col * stride + ent[G.e0 + er].off + idx] = a;
+        for (int t0 = 0; t0 < tasks; t0 += 128) {   // more than one round only with NS = 1
+            const int task = (t0 + (int)threadIdx.x) % max(tasks, 1), sl = NS > 1 ? (int)threadIdx.x / tasks : 0;
+            const bool live = NS > 1 ? sl < NS : t0 + (int)threadIdx.x < tasks;
+            const int er = task / np1, k2 = task - er * np1;
+            if (live) {
+                const int b0 = max(soff[er], p0), b1 = min(soff[er + 1], p0 + np);
+                const cd* b = basis + (ent[G.e0 + er].brow - soff[er]) * (int64_t)bstride + k2;
+                const cd* g = gbasis ? gbasis + (ent[G.e0 + er].brow - soff[er]) * (int64_t)bstride + k2 : nullptr;
+#pragma unroll 4
+                for (int t = b0 + sl; t < b1; t += NS) {
+                    const cd v = b[(int64_t)t * bstride];
+#pragma unroll
+                    for (int c = 0; c < CB; ++c) {
+                        const cd q = sq[c][t - p0];
+                        a[c][0] = fma(q.x, v.x, a[c][0]);
+                        a[c][1] = fma(q.y, v.y, a[c][1]);
+                        a[c][2] = fma(q.y, v.x, a[c][2]);
+                        a[c][3] = fma(q.x, v.y, a[c][3]);
+                    }
+                    if (g) {
+                        const cd w = g[(int64_t)t * bstride];
+#pragma unroll
+                        for (int c = 0; c < CB; ++c) {
+                            const cd q = sq[c][t - p0];
+                            d[c][0] = fma(q.x, w.x, d[c][0]);
+                            d[c][1] = fma(q.y, w.y, d[c][1]);
+                            d[c][2] = fma(q.y, w.x, d[c][2]);
+                            d[c][3] = fma(q.x, w.y, d[c][3]);
+                        }
+                    }
+                }
+            }
+            if (!last) continue;
+            if (NS > 1) {
+#pragma unroll
+                for (int c = 0; c < CB; ++c)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { red[c][i][threadIdx.x] = a[c][i]; red[c][4 + i][threadIdx.x] = d[c][i]; }
+                __syncthreads();
+            }
+            if (live && sl == 0) {
+                const double k = m.k[ent[G.e0 + er].lay];
+#pragma unroll
+                for (int c = 0; c < CB; ++c) {
+                    if (c >= ncb) break;
+                    for (int q = 1; q < NS; ++q)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) { a[c][i] += red[c][i][q * tasks + task]; d[c][i] += red[c][4 + i][q * tasks + task]; }
+                    cd up = mk(a[c][0] + a[c][1], a[c][2] - a[c][3]), dn = mk(a[c][0] - a[c][1], a[c][2] + a[c][3]);
+                    if (gbasis) {   // G - i k u
+                        up = mk(fma(k, up.y, d[c][0] + d[c][1]), fma(-k, up.x, d[c][2] - d[c][3]));
+                        dn = mk(fma(k, dn.y, d[c][0] - d[c][1]), fma(-k, dn.x, d[c][2] + d[c][3]));
+                    }
+                    cd* out = M + (int64_t)(col0 + c) * stride + ent[G.e0 + er].off + p;
+                    out[k2] = up;
+                    if (k2 > 0) out[-k2] = csign(dn, k2);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < CB; ++c)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { a[c][i] = 0.0; d[c][i] = 0.0; }
         }
     }
 }
-__global__ void __launch_bounds__(128) k_p2m(const ExpGroup* __restrict__ groups, const ExpEntry* __restrict__ ent,
-                      MediumDev m, const double* __restrict__ pw, const double* __restrict__ nx,
-                      const double* __restrict__ ny, const cd* __restrict__ basis, int bstride,
-                      const cd* __restrict__ phi, int64_t n, int nrhs, int64_t stride, cd* __restrict__ M) {
-    p2m_group(blockIdx.x, groups, ent, m, pw, nx, ny, basis, bstride, phi, n, nrhs, stride, M);
+// leaf groups first, then the straddling leaves' reaction-centre groups
+struct P2MArgs {
+    const ExpGroup *groups, *sgroups;
+    const ExpEntry *ent, *sent;
+    int ngroups;
+    MediumDev m;
+    const double* pw;
+    const cd *basis, *gbasis;
+    int bstride;
+    const cd* phi;
+    int64_t n, ncoef, nslotcoef;
+    int nrhs;
+    cd *M, *Mp;
+};
+template <int CB>
+__device__ __forceinline__ void p2m_block(const P2MArgs& P, int b, int col0) {
+    const bool slot = b >= P.ngroups;
+    p2m_group<CB>(slot ? P.sgroups[b - P.ngroups] : P.groups[b], slot ? P.sent : P.ent, P.m, P.pw, P.basis, P.gbasis,
+                  P.bstride, P.phi, P.n, col0, P.nrhs, slot ? P.nslotcoef : P.ncoef, slot ? P.Mp : P.M);
 }
+template <int CB>
+__global__ void __launch_bounds__(128) k_p2m(const P2MArgs P) { p2m_block<CB>(P, blockIdx.x, blockIdx.y * CB); }
 
 // The expansion basis of every (entry, point), computed once per geometry:
 // b_n = J_n(k rho) e^{i n theta}, n = 0..ord, with (rho, theta) the point's polar
 // coordinates about the entry's centre (the cell centre, or a straddling leaf's reaction
 // centre).  L2P uses b_n, P2M its conjugate.  e^{i n theta} by powers upward from 1.
+// Combined field: also gb_n = conj(n_j . grad u_n) for n < ord, u = conj(b), with
+// n . grad u_n = (k/2)(conj(nu) u_{n-1} - nu u_{n+1}), nu = n_x + i n_y (from
+// (d_x +- i d_y) J_m e^{i m theta} = -+k J_{m+-1} e^{i (m+-1) theta}).
 __global__ void __launch_bounds__(128) k_basis(const ExpGroup* __restrict__ groups, const ExpEntry* __restrict__ ent,
                                                MediumDev m, const double* __restrict__ px,
-                                               const double* __restrict__ py, int ord, cd* __restrict__ basis) {
+                                               const double* __restrict__ py, const double* __restrict__ nx,
+                                               const double* __restrict__ ny, int ord, cd* __restrict__ basis,
+                                               cd* __restrict__ gbasis) {
     extern __shared__ double sjb[];   // [npts][ord + 1] J_n
     const ExpGroup G = groups[blockIdx.x];
     for (int t = threadIdx.x; t < G.npts; t += blockDim.x) {
@@ -146,6 +205,15 @@ __global__ void __launch_bounds__(128) k_basis(const ExpGroup* __restrict__ grou
         for (int k2 = 1; k2 <= ord; ++k2) {
             zz = zz * z;
             b[k2] = mk(J[k2] * zz.x, J[k2] * zz.y);
+        }
+        if (gbasis) {
+            cd* g = gbasis + (E.brow + (j - E.beg)) * (int64_t)(ord + 1);
+            const cd nu = mk(nx[j], ny[j]), nub = conjc(nu);
+            for (int k2 = 0; k2 < ord; ++k2) {
+                const cd bm = k2 > 0 ? b[k2 - 1] : mk(-b[1].x, b[1].y);   // b_{-1} = -conj(b_1)
+                g[k2] = (0.5 * m.k[E.lay]) * (nu * bm - nub * b[k2 + 1]);
+            }
+            g[ord] = mk(0.0, 0.0);
         }
     }
 }
@@ -171,52 +239,104 @@ __global__ void __launch_bounds__(64) k_m2l_reduce(const M2LReduce* __restrict__
         else Lp[(int64_t)col * nslotcoef + slot_coef[ts] + idx] = t;
     }
 }
-// L2P over a list of point ranges: y_i += sum_n L_n J_n(k rho_i) e^{i n theta_i}
-// about (cx, cy).  Leaves (cell centres) and straddling leaves (reaction centres).
-__device__ __forceinline__ void l2p_group(int gi, const ExpGroup* __restrict__ groups,
-                      const ExpEntry* __restrict__ ent, const cd* __restrict__ basis, int bstride, int64_t n,
-                      int nrhs, int64_t stride, const cd* __restrict__ L, cd* __restrict__ y) {
-    // y_j += sum_n L_n J_n(k rho_j) e^{i n theta_j}.  Per entry, A_n = L_n and
-    // B_n = (-1)^n L_{-n} are folded into P_n = A_n + B_n and Q_n = A_n - B_n, so
-    // that A_n z^n + B_n conj(z^n) = P_n cos(n theta) + i Q_n sin(n theta); the point's
-    // J_n cos(n theta) and J_n sin(n theta) are its stored basis row.
-    extern __shared__ cd sPQ[];   // [nent][2][p+1] (P, Q)
-    const ExpGroup G = groups[gi];
-    const int p = ent[G.e0].p, np1 = p + 1;
-    const int ne = G.e1 - G.e0;
-    for (int col = 0; col < nrhs; ++col) {
+// L2P: y_j += sum_n L_n J_n(k rho_j) e^{i n theta_j} over the leaf's cell centre and, for a
+// straddling leaf, its reaction centres.  Per entry, A_n = L_n and B_n = (-1)^n L_{-n} are
+// folded into P_n = A_n + B_n and Q_n = A_n - B_n, so that A_n z^n + B_n conj(z^n) =
+// P_n cos(n theta) + i Q_n sin(n theta); the point's J_n cos(n theta) and J_n sin(n theta) are
+// its stored basis row.  A CTA takes one group, L2P_PTS points at a time: their basis rows come
+// to shared memory in whole lines and two threads share a point's orders; the reaction
+// centres' terms, a few leaves, read their rows directly.  N = 65,536: 29 us; a thread reading
+// its own point's row 19 us, and 15 us for a second launch of the reaction-centre groups
+// (which add into the same points).
+#define L2P_PTS 64
+struct L2PArgs {
+    const ExpGroup* groups;
+    const ExpEntry *ent, *sent;   // leaf entries; reaction-centre entries (ExpEntry::slot)
+    const cd* basis;
+    int bstride;
+    int64_t n, ncoef, nslotcoef;
+    int nrhs;
+    const cd *L, *Lp;
+    cd* y;
+};
+inline size_t l2p_smem(int cb, int ne, int p) { return sizeof(cd) * ((size_t)L2P_PTS * (p + 1) + (size_t)cb * ne * 2 * (p + 1)); }
+template <int CB>
+__device__ __forceinline__ void l2p_group(const L2PArgs& A, int gi, int col0) {
+    extern __shared__ cd l2p_sm[];   // [L2P_PTS][p + 1] basis rows, then [CB][ne][2][p + 1] (P, Q)
+    __shared__ cd half[CB][L2P_PTS];
+    const ExpGroup G = A.groups[gi];
+    const int p = A.ent[G.e0].p, np1 = p + 1, ne = G.e1 - G.e0, ncb = min(CB, A.nrhs - col0);
+    cd* sb = l2p_sm;
+    cd* pq = sb + L2P_PTS * np1;
+    for (int i = threadIdx.x; i < ncb * ne * np1; i += blockDim.x) {
+        const int c = i / (ne * np1), er = (i - c * ne * np1) / np1, k2 = i % np1;
+        const cd* Le = A.L + (int64_t)(col0 + c) * A.ncoef + A.ent[G.e0 + er].off;
+        const cd a = Le[p + k2], b = csign(Le[p - k2], k2);
+        cd* o = pq + (size_t)((c * ne + er) * 2) * np1 + k2;
+        o[0] = k2 == 0 ? a : a + b;
+        o[np1] = k2 == 0 ? mk(0, 0) : a - b;
+    }
+    const int h = threadIdx.x >> 6, t = threadIdx.x & 63;   // half of the orders, point
+    const int k0 = h ? (np1 + 1) / 2 : 0, k1 = h ? np1 : (np1 + 1) / 2;
+    for (int p0 = 0; p0 < G.npts; p0 += L2P_PTS) {
+        const int np = min(L2P_PTS, G.npts - p0);
         __syncthreads();
-        for (int i = threadIdx.x; i < ne * np1; i += blockDim.x) {
-            const int er = i / np1, k2 = i - er * np1;
-            const cd* Le = L + (int64_t)col * stride + ent[G.e0 + er].off;
-            const cd A = Le[p + k2];
-            const cd B = csign(Le[p - k2], k2);
-            if (k2 == 0) { sPQ[(er * 2) * np1] = A; sPQ[(er * 2 + 1) * np1] = mk(0, 0); }
-            else { sPQ[(er * 2) * np1 + k2] = A + B; sPQ[(er * 2 + 1) * np1 + k2] = A - B; }
+        // consecutive leaves' points are consecutive, and so are their basis rows
+        const cd* b = A.basis + (A.ent[G.e0].brow + p0) * (int64_t)A.bstride;
+        if (A.bstride == np1) {
+            for (int i = threadIdx.x; i < np * np1; i += blockDim.x) sb[i] = b[i];
+        } else {
+            for (int i = threadIdx.x; i < np * np1; i += blockDim.x) sb[i] = b[(int64_t)(i / np1) * A.bstride + i % np1];
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < G.npts; t += blockDim.x) {
-            int er, j;
-            group_point(ent, G.e0, G.e1, t, &er, &j);
-            const ExpEntry& E = ent[G.e0 + er];
-            const cd* b = basis + (E.brow + (j - E.beg)) * (int64_t)bstride;
-            const cd* P = sPQ + (er * 2) * np1;
-            const cd* Q = P + np1;
-            cd acc = P[0] * b[0].x;
-            for (int k2 = 1; k2 <= p; ++k2) {
-                const cd v = b[k2];
-                acc.x = fma(P[k2].x, v.x, fma(-Q[k2].y, v.y, acc.x));
-                acc.y = fma(P[k2].y, v.x, fma(Q[k2].x, v.y, acc.y));
+        int er = 0, j = 0;
+        cd acc[CB];
+#pragma unroll
+        for (int c = 0; c < CB; ++c) acc[c] = mk(0, 0);
+        if (t < np) {
+            group_point(A.ent, G.e0, G.e1, p0 + t, &er, &j);
+            const cd* v = sb + t * np1;
+#pragma unroll
+            for (int c = 0; c < CB; ++c) {
+                if (c >= ncb) break;
+                const cd *P = pq + (size_t)((c * ne + er) * 2) * np1, *Q = P + np1;
+                for (int k2 = k0; k2 < k1; ++k2) {
+                    const cd w = v[k2];
+                    acc[c].x = fma(P[k2].x, w.x, fma(-Q[k2].y, w.y, acc[c].x));
+                    acc[c].y = fma(P[k2].y, w.x, fma(Q[k2].x, w.y, acc[c].y));
+                }
             }
-            y[(int64_t)col * n + j] += acc;
+            const ExpEntry& E = A.ent[G.e0 + er];
+            for (int side = 0; side < 2; ++side) {
+                if (E.slot[side] < 0) continue;
+                const ExpEntry& R = A.sent[E.slot[side]];
+                const cd* br = A.basis + (R.brow + (j - R.beg)) * (int64_t)A.bstride;
+#pragma unroll
+                for (int c = 0; c < CB; ++c) {
+                    if (c >= ncb) break;
+                    const cd* Le = A.Lp + (int64_t)(col0 + c) * A.nslotcoef + R.off + p;
+                    for (int k2 = k0; k2 < k1; ++k2) {
+                        const cd w = br[k2];
+                        cfma(acc[c], Le[k2], w);
+                        if (k2 > 0) cfma(acc[c], csign(Le[-k2], k2), conjc(w));
+                    }
+                }
+            }
+            if (h == 1) {
+#pragma unroll
+                for (int c = 0; c < CB; ++c) half[c][t] = acc[c];
+            }
+        }
+        __syncthreads();
+        if (h == 0 && t < np) {
+#pragma unroll
+            for (int c = 0; c < CB; ++c)
+                if (c < ncb) A.y[(int64_t)(col0 + c) * A.n + j] += acc[c] + half[c][t];
         }
     }
 }
-__global__ void __launch_bounds__(128) k_l2p(const ExpGroup* __restrict__ groups, const ExpEntry* __restrict__ ent,
-                      const cd* __restrict__ basis, int bstride, int64_t n, int nrhs, int64_t stride,
-                      const cd* __restrict__ L, cd* __restrict__ y) {
-    l2p_group(blockIdx.x, groups, ent, basis, bstride, n, nrhs, stride, L, y);
-}
+template <int CB>
+__global__ void __launch_bounds__(128) k_l2p(const L2PArgs A) { l2p_group<CB>(A, blockIdx.x, blockIdx.y * CB); }
 
 // Multipole-to-multipole and local-to-local translations (Graf's addition theorem),
 // one launch per level and pass over two kinds of work:

@@ -55,6 +55,7 @@ struct ExpEntry {
     double cx, cy;
     int64_t off;   // coefficient offset in the output/input array
     int64_t brow;  // row of the entry's first point in the stored expansion basis
+    int slot[2] = {-1, -1};   // leaf: its reaction-centre entries (side 0, 1), -1: none
 };
 // consecutive entries processed by one CTA (at most EXP_GROUP_PTS points and
 // EXP_GROUP_ENTRIES entries, or a single larger entry)
@@ -263,6 +264,7 @@ struct lfmm_geometry_s {
     // J_n(k rho) e^{i n theta}, n = 0..basis_ord, one row per (entry, point): leaf entries at
     // rows 0..n-1 (the point's index), straddling leaves' reaction-centre entries after them
     cd* d_basis = nullptr;
+    cd* d_gbasis = nullptr;            // combined field: the dipoles' basis, rows as d_basis
     int basis_ord = 0;
     int n_leaf_groups = 0, n_slot_groups = 0, group_max_pts = 1, group_max_ent = 1;
     // M2M (up) and L2L (down) passes: per level, a range of destinations
