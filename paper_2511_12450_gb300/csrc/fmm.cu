@@ -208,31 +208,42 @@ static void split_alloc(lfmm_geometry_s* g, int cols) {   // products, then digi
     g->d_sp_vexp = (int*)(g->d_sp_vdig + (size_t)g->sp_nvec * cols * SP_ND * SP_POS);
     g->sp_ws_cols = cols;
 }
-// Units: a matrix's pairs in groups of up to cap, of nearly equal size, by row tiles of up
-// to 64 complex rows.  Replaces the geometry's units.
-static void make_split_units(lfmm_geometry_s* g, int cap) {
+// Units: a matrix's (pair, column) columns in groups of up to sp_cap, of nearly equal size, by
+// row tiles of up to 64 complex rows.
+static void make_split_plan(lfmm_geometry_s* g, SplitPlan& P, int ncols) {
     std::vector<SplitUnit> units;
-    const int nlev = g->tree.D + 1;
-    g->sp_unit_start.assign(nlev + 2, -1);
-    g->sp_max_cnt = 0;
+    const int nlev = g->tree.D + 1, cap = g->sp_cap;
+    P.start.assign(nlev + 2, -1);
     for (const SplitTab& s : g->sp_tabs_host) {
-        if (g->sp_unit_start[s.level] < 0) g->sp_unit_start[s.level] = (int)units.size();
-        const int nco = 2 * s.pT + 1, nu = (s.npairs + cap - 1) / cap;
+        if (P.start[s.level] < 0) P.start[s.level] = (int)units.size();
+        const int nco = 2 * s.pT + 1, Q = s.npairs * ncols, nu = (Q + cap - 1) / cap;
         for (int u = 0; u < nu; ++u) {
-            const int q0 = (int)((int64_t)s.npairs * u / nu), q1 = (int)((int64_t)s.npairs * (u + 1) / nu);
-            g->sp_max_cnt = std::max(g->sp_max_cnt, q1 - q0);
+            const int q0 = (int)((int64_t)Q * u / nu), q1 = (int)((int64_t)Q * (u + 1) / nu);
             for (int k = 0; k * split_tile(nco) < nco; ++k)
-                units.push_back(SplitUnit{s.base, s.out0 + (int64_t)q0 * 2 * nco, s.sr, s.sc, s.pT, s.pS, s.rexp, s.dexp, s.react,
-                                          s.pair0 + q0, q1 - q0, k});
+            {
+                const int nr8 = (split_tile(nco) + 7) & ~7;
+                units.push_back(SplitUnit{s.dig + k * split_tile_bytes(s.pS, nr8), s.out0 * ncols + (int64_t)q0 * 2 * nco, s.pT,
+                                          s.pS, s.rexp, s.pair0, q0, q1 - q0, k});
+            }
         }
     }
     for (int l = nlev + 1, next = (int)units.size(); l >= 0; --l) {
-        if (g->sp_unit_start[l] < 0) g->sp_unit_start[l] = next;
-        next = g->sp_unit_start[l];
+        if (P.start[l] < 0) P.start[l] = next;
+        next = P.start[l];
     }
-    auto it = std::find(g->allocs.begin(), g->allocs.end(), (void*)g->d_sp_unit);
-    if (g->d_sp_unit && it != g->allocs.end()) { g->allocs.erase(it); dev_release(g->d_sp_unit); }   // units being replaced
-    g->d_sp_unit = dupload(g, units);
+    if (P.d_unit) {   // units being replaced; work queued on any stream may still read them
+        g->allocs.erase(std::find(g->allocs.begin(), g->allocs.end(), (void*)P.d_unit));
+        dev_release_now(P.d_unit);
+        P.d_unit = nullptr;
+    }
+    P.d_unit = dupload(g, units);
+    cuda_check(cudaStreamSynchronize(cudaStreamPerThread), "split M2L units");
+    P.ncols = ncols;
+}
+static const SplitPlan& split_plan(lfmm_geometry_s* g, int ncols) {
+    SplitPlan& P = g->sp_plan[ncols == 1 ? 0 : 1];
+    if (P.ncols != ncols) make_split_plan(g, P, ncols);
+    return P;
 }
 static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, const std::vector<int>& vr_src,
                         const std::vector<int>& vr_key, const std::vector<int>& vr_comp,
@@ -258,14 +269,28 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
             dexp.insert(dexp.end(), d.begin(), d.end());
         }
     // pairs per matrix: free-space canonical tables, then reaction keys
-    std::vector<int> cnt(nF + nR, 0);
-    for (int v : g->vf_tab_host) ++cnt[g->ftab_canon[v]];
-    for (int v : vr_key) ++cnt[nF + v];
+    // and, within one, per symmetry (reversal and quarter turns): sorted by it, a unit's columns
+    // are staged alike
+    std::vector<int> cnt(nF + nR, 0), var((size_t)(nF + nR) * 8, 0);
+    auto free_flags = [&](int tab) {
+        const int turn = g->ftab_turn[tab], mir = turn >> 2;
+        return (mir ? SP_REV : 0) | (((turn + 2 * mir) & 3) << SP_Q_SHIFT);
+    };
+    auto react_flags = [&](int e) {
+        const Component& C = t.comps[vr_comp[e]];
+        return (((C.a ? 0 : 1) ^ vr_flip[e]) ? SP_REV : 0) | ((C.a ? 0 : 2) << SP_Q_SHIFT);
+    };
+    auto variant = [](int flags) { return (flags & SP_REV) | (((flags >> SP_Q_SHIFT) & 3) << 1); };
+    for (int v : g->vf_tab_host) { ++cnt[g->ftab_canon[v]]; ++var[(size_t)g->ftab_canon[v] * 8 + variant(free_flags(v))]; }
+    for (size_t e = 0; e < vr_key.size(); ++e) { ++cnt[nF + vr_key[e]]; ++var[(size_t)(nF + vr_key[e]) * 8 + variant(react_flags((int)e))]; }
+    for (int i = 0; i < nF + nR; ++i)   // counts to first positions
+        for (int k = 0, o = 0; k < 8; ++k) { const int c = var[(size_t)i * 8 + k]; var[(size_t)i * 8 + k] = o; o += c; }
     std::vector<std::vector<int>> by_level(nlev);
     for (int i = 0; i < nF; ++i) if (cnt[i]) by_level[g->ftab_lev[i]].push_back(i);
     for (int i = 0; i < nR; ++i) if (cnt[nF + i]) by_level[keys[i].level].push_back(nF + i);
     std::vector<SplitTab> tabs;
-    std::vector<int> tab_of(nF + nR, -1), fill(nF + nR, 0);
+    std::vector<int> tab_of(nF + nR, -1);
+    int64_t dig = 0;
     int np = 0, nrexp = 0;
     int64_t rows = 0;
     for (int l = 0; l < nlev; ++l) {
@@ -285,6 +310,9 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
             s.rexp = nrexp; nrexp += nco * split_nseg(p);
             s.pair0 = np; s.npairs = cnt[i]; np += cnt[i];
             s.out0 = rows; rows += (int64_t)cnt[i] * 2 * nco;
+            const int tiles = (nco + split_tile(nco) - 1) / split_tile(nco);
+            s.dig = dig; dig += tiles * split_tile_bytes(p, (split_tile(nco) + 7) & ~7);
+            g->sp_max_tiles = std::max(g->sp_max_tiles, tiles);
             tab_of[i] = (int)tabs.size();
             s.level = l;
             tabs.push_back(s);
@@ -324,16 +352,14 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
         const int p = t.p_level[l], nco = 2 * p + 1;
         auto add = [&](int i, int vec, int fin, int fout, int d) {
             const SplitTab& s = tabs[tab_of[i]];
-            const int q = fill[i]++;
+            const int q = var[(size_t)i * 8 + variant(fin)]++;
             pairs[s.pair0 + q] = SplitPair{vec, fin};
             rowv[d].push_back(SplitRow{s.out0 + (int64_t)q * 2 * nco, fout, 0});
         };
         for (int T = t.level_start[l]; T < t.level_start[l + 1]; ++T) {
             for (int e = g->vf_ptr_host[T]; e < g->vf_ptr_host[T + 1]; ++e) {
-                const int tab = g->vf_tab_host[e], turn = g->ftab_turn[tab];
-                const int mir = turn >> 2, q = (turn + 2 * mir) & 3;
-                add(g->ftab_canon[tab], vec_of[g->vf_src_host[e]], (mir ? SP_REV : 0) | (q << SP_Q_SHIFT),
-                    (mir ? SP_REV : 0) | (((4 - q) & 3) << SP_Q_SHIFT), 0);
+                const int tab = g->vf_tab_host[e], fin = free_flags(tab), q = (fin >> SP_Q_SHIFT) & 3;
+                add(g->ftab_canon[tab], vec_of[g->vf_src_host[e]], fin, (fin & SP_REV) | (((4 - q) & 3) << SP_Q_SHIFT), 0);
             }
             for (int e = vr_ptr[T]; e < vr_ptr[T + 1]; ++e) {
                 const int S = vr_src[e];
@@ -341,10 +367,9 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
                 const int ssl = g->slot_of_host[2 * S + (C.a == 0 ? 0 : 1)];
                 const int side = (C.b == 0) ? 1 : 0;
                 const int d = (g->slot_of_host[2 * T + side] >= 0) ? 1 + side : 0;
-                const int rin = (C.a ? 0 : 1) ^ vr_flip[e], rout = (C.b ? 0 : 1) ^ vr_flip[e];
+                const int rout = (C.b ? 0 : 1) ^ vr_flip[e];
                 add(nF + vr_key[e], ssl >= 0 ? vec_of_slot[ssl] : vec_of[S],
-                    (rin ? SP_REV : 0) | ((C.a ? 0 : 2) << SP_Q_SHIFT),
-                    (rout ? SP_REV : 0) | ((C.b ? 0 : 2) << SP_Q_SHIFT), d);
+                    react_flags(e), (rout ? SP_REV : 0) | ((C.b ? 0 : 2) << SP_Q_SHIFT), d);
             }
             for (int d = 0; d < 3; ++d) {
                 const int ts = d == 0 ? -1 : g->slot_of_host[2 * T + d - 1];
@@ -368,7 +393,11 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     g->d_sp_rexp = dalloc<int>(g, (size_t)std::max(nrexp, 1));
     g->sp_ntab = (int)tabs.size();
     g->sp_tabs_host = tabs;
-    make_split_units(g, SP_COLS);
+    g->sp_dig_bytes = dig;
+    g->d_sp_dig = dalloc<unsigned char>(g, (size_t)dig);
+    g->d_sp_ctr = dalloc<int>(g, 1);
+    g->sp_cap = SP_COLS;
+    make_split_plan(g, g->sp_plan[0], 1);
     g->sp_rows = rows;
     split_alloc(g, 1);
     cuda_check(cudaHostAlloc((void**)&g->wait_err, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable), "wait status");
@@ -795,6 +824,9 @@ void fmm_build(lfmm_geometry_s* g) {
         if (g->sp_ntab > 0) {
             k_split_rexp<<<g->sp_ntab, 128>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_sp_dexp, g->d_sp_rexp);
             cuda_check(cudaGetLastError(), "k_split_rexp");
+            k_split_digits<<<dim3(g->sp_ntab, g->sp_max_tiles), 256>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_sp_dexp,
+                                                                      g->d_sp_rexp, g->d_sp_dig);
+            cuda_check(cudaGetLastError(), "k_split_digits");
         }
     }
     cuda_check(cudaStreamSynchronize(cudaStreamPerThread), "fmm_build");
@@ -863,6 +895,7 @@ static void launch_m2l_reduce(lfmm_geometry_s* g, int nrhs, int r1, cudaStream_t
 // The split M2L's workspace: one row of products per (pair, column), for as many columns
 // at once as fit SP_WS_BYTES (at least one); a wider block takes several rounds.
 #define SP_WS_BYTES (2ll << 30)
+#define SP_SMS 152   // persistent CTAs of k_split: one per SM
 static int split_round(const lfmm_geometry_s* g, int nrhs) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(nrhs, 2048), SP_WS_BYTES / (int64_t)split_col_bytes(g)));
 }
@@ -880,25 +913,26 @@ void split_check_waits(lfmm_geometry_s* g) {
     throw TimeoutError{"split M2L: an mbarrier wait gave up; that product's M2L contributions were zeroed"};
 }
 static SplitArgs split_args(lfmm_geometry_s* g, int col0, int ncols) {
-    return SplitArgs{g->d_sp_vec, g->d_sp_pair, g->d_sp_unit, g->d_sp_row, g->d_sp_dst, g->d_sp_rexp, g->d_sp_dexp,
-                     g->d_m2lf, g->d_m2lr, g->d_M, g->d_Mp, g->d_L, g->d_Lp, g->ncoef, g->nslotcoef,
+    const SplitPlan& P = split_plan(g, ncols);
+    return SplitArgs{g->d_sp_vec, g->d_sp_pair, P.d_unit, g->d_sp_ctr, g->d_sp_row, g->d_sp_dst, g->d_sp_rexp, g->d_sp_dexp,
+                     g->d_sp_dig, g->d_M, g->d_Mp, g->d_L, g->d_Lp, g->ncoef, g->nslotcoef,
                      g->d_sp_vdig, g->d_sp_vexp, g->sp_nvec, g->d_sp_ws, col0, ncols, g->wait_err};
 }
-static int split_chunks(const lfmm_geometry_s* g, int ncols) { return (g->sp_max_cnt * ncols + SP_COLS - 1) / SP_COLS; }
 // FP64 M2L of the levels below lm
 static void launch_split(lfmm_geometry_s* g, int nrhs, int lm, cudaStream_t s) {
     split_check_waits(g);
     ensure_split(g, nrhs);
-    const int nu = g->sp_unit_start[lm], nd = g->sp_dst_start[lm];
+    const int nd = g->sp_dst_start[lm];
     raise_smem_limit((const void*)k_split, SP_SMEM, "split M2L smem");
     for (int c0 = 0; c0 < nrhs && nd > 0; c0 += g->sp_ws_cols) {
         const SplitArgs a = split_args(g, c0, std::min(nrhs - c0, g->sp_ws_cols));
+        const int nu = split_plan(g, a.ncols).start[lm];
         if (nu > 0) {
             const int nv = g->sp_vec_start[lm];
             k_split_vec<<<dim3((nv + 3) / 4, a.ncols), 128, 0, s>>>(a, 0, nv);
             cuda_check(cudaGetLastError(), "k_split_vec");
             ++g->n_launches;
-            k_split<<<dim3(nu, split_chunks(g, a.ncols)), 256, SP_SMEM, s>>>(a);
+            k_split<<<std::min(nu, SP_SMS), SP_THREADS, SP_SMEM, s>>>(a, nu);
             cuda_check(cudaGetLastError(), "k_split");
             ++g->n_launches;
         }
@@ -1050,7 +1084,6 @@ struct XJob {
 };
 struct SplitJob {
     SplitArgs a;
-    int chunks;   // column chunks per unit
     int vblocks;  // blocks of k_split_vec per column
 };
 
@@ -1089,12 +1122,6 @@ __global__ void __launch_bounds__(128) k_split_vec_multi(const SplitJob* __restr
     const int j = job_of(prefix, njobs, blockIdx.x);
     const int b = blockIdx.x - prefix[j], vb = jobs[j].vblocks;
     split_vec(jobs[j].a, b % vb, b / vb, 0, (int)jobs[j].a.nvec);
-}
-__global__ void __launch_bounds__(256, 2) k_split_multi(const SplitJob* __restrict__ jobs,
-                                                        const int* __restrict__ prefix, int njobs) {
-    const int j = job_of(prefix, njobs, blockIdx.x);
-    const int b = blockIdx.x - prefix[j], ch = jobs[j].chunks;
-    split_unit(jobs[j].a, b / ch, b % ch);
 }
 __global__ void __launch_bounds__(192) k_split_reduce_multi(const SplitJob* __restrict__ jobs,
                                                             const int* __restrict__ prefix, int njobs) {
@@ -1192,21 +1219,33 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
     raise_smem_limit((const void*)k_split_multi, SP_SMEM, "split M2L smem");
     for (int round = 0;; ++round) {
         std::vector<SplitJob> jobs;
-        std::vector<int> blocks, rblocks, vblocks;
+        std::vector<SplitArgs> args;
+        std::vector<int> rblocks, vblocks, prefix(1, 0);
         for (const BatchOp* op : far) {
             lfmm_geometry_s* g = op->g;
             const int c0 = round * g->sp_ws_cols, D = g->tree.D;
             if (c0 >= op->nrhs) continue;
             const int nc = std::min(op->nrhs - c0, g->sp_ws_cols);
             const int vb = (g->sp_nvec + 3) / 4;
-            jobs.push_back(SplitJob{split_args(g, c0, nc), split_chunks(g, nc), vb});
+            jobs.push_back(SplitJob{split_args(g, c0, nc), vb});
+            args.push_back(jobs.back().a);
             vblocks.push_back(vb * nc);
-            blocks.push_back(g->sp_unit_start[D + 1] * split_chunks(g, nc));
+            prefix.push_back(prefix.back() + split_plan(g, nc).start[D + 1]);
             rblocks.push_back(g->sp_dst_start[D + 1] * nc);
         }
         if (jobs.empty()) break;
         launch_jobs(jobs, vblocks, k_split_vec_multi, 128, 0, s, "k_split_vec_multi");
-        launch_jobs(jobs, blocks, k_split_multi, 256, SP_SMEM, s, "k_split_multi");
+        if (prefix.back() > 0) {   // persistent: a CTA takes units of every geometry in turn
+            JobTables t;
+            const size_t oj = t.add(args.data(), sizeof(SplitArgs) * args.size());
+            const size_t op = t.add(prefix.data(), sizeof(int) * prefix.size());
+            t.upload(s);
+            k_split_multi<<<std::min(prefix.back(), SP_SMS), SP_THREADS, SP_SMEM, s>>>(t.at<SplitArgs>(oj), t.at<int>(op),
+                                                                                      (int)args.size());
+            const cudaError_t e = cudaGetLastError();
+            t.release(s);
+            cuda_check(e, "k_split_multi");
+        }
         launch_jobs(jobs, rblocks, k_split_reduce_multi, 192, 0, s, "k_split_reduce_multi");
     }
     // L2L: pass k takes each geometry's children at level l0 + 1 + k
@@ -1260,7 +1299,8 @@ void fmm_autotune(lfmm_geometry_s* g) {
     int best_work = M2L_ITEM_WORK;
     double best = 1e300, dflt = 0.0;
     for (int work : {1024, M2L_ITEM_WORK}) {   // 16 and 32 pairs
-        make_split_units(g, std::min(SP_COLS, work / 64));
+        g->sp_cap = std::min(SP_COLS, work / 64);
+        make_split_plan(g, g->sp_plan[0], 1);
         for (int r = 0; r < 2; ++r) launch_split(g, 1, t.D + 1, s);
         cuda_check(cudaEventRecord(e0, s), "event");
         for (int r = 0; r < 3; ++r) launch_split(g, 1, t.D + 1, s);
@@ -1274,7 +1314,8 @@ void fmm_autotune(lfmm_geometry_s* g) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    make_split_units(g, std::min(SP_COLS, best_work / 64));
+    g->sp_cap = std::min(SP_COLS, best_work / 64);
+    make_split_plan(g, g->sp_plan[0], 1);
     make_m2l_items(g, best_work, 1);
     cuda_check(cudaStreamSynchronize(s), "tune");
     g->n_launches = launches;

@@ -142,6 +142,7 @@ struct M2LReduce {
 struct SplitTab {
     int64_t base;
     int64_t out0;      // first workspace row of its pairs (doubles, one column)
+    int64_t dig;       // its digits (bytes)
     int sr, sc;
     int pT, pS;        // orders of the result and of the source
     int rexp, dexp;    // offsets of its row exponents and of its source scales (by |n|)
@@ -166,10 +167,16 @@ struct SplitRow {
     int64_t row;       // the pair's workspace row (doubles, one column)
     int flags, pad;
 };
-struct SplitUnit {     // up to SP_COLS pairs of one matrix, one row tile
-    int64_t base, out0;         // as the matrix's; out0 of the first pair
-    int sr, sc, pT, pS, rexp, dexp, react;
-    int pair0, cnt, tile;
+struct SplitUnit {     // up to SP_COLS (pair, right-hand side) columns of one matrix, one row tile
+    int64_t dig, out0;          // the tile's digits; workspace row of the first column
+    int pT, pS, rexp;           // as the matrix's
+    int pair0, col0, cnt, tile; // the matrix's first pair; column c is pair c / ncols
+};
+// the units for blocks of ncols right-hand sides, coarse levels first
+struct SplitPlan {
+    int ncols = 0;
+    SplitUnit* d_unit = nullptr;
+    std::vector<int> start;     // [nlev + 2]: first unit of each level
 };
 struct SplitDst {
     int64_t off;       // coefficient offset of the local expansion (L, or Lp with slot)
@@ -180,10 +187,11 @@ struct SplitArgs {
     const SplitVec* vec;
     const SplitPair* pair;
     const SplitUnit* unit;
+    int* ctr;                     // next unit
     const SplitRow* row;
     const SplitDst* dst;
     const int *rexp, *dexp;
-    const cd *tf, *tr;            // Toeplitz vectors, reaction tables
+    const unsigned char* dig;     // the matrices' digits
     const cd *M, *Mp;
     cd *L, *Lp;
     int64_t ncoef, nslotcoef;
@@ -328,16 +336,20 @@ struct lfmm_geometry_s {
     lfmm::SplitTab* d_sp_tab = nullptr;
     lfmm::SplitVec* d_sp_vec = nullptr;
     lfmm::SplitPair* d_sp_pair = nullptr;
-    lfmm::SplitUnit* d_sp_unit = nullptr;
     lfmm::SplitRow* d_sp_row = nullptr;
     lfmm::SplitDst* d_sp_dst = nullptr;
     int *d_sp_rexp = nullptr, *d_sp_dexp = nullptr;
-    std::vector<int> sp_unit_start, sp_dst_start, sp_vec_start;   // [nlev + 2]: first unit / destination / vector of each level
+    unsigned char* d_sp_dig = nullptr;              // the matrices' digits
+    int64_t sp_dig_bytes = 0;
+    int* d_sp_ctr = nullptr;
+    int sp_max_tiles = 1;
+    lfmm::SplitPlan sp_plan[2];                     // one column; the block width used last
+    int sp_cap = 0;                                 // most columns of a unit (LFMM_AUTOTUNE)
+    std::vector<int> sp_dst_start, sp_vec_start;    // [nlev + 2]: first destination / vector of each level
     uint32_t* d_sp_vdig = nullptr;                  // digits and exponents of the vectors, sp_ws_cols columns
     int* d_sp_vexp = nullptr;
     int sp_nvec = 0;
     int sp_ntab = 0;
-    int sp_max_cnt = 0;                             // largest pair count of a unit
     int64_t sp_rows = 0;                            // workspace doubles per column
     double* d_sp_ws = nullptr;
     int sp_ws_cols = 0;                             // columns it holds

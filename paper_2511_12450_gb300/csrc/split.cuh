@@ -34,30 +34,26 @@
 // gave 9.9e-8.)  The sums of digits are exact, so a product does not depend on how pairs
 // are grouped into CTAs, on the columns beside it or on the launch it is part of.
 //
-// k_split_vec writes every source vector's digits once (a vector serves about 7 pairs).
-// k_split: one CTA (8 warps) per unit, up to 32 (pair, right-hand side) columns of one
-// matrix and up to 64 of its complex rows.  Real form, one MMA tile of 128 rows:
-//   [Re y; Im y] = [zr, -zi; zi, zr] [vr; vi], K index 2 position + part,
-// the unit's Re rows first, its Im rows from the next multiple of 8.  Positions run over a
+// k_split_digits writes every matrix's digits once per geometry (5 times its FP64 size),
+// k_split_vec every source vector's once per product (a vector serves about 7 pairs).
+// k_split: a unit is up to 32 (pair, right-hand side) columns of one matrix and up to 64 of its
+// complex rows: one MMA tile of 128 rows, K index 2 position + part.  Positions run over a
 // segment's n = -h..-0, 0..h, so that n -> -n reverses them (the second 0 has a zero column).
-// The matrix is staged in chunks of 24 (up to 96 rows) or 16 positions straight from its FP64
-// values (a digit costs about three integer instructions; keeping the matrices as digits
-// would cost 4 times their memory and traffic), in the K-major canonical layout without
-// swizzle.  The vectors' digits lie side by side along N, digit j in columns
-// [j C, (j + 1) C), so that A_i times the first 8 - i digits is ONE MMA into the
-// accumulator columns from i C on: its digit j lands in accumulator i + j.  The first MMA
-// (N = 8 C) initialises all eight accumulators.  A digit's rows end where the next digit's
-// begin: an MMA of 128 rows over a unit of fewer reads on into them, and the product's rows
-// past the unit's are not read back.  Two CTAs fit an SM (96 KB of shared memory, 256 TMEM
-// columns each) and overlap staging with the other's MMAs.
+// The vectors' digits lie side by side along N, digit j in columns [j C, (j + 1) C), so that
+// A_i times the first 8 - i digits is ONE MMA into the accumulator columns from i C on: its
+// digit j lands in accumulator i + j.  The first MMA (N = 8 C) initialises all eight
+// accumulators.  A digit's rows end where the next digit's begin: an MMA of 128 rows over a
+// unit of fewer reads on into them, and the product's rows past the unit's are not read back.
+// Operands are in the K-major canonical layout without swizzle.
 //
 // The products are written to a workspace, one row of 2 (2p + 1) doubles per (pair,
 // column); k_split_reduce adds every target's rows in list order.
 //
-// Measured at N = 65,536, three layers (72,000 pairs, 2,700 matrices, orders 57 to 20): 270 us
-// for the three kernels where the FP64 FMA kernel took 1,040 us at 97% of the FP64 pipe.
-// Bound by the issue of the staging and of the combination of accumulators (tensor pipe
-// 14% busy, 1.5 of 4 instructions per cycle).
+// Measured at N = 65,536, three layers (72,000 pairs, 2,000 matrices, orders 57 to 20): k_split
+// 172 us, k_split_vec 9, k_split_reduce 34, where the FP64 FMA kernel took 1,040 us at 97% of
+// the FP64 pipe; at N = 262,144 1.0 ms against 5.7.  About equally bound by the MMAs' issue (112 us
+// with nothing else left in the kernel), the gathering of the columns and the combination of
+// the accumulators.
 #pragma once
 
 #include "devmath.cuh"
@@ -72,8 +68,6 @@ namespace lfmm {
 #define SP_COLS 32                  // columns per unit
 #define SP_ND 8                     // digits
 #define SP_PLANE 9216u              // most bytes of one digit of A: 96 rows x 48, 128 x 32
-#define SP_SMEM (SP_ND * SP_PLANE + SP_ND * SP_COLS * 96u)
-#define SP_TMEM 256u
 #define SP_NONE (-100000)           // column exponents: all zero, not finite
 #define SP_INF (1 << 20)
 #define SP_WAIT_LIMIT (1 << 24)
@@ -98,12 +92,6 @@ __device__ __forceinline__ bool sp_wait(uint32_t mbar, uint32_t parity) {
                      "selp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done) : "r"(mbar), "r"(parity));
     return done != 0;
-}
-
-// The whole CTA's wait: one thread polls, the others stand at the barrier (eight polling
-// warps took half of the SM's issue slots from the staging of the CTA beside this one)
-__device__ __forceinline__ bool sp_wait_all(uint32_t mbar, uint32_t parity, int tid) {
-    return __syncthreads_and(tid == 0 ? sp_wait(mbar, parity) : 1) != 0;
 }
 
 // biased exponent field of a double (0: zero or subnormal, taken as zero; 2047: not finite)
@@ -154,17 +142,23 @@ __device__ __forceinline__ cd sp_turn(cd z, int s) {
     return mk(dsign(x, ((s + 1) >> 1)), dsign(y, s >> 1));
 }
 
-// T 2^x as a double, rounded to nearest (integer instructions only: the FP64 pipe is slow)
-__device__ __forceinline__ double sp_value(long long T, int x) {
+// (2^32 hi + lo) 2^x as a double, for |hi| < 2^43 and |lo| < 2^48, in integer instructions (three
+// FP64 additions instead made the epilogue the longest part of a unit: the FP64 pipe takes 16
+// cycles for a warp's).  The sum is cut at 2^12, or for |hi| < 2^30 not at all (terms that
+// cancel, or a vector that is small where the row is large: a fixed cut left 1.4e-9 in the
+// sparse four-layer case), and the 63 bits are rounded to nearest.
+__device__ __forceinline__ double sp_value(long long hi, long long lo, int x) {
+    const bool fits = (unsigned long long)(hi + (1ll << 30)) < (1ull << 31);
+    const long long T = fits ? hi * (1ll << 32) + lo : hi * (1ll << 20) + (lo >> 12);
     const uint64_t m = T < 0 ? 0ull - (uint64_t)T : (uint64_t)T;
-    if (m == 0) return 0.0;
     const int lz = __clzll((long long)m);
-    const uint64_t s = m << lz;                                // top bit at 63
+    const uint64_t s = m << (lz & 63);                         // top bit at 63
     const uint64_t f = (s >> 11) + ((s >> 10) & 1);            // 53 bits (or 2^53)
-    const int e = 1023 + 63 - lz + x;
-    if (e < 1) return 0.0;
-    uint64_t b = ((uint64_t)(e - 1) << 52) + f;
-    if (e > 2046 || b >= 0x7ff0000000000000ull) b = 0x7ff0000000000000ull;
+    const int e = 1023 + 63 + (fits ? 0 : 12) - lz + x;
+    // selects, not branches: the columns of a group run side by side
+    uint64_t b = ((uint64_t)(uint32_t)(e - 1) << 52) + f;
+    b = e > 2046 || b >= 0x7ff0000000000000ull ? 0x7ff0000000000000ull : b;
+    b = m == 0 || e < 1 ? 0ull : b;
     return __longlong_as_double((long long)(b | ((uint64_t)T & 0x8000000000000000ull)));
 }
 
@@ -181,6 +175,13 @@ __host__ __device__ inline int split_vals(int p, int seg) {
     return h < z ? h : z;
 }
 __host__ __device__ inline int split_half(int p, int seg) { return (split_vals(p, seg) + 3) & ~3; }
+// positions of all segments, and the digits of one row tile of nr8 rows of each part
+__host__ __device__ inline int split_positions(int p) {
+    int n = 0;
+    for (int seg = 0; seg < split_nseg(p); ++seg) n += 2 * split_half(p, seg);
+    return n;
+}
+__host__ __device__ inline int64_t split_tile_bytes(int p, int nr8) { return (int64_t)split_positions(p) * nr8 * (8 * SP_ND); }
 // |n| less the segment's first at position k of a segment of half length H; n < 0 in the first half
 __device__ __forceinline__ int split_abs(int k, int H) { return k < H ? H - 1 - k : k - H; }
 
@@ -205,11 +206,76 @@ __global__ void __launch_bounds__(128) k_split_rexp(const SplitTab* __restrict__
     }
 }
 
+// The matrices as digits, once per geometry, in the order the MMAs read them: per row tile
+// and chunk of positions eight planes in the K-major canonical layout (core matrices of 8
+// rows x 16 bytes, contiguous along K), Re rows first, Im rows from nr8:
+//   [Re y; Im y] = [zr, -zi; zi, zr] [vr; vi].
+// A chunk is one contiguous block, so a bulk copy stages it.  Converting the FP64 tables in
+// every product instead took a third of the instructions of the product kernel (256 us at N =
+// 65,536, where copies of the 330 MB of digits take about 50).  One CTA per (matrix, tile).
+__device__ __forceinline__ void split_load(cd (&z)[4], const cd* __restrict__ A, int sr, int sc, int r, int k, int H,
+                                           int h, int n1) {
+    // row r's entries at positions k..k+3 of a segment (A at column n = 0); the positions past
+    // |n| = p and the second one of n = 0 are zero
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int j = split_abs(k + i, H), a = n1 + j;
+        z[i] = mk(0, 0);
+        if (j < h && !(k + i >= H && a == 0)) z[i] = A[(int64_t)r * sr + (int64_t)(k + i < H ? -a : a) * sc];
+    }
+}
+__global__ void __launch_bounds__(256) k_split_digits(const SplitTab* __restrict__ tabs, const cd* __restrict__ tf,
+                                                      const cd* __restrict__ tr, const int* __restrict__ dexp,
+                                                      const int* __restrict__ rexp, unsigned char* __restrict__ dig) {
+    const SplitTab t = tabs[blockIdx.x];
+    const int nT = 2 * t.pT + 1, per = split_tile(nT), n0 = blockIdx.y * per;
+    if (n0 >= nT) return;
+    const int nt = min(per, nT - n0), nr8 = (per + 7) & ~7, KC = split_chunk(nT);
+    const cd* A = (t.react ? tr : tf) + t.base + (int64_t)n0 * t.sr + (int64_t)t.pS * t.sc;   // column n = 0
+    unsigned char* out = dig + t.dig + (int64_t)blockIdx.y * split_tile_bytes(t.pS, nr8);
+    for (int seg = 0; seg < split_nseg(t.pS); ++seg) {
+        const int H = split_half(t.pS, seg), h = split_vals(t.pS, seg), n1 = split_size(t.pS) * seg;
+        for (int k0 = 0; k0 < 2 * H; k0 += KC) {
+            const int ng = min(2 * H - k0, KC) >> 2;
+            const uint32_t sbo = (uint32_t)ng * 128u, plane = (uint32_t)(nr8 >> 2) * sbo;
+            for (int q = threadIdx.x; q < nr8 * ng; q += blockDim.x) {
+                const int g = q / nr8, r = q - g * nr8, k = k0 + 4 * g;
+                uint2 dr[4], di[4];
+                cd z[4] = {mk(0, 0), mk(0, 0), mk(0, 0), mk(0, 0)};
+                if (r < nt) split_load(z, A, t.sr, t.sc, r, k, H, h, n1);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int adj = 1022 + (r < nt ? rexp[t.rexp + seg * nT + n0 + r] : 0) +
+                                    dexp[t.dexp + min(n1 + split_abs(k + i, H), t.pS)];
+                    dr[i] = sp_digits(z[i].x, adj);
+                    di[i] = sp_digits(z[i].y, adj);
+                }
+                const int rr = nr8 + r;
+                unsigned char* ar = out + (uint32_t)(r >> 3) * sbo + (uint32_t)g * 128u + (uint32_t)(r & 7) * 16u;
+                unsigned char* ai = out + (uint32_t)(rr >> 3) * sbo + (uint32_t)g * 128u + (uint32_t)(rr & 7) * 16u;
+#define SP_STORE_A(J)                                                                                          \
+    {                                                                                                          \
+        const uint32_t h0 = sp_digit<J>(dr[0], di[0]), h1 = sp_digit<J>(dr[1], di[1]),                         \
+                       h2 = sp_digit<J>(dr[2], di[2]), h3 = sp_digit<J>(dr[3], di[3]);                         \
+        *(uint4*)(ar + J * plane) =                                                                            \
+            make_uint4(h0 ^ 0x80000000u, h1 ^ 0x80000000u, h2 ^ 0x80000000u, h3 ^ 0x80000000u);                \
+        *(uint4*)(ai + J * plane) = make_uint4(__byte_perm(h0, h0, 0x1032), __byte_perm(h1, h1, 0x1032),       \
+                                               __byte_perm(h2, h2, 0x1032), __byte_perm(h3, h3, 0x1032));      \
+    }
+                SP_STORE_A(0) SP_STORE_A(1) SP_STORE_A(2) SP_STORE_A(3) SP_STORE_A(4) SP_STORE_A(5) SP_STORE_A(6) SP_STORE_A(7)
+#undef SP_STORE_A
+            }
+            out += (int64_t)SP_ND * plane;
+        }
+    }
+}
+
 // The source vectors as digits: per (vector, segment) eight planes of SP_POS words (a word is
 // the FP16 pair (re, im) of one coefficient's digit) and the exponent.  One warp per (vector,
 // segment); a vector serves all its pairs (about 7 at one column).
 __device__ __forceinline__ void split_vec(const SplitArgs& S, int block, int column, int v0, int nv) {
     const int w = block * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (block == 0 && column == 0 && threadIdx.x == 0) *S.ctr = 0;   // k_split's counter
     if (w >= nv) return;
     const SplitVec V = S.vec[v0 + w];
     const int col = S.col0 + column;
@@ -256,228 +322,487 @@ __global__ void __launch_bounds__(128) k_split_vec(const SplitArgs S, int v0, in
     split_vec(S, blockIdx.x, blockIdx.y, v0, nv);
 }
 
-// row r's entries at positions k..k+3 of a segment (A at column n = 0); the positions past
-// |n| = p and the second one of n = 0 are zero
-__device__ __forceinline__ void split_load(cd (&z)[4], const cd* __restrict__ A, int sr, int sc, int r, int k, int H,
-                                           int h, int n1) {
+// ---- k_split: one persistent CTA per SM of 23 warps, each unit's work passing through
+//  - a warp that loads the units' descriptors ahead into a ring of eight;
+//  - a thread that brings the matrix's chunks by bulk copies into two buffers (a chunk that a
+//    buffer still holds, as when the next unit has the same matrix of two chunks, is kept);
+//  - two staging groups of 4 warps, taking turns by chunk, which gather the chunk's part of the
+//    columns' digits (a group's loads run while the other group stores);
+//  - the MMA warp, which issues a chunk's MMAs when its group has staged it, into the
+//    accumulator set of the chunk's segment (two sets);
+//  - twelve epilogue warps, which combine a segment's accumulators while the next one is built.
+// A CTA takes runs of consecutive units (often of one matrix) from a counter, the coarse
+// levels' long ones first.  The warps meet at
+// mbarriers: info (descriptor there), slotfree (everyone is done with it), full
+// (staged), empty (its MMAs are done), accfull, accempty.
+#define SP_STAGE_WARPS 8
+#define SP_EPI_WARPS 12
+#define SP_MMA_WARP (SP_STAGE_WARPS + SP_EPI_WARPS)
+#define SP_THREADS (32 * (SP_MMA_WARP + 3))
+#define SP_BUF (SP_ND * SP_PLANE + SP_ND * SP_COLS * 96u)   // A's planes, then B's
+#define SP_SMEM (2u * SP_BUF)
+#define SP_TMEM 512u
+#define SP_RING 8
+#define SP_RUN 4          // units a CTA takes at a time
+struct SplitSlot {   // a unit's descriptor; u.cnt = 0: no more
+    SplitUnit u;
+    const SplitArgs* args;
+    int flag[SP_COLS];
+    int64_t vec[SP_COLS];   // the columns' vectors (index of their first segment)
+};
+struct SplitShared {
+    SplitSlot ring[SP_RING];
+    uint64_t full[2], empty[2], accfull[2], accempty[2], info[SP_RING], slotfree[SP_RING];
+    uint32_t tmem;
+    volatile int dead;   // a wait gave up: everyone leaves
+};
+
+// a warp's wait on an mbarrier phase; false once any wait of the CTA has given up
+__device__ __forceinline__ bool sp_wait_warp(SplitShared& sh, uint64_t* bar, uint32_t parity) {
+    if ((threadIdx.x & 31) == 0) {
+        const uint32_t mb = sp_saddr(bar);
+        uint32_t done = 0;
+        for (int it = 0; it < SP_WAIT_LIMIT && !done; ++it) {
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                         "selp.u32 %0, 1, 0, p;\n\t}"
+                         : "=r"(done) : "r"(mb), "r"(parity) : "memory");
+            if (!done && (it & 255) == 255 && sh.dead) break;
+        }
+        if (!done) sh.dead = 1;
+    }
+    __syncwarp();
+    return sh.dead == 0;
+}
+__device__ __forceinline__ void sp_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sp_saddr(bar)) : "memory");
+}
+__device__ __forceinline__ void sp_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sp_saddr(bar)) : "memory");
+}
+
+__device__ __forceinline__ bool sp_elect() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
+// one chunk's MMAs, KS K steps: A_i times the first 8 - i digits into accumulators i..7.  The
+// flow around an MMA is free of branches and of predicates but for the very first one's: 43
+// cycles an MMA at small N and the full rate (128) at N = 256, with one condition per MMA 92
+template <int KS>
+__device__ __forceinline__ void sp_chunk(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t first, uint32_t astep,
+                                         uint32_t C) {
+    sp_mma(d, da, db, idesc, first);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int j = split_abs(k + i, H), a = n1 + j;
-        z[i] = mk(0, 0);
-        if (j < h && !(k + i >= H && a == 0)) z[i] = A[(int64_t)r * sr + (int64_t)(k + i < H ? -a : a) * sc];
+    for (int ks = 1; ks < KS; ++ks) sp_mma(d, da + ks * 16, db + ks * 16, idesc, 1u);
+#pragma unroll 1
+    for (int i = 1; i < SP_ND; ++i) {
+        da += astep;
+        d += C;
+        idesc -= C >> 3 << 17;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) sp_mma(d, da + ks * 16, db + ks * 16, idesc, 1u);
     }
 }
 
-// shared memory of one unit beside the operands
-struct SplitShared {
-    int rexp[SP_MAXSEG * 64], dexp[LFMM_PMAX + 1], flag[SP_COLS];
-    int64_t vec[SP_COLS];   // the columns' vectors (index of their first segment)
+// geometry of a unit
+struct SplitGeo {
+    int nT, pS, nseg, n0, nt, nr8, KC, lc, C;
+    __device__ __forceinline__ explicit SplitGeo(const SplitUnit& U) {
+        nT = 2 * U.pT + 1;
+        pS = U.pS;
+        nseg = split_nseg(pS);
+        const int per = split_tile(nT);
+        n0 = U.tile * per;
+        nt = min(per, nT - n0);
+        nr8 = (per + 7) & ~7;
+        KC = split_chunk(nT);   // positions per chunk: 24 up to 96 rows, else 16
+        lc = U.cnt <= 16 ? 4 : 5;
+        C = 1 << lc;
+    }
 };
 
-__device__ __forceinline__ void split_unit(const SplitArgs& S, int ui, int chunk) {
-    extern __shared__ __align__(1024) unsigned char sp_sm[];
-    __shared__ __align__(8) uint64_t mbar;
-    __shared__ uint32_t tmem_base;
-    __shared__ SplitShared sh;
-    const SplitUnit U = S.unit[ui];
-    const int tot = U.cnt * S.ncols, c0 = chunk * SP_COLS;
-    if (c0 >= tot) return;
-    const int cnt = min(SP_COLS, tot - c0);
-    const int lc = cnt <= 16 ? 4 : 5, C = 1 << lc;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid < cnt) {   // first: a chain of loads hangs on the columns' vectors
-        const int q = (c0 + tid) / S.ncols, rhs = (c0 + tid) - q * S.ncols;
-        const SplitPair P = S.pair[U.pair0 + q];
-        sh.flag[tid] = P.flags;
-        sh.vec[tid] = (int64_t)rhs * S.nvec + P.vec;
+// four coefficients' digit words, turned by i^t of each (sel, sgn) and, with REV, in reverse
+template <bool REV, bool ODD>
+__device__ __forceinline__ uint4 sp_turned(uint4 w, const uint32_t (&sel)[4], const uint32_t (&sgn)[4]) {
+    if (REV) w = make_uint4(w.w, w.z, w.y, w.x);
+    if (ODD)
+        w = make_uint4(__byte_perm(w.x, w.x, sel[0]), __byte_perm(w.y, w.y, sel[1]), __byte_perm(w.z, w.z, sel[2]),
+                       __byte_perm(w.w, w.w, sel[3]));
+    return make_uint4(w.x ^ sgn[0], w.y ^ sgn[1], w.z ^ sgn[2], w.w ^ sgn[3]);
+}
+// B: the digits of 4 positions at k (group g of the chunk, 8-row groups sbo apart) of column bc
+// (the words are loaded beforehand by split_load_b)
+__device__ __forceinline__ void split_load_b(uint4 (&w)[SP_ND], const SplitArgs& S, const SplitSlot& sl, int bc, int k, int seg,
+                                             int H) {
+    if (bc >= sl.u.cnt) return;
+    const int P = k >> 2;
+    const uint4* src = (const uint4*)(S.vdig + (sl.vec[bc] + seg) * (SP_ND * SP_POS)) +
+                       ((sl.flag[bc] & SP_REV) ? (H >> 1) - 1 - P : P);
+#pragma unroll
+    for (int j = 0; j < SP_ND; ++j) w[j] = src[j * (SP_POS / 4)];
+}
+__device__ __forceinline__ void split_stage_b(const uint4 (&w)[SP_ND], const SplitSlot& sl, int C, uint32_t sbo, unsigned char* sB,
+                                              int bc, int g, int k, int seg, int H, int n1) {
+    unsigned char* bp = sB + (uint32_t)(bc >> 3) * sbo + (uint32_t)g * 128u + (uint32_t)(bc & 7) * 16u;
+    const uint32_t bs = (uint32_t)(C >> 3) * sbo;   // a digit's rows
+    if (bc >= sl.u.cnt) {
+#pragma unroll
+        for (int j = 0; j < SP_ND; ++j) *(uint4*)(bp + j * bs) = make_uint4(0, 0, 0, 0);
+        return;
     }
-    const int nT = 2 * U.pT + 1, pS = U.pS, nseg = split_nseg(pS);
-    const int per = split_tile(nT), n0 = U.tile * per, nt = min(per, nT - n0), nr8 = (per + 7) & ~7;
-    const cd* A = (U.react ? S.tr : S.tf) + U.base + (int64_t)n0 * U.sr + (int64_t)pS * U.sc;   // column n = 0
-    // positions per chunk: 24 up to 96 rows, else 16; 8-row groups sbo apart
-    const int KC = split_chunk(nT);
-    const uint32_t sbo = (uint32_t)KC * 32u, plane = (uint32_t)(nr8 >> 2) * sbo;
-    unsigned char* sA = sp_sm;
-    unsigned char* sB = sp_sm + SP_ND * SP_PLANE;
-    const uint32_t mb = sp_saddr(&mbar);
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sp_saddr(&tmem_base)),
+    const int f = sl.flag[bc], turn = (f >> SP_Q_SHIFT) & 3;
+    const bool rev = (f & SP_REV) != 0;
+    // i^(turn m) v_m, m the coefficient's index: n at its position, -n reversed; n grows by one
+    // along the group (H is a multiple of 4, so a group lies in one half)
+    const int nf = k < H ? -(n1 + H - 1 - k) : n1 + k - H, m0 = rev ? -nf : nf, dm = rev ? -turn : turn;
+    uint32_t sel[4], sgn[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int t = (turn * m0 + dm * i) & 3;
+        sel[i] = (t & 1) ? 0x1032u : 0x3210u;
+        sgn[i] = (((t + 1) & 2) << 14) | ((uint32_t)(t & 2) << 30);   // real part: t = 1, 2; imaginary: 2, 3
+    }
+    // pairs are sorted by their symmetry, so a warp's columns mostly take one branch
+    if (rev) {
+        if (turn & 1) {
+#pragma unroll
+            for (int j = 0; j < SP_ND; ++j) *(uint4*)(bp + j * bs) = sp_turned<true, true>(w[j], sel, sgn);
+        } else {
+#pragma unroll
+            for (int j = 0; j < SP_ND; ++j) *(uint4*)(bp + j * bs) = sp_turned<true, false>(w[j], sel, sgn);
+        }
+    } else if (turn & 1) {
+#pragma unroll
+        for (int j = 0; j < SP_ND; ++j) *(uint4*)(bp + j * bs) = sp_turned<false, true>(w[j], sel, sgn);
+    } else if (turn) {
+#pragma unroll
+        for (int j = 0; j < SP_ND; ++j) *(uint4*)(bp + j * bs) = sp_turned<false, false>(w[j], sel, sgn);
+    } else {
+#pragma unroll
+        for (int j = 0; j < SP_ND; ++j) *(uint4*)(bp + j * bs) = w[j];
+    }
+}
+
+// The units of a launch: one geometry's, or several' one after another (prefix: their unit
+// counts).
+struct SplitOne {
+    const SplitArgs* a;
+    int n;
+    __device__ __forceinline__ int count() const { return n; }
+    __device__ __forceinline__ const SplitArgs* at(int t, int* u) const { *u = t; return a; }
+};
+struct SplitMany {
+    const SplitArgs* a;
+    const int* prefix;
+    int njobs;
+    __device__ __forceinline__ int count() const { return prefix[njobs]; }
+    __device__ __forceinline__ const SplitArgs* at(int t, int* u) const {
+        int lo = 0, hi = njobs - 1;   // the last job whose first unit is <= t
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (prefix[mid] <= t) lo = mid;
+            else hi = mid - 1;
+        }
+        *u = t - prefix[lo];
+        return a + lo;
+    }
+};
+
+template <class JOBS>
+__device__ __forceinline__ void split_units(const JOBS& jobs) {
+    extern __shared__ __align__(1024) unsigned char sp_sm[];
+    __shared__ SplitShared sh;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (warp == SP_MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sp_saddr(&sh.tmem)),
                      "r"(SP_TMEM));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb));
+        auto init = [](uint64_t* b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sp_saddr(b)), "r"(n)); };
+        for (int i = 0; i < 2; ++i) {
+            init(&sh.full[i], SP_STAGE_WARPS / 2 + 1);   // the group's warps and the copying thread
+            init(&sh.empty[i], 1);
+            init(&sh.accfull[i], 1);
+            init(&sh.accempty[i], SP_EPI_WARPS);
+        }
+        for (int i = 0; i < SP_RING; ++i) { init(&sh.info[i], 1); init(&sh.slotfree[i], SP_MMA_WARP + 2); }
+        sh.dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
-    const uint32_t inv = (uint32_t)((0x100000000ull + nt - 1) / nt);   // q / nt = umulhi(q, inv) for the q here (< 2^10)
-    for (int i = tid; i < nt * nseg; i += 256) {
-        const int g = (int)__umulhi((uint32_t)i, inv), r = i - g * nt;
-        sh.rexp[g * 64 + r] = S.rexp[U.rexp + g * nT + n0 + r];
-    }
-    for (int i = tid; i <= pS; i += 256) sh.dexp[i] = S.dexp[U.dexp + i];
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tb = tmem_base;
-    const int half = warp >> 2, R = (warp & 3) * 32 + lane;             // epilogue: columns, row
-    const int part = R >= nr8 ? 1 : 0, r0 = min(R - part * nr8, nt - 1);
-    const int bc = tid & (C - 1), bg0 = tid >> lc;                      // staging of B: column, first group of 4
-    double acc[SP_COLS / 2];
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int seg = 0; seg < nseg && ok; ++seg) {
-        const int H = split_half(pS, seg), h = split_vals(pS, seg), len = 2 * H, n1 = split_size(pS) * seg;
-        const int* rexp = sh.rexp + seg * 64;
-        for (int k0 = 0; k0 < len; k0 += KC) {
-            const int ng = min(len - k0, KC) >> 2;   // groups of 4 positions (an even number)
-            // this thread's first matrix entries and its vectors' digits are loaded before the
-            // wait for the previous chunk's MMAs, which read the buffers
-            cd z[4];
-            const int g1 = (int)__umulhi((uint32_t)tid, inv), r1 = tid - g1 * nt;
-            if (g1 < ng) split_load(z, A, U.sr, U.sc, r1, k0 + 4 * g1, H, h, n1);
-            if (k0 > 0) {
-                ok = sp_wait_all(mb, phase, tid);
-                phase ^= 1u;
-                if (!ok) break;
-            }
-            for (int g = bg0; g < ng; g += 256 >> lc) {
-                unsigned char* bp = sB + (uint32_t)(bc >> 3) * sbo + (uint32_t)g * 128u + (uint32_t)(bc & 7) * 16u;
-                const uint32_t bs = (uint32_t)(C >> 3) * sbo;   // a digit's rows
-                if (bc < cnt) {
-                    const int f = sh.flag[bc], G = (k0 >> 2) + g, k = k0 + 4 * g;
-                    const bool rev = (f & SP_REV) != 0;
-                    const int turn = (f >> SP_Q_SHIFT) & 3;
-                    const uint4* src = (const uint4*)(S.vdig + (sh.vec[bc] + seg) * (SP_ND * SP_POS)) +
-                                       (rev ? (len >> 2) - 1 - G : G);
+    const uint32_t tb = sh.tmem;
+
+    if (warp < SP_STAGE_WARPS) {
+        // ---------------------------------------------------------------- staging
+        const int grp = warp >> 2, t = tid & 127;
+        unsigned char* sB = sp_sm + grp * SP_BUF + SP_ND * SP_PLANE;
+        int chunk = 0, k = 0;
+        bool ok = true;
+        for (; ok; ++k) {
+            ok = sp_wait_warp(sh, &sh.info[k & (SP_RING - 1)], (k / SP_RING) & 1);
+            if (!ok || sh.ring[k & (SP_RING - 1)].u.cnt == 0) break;
+            const SplitSlot& sl = sh.ring[k & (SP_RING - 1)];
+            const SplitArgs& S = *sl.args;
+            const SplitGeo G(sl.u);
+            for (int seg = 0; seg < G.nseg && ok; ++seg) {
+                const int H = split_half(G.pS, seg), n1 = split_size(G.pS) * seg;
+                for (int k0 = 0; k0 < 2 * H; k0 += G.KC, ++chunk) {
+                    if ((chunk & 1) != grp) continue;
+                    const int ng = min(2 * H - k0, G.KC) >> 2;   // groups of 4 positions (an even number)
+                    const int nq = ng << G.lc, bc = t & (G.C - 1);
                     uint4 w[SP_ND];
-#pragma unroll
-                    for (int j = 0; j < SP_ND; ++j) w[j] = src[j * (SP_POS / 4)];
-                    // i^(turn m) v_m, m the coefficient's index: n at its position, -n reversed
-                    uint32_t sel[4], sgn[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int a = n1 + split_abs(k + i, H), n = (k + i < H) != rev ? -a : a;
-                        const int t = (turn * n) & 3;
-                        sel[i] = (t & 1) ? 0x1032u : 0x3210u;
-                        sgn[i] = t == 0 ? 0u : t == 1 ? 0x8000u : t == 2 ? 0x80008000u : 0x80000000u;
+                    if (t < nq) split_load_b(w, S, sl, bc, k0 + 4 * (t >> G.lc), seg, H);
+                    if (chunk >= 2) {   // the MMAs that read this buffer
+                        ok = sp_wait_warp(sh, &sh.empty[grp], ((chunk >> 1) - 1) & 1);
+                        if (!ok) break;
                     }
-#pragma unroll
-                    for (int j = 0; j < SP_ND; ++j) {
-                        const uint4 v = rev ? make_uint4(w[j].w, w[j].z, w[j].y, w[j].x) : w[j];
-                        *(uint4*)(bp + j * bs) = make_uint4(__byte_perm(v.x, v.x, sel[0]) ^ sgn[0], __byte_perm(v.y, v.y, sel[1]) ^ sgn[1],
-                                                            __byte_perm(v.z, v.z, sel[2]) ^ sgn[2], __byte_perm(v.w, v.w, sel[3]) ^ sgn[3]);
+#pragma unroll 1
+                    for (int q = t; q < nq; q += 128) {
+                        const int g = q >> G.lc;
+                        if (q != t) split_load_b(w, S, sl, bc, k0 + 4 * g, seg, H);
+                        split_stage_b(w, sl, G.C, (uint32_t)ng * 128u, sB, bc, g, k0 + 4 * g, seg, H, n1);
                     }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < SP_ND; ++j) *(uint4*)(bp + j * bs) = make_uint4(0, 0, 0, 0);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) sp_arrive(&sh.full[grp]);
                 }
             }
-            for (int q = tid; q < nt * ng; q += 256) {
-                const int g = (int)__umulhi((uint32_t)q, inv), r = q - g * nt, k = k0 + 4 * g;
-                if (q != tid) split_load(z, A, U.sr, U.sc, r, k, H, h, n1);
-                const int adj0 = 1022 + rexp[r];
-                uint2 dr[4], di[4];
+            __syncwarp();
+            if (lane == 0) sp_arrive(&sh.slotfree[k & (SP_RING - 1)]);
+        }
+    } else if (warp < SP_MMA_WARP) {
+        // ---------------------------------------------------------------- epilogue
+        const int part3 = (warp - SP_STAGE_WARPS) >> 2, R = (warp & 3) * 32 + lane;   // columns, row
+        int sgc = 0, k = 0;
+        bool ok = true;
+        for (; ok; ++k) {
+            ok = sp_wait_warp(sh, &sh.info[k & (SP_RING - 1)], (k / SP_RING) & 1);
+            if (!ok || sh.ring[k & (SP_RING - 1)].u.cnt == 0) break;
+            const SplitSlot& sl = sh.ring[k & (SP_RING - 1)];
+            const SplitArgs& S = *sl.args;
+            const SplitGeo G(sl.u);
+            const int cnt = sl.u.cnt, part = R >= G.nr8 ? 1 : 0, r0 = min(R - part * G.nr8, G.nt - 1);
+            const bool live = R - part * G.nr8 < G.nt;
+            const bool any = (warp & 3) * 32 < 2 * G.nr8;   // some row of this warp belongs to the unit
+            const int64_t vec = sl.vec[min(lane, cnt - 1)];
+            double* out = S.ws + sl.u.out0 + part * G.nT + G.n0 + r0;   // this row's result, column 0
+            for (int seg = 0; seg < G.nseg; ++seg, ++sgc) {
+                const int xv = S.vexp[vec + seg];   // lane's column
+                const int xe = S.rexp[sl.u.rexp + seg * G.nT + G.n0 + r0] - 68;
+                ok = sp_wait_warp(sh, &sh.accfull[sgc & 1], (sgc >> 1) & 1);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                // accumulators v_0..v_7 of a column: y = 2^56 sum_g v_g 256^(7-g), |v_0| <= 64^2 * 96
+                // and |v_g| <= g 128^2 96; y 2^-56 = 2^32 hi + lo with hi = 2^16 (256 v_0 + v_1) + 256
+                // v_2 + v_3 (|hi| < 2^43) and lo likewise (|lo| < 2^48, its last term in 64 bits).
+                // Groups of 4 columns, taken in turn by the two warps of a row range
+                const uint32_t trow = tb + (uint32_t)(sgc & 1) * (SP_ND * SP_COLS) + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll 1
+                for (int col = 4 * part3; any && col < cnt; col += SP_EPI_WARPS) {
+                    int x[4];
+                    double sum[4], y[4];   // sum: of the segments before
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int adj = adj0 + sh.dexp[min(n1 + split_abs(k + i, H), pS)];
-                    dr[i] = sp_digits(z[i].x, adj);
-                    di[i] = sp_digits(z[i].y, adj);
+                    for (int c = 0; c < 4; ++c) {
+                        x[c] = __shfl_sync(0xffffffffu, xv, min(col + c, cnt - 1));
+                        sum[c] = seg > 0 ? out[(int64_t)min(col + c, cnt - 1) * (2 * G.nT)] : 0.0;
+                    }
+                    uint32_t w8[8][4];
+#pragma unroll
+                    for (int g = 0; g < 8; ++g)
+                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                                     : "=r"(w8[g][0]), "=r"(w8[g][1]), "=r"(w8[g][2]), "=r"(w8[g][3])
+                                     : "r"(trow + (uint32_t)(g * G.C + col)));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        int w[8];
+#pragma unroll
+                        for (int g = 0; g < 8; ++g) w[g] = __float2int_rn(__uint_as_float(w8[g][c]));
+                        const int a = w[0] * 256 + w[1], b = w[2] * 256 + w[3], d = w[4] * 256 + w[5];
+                        const long long hi = (long long)a * 65536 + b;
+                        const long long lo = (long long)d * 65536 + ((long long)w[6] * 256 + w[7]);
+                        y[c] = sp_value(hi, lo, xe + x[c]);
+                        y[c] = x[c] == SP_INF ? __longlong_as_double(0x7ff8000000000000ll) : y[c];
+                    }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (live && col + c < cnt) out[(int64_t)(col + c) * (2 * G.nT)] = seg == 0 ? y[c] : sum[c] + y[c];
                 }
-                const int rr = nr8 + r;
-                unsigned char* ar = sA + (uint32_t)(r >> 3) * sbo + (uint32_t)g * 128u + (uint32_t)(r & 7) * 16u;
-                unsigned char* ai = sA + (uint32_t)(rr >> 3) * sbo + (uint32_t)g * 128u + (uint32_t)(rr & 7) * 16u;
-#define SP_STORE_A(J)                                                                                          \
-    {                                                                                                          \
-        const uint32_t h0 = sp_digit<J>(dr[0], di[0]), h1 = sp_digit<J>(dr[1], di[1]),                         \
-                       h2 = sp_digit<J>(dr[2], di[2]), h3 = sp_digit<J>(dr[3], di[3]);                         \
-        *(uint4*)(ar + J * plane) =                                                                            \
-            make_uint4(h0 ^ 0x80000000u, h1 ^ 0x80000000u, h2 ^ 0x80000000u, h3 ^ 0x80000000u);                \
-        *(uint4*)(ai + J * plane) = make_uint4(__byte_perm(h0, h0, 0x1032), __byte_perm(h1, h1, 0x1032),       \
-                                               __byte_perm(h2, h2, 0x1032), __byte_perm(h3, h3, 0x1032));      \
-    }
-                SP_STORE_A(0) SP_STORE_A(1) SP_STORE_A(2) SP_STORE_A(3) SP_STORE_A(4) SP_STORE_A(5) SP_STORE_A(6) SP_STORE_A(7)
-#undef SP_STORE_A
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                __syncwarp();
+                if (lane == 0) sp_arrive(&sh.accempty[sgc & 1]);
             }
-            asm volatile("fence.proxy.async.shared::cta;");
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            __syncthreads();
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            if (tid == 0) {
-                const uint32_t a0 = sp_saddr(sA), b0 = sp_saddr(sB);
-                for (int i = 0; i < SP_ND; ++i) {
+            if (lane == 0) sp_arrive(&sh.slotfree[k & (SP_RING - 1)]);
+        }
+    } else if (warp == SP_MMA_WARP) {
+        // ---------------------------------------------------------------- MMAs
+        // The issuing lane is elected inside the warp's uniform flow (sp_chunk); from a lane-index
+        // branch with descriptors built in the loop an MMA took 180 cycles to issue whatever its N.
+        int chunk = 0, sgc = 0, k = 0;
+        bool ok = true;
+        const uint32_t sm0 = sp_saddr(sp_sm);
+        for (; ok; ++k) {
+            ok = sp_wait_warp(sh, &sh.info[k & (SP_RING - 1)], (k / SP_RING) & 1);
+            if (!ok || sh.ring[k & (SP_RING - 1)].u.cnt == 0) break;
+            const SplitGeo G(sh.ring[k & (SP_RING - 1)].u);
+            for (int seg = 0; seg < G.nseg && ok; ++seg, ++sgc) {
+                const int len = 2 * split_half(G.pS, seg);
+                const uint32_t acc = tb + (uint32_t)(sgc & 1) * (SP_ND * SP_COLS);
+                if (sgc >= 2) {
+                    ok = sp_wait_warp(sh, &sh.accempty[sgc & 1], ((sgc >> 1) - 1) & 1);
+                    if (!ok) break;
+                }
+                for (int k0 = 0; k0 < len; k0 += G.KC, ++chunk) {
+                    const int kst = min(len - k0, G.KC) >> 3;   // K steps of 16: 1 to 3
+                    ok = sp_wait_warp(sh, &sh.full[chunk & 1], (chunk >> 1) & 1);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t a0 = sm0 + (uint32_t)(chunk & 1) * SP_BUF;
+                    const uint32_t sbo = (uint32_t)kst * 256u;   // bytes between 8-row groups
+                    uint64_t da = sp_desc(a0, sbo);
+                    const uint64_t db = sp_desc(a0 + SP_ND * SP_PLANE, sbo);
                     // D FP32, A and B FP16, K-major, M = 128, N = (8 - i) C
-                    const uint32_t idesc = (1u << 4) | ((uint32_t)(128 >> 4) << 24) | ((uint32_t)((8 - i) * C) >> 3 << 17);
-                    for (int ks = 0; ks < ng / 2; ++ks)
-                        sp_mma(tb + (uint32_t)(i * C), sp_desc(a0 + i * plane + ks * 256, sbo), sp_desc(b0 + ks * 256, sbo),
-                               idesc, (k0 > 0 || i > 0 || ks > 0) ? 1u : 0u);
-                }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mb));
-            }
-        }
-        if (!ok) break;
-        ok = sp_wait_all(mb, phase, tid);
-        phase ^= 1u;
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        // accumulators v_0..v_7 of a column: y = 2^56 sum_g v_g 256^(7-g), |v_0| <= 64^2 * 96 and
-        // |v_g| <= g 128^2 96.  y 2^-56 = 2^32 hi + lo with hi = 2^16 (256 v_0 + v_1) + 256 v_2 + v_3
-        // (|hi| < 2^43) and lo likewise (|lo| < 2^48, its last term in 64 bits).  T = y 2^-68 cut to
-        // an integer or, for |hi| < 2^30 (terms that cancel, or a vector that is small where the row
-        // is large), y 2^-56: a fixed 2^-68 left 1.4e-9 in the sparse four-layer case
-        // Groups of 4 columns, taken in turn by the two warps of a row range
-        const uint32_t trow = tb + ((uint32_t)((warp & 3) * 32) << 16);
-        const int xe = rexp[r0] - 56;
-#pragma unroll
-        for (int cb = 0; cb < SP_COLS / 2; cb += 4) {
-            const int col = 2 * cb + 4 * half;
-            if (col < cnt) {
-                uint32_t t[8][4];
-#pragma unroll
-                for (int g = 0; g < 8; ++g)
-                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                                 : "=r"(t[g][0]), "=r"(t[g][1]), "=r"(t[g][2]), "=r"(t[g][3])
-                                 : "r"(trow + (uint32_t)(g * C + col)));
-                asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    int w[8];
-#pragma unroll
-                    for (int g = 0; g < 8; ++g) w[g] = __float2int_rn(__uint_as_float(t[g][c]));
-                    const int a = w[0] * 256 + w[1], b = w[2] * 256 + w[3], d = w[4] * 256 + w[5];
-                    const long long hi = (long long)a * 65536 + b;
-                    const long long lo = (long long)d * 65536 + ((long long)w[6] * 256 + w[7]);
-                    const bool fits = (unsigned long long)(hi + (1ll << 30)) < (1ull << 31);
-                    const long long T = fits ? hi * (1ll << 32) + lo : hi * (1ll << 20) + (lo >> 12);
-                    const int x = S.vexp[sh.vec[min(col + c, cnt - 1)] + seg];
-                    const double y = x == SP_INF ? __longlong_as_double(0x7ff8000000000000ll) : sp_value(T, xe + x - (fits ? 12 : 0));
-                    acc[cb + c] = seg == 0 ? y : acc[cb + c] + y;
+                    uint32_t idesc = (1u << 4) | ((uint32_t)(128 >> 4) << 24) | ((uint32_t)(8 * G.C) >> 3 << 17), d = acc;
+                    const uint32_t first = k0 > 0 ? 1u : 0u;
+                    const uint32_t astep = ((uint32_t)(G.nr8 >> 2) * sbo) >> 4;
+                    if (sp_elect()) {
+                        if (kst == 3) sp_chunk<3>(d, da, db, idesc, first, astep, (uint32_t)G.C);
+                        else if (kst == 2) sp_chunk<2>(d, da, db, idesc, first, astep, (uint32_t)G.C);
+                        else sp_chunk<1>(d, da, db, idesc, first, astep, (uint32_t)G.C);
+                        sp_commit(&sh.empty[chunk & 1]);
+                        if (k0 + G.KC >= len) sp_commit(&sh.accfull[sgc & 1]);
+                    }
+                    __syncwarp();
                 }
             }
+            if (lane == 0) sp_arrive(&sh.slotfree[k & (SP_RING - 1)]);
         }
-        if (seg + 1 < nseg) {
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            __syncthreads();   // the next segment's first MMA overwrites the accumulators
-            asm volatile("tcgen05.fence::after_thread_sync;");
+        // the last MMAs are done before the TMEM is freed (bounded, also after a wait gave up)
+        if (chunk > 0 && lane == 0) {
+            sp_wait(sp_saddr(&sh.empty[(chunk - 1) & 1]), ((chunk - 1) >> 1) & 1);
+            if (chunk > 1) sp_wait(sp_saddr(&sh.empty[chunk & 1]), ((chunk - 2) >> 1) & 1);
         }
-    }
-    if (!ok) {
-        sp_wait(mb, phase);   // the MMAs in flight, once more (bounded), before the TMEM is freed
-        if (tid == 0) { *(volatile int*)S.err = 1; __threadfence_system(); }
-    }
-    if (R - part * nr8 < nt) {
-        double* out = S.ws + (U.out0 * S.ncols + (int64_t)c0 * (2 * nT)) + part * nT + n0 + r0;
+        __syncwarp();
+    } else if (warp == SP_MMA_WARP + 1) {
+        // ---------------------------------------------------------------- matrix chunks
+        int chunk = 0, k = 0;
+        bool ok = true;
+        const unsigned char* held[2] = {nullptr, nullptr};
+        for (; ok; ++k) {
+            ok = sp_wait_warp(sh, &sh.info[k & (SP_RING - 1)], (k / SP_RING) & 1);
+            if (!ok || sh.ring[k & (SP_RING - 1)].u.cnt == 0) break;
+            const SplitGeo G(sh.ring[k & (SP_RING - 1)].u);
+            const unsigned char* src = sh.ring[k & (SP_RING - 1)].args->dig + sh.ring[k & (SP_RING - 1)].u.dig;
+            for (int seg = 0; seg < G.nseg && ok; ++seg) {
+                const int len = 2 * split_half(G.pS, seg);
+                for (int k0 = 0; k0 < len; k0 += G.KC, ++chunk) {
+                    const int b = chunk & 1;
+                    const uint32_t bytes = (uint32_t)min(len - k0, G.KC) * (uint32_t)G.nr8 * (8 * SP_ND);
+                    if (chunk >= 2) {
+                        ok = sp_wait_warp(sh, &sh.empty[b], ((chunk >> 1) - 1) & 1);
+                        if (!ok) break;
+                    }
+                    if (lane == 0) {
+                        const uint32_t mb = sp_saddr(&sh.full[b]);
+                        if (held[b] == src) {
+                            sp_arrive(&sh.full[b]);
+                        } else {
+                            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(bytes) : "memory");
+                            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                         ::"r"(sp_saddr(sp_sm + b * SP_BUF)), "l"(src), "r"(bytes), "r"(mb)
+                                         : "memory");
+                        }
+                    }
+                    held[b] = src;
+                    src += bytes;
+                    __syncwarp();
+                }
+            }
+            if (lane == 0) sp_arrive(&sh.slotfree[k & (SP_RING - 1)]);
+        }
+        // a copy in flight lands before the CTA ends (after a wait gave up; else the MMAs waited for it)
+        if (!ok && lane == 0)
+            for (int c = max(0, chunk - 2); c < chunk; ++c) sp_wait(sp_saddr(&sh.full[c & 1]), (c >> 1) & 1);
+        __syncwarp();
+    } else {
+        // ---------------------------------------------------------------- descriptors
+        // a run of units at a time, so that their chains of loads run side by side
+        const int nun = jobs.count(), run = max(1, min(SP_RUN, nun / (8 * (int)gridDim.x)));
+        bool ok = true, more = true;
+        for (int k = 0; more && ok;) {
+            int un = 0;
+            if (lane == 0) un = atomicAdd(jobs.a->ctr, run);
+            un = __shfl_sync(0xffffffffu, un, 0);
+            const int cnt = max(0, min(run, nun - un));
+            more = cnt == run;
+            for (int i = 0; i < cnt && ok; ++i)
+                if (k + i >= SP_RING) ok = sp_wait_warp(sh, &sh.slotfree[(k + i) & (SP_RING - 1)], ((k + i) / SP_RING - 1) & 1);
+            if (!ok) break;
+            const SplitArgs* SA[SP_RUN];
+            int word[SP_RUN];
+            static_assert(sizeof(SplitUnit) <= 128, "a lane per word");
 #pragma unroll
-        for (int c = 0; c < SP_COLS / 2; ++c) {
-            const int cc = 2 * (c & ~3) + 4 * half + (c & 3);
-            if (cc < cnt) out[(int64_t)cc * (2 * nT)] = ok ? acc[c] : 0.0;
+            for (int i = 0; i < SP_RUN; ++i) {
+                if (i >= cnt) break;
+                int ui;
+                SA[i] = jobs.at(un + i, &ui);
+                word[i] = lane < (int)(sizeof(SplitUnit) / 4) ? ((const int*)(SA[i]->unit + ui))[lane] : 0;
+            }
+#pragma unroll
+            for (int i = 0; i < SP_RUN; ++i) {
+                if (i >= cnt) break;
+                SplitSlot& sl = sh.ring[(k + i) & (SP_RING - 1)];
+                if (lane < (int)(sizeof(SplitUnit) / 4)) ((int*)&sl.u)[lane] = word[i];
+                if (lane == 0) sl.args = SA[i];
+            }
+            __syncwarp();
+            SplitPair P[SP_RUN];
+            int rhs[SP_RUN];
+#pragma unroll
+            for (int i = 0; i < SP_RUN; ++i) {
+                if (i >= cnt) break;
+                const SplitUnit& U = sh.ring[(k + i) & (SP_RING - 1)].u;
+                const int c = U.col0 + min(lane, U.cnt - 1), q = c / SA[i]->ncols;
+                rhs[i] = c - q * SA[i]->ncols;
+                P[i] = SA[i]->pair[U.pair0 + q];
+            }
+#pragma unroll
+            for (int i = 0; i < SP_RUN; ++i) {
+                if (i >= cnt) break;
+                SplitSlot& sl = sh.ring[(k + i) & (SP_RING - 1)];
+                sl.flag[lane] = P[i].flags;
+                sl.vec[lane] = (int64_t)rhs[i] * SA[i]->nvec + P[i].vec;
+                __syncwarp();
+                if (lane == 0) sp_arrive(&sh.info[(k + i) & (SP_RING - 1)]);
+            }
+            k += cnt;
+            if (!more) {   // the end, for everyone
+                if (k >= SP_RING) ok = sp_wait_warp(sh, &sh.slotfree[k & (SP_RING - 1)], (k / SP_RING - 1) & 1);
+                if (lane == 0) {
+                    sh.ring[k & (SP_RING - 1)].u.cnt = 0;
+                    sp_arrive(&sh.info[k & (SP_RING - 1)]);
+                }
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tb), "r"(SP_TMEM));
+    if (sh.dead && tid == 0) { *(volatile int*)jobs.a->err = 1; __threadfence_system(); }
+    if (warp == SP_MMA_WARP)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tb), "r"(SP_TMEM));
 }
 
-__global__ void __launch_bounds__(256, 2) k_split(const SplitArgs S) { split_unit(S, blockIdx.x, blockIdx.y); }
+__global__ void __launch_bounds__(SP_THREADS, 1) k_split(const __grid_constant__ SplitArgs S, int nunits) {
+    split_units(SplitOne{&S, nunits});
+}
+__global__ void __launch_bounds__(SP_THREADS, 1) k_split_multi(const SplitArgs* __restrict__ jobs,
+                                                              const int* __restrict__ prefix, int njobs) {
+    split_units(SplitMany{jobs, prefix, njobs});
+}
 
 // Every destination's sum over its products, in list order within a slice; the slices
 // (192 / (2p + 1) of them) in order.
