@@ -162,6 +162,13 @@ static void make_m2l_items(lfmm_geometry_s* g, int item_work, int wide) {
 // kernel adds in a fixed order, so the few large boxes of the coarse levels
 // spread over the GPU instead of running as a handful of long CTAs.
 #define M2L_ITEM_WORK 2048
+// families (parent cells) from which an M2M or L2L pass runs as products on the tensor cores
+// (two launches) instead of FP64 FMAs (one).  Alone and cold: 2,466 families 39 against 60 us,
+// 1,240 34 against 38, 610 36 against 30, 12,700 74 against 247.  Whole products with the line
+// at 200, 700, 1,500 and never: N = 65,536 726, 687, 700, 748 us; N = 262,144 2.00, 1.99, 2.01,
+// 2.59 ms; N = 19,871 357, 340, 327, 326 us.  By the families alone, not the right-hand sides,
+// so that a block's columns equal single products.
+#define SP_MIN_FAMILIES 1200
 static void build_m2l_work(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, const std::vector<int>& vr_src,
                            const std::vector<int>& vr_key, const std::vector<int>& vr_comp,
                            const std::vector<int>& vr_flip, const std::vector<ReactKey>& keys) {
@@ -212,8 +219,8 @@ static void split_alloc(lfmm_geometry_s* g, int cols) {   // products, then digi
 // row tiles of up to 64 complex rows.
 static void make_split_plan(lfmm_geometry_s* g, SplitPlan& P, int ncols) {
     std::vector<SplitUnit> units;
-    const int nlev = g->tree.D + 1, cap = g->sp_cap;
-    P.start.assign(nlev + 2, -1);
+    const int nst = 3 * (g->tree.D + 1), cap = g->sp_cap;
+    P.start.assign(nst + 1, -1);
     for (const SplitTab& s : g->sp_tabs_host) {
         if (P.start[s.level] < 0) P.start[s.level] = (int)units.size();
         const int nco = 2 * s.pT + 1, Q = s.npairs * ncols, nu = (Q + cap - 1) / cap;
@@ -227,7 +234,7 @@ static void make_split_plan(lfmm_geometry_s* g, SplitPlan& P, int ncols) {
             }
         }
     }
-    for (int l = nlev + 1, next = (int)units.size(); l >= 0; --l) {
+    for (int l = nst, next = (int)units.size(); l >= 0; --l) {
         if (P.start[l] < 0) P.start[l] = next;
         next = P.start[l];
     }
@@ -268,6 +275,8 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
             }
             dexp.insert(dexp.end(), d.begin(), d.end());
         }
+    g->sp_ndexp = (int)dexp.size();   // the locals' scales: L_n has about the size of 1 / J_n
+    for (int i = 0; i < g->sp_ndexp; ++i) dexp.push_back(-dexp[i]);
     // pairs per matrix: free-space canonical tables, then reaction keys
     // and, within one, per symmetry (reversal and quarter turns): sorted by it, a unit's columns
     // are staged alike
@@ -383,6 +392,83 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
         }
     }
     for (int l = nlev; l <= nlev + 1; ++l) g->sp_dst_start[l] = (int)dst.size();
+    // M2M and L2L passes over many families (SP_MIN_FAMILIES) as products: per (layer, child level)
+    // one matrix, the quadrant-3 child's translation; child q's is that one with row n and column
+    // m turned by w quarters, w = 0, 3, 2, 1 for the quadrants 3, 2, 0, 1 (om_q = i^w, fam_up)
+    g->sp_up.assign(nlev, 0);
+    g->sp_dn.assign(nlev, 0);
+    g->sp_fin_up.assign(2 * nlev, 0);
+    g->sp_fin_dn.assign(2 * nlev, 0);
+    std::vector<SplitFin> fins;
+    const int wq[4] = {2, 1, 3, 0};
+    for (int down = 0; down < 2; ++down)
+        for (int l = l0 + 1; l <= D; ++l) {
+            if (g->q_end[l] - g->q_begin[l] < SP_MIN_FAMILIES) continue;
+            (down ? g->sp_dn : g->sp_up)[l] = 1;
+            const int pS = t.p_level[down ? l - 1 : l], pT = t.p_level[down ? l : l - 1], nT = 2 * pT + 1;
+            // pairs of each layer by turn, in family order within one
+            std::vector<int> lay_tab(nl, -1), cntv((size_t)nl * 4, 0), nlay(nl, 0);
+            auto each = [&](auto&& f) {
+                for (int q = g->q_begin[l]; q < g->q_end[l]; ++q) {
+                    const int P = t.level_start[l - 1] + (q - g->q_begin[l]);
+                    for (int c = t.child_begin[P]; c < t.child_end[P]; ++c) {
+                        const int qd = (t.box_ix[c] & 1) | ((t.box_iy[c] & 1) << 1);
+                        if (down && ((g->qx_host[q].dn_skip >> qd) & 1)) continue;
+                        f(P, c, g->qx_host[q].lay, wq[qd]);
+                    }
+                }
+            };
+            each([&](int, int, int lay, int w) { ++cntv[(size_t)lay * 4 + w]; ++nlay[lay]; });
+            int64_t lrows = 0;
+            for (int lay = 0; lay < nl; ++lay) {
+                if (!nlay[lay]) continue;
+                SplitTab s{};
+                s.base = g->qvec_host[2 * ((size_t)lay * nlev + l) + down] + 2 * pS;   // element (r, c) at r - c + 2 pS
+                s.sr = 1; s.sc = -1; s.react = 2; s.pT = pT; s.pS = pS;
+                s.dexp = down ? g->sp_ndexp + dexp_off[lay * nlev + l - 1] : dexp_off[lay * nlev + l];
+                s.rexp = nrexp; nrexp += nT * split_nseg(pS);
+                s.pair0 = (int)pairs.size(); s.npairs = nlay[lay];
+                s.out0 = lrows; lrows += (int64_t)nlay[lay] * 2 * nT;
+                const int tiles = (nT + split_tile(nT) - 1) / split_tile(nT);
+                s.dig = dig; dig += tiles * split_tile_bytes(pS, (split_tile(nT) + 7) & ~7);
+                g->sp_max_tiles = std::max(g->sp_max_tiles, tiles);
+                s.level = (down ? 2 : 1) * nlev + l;
+                lay_tab[lay] = (int)tabs.size();
+                tabs.push_back(s);
+                pairs.resize(pairs.size() + nlay[lay]);
+                for (int w = 0, o = 0; w < 4; ++w) { const int c = cntv[(size_t)lay * 4 + w]; cntv[(size_t)lay * 4 + w] = o; o += c; }
+            }
+            rows = std::max(rows, lrows);
+            std::vector<int>& range = down ? g->sp_fin_dn : g->sp_fin_up;
+            range[2 * l] = (int)fins.size();
+            int lastP = -1;
+            each([&](int P, int c, int lay, int w) {
+                const SplitTab& s = tabs[lay_tab[lay]];
+                const int q = cntv[(size_t)lay * 4 + w]++;
+                pairs[s.pair0 + q] = SplitPair{vec_of[down ? P : c], ((4 - w) & 3) << SP_Q_SHIFT};
+                const int dst = down ? c : P;
+                if (down || P != lastP)
+                    fins.push_back(SplitFin{g->box_coef_off_host[dst], pT, (int)rlist.size(), (int)rlist.size(), vec_of[dst],
+                                            (down ? g->sp_ndexp : 0) + dexp_off[t.box_layer[dst] * nlev + t.box_level[dst]], 0});
+                lastP = P;
+                rlist.push_back(SplitRow{s.out0 + (int64_t)q * 2 * nT, w << SP_Q_SHIFT, 0});
+                fins.back().r1 = (int)rlist.size();
+            });
+            range[2 * l + 1] = (int)fins.size();
+        }
+    std::vector<int2> xv(g->xdst_host.size());
+    for (int l = l0; l <= D; ++l)
+        for (int down = 0; down < 2; ++down) {
+            const int b0 = down ? g->dn_begin[l] : g->up_begin[l], b1 = down ? g->dn_end[l] : g->up_end[l];
+            for (int i = b0; i < b1; ++i) {
+                const int r = g->xd_ref_host[i], slot = g->xdst_host[i].in_slots;
+                const int box = slot ? g->slot_box_host[r] : r;
+                xv[i] = make_int2(slot ? vec_of_slot[r] : vec_of[r],
+                                  (down ? g->sp_ndexp : 0) + dexp_off[t.box_layer[box] * nlev + t.box_level[box]]);
+            }
+        }
+    g->d_sp_fin = dupload(g, fins);
+    g->d_xdst_vec = dupload(g, xv);
     g->d_sp_tab = dupload(g, tabs);
     g->d_sp_vec = dupload(g, vecs);
     g->sp_nvec = (int)vecs.size();
@@ -585,6 +671,7 @@ void fmm_build(lfmm_geometry_s* g) {
                     d.src_end = (int)xs.size();
                     xd.push_back(d);
                     xd_layer.push_back(t.box_layer[b]);
+                    g->xd_ref_host.push_back(sp);
                 }
             g->up_end[lp] = (int)xd.size();
         }
@@ -610,6 +697,7 @@ void fmm_build(lfmm_geometry_s* g) {
                     d.src_end = (int)xs.size();
                     xd.push_back(d);
                     xd_layer.push_back(t.box_layer[c]);
+                    g->xd_ref_host.push_back(c);
                 }
             }
             for (int side = 0; side < 2; ++side)
@@ -626,6 +714,7 @@ void fmm_build(lfmm_geometry_s* g) {
                     d.src_end = (int)xs.size();
                     xd.push_back(d);
                     xd_layer.push_back(t.box_layer[b]);
+                    g->xd_ref_host.push_back(sb);
                 }
             g->dn_end[l] = (int)xd.size();
         }
@@ -822,10 +911,11 @@ void fmm_build(lfmm_geometry_s* g) {
             }
         }
         if (g->sp_ntab > 0) {
-            k_split_rexp<<<g->sp_ntab, 128>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_sp_dexp, g->d_sp_rexp);
+            k_split_rexp<<<g->sp_ntab, 128>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_xvec, g->d_sp_dexp,
+                                              g->d_sp_rexp);
             cuda_check(cudaGetLastError(), "k_split_rexp");
-            k_split_digits<<<dim3(g->sp_ntab, g->sp_max_tiles), 256>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_sp_dexp,
-                                                                      g->d_sp_rexp, g->d_sp_dig);
+            k_split_digits<<<dim3(g->sp_ntab, g->sp_max_tiles), 256>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_xvec,
+                                                                      g->d_sp_dexp, g->d_sp_rexp, g->d_sp_dig);
             cuda_check(cudaGetLastError(), "k_split_digits");
         }
     }
@@ -918,28 +1008,81 @@ static SplitArgs split_args(lfmm_geometry_s* g, int col0, int ncols) {
                      g->d_sp_dig, g->d_M, g->d_Mp, g->d_L, g->d_Lp, g->ncoef, g->nslotcoef,
                      g->d_sp_vdig, g->d_sp_vexp, g->sp_nvec, g->d_sp_ws, col0, ncols, g->wait_err};
 }
-// FP64 M2L of the levels below lm
+static void launch_split_vec(lfmm_geometry_s* g, const SplitArgs& a, int v0, int v1, cudaStream_t s) {
+    if (v1 <= v0) return;
+    k_split_vec<<<dim3((v1 - v0 + 3) / 4, a.ncols), 128, 0, s>>>(a, v0, v1 - v0);
+    cuda_check(cudaGetLastError(), "k_split_vec");
+    ++g->n_launches;
+}
+// the products of the stages [st0, st1)
+static void launch_split_units(lfmm_geometry_s* g, SplitArgs a, int st0, int st1, cudaStream_t s) {
+    const SplitPlan& P = split_plan(g, a.ncols);
+    const int n = P.start[st1] - P.start[st0];
+    if (n <= 0) return;
+    raise_smem_limit((const void*)k_split, SP_SMEM, "split M2L smem");
+    a.unit += P.start[st0];
+    k_split<<<std::min(n, SP_SMS), SP_THREADS, SP_SMEM, s>>>(a, n);
+    cuda_check(cudaGetLastError(), "k_split");
+    ++g->n_launches;
+}
+// M2L destinations of 2p + 1 > 64 (the coarse levels', first) among the first nd
+static int split_big(const lfmm_geometry_s* g, int nd) {
+    int l = g->tree.l0;
+    while (l <= g->tree.D && 2 * g->tree.p_level[l] + 1 > 64) ++l;
+    return std::min(nd, g->sp_dst_start[l]);
+}
+static void launch_split_reduce(lfmm_geometry_s* g, const SplitArgs& a, int nd, cudaStream_t s) {
+    if (nd <= 0) return;
+    const int nbig = split_big(g, nd);
+    k_split_reduce<<<dim3(split_red_ctas(nbig, nd - nbig), a.ncols), 192, 0, s>>>(a, nbig, nd);
+    cuda_check(cudaGetLastError(), "k_split_reduce");
+    ++g->n_launches;
+}
+// FP64 M2L of the levels below lm, digits included
 static void launch_split(lfmm_geometry_s* g, int nrhs, int lm, cudaStream_t s) {
     split_check_waits(g);
     ensure_split(g, nrhs);
-    const int nd = g->sp_dst_start[lm];
-    raise_smem_limit((const void*)k_split, SP_SMEM, "split M2L smem");
-    for (int c0 = 0; c0 < nrhs && nd > 0; c0 += g->sp_ws_cols) {
+    for (int c0 = 0; c0 < nrhs; c0 += g->sp_ws_cols) {
         const SplitArgs a = split_args(g, c0, std::min(nrhs - c0, g->sp_ws_cols));
-        const int nu = split_plan(g, a.ncols).start[lm];
-        if (nu > 0) {
-            const int nv = g->sp_vec_start[lm];
-            k_split_vec<<<dim3((nv + 3) / 4, a.ncols), 128, 0, s>>>(a, 0, nv);
-            cuda_check(cudaGetLastError(), "k_split_vec");
-            ++g->n_launches;
-            k_split<<<std::min(nu, SP_SMS), SP_THREADS, SP_SMEM, s>>>(a, nu);
-            cuda_check(cudaGetLastError(), "k_split");
-            ++g->n_launches;
-        }
-        k_split_reduce<<<dim3(nd, a.ncols), 192, 0, s>>>(a, 0);
-        cuda_check(cudaGetLastError(), "k_split_reduce");
-        ++g->n_launches;
+        launch_split_vec(g, a, 0, g->sp_vec_start[lm], s);
+        launch_split_units(g, a, 0, lm, s);
+        launch_split_reduce(g, a, g->sp_dst_start[lm], s);
     }
+}
+// the arguments of a pass into the cells at child level (down) or into their parents
+static FinArgs fin_args(lfmm_geometry_s* g, const SplitArgs& a, int level, int down) {
+    const TreeHost& t = g->tree;
+    FinArgs F;
+    F.s = a;
+    F.X = down ? g->d_L : g->d_M;
+    F.Xp = down ? g->d_Lp : g->d_Mp;
+    F.s.M = F.X;
+    F.s.Mp = F.Xp;
+    const std::vector<int>& r = down ? g->sp_fin_dn : g->sp_fin_up;
+    F.fin = g->d_sp_fin + r[2 * level];
+    F.ncell = r[2 * level + 1] - r[2 * level];
+    const int b0 = down ? g->dn_begin[level] : g->up_begin[level - 1];
+    F.nd = (down ? g->dn_end[level] : g->up_end[level - 1]) - b0;
+    F.dsts = g->d_xdst + b0;
+    F.dvec = g->d_xdst_vec + b0;
+    F.srcs = g->d_xsrc;
+    F.vec = g->d_xvec;
+    F.pS = t.p_level[down ? level - 1 : level];
+    F.add = down;
+    F.big = 2 * t.p_level[down ? level : level - 1] + 1 > 64;
+    F.digits = down ? (level < t.D && g->sp_dn[level + 1]) : 1;   // multipoles: the M2L takes them all
+    return F;
+}
+static size_t fin_smem_of(const lfmm_geometry_s* g, int level, int down) {
+    const TreeHost& t = g->tree;
+    return fin_smem(t.p_level[down ? level - 1 : level], t.p_level[down ? level : level - 1]);
+}
+// the digits of the locals
+static SplitArgs local_args(lfmm_geometry_s* g, SplitArgs a) {
+    a.M = g->d_L;
+    a.Mp = g->d_Lp;
+    a.dexp += g->sp_ndexp;   // the vectors' scales
+    return a;
 }
 
 // one level's M2M (into parents at level - 1: down = 0) or L2L (into children at level:
@@ -978,6 +1121,68 @@ static void launch_pass(lfmm_geometry_s* g, const XPass& P, int nrhs, cudaStream
     ++g->n_launches;
 }
 
+// M2M, M2L and L2L in FP64: passes over many families and every M2L as products on the tensor
+// cores, the other passes as FP64 translations.  Columns in rounds that fit the workspace.
+static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
+    const TreeHost& t = g->tree;
+    const int D = t.D, l0 = t.l0, nlev = D + 1;
+    split_check_waits(g);
+    ensure_split(g, nrhs);
+    for (int c0 = 0; c0 < nrhs; c0 += g->sp_ws_cols) {
+        const int nc = std::min(nrhs - c0, g->sp_ws_cols);
+        const SplitArgs a = split_args(g, c0, nc);
+        auto columns = [&](XPass P) {
+            P.X += (int64_t)c0 * g->ncoef;
+            P.Xp += (int64_t)c0 * g->nslotcoef;
+            return P;
+        };
+        auto finish = [&](int level, int down) {
+            const FinArgs F = fin_args(g, a, level, down);
+            const size_t smem = fin_smem_of(g, level, down);
+            raise_smem_limit((const void*)k_split_fin, smem, "translation smem");
+            k_split_fin<<<dim3(fin_ctas(F), nc), 192, smem, s>>>(F);
+            cuda_check(cudaGetLastError(), "k_split_fin");
+            ++g->n_launches;
+        };
+        prof_begin(g, ST_M2M, s);
+        std::vector<char> ready(nlev + 1, 0);   // levels whose multipoles' digits are written
+        for (int l = D; l > l0; --l) {
+            if (!g->sp_up[l]) {
+                launch_pass(g, columns(make_pass(g, l, 0, 0, nc)), nc, s, "k_translate (M2M)");
+                continue;
+            }
+            if (!ready[l]) { launch_split_vec(g, a, g->sp_vec_start[l], g->sp_vec_start[l + 1], s); ready[l] = 1; }
+            launch_split_units(g, a, nlev + l, nlev + l + 1, s);
+            finish(l, 0);
+            ready[l - 1] = 1;
+        }
+        prof_end(g, ST_M2M, s);
+        prof_begin(g, ST_M2L, s);
+        for (int l = l0; l <= D; ++l) {   // the levels without digits, whole runs at a time
+            if (ready[l]) continue;
+            int e = l;
+            while (e + 1 <= D && !ready[e + 1]) ++e;
+            launch_split_vec(g, a, g->sp_vec_start[l], g->sp_vec_start[e + 1], s);
+            l = e;
+        }
+        launch_split_units(g, a, 0, nlev, s);
+        launch_split_reduce(g, a, g->sp_dst_start[nlev], s);
+        prof_end(g, ST_M2L, s);
+        prof_begin(g, ST_L2L, s);
+        for (int l = l0 + 1; l <= D; ++l) {
+            if (!g->sp_dn[l]) {
+                launch_pass(g, columns(make_pass(g, l, 1, 1, nc)), nc, s, "k_translate (L2L)");
+                continue;
+            }
+            if (l == l0 + 1 || !g->sp_dn[l - 1])
+                launch_split_vec(g, local_args(g, a), g->sp_vec_start[l - 1], g->sp_vec_start[l], s);
+            launch_split_units(g, a, 2 * nlev + l, 2 * nlev + l + 1, s);
+            finish(l, 1);
+        }
+        prof_end(g, ST_L2L, s);
+    }
+}
+
 static P2MArgs p2m_args(lfmm_geometry_s* g, const cd* x, int nrhs) {
     return P2MArgs{g->d_leaf_groups, g->d_slot_groups, g->d_leaf_entries, g->d_slot_entries, g->n_leaf_groups, g->m, g->d_w,
                    g->d_basis, g->d_gbasis, g->basis_ord + 1, x, g->n, g->ncoef, g->nslotcoef, nrhs, g->d_M, g->d_Mp};
@@ -1012,38 +1217,42 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
         }
         prof_end(g, ST_P2M, s);
     }
-    prof_begin(g, ST_M2M, s);
-    for (int lp = D - 1; lp >= l0; --lp) {   // M2M: children at lp + 1 -> parents (cells and reaction centres) at lp
-        if (lp >= lm) { mixed_m2m(g, lp, nrhs, s); continue; }
-        if (lp == lm - 1) mixed_m_to64(g, lm, nrhs, s);   // the FP64 levels start from the FP32 ones' multipoles
-        launch_pass(g, make_pass(g, lp + 1, 0, 0, nrhs), nrhs, s, "k_translate (M2M)");
-    }
-    prof_end(g, ST_M2M, s);
-    {   // M2L, all levels (precision form: the levels >= lm in FP32)
-        prof_begin(g, ST_M2L, s);
-        const int n64 = g->m2l_item_level_start[lm];
-        const int r64 = g->m2l_red_level_start[lm];
-        if (lm <= D && mixed_coarse_df(g)) {
-            // precision form: the coarse (wide-band) levels in double-float, the rest in FP32
-            ensure_m2l_part(g, nrhs);
-            mixed_m2l_coarse(g, nrhs, n64, s);
-            launch_m2l_reduce(g, nrhs, r64, s);
-        } else {
-            launch_split(g, nrhs, lm, s);
+    if (lm > D) {
+        far_fp64(g, nrhs, s);
+    } else {
+        prof_begin(g, ST_M2M, s);
+        for (int lp = D - 1; lp >= l0; --lp) {   // M2M: children at lp + 1 -> parents (cells and reaction centres) at lp
+            if (lp >= lm) { mixed_m2m(g, lp, nrhs, s); continue; }
+            if (lp == lm - 1) mixed_m_to64(g, lm, nrhs, s);   // the FP64 levels start from the FP32 ones' multipoles
+            launch_pass(g, make_pass(g, lp + 1, 0, 0, nrhs), nrhs, s, "k_translate (M2M)");
         }
-        if (lm <= D) mixed_m2l(g, nrhs, lm, s);
-        prof_end(g, ST_M2L, s);
+        prof_end(g, ST_M2M, s);
+        {   // M2L, all levels (precision form: the levels >= lm in FP32)
+            prof_begin(g, ST_M2L, s);
+            const int n64 = g->m2l_item_level_start[lm];
+            const int r64 = g->m2l_red_level_start[lm];
+            if (lm <= D && mixed_coarse_df(g)) {
+                // precision form: the coarse (wide-band) levels in double-float, the rest in FP32
+                ensure_m2l_part(g, nrhs);
+                mixed_m2l_coarse(g, nrhs, n64, s);
+                launch_m2l_reduce(g, nrhs, r64, s);
+            } else {
+                launch_split(g, nrhs, lm, s);
+            }
+            if (lm <= D) mixed_m2l(g, nrhs, lm, s);
+            prof_end(g, ST_M2L, s);
+        }
+        prof_begin(g, ST_L2L, s);
+        for (int l = l0 + 1; l <= D; ++l) {   // L2L: parents at l - 1 -> children (cells and reaction centres) at l
+            if (l > lm) { mixed_l2l(g, l, nrhs, s); continue; }
+            // at the first FP32 level the FP64 translation writes (not adds) and is then added
+            // into the FP32 locals, which the FP32 M2L has written
+            const int acc = (l == lm) ? 0 : 1;
+            launch_pass(g, make_pass(g, l, 1, acc, nrhs), nrhs, s, "k_translate (L2L)");
+            if (l == lm) mixed_l_add(g, lm, nrhs, s);
+        }
+        prof_end(g, ST_L2L, s);
     }
-    prof_begin(g, ST_L2L, s);
-    for (int l = l0 + 1; l <= D; ++l) {   // L2L: parents at l - 1 -> children (cells and reaction centres) at l
-        if (l > lm) { mixed_l2l(g, l, nrhs, s); continue; }
-        // at the first FP32 level the FP64 translation writes (not adds) and is then added
-        // into the FP32 locals, which the FP32 M2L has written
-        const int acc = (l == lm) ? 0 : 1;
-        launch_pass(g, make_pass(g, l, 1, acc, nrhs), nrhs, s, "k_translate (L2L)");
-        if (l == lm) mixed_l_add(g, lm, nrhs, s);
-    }
-    prof_end(g, ST_L2L, s);
     {   // L2P: leaves from cell centres, straddling leaves from their reaction centres
         // (after the near field, which adds into the same y on the side stream)
         if (before_l2p) cuda_check(cudaStreamWaitEvent(s, before_l2p, 0), "wait for the near field");
@@ -1084,7 +1293,10 @@ struct XJob {
 };
 struct SplitJob {
     SplitArgs a;
-    int vblocks;  // blocks of k_split_vec per column
+    int v0, nv;   // k_split_vec's vectors; k_split_reduce: large destinations, all of them
+};
+struct FinJob {
+    FinArgs F;
 };
 
 __device__ __forceinline__ int job_of(const int* __restrict__ prefix, int njobs, int b) {
@@ -1120,14 +1332,20 @@ __global__ void __launch_bounds__(128) k_translate_multi(const XJob* __restrict_
 __global__ void __launch_bounds__(128) k_split_vec_multi(const SplitJob* __restrict__ jobs,
                                                          const int* __restrict__ prefix, int njobs) {
     const int j = job_of(prefix, njobs, blockIdx.x);
-    const int b = blockIdx.x - prefix[j], vb = jobs[j].vblocks;
-    split_vec(jobs[j].a, b % vb, b / vb, 0, (int)jobs[j].a.nvec);
+    const int b = blockIdx.x - prefix[j], vb = (jobs[j].nv + 3) / 4;
+    split_vec(jobs[j].a, b % vb, b / vb, jobs[j].v0, jobs[j].nv);
+}
+__global__ void __launch_bounds__(192) k_split_fin_multi(const FinJob* __restrict__ jobs, const int* __restrict__ prefix,
+                                                         int njobs) {
+    const int j = job_of(prefix, njobs, blockIdx.x);
+    const int b = blockIdx.x - prefix[j], n = fin_ctas(jobs[j].F);
+    split_fin(jobs[j].F, b % n, b / n);
 }
 __global__ void __launch_bounds__(192) k_split_reduce_multi(const SplitJob* __restrict__ jobs,
                                                             const int* __restrict__ prefix, int njobs) {
     const int j = job_of(prefix, njobs, blockIdx.x);
-    const int b = blockIdx.x - prefix[j], nc = jobs[j].a.ncols;
-    split_reduce(jobs[j].a, b / nc, b % nc);
+    const int b = blockIdx.x - prefix[j], n = split_red_ctas(jobs[j].v0, jobs[j].nv - jobs[j].v0);
+    split_reduce(jobs[j].a, jobs[j].v0, jobs[j].nv, b % n, b / n);   // (v0, nv): large destinations, all
 }
 
 void JobTables::upload(cudaStream_t s) {
@@ -1196,76 +1414,116 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
         if (cb > 1) launch_jobs(jobs, blocks, k_p2m_multi<4>, 128, 0, s, "k_p2m_multi");
         else launch_jobs(jobs, blocks, k_p2m_multi<1>, 128, 0, s, "k_p2m_multi");
     }
-    // M2M: pass k takes each geometry's parents at level D - 1 - k (down to its l0)
-    for (int k = 0; k < max_up; ++k) {
-        std::vector<XJob> jobs;
-        std::vector<int> blocks;
-        size_t smem = 0;
-        for (const BatchOp* op : far) {
-            lfmm_geometry_s* g = op->g;
-            const TreeHost& t = g->tree;
-            const int lp = t.D - 1 - k;
-            if (lp < t.l0) continue;
-            const XPass P = make_pass(g, lp + 1, 0, 0, op->nrhs);
-            jobs.push_back(XJob{P, op->nrhs});
-            blocks.push_back(xpass_fam_ctas(P.nq, P.fch) + P.nd * P.nch);
-            smem = std::max(smem, xpass_smem(0, P.pS, P.pD, P.w));
-        }
-        raise_smem_limit((const void*)k_translate_multi, smem, "translate smem");
-        launch_jobs(jobs, blocks, k_translate_multi, 128, smem, s, "k_translate_multi (M2M)");
+    // a block too wide for its workspace: its own rounds; the others share every launch
+    std::vector<const BatchOp*> sh;
+    for (const BatchOp* op : far) {
+        if (op->nrhs > op->g->sp_ws_cols) far_fp64(op->g, op->nrhs, s);
+        else sh.push_back(op);
     }
-    // M2L of every level: products, then each destination's sum; a block too wide for its
-    // workspace takes several rounds
-    raise_smem_limit((const void*)k_split_multi, SP_SMEM, "split M2L smem");
-    for (int round = 0;; ++round) {
-        std::vector<SplitJob> jobs;
+    auto vec_jobs = [&](const std::vector<SplitJob>& jobs) {
+        std::vector<int> blocks;
+        for (const SplitJob& j : jobs) blocks.push_back((j.nv + 3) / 4 * j.a.ncols);
+        launch_jobs(jobs, blocks, k_split_vec_multi, 128, 0, s, "k_split_vec_multi");
+    };
+    // the products of a stage range of each geometry; the counter is the first one's
+    auto unit_jobs = [&](const std::vector<const BatchOp*>& ops2, auto&& range) {
         std::vector<SplitArgs> args;
-        std::vector<int> rblocks, vblocks, prefix(1, 0);
-        for (const BatchOp* op : far) {
+        std::vector<int> prefix(1, 0);
+        for (const BatchOp* op : ops2) {
+            const SplitPlan& P = split_plan(op->g, op->nrhs);
+            const std::pair<int, int> st = range(op->g);
+            args.push_back(split_args(op->g, 0, op->nrhs));
+            args.back().unit += P.start[st.first];
+            prefix.push_back(prefix.back() + P.start[st.second] - P.start[st.first]);
+        }
+        if (prefix.back() == 0) return;
+        raise_smem_limit((const void*)k_split_multi, SP_SMEM, "split M2L smem");
+        JobTables t;   // persistent: a CTA takes units of every geometry in turn
+        const size_t oj = t.add(args.data(), sizeof(SplitArgs) * args.size());
+        const size_t op = t.add(prefix.data(), sizeof(int) * prefix.size());
+        t.upload(s);
+        k_split_multi<<<std::min(prefix.back(), SP_SMS), SP_THREADS, SP_SMEM, s>>>(t.at<SplitArgs>(oj), t.at<int>(op),
+                                                                                  (int)args.size());
+        const cudaError_t e = cudaGetLastError();
+        t.release(s);
+        cuda_check(e, "k_split_multi");
+    };
+    // one pass of each geometry: products and their ends, or FP64 translations
+    auto pass = [&](int down, auto&& level_of, auto&& vec_of_level) {
+        std::vector<XJob> xj;
+        std::vector<int> xb;
+        std::vector<const BatchOp*> sp;
+        std::vector<SplitJob> vj;
+        std::vector<FinJob> fj;
+        std::vector<int> fb;
+        size_t xs = 0, fs = 0;
+        for (const BatchOp* op : sh) {
             lfmm_geometry_s* g = op->g;
-            const int c0 = round * g->sp_ws_cols, D = g->tree.D;
-            if (c0 >= op->nrhs) continue;
-            const int nc = std::min(op->nrhs - c0, g->sp_ws_cols);
-            const int vb = (g->sp_nvec + 3) / 4;
-            jobs.push_back(SplitJob{split_args(g, c0, nc), vb});
-            args.push_back(jobs.back().a);
-            vblocks.push_back(vb * nc);
-            prefix.push_back(prefix.back() + split_plan(g, nc).start[D + 1]);
-            rblocks.push_back(g->sp_dst_start[D + 1] * nc);
+            const int l = level_of(g);
+            if (l <= g->tree.l0 || l > g->tree.D) continue;
+            if (!(down ? g->sp_dn : g->sp_up)[l]) {
+                const XPass P = make_pass(g, l, down, down, op->nrhs);
+                xj.push_back(XJob{P, op->nrhs});
+                xb.push_back(xpass_fam_ctas(P.nq, P.fch) + P.nd * P.nch);
+                xs = std::max(xs, xpass_smem(down, P.pS, P.pD, P.w));
+                continue;
+            }
+            sp.push_back(op);
+            vec_of_level(op, l, vj);
+            fj.push_back(FinJob{fin_args(g, split_args(g, 0, op->nrhs), l, down)});
+            fb.push_back(fin_ctas(fj.back().F) * op->nrhs);
+            fs = std::max(fs, fin_smem_of(g, l, down));
         }
-        if (jobs.empty()) break;
-        launch_jobs(jobs, vblocks, k_split_vec_multi, 128, 0, s, "k_split_vec_multi");
-        if (prefix.back() > 0) {   // persistent: a CTA takes units of every geometry in turn
-            JobTables t;
-            const size_t oj = t.add(args.data(), sizeof(SplitArgs) * args.size());
-            const size_t op = t.add(prefix.data(), sizeof(int) * prefix.size());
-            t.upload(s);
-            k_split_multi<<<std::min(prefix.back(), SP_SMS), SP_THREADS, SP_SMEM, s>>>(t.at<SplitArgs>(oj), t.at<int>(op),
-                                                                                      (int)args.size());
-            const cudaError_t e = cudaGetLastError();
-            t.release(s);
-            cuda_check(e, "k_split_multi");
+        raise_smem_limit((const void*)k_translate_multi, xs, "translate smem");
+        raise_smem_limit((const void*)k_split_fin_multi, fs, "translation smem");
+        launch_jobs(xj, xb, k_translate_multi, 128, xs, s, "k_translate_multi");
+        vec_jobs(vj);
+        unit_jobs(sp, [&](lfmm_geometry_s* g) {
+            const int st = (down ? 2 : 1) * (g->tree.D + 1) + level_of(g);
+            return std::make_pair(st, st + 1);
+        });
+        launch_jobs(fj, fb, k_split_fin_multi, 192, fs, s, "k_split_fin_multi");
+    };
+    // M2M: pass k takes each geometry's children at level D - k
+    std::vector<std::vector<char>> ready;   // per shared geometry: levels whose multipoles' digits are written
+    for (const BatchOp* op : sh) ready.push_back(std::vector<char>(op->g->tree.D + 2, 0));
+    auto ready_of = [&](const BatchOp* op) -> std::vector<char>& { return ready[std::find(sh.begin(), sh.end(), op) - sh.begin()]; };
+    for (int k = 0; k < max_up; ++k)
+        pass(0, [&](lfmm_geometry_s* g) { return g->tree.D - k; },
+             [&](const BatchOp* op, int l, std::vector<SplitJob>& vj) {
+                 lfmm_geometry_s* g = op->g;
+                 std::vector<char>& r = ready_of(op);
+                 if (!r[l])
+                     vj.push_back(SplitJob{split_args(g, 0, op->nrhs), g->sp_vec_start[l], g->sp_vec_start[l + 1] - g->sp_vec_start[l]});
+                 r[l] = r[l - 1] = 1;
+             });
+    {   // M2L of every level: the digits still missing, products, each destination's sum
+        std::vector<SplitJob> vj, jobs;
+        std::vector<int> rblocks;
+        for (const BatchOp* op : sh) {
+            lfmm_geometry_s* g = op->g;
+            const int D = g->tree.D;
+            std::vector<char>& r = ready_of(op);
+            for (int l = g->tree.l0; l <= D; ++l)
+                if (!r[l])
+                    vj.push_back(SplitJob{split_args(g, 0, op->nrhs), g->sp_vec_start[l], g->sp_vec_start[l + 1] - g->sp_vec_start[l]});
+            const int nd = g->sp_dst_start[D + 1], nbig = split_big(g, nd);
+            jobs.push_back(SplitJob{split_args(g, 0, op->nrhs), nbig, nd});
+            rblocks.push_back(split_red_ctas(nbig, nd - nbig) * op->nrhs);
         }
+        vec_jobs(vj);
+        unit_jobs(sh, [&](lfmm_geometry_s* g) { return std::make_pair(0, g->tree.D + 1); });
         launch_jobs(jobs, rblocks, k_split_reduce_multi, 192, 0, s, "k_split_reduce_multi");
     }
     // L2L: pass k takes each geometry's children at level l0 + 1 + k
-    for (int k = 0; k < max_dn; ++k) {
-        std::vector<XJob> jobs;
-        std::vector<int> blocks;
-        size_t smem = 0;
-        for (const BatchOp* op : far) {
-            lfmm_geometry_s* g = op->g;
-            const TreeHost& t = g->tree;
-            const int l = t.l0 + 1 + k;
-            if (l > t.D) continue;
-            const XPass P = make_pass(g, l, 1, 1, op->nrhs);
-            jobs.push_back(XJob{P, op->nrhs});
-            blocks.push_back(xpass_fam_ctas(P.nq, P.fch) + P.nd * P.nch);
-            smem = std::max(smem, xpass_smem(1, P.pS, P.pD, P.w));
-        }
-        raise_smem_limit((const void*)k_translate_multi, smem, "translate smem");
-        launch_jobs(jobs, blocks, k_translate_multi, 128, smem, s, "k_translate_multi (L2L)");
-    }
+    for (int k = 0; k < max_dn; ++k)
+        pass(1, [&](lfmm_geometry_s* g) { return g->tree.l0 + 1 + k; },
+             [&](const BatchOp* op, int l, std::vector<SplitJob>& vj) {
+                 lfmm_geometry_s* g = op->g;
+                 if (l == g->tree.l0 + 1 || !g->sp_dn[l - 1])
+                     vj.push_back(SplitJob{local_args(g, split_args(g, 0, op->nrhs)), g->sp_vec_start[l - 1],
+                                           g->sp_vec_start[l] - g->sp_vec_start[l - 1]});
+             });
     // L2P after the near field, which adds into the same y
     if (before_l2p) cuda_check(cudaStreamWaitEvent(s, before_l2p, 0), "wait for the near field");
     std::vector<L2PJob> jobs;

@@ -147,8 +147,8 @@ struct SplitTab {
     int pT, pS;        // orders of the result and of the source
     int rexp, dexp;    // offsets of its row exponents and of its source scales (by |n|)
     int pair0, npairs;
-    int react;         // 0: Toeplitz vectors, 1: reaction tables
-    int level;
+    int react;         // 0: free-space Toeplitz vectors, 1: reaction tables, 2: translation vectors
+    int level;         // M2L: level l; M2M from level l: nlev + l; L2L into it: 2 nlev + l
 };
 // Its pairs: the source vector enters as v_c = i^(q m) M_m with m = c - p, or p - c with
 // SP_REV, and the result leaves as L_n = i^(q n) y_n, or y_-n with SP_REV (SplitRow); the
@@ -176,7 +176,15 @@ struct SplitUnit {     // up to SP_COLS (pair, right-hand side) columns of one m
 struct SplitPlan {
     int ncols = 0;
     SplitUnit* d_unit = nullptr;
-    std::vector<int> start;     // [nlev + 2]: first unit of each level
+    std::vector<int> start;     // [3 nlev + 1]: first unit of each SplitTab::level
+};
+// A cell's expansion from its products in an M2M or L2L pass (split.cuh: split_fin), and where
+// its digits go for the next product
+struct SplitFin {
+    int64_t off;       // coefficient offset (M, or L)
+    int p, r0, r1;     // order, its rows
+    int vec, dexp;     // its vector and source scales
+    int pad;
 };
 struct SplitDst {
     int64_t off;       // coefficient offset of the local expansion (L, or Lp with slot)
@@ -289,6 +297,7 @@ struct lfmm_geometry_s {
     std::vector<lfmm::XDst> xdst_host;
     std::vector<lfmm::XSrc> xsrc_host;
     std::vector<int> xd_layer_host;
+    std::vector<int> xd_ref_host;      // per destination its reaction centre, or its cell
     // near field: block-sparse rows over target leaves
     int *d_nb_ptr = nullptr;          // nleaf + 1
     int *d_nb_src = nullptr;          // source leaf (box id) per block
@@ -338,6 +347,13 @@ struct lfmm_geometry_s {
     lfmm::SplitPair* d_sp_pair = nullptr;
     lfmm::SplitRow* d_sp_row = nullptr;
     lfmm::SplitDst* d_sp_dst = nullptr;
+    // M2M / L2L passes as products: per child level whether, and the cells' range in d_sp_fin;
+    // the reaction-centre destinations' vectors and scales (with d_xdst)
+    std::vector<char> sp_up, sp_dn;
+    std::vector<int> sp_fin_up, sp_fin_dn;          // [2 l], [2 l + 1]
+    lfmm::SplitFin* d_sp_fin = nullptr;
+    int2* d_xdst_vec = nullptr;
+    int sp_ndexp = 0;                               // scales of the multipoles; the locals' follow
     int *d_sp_rexp = nullptr, *d_sp_dexp = nullptr;
     unsigned char* d_sp_dig = nullptr;              // the matrices' digits
     int64_t sp_dig_bytes = 0;

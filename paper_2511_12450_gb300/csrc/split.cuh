@@ -188,10 +188,10 @@ __device__ __forceinline__ int split_abs(int k, int H) { return k < H ? H - 1 - 
 // The row exponents of the matrices: rexp[seg nT + r] = smallest e with |A_rc| 2^-d_c < 2^e
 // over the row's segment (both components).  One CTA per matrix.
 __global__ void __launch_bounds__(128) k_split_rexp(const SplitTab* __restrict__ tabs, const cd* __restrict__ tf,
-                                                    const cd* __restrict__ tr, const int* __restrict__ dexp,
-                                                    int* __restrict__ rexp) {
+                                                    const cd* __restrict__ tr, const cd* __restrict__ tx,
+                                                    const int* __restrict__ dexp, int* __restrict__ rexp) {
     const SplitTab t = tabs[blockIdx.x];
-    const cd* a = (t.react ? tr : tf) + t.base + (int64_t)t.pS * t.sc;
+    const cd* a = (t.react == 2 ? tx : t.react ? tr : tf) + t.base + (int64_t)t.pS * t.sc;
     const int nT = 2 * t.pT + 1, nseg = split_nseg(t.pS);
     for (int i = threadIdx.x; i < nT * nseg; i += blockDim.x) {
         const int seg = i / nT, r = i - seg * nT;
@@ -225,13 +225,14 @@ __device__ __forceinline__ void split_load(cd (&z)[4], const cd* __restrict__ A,
     }
 }
 __global__ void __launch_bounds__(256) k_split_digits(const SplitTab* __restrict__ tabs, const cd* __restrict__ tf,
-                                                      const cd* __restrict__ tr, const int* __restrict__ dexp,
-                                                      const int* __restrict__ rexp, unsigned char* __restrict__ dig) {
+                                                      const cd* __restrict__ tr, const cd* __restrict__ tx,
+                                                      const int* __restrict__ dexp, const int* __restrict__ rexp,
+                                                      unsigned char* __restrict__ dig) {
     const SplitTab t = tabs[blockIdx.x];
     const int nT = 2 * t.pT + 1, per = split_tile(nT), n0 = blockIdx.y * per;
     if (n0 >= nT) return;
     const int nt = min(per, nT - n0), nr8 = (per + 7) & ~7, KC = split_chunk(nT);
-    const cd* A = (t.react ? tr : tf) + t.base + (int64_t)n0 * t.sr + (int64_t)t.pS * t.sc;   // column n = 0
+    const cd* A = (t.react == 2 ? tx : t.react ? tr : tf) + t.base + (int64_t)n0 * t.sr + (int64_t)t.pS * t.sc;   // column n = 0
     unsigned char* out = dig + t.dig + (int64_t)blockIdx.y * split_tile_bytes(t.pS, nr8);
     for (int seg = 0; seg < split_nseg(t.pS); ++seg) {
         const int H = split_half(t.pS, seg), h = split_vals(t.pS, seg), n1 = split_size(t.pS) * seg;
@@ -273,31 +274,25 @@ __global__ void __launch_bounds__(256) k_split_digits(const SplitTab* __restrict
 // The source vectors as digits: per (vector, segment) eight planes of SP_POS words (a word is
 // the FP16 pair (re, im) of one coefficient's digit) and the exponent.  One warp per (vector,
 // segment); a vector serves all its pairs (about 7 at one column).
-__device__ __forceinline__ void split_vec(const SplitArgs& S, int block, int column, int v0, int nv) {
-    const int w = block * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (block == 0 && column == 0 && threadIdx.x == 0) *S.ctr = 0;   // k_split's counter
-    if (w >= nv) return;
-    const SplitVec V = S.vec[v0 + w];
-    const int col = S.col0 + column;
-    const cd* m = (V.slot ? S.Mp + (int64_t)col * S.nslotcoef : S.M + (int64_t)col * S.ncoef) + V.src + V.p;
-    const int H = split_half(V.p, V.seg), h = split_vals(V.p, V.seg);
+// One warp writes one segment's digits and exponent: m the vector at n = 0, o its index.
+__device__ __forceinline__ void split_vec_seg(const SplitArgs& S, const cd* m, int p, int seg, int dexp, int64_t o, int lane) {
+    const int H = split_half(p, seg), h = split_vals(p, seg);
     cd z[2];
     int d[2], e = SP_NONE;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        const int k = lane + 32 * i, j = split_abs(k, H), n = split_size(V.p) * V.seg + j;
+        const int k = lane + 32 * i, j = split_abs(k, H), n = split_size(p) * seg + j;
         z[i] = mk(0, 0);
         d[i] = 0;
         if (k < 2 * H && j < h) {
             z[i] = m[k < H ? -n : n];
-            d[i] = S.dexp[V.dexp + n];
+            d[i] = S.dexp[dexp + n];
             const int eb = max(sp_expo(z[i].x), sp_expo(z[i].y));
             if (eb == 2047) e = SP_INF;
             else if (eb > 0) e = max(e, eb - 1022 + d[i]);
         }
     }
     e = __reduce_max_sync(0xffffffffu, e);
-    const int64_t o = (int64_t)column * S.nvec + v0 + w;
     if (lane == 0) S.vexp[o] = e;
     uint32_t* out = S.vdig + o * (SP_ND * SP_POS);
     const bool live = e > SP_NONE && e < SP_INF;
@@ -317,7 +312,15 @@ __device__ __forceinline__ void split_vec(const SplitArgs& S, int block, int col
         out[7 * SP_POS + k] = sp_digit<7>(a, b);
     }
 }
-
+__device__ __forceinline__ void split_vec(const SplitArgs& S, int block, int column, int v0, int nv) {
+    const int w = block * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (block == 0 && column == 0 && threadIdx.x == 0) *S.ctr = 0;   // k_split's counter
+    if (w >= nv) return;
+    const SplitVec V = S.vec[v0 + w];
+    const int col = S.col0 + column;
+    const cd* m = (V.slot ? S.Mp + (int64_t)col * S.nslotcoef : S.M + (int64_t)col * S.ncoef) + V.src + V.p;
+    split_vec_seg(S, m, V.p, V.seg, V.dexp, (int64_t)column * S.nvec + v0 + w, lane);
+}
 __global__ void __launch_bounds__(128) k_split_vec(const SplitArgs S, int v0, int nv) {
     split_vec(S, blockIdx.x, blockIdx.y, v0, nv);
 }
@@ -804,33 +807,175 @@ __global__ void __launch_bounds__(SP_THREADS, 1) k_split_multi(const SplitArgs* 
     split_units(SplitMany{jobs, prefix, njobs});
 }
 
-// Every destination's sum over its products, in list order within a slice; the slices
-// (192 / (2p + 1) of them) in order.
-__device__ __forceinline__ void split_reduce(const SplitArgs& S, int di, int col) {
-    __shared__ cd red[192];
-    const SplitDst d = S.dst[di];
-    const int n = 2 * d.p + 1, NS = 192 / n;
-    const int sl = threadIdx.x / n, i = threadIdx.x - sl * n;
+// The sum of rows r0.. of an order-p destination by one warp, in list order: coefficients
+// lane and lane + 32 (2 p + 1 <= 64).  The rows' places are read 32 at a time, so that only the
+// products' loads stand in the loop.
+__device__ __forceinline__ void split_sum_warp(const SplitArgs& S, int p, int r0, int r1, int col, int lane, cd (&a)[2]) {
+    const int n = 2 * p + 1;
+    const double* w = S.ws + (int64_t)col * (2 * n);
+    const bool two = lane + 32 < n;
+    a[0] = a[1] = mk(0, 0);
+    for (int b = r0; b < r1; b += 32) {
+        const SplitRow mine = S.row[min(b + lane, r1 - 1)];
+        const int cnt = min(32, r1 - b);
+#pragma unroll 4
+        for (int r = 0; r < cnt; ++r) {
+            const int64_t row = __shfl_sync(0xffffffffu, mine.row, r);
+            const int flags = __shfl_sync(0xffffffffu, mine.flags, r), turn = (flags >> SP_Q_SHIFT) & 3;
+            const double* y = w + row * S.ncols + ((flags & SP_REV) ? 2 * p - lane : lane);
+            const int step = (flags & SP_REV) ? -32 : 32;
+            const cd u = lane < n ? mk(y[0], y[n]) : mk(0, 0), v = two ? mk(y[step], y[step + n]) : mk(0, 0);
+            a[0] += sp_turn(u, (turn * (lane - p)) & 3);
+            a[1] += sp_turn(v, (turn * (lane + 32 - p)) & 3);
+        }
+    }
+}
+// the same by a CTA of 192 threads, in list order within a slice; the slices (192 / (2p + 1) of
+// them) in order.  Thread i < 2p + 1 returns coefficient i.
+__device__ __forceinline__ cd split_sum_cta(const SplitArgs& S, int p, int r0, int r1, int col, cd* red) {
+    const int n = 2 * p + 1, NS = 192 / n, sl = threadIdx.x / n, i = threadIdx.x - sl * n;
     cd a = mk(0, 0);
     if (sl < NS) {
         const double* w = S.ws + (int64_t)col * (2 * n);
 #pragma unroll 4
-        for (int r = d.r0 + sl; r < d.r1; r += NS) {
+        for (int r = r0 + sl; r < r1; r += NS) {
             const SplitRow q = S.row[r];
-            const double* y = w + q.row * S.ncols + ((q.flags & SP_REV) ? 2 * d.p - i : i);
-            a += sp_turn(mk(y[0], y[n]), (((q.flags >> SP_Q_SHIFT) & 3) * (i - d.p)) & 3);
+            const double* y = w + q.row * S.ncols + ((q.flags & SP_REV) ? 2 * p - i : i);
+            a += sp_turn(mk(y[0], y[n]), (((q.flags >> SP_Q_SHIFT) & 3) * (i - p)) & 3);
         }
         red[threadIdx.x] = a;
     }
     __syncthreads();
-    if (threadIdx.x < n) {
+    if (threadIdx.x < n)
         for (int q = 1; q < NS; ++q) a += red[q * n + threadIdx.x];
-        if (d.slot) S.Lp[(int64_t)(S.col0 + col) * S.nslotcoef + d.off + threadIdx.x] = a;
-        else S.L[(int64_t)(S.col0 + col) * S.ncoef + d.off + threadIdx.x] = a;
+    return a;
+}
+#define SP_RED_WARPS 6
+// CTAs of 192 threads for nbig large destinations (2p + 1 > 64) and nsmall others, a warp each
+__host__ __device__ inline int split_red_ctas(int nbig, int nsmall) { return nbig + (nsmall + SP_RED_WARPS - 1) / SP_RED_WARPS; }
+// M2L: every destination's sum over its products
+__device__ __forceinline__ void split_reduce(const SplitArgs& S, int nbig, int nd, int b, int col) {
+    __shared__ cd red[192];
+    const int lane = threadIdx.x & 31;
+    if (b < nbig) {
+        const SplitDst d = S.dst[b];
+        const cd a = split_sum_cta(S, d.p, d.r0, d.r1, col, red);
+        cd* out = d.slot ? S.Lp + (int64_t)(S.col0 + col) * S.nslotcoef : S.L + (int64_t)(S.col0 + col) * S.ncoef;
+        if (threadIdx.x < 2 * d.p + 1) out[d.off + threadIdx.x] = a;
+        return;
     }
+    const int di = nbig + (b - nbig) * SP_RED_WARPS + (threadIdx.x >> 5);
+    if (di >= nd) return;
+    const SplitDst d = S.dst[di];
+    cd a[2];
+    split_sum_warp(S, d.p, d.r0, d.r1, col, lane, a);
+    cd* out = (d.slot ? S.Lp + (int64_t)(S.col0 + col) * S.nslotcoef : S.L + (int64_t)(S.col0 + col) * S.ncoef) + d.off;
+    if (lane < 2 * d.p + 1) out[lane] = a[0];
+    if (lane + 32 < 2 * d.p + 1) out[lane + 32] = a[1];
 }
-__global__ void __launch_bounds__(192) k_split_reduce(const SplitArgs S, int d0) {
-    split_reduce(S, d0 + blockIdx.x, blockIdx.y);
+__global__ void __launch_bounds__(192) k_split_reduce(const SplitArgs S, int nbig, int nd) {
+    split_reduce(S, nbig, nd, blockIdx.x, blockIdx.y);
 }
+
+// The end of an M2M or L2L pass on the tensor cores: the cells' expansions from their products
+// (a parent's from up to four children's; a child's local plus its parent's), and the
+// destinations with translations of their own -- reaction centres, and cells that take a
+// straddling parent's reaction-centre local (XDst) -- in FP64, each written, and its digits for
+// the next product with it.  CTAs of 192 threads: one per XDst, one per cell of a large order,
+// else a warp per cell; k_split's counter is reset.
+struct FinArgs {
+    SplitArgs s;               // M, Mp: the expansions of the pass (multipoles, or locals)
+    cd *X, *Xp;                // the same, to write
+    const SplitFin* fin;
+    int ncell, nd;
+    const XDst* dsts;
+    const int2* dvec;          // their vectors and source scales
+    const XSrc* srcs;
+    const cd* vec;
+    int pS, add, digits;       // XSrc order; add into the expansions; write digits
+    int big;                   // 1: cells of 2p + 1 > 64
+};
+#define SP_XSTAGE 4            // sources of an XDst staged together
+inline size_t fin_smem(int pS, int pD) { return sizeof(cd) * SP_XSTAGE * (size_t)(2 * pS + 1 + 2 * (pS + pD) + 1); }
+__host__ __device__ inline int fin_ctas(const FinArgs& F) { return F.nd + split_red_ctas(F.big ? F.ncell : 0, F.big ? 0 : F.ncell); }
+__device__ __forceinline__ void split_fin(const FinArgs& F, int b, int column) {
+    extern __shared__ __align__(16) cd fin_sm[];   // XDst: sources, then their translation vectors
+    __shared__ cd red[192], z[SP_RED_WARPS * 64 > 2 * LFMM_PMAX + 1 ? SP_RED_WARPS * 64 : 2 * LFMM_PMAX + 1];
+    const SplitArgs& S = F.s;
+    const int tid = threadIdx.x, lane = tid & 31, col = S.col0 + column;
+    if (b == 0 && column == 0 && tid == 0) *S.ctr = 0;
+    int p, vec, dexp;
+    if (b >= F.nd && !F.big) {   // a warp per cell
+        const int w = tid >> 5, ci = (b - F.nd) * SP_RED_WARPS + w;
+        if (ci >= F.ncell) return;
+        const SplitFin f = F.fin[ci];
+        cd* out = F.X + (int64_t)col * S.ncoef + f.off;
+        cd a[2];
+        split_sum_warp(S, f.p, f.r0, f.r1, column, lane, a);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = lane + 32 * h;
+            if (i < 2 * f.p + 1) {
+                if (F.add) a[h] += out[i];
+                out[i] = a[h];
+                z[w * 64 + i] = a[h];
+            }
+        }
+        if (!F.digits) return;
+        __syncwarp();
+        for (int seg = 0; seg < split_nseg(f.p); ++seg)
+            split_vec_seg(S, z + w * 64 + f.p, f.p, seg, f.dexp, (int64_t)column * S.nvec + f.vec + seg, lane);
+        return;
+    }
+    cd* out;
+    cd a = mk(0, 0);
+    if (b >= F.nd) {
+        const SplitFin f = F.fin[b - F.nd];
+        p = f.p; vec = f.vec; dexp = f.dexp;
+        out = F.X + (int64_t)col * S.ncoef + f.off;
+        a = split_sum_cta(S, p, f.r0, f.r1, column, red);
+    } else {
+        const XDst d = F.dsts[b];
+        const int2 v = F.dvec[b];
+        p = d.p; vec = v.x; dexp = v.y;
+        out = (d.in_slots ? F.Xp + (int64_t)col * S.nslotcoef : F.X + (int64_t)col * S.ncoef) + d.off;
+        const int n = 2 * p + 1, NS = 192 / n, sl = tid / n, i = tid - sl * n;
+        const int ncS = 2 * F.pS + 1, nv = 2 * (F.pS + p) + 1;
+        for (int j0 = d.src_begin; j0 < d.src_end; j0 += SP_XSTAGE) {
+            const int js = min(SP_XSTAGE, d.src_end - j0);
+            __syncthreads();
+            for (int j = 0; j < js; ++j) {
+                const XSrc sr = F.srcs[j0 + j];
+                const cd* src = (sr.in_slots ? S.Mp + (int64_t)col * S.nslotcoef : S.M + (int64_t)col * S.ncoef) + sr.off;
+                cd* xs = fin_sm + j * ncS;
+                cd* vs = fin_sm + SP_XSTAGE * ncS + j * nv;
+                for (int k = tid; k < ncS; k += 192) xs[k] = src[k];
+                for (int k = tid; k < nv; k += 192) vs[k] = F.vec[sr.vec_off + k];
+            }
+            __syncthreads();
+            // V[n - m + hw] with n = i - p, m = mi - pS, hw = pS + p
+            if (sl < NS)
+                for (int j = 0; j < js; ++j) {
+                    const cd *xs = fin_sm + j * ncS, *vs = fin_sm + SP_XSTAGE * ncS + j * nv + i + 2 * F.pS;
+#pragma unroll 4
+                    for (int mi = sl; mi < ncS; mi += NS) cfma(a, xs[mi], vs[-mi]);
+                }
+        }
+        if (sl < NS) red[tid] = a;
+        __syncthreads();
+        if (tid < n)
+            for (int q = 1; q < NS; ++q) a += red[q * n + tid];
+    }
+    if (tid < 2 * p + 1) {
+        if (F.add) a += out[tid];
+        out[tid] = a;
+        z[tid] = a;
+    }
+    if (!F.digits) return;
+    __syncthreads();
+    for (int seg = tid >> 5; seg < split_nseg(p); seg += 6)
+        split_vec_seg(S, z + p, p, seg, dexp, (int64_t)column * S.nvec + vec + seg, lane);
+}
+__global__ void __launch_bounds__(192) k_split_fin(const FinArgs F) { split_fin(F, blockIdx.x, blockIdx.y); }
 
 }  // namespace lfmm

@@ -71,3 +71,29 @@ def test_scales_zeros_and_values_that_are_not_finite(gpu_lib):
         xb[5] = bad
         assert not np.any(np.isfinite(lf.matvec(G, xb)))
     assert np.array_equal(lf.matvec(G, x), y)
+
+
+def test_passes_as_products_in_blocks_and_batches(gpu_lib):
+    """A geometry whose finest M2M and L2L passes are products too (over 1,200 families): a block's
+    columns, and its share of a batch with a small geometry, equal its own single products."""
+    import torch
+
+    from workloads import config_c2
+
+    lf = gpu_lib
+    geos = []
+    for wl, leaf in ((config_c2(), 64), (layered_small(n_bodies=3, nodes=150, seed=7), 16)):
+        pts, w, _, _ = onys.elements(wl.bodies)
+        M = lf.medium_create(wl.medium.interfaces, wl.medium.k, wl.medium.eta)
+        geos.append(lf.geometry_build(M, pts, w, p=20, leaf_size=leaf))
+    rng = np.random.default_rng(6)
+    xs = [torch.from_numpy(rng.standard_normal((3, G.n)) + 1j * rng.standard_normal((3, G.n))).cuda() for G in geos]
+    own = [torch.stack([lf.matvec(G, x[c].contiguous()) for c in range(3)]) for G, x in zip(geos, xs)]
+    for G, x, y in zip(geos, xs, own):
+        assert torch.equal(lf.matvec(G, x), y)
+    for order in (slice(None), slice(None, None, -1)):
+        for y, ref in zip(lf.matvec_batch(geos[order], xs[order]), own[order]):
+            assert torch.equal(y, ref)
+    single = [x[0].contiguous() for x in xs]
+    for y, ref in zip(lf.matvec_batch(geos, single), own):
+        assert torch.equal(y, ref[0])
