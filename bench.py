@@ -392,7 +392,7 @@ def run_c3(lfmm, steps=5):
                                                 torch.linalg.norm(ys["fp64"]))
     pf = lfmm.geometry_query(G, "precision_form", np.float64)
     out["mixed"]["fp32_from_level"] = int(pf[0])
-    out["mixed"]["coarse_m2l"] = "double-float" if pf[1] == 1 else "FP64"
+    out["mixed"]["coarse_m2l"] = "FP64 (split integer products)"
     out["mixed"]["coarse_log10_ranges"] = [float(v) for v in pf[2:]]
     # the precision form's near field against HBM (complex64 regular blocks, FP64 reaction
     # blocks and diagonal, x in FP64 and complex64, y read and written); the stage runs
@@ -765,7 +765,7 @@ def run_ours(args):
              "op_rel_diff": float(torch.linalg.norm(ym - y) / torch.linalg.norm(y))}
     pf = lfmm.geometry_query(G, "precision_form", np.float64)
     mixed["fp32_from_level"] = int(pf[0])
-    mixed["coarse_m2l"] = "double-float" if pf[1] == 1 else "FP64"
+    mixed["coarse_m2l"] = "FP64 (split integer products)"
     # the precision form's near field against HBM: complex64 regular blocks, FP64 reaction
     # blocks, the FP64 diagonal, x in FP64 and complex64, y read and written
     ne = lfmm.geometry_query(G, "near_entries", np.float64)

@@ -95,7 +95,7 @@ static std::vector<ExpGroup> make_groups(const std::vector<ExpEntry>& e, int* ma
 
 // M2L work items over the entry ranges: (box, chunk of output coefficients,
 // entry range).  item_work caps the entry x coefficient units of one item (heavy
-// (box, chunk)s are split, their parts reduced by k_m2l_reduce); with wide = 1 an
+// (box, chunk)s are split, their parts reduced by k_m2l32_reduce); with wide = 1 an
 // unsplit box whose coefficients fill a 128-thread CTA better as one row
 // (lane_width) gets a single item.  Replaces the geometry's items.
 static void make_m2l_items(lfmm_geometry_s* g, int item_work, int wide) {
@@ -147,9 +147,6 @@ static void make_m2l_items(lfmm_geometry_s* g, int item_work, int wide) {
     g->m2l_item_work = item_work;
     g->m2l_wide = wide;
     // the partial-sum buffer is sized for the parts: make the next matvec size it again
-    dev_release_now(g->d_m2l_part);
-    g->d_m2l_part = nullptr;
-    g->m2l_part_cols = 0;
 }
 
 // M2L entry descriptors and work items.  Every list entry of a target box
@@ -948,9 +945,6 @@ static void ensure_coef(lfmm_geometry_s* g, int nrhs) {
 }
 
 void fmm_free(lfmm_geometry_s* g) {
-    dev_release(g->d_m2l_part);
-    g->d_m2l_part = nullptr;
-    g->m2l_part_cols = 0;
     dev_release(g->d_sp_ws);
     g->d_sp_ws = nullptr;
     g->sp_ws_cols = 0;
@@ -960,26 +954,6 @@ void fmm_free(lfmm_geometry_s* g) {
     dev_release(g->d_Mp); dev_release(g->d_Lp);
     g->d_M = g->d_L = g->d_Mp = g->d_Lp = nullptr;
     g->coef_cols = 0;
-}
-
-// partial sums of the precision form's double-float M2L
-static void ensure_m2l_part(lfmm_geometry_s* g, int nrhs) {
-    if (g->n_m2l_parts > 0 && g->m2l_part_cols < nrhs) {
-        dev_release_now(g->d_m2l_part);
-        g->d_m2l_part = nullptr;
-        g->d_m2l_part = (cd*)dev_alloc_ready(sizeof(cd) * (size_t)g->n_m2l_parts * 3 * XT_W * nrhs,
-                                             "M2L partial sums");
-        g->m2l_part_cols = nrhs;
-    }
-}
-// reductions [0, r1) of the double-float M2L's split items
-static void launch_m2l_reduce(lfmm_geometry_s* g, int nrhs, int r1, cudaStream_t s) {
-    if (r1 <= 0) return;
-    k_m2l_reduce<<<r1, 64, 0, s>>>(g->d_m2l_reds, g->d_box_level, g->d_p_level, g->d_coef_off, g->d_slot_of,
-                                   g->d_slot_coef, nrhs, g->ncoef, g->nslotcoef, g->n_m2l_parts, g->d_m2l_part, g->d_L,
-                                   g->d_Lp);
-    cuda_check(cudaGetLastError(), "k_m2l_reduce");
-    ++g->n_launches;
 }
 
 // The split M2L's workspace: one row of products per (pair, column), for as many columns
@@ -1227,19 +1201,10 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
             launch_pass(g, make_pass(g, lp + 1, 0, 0, nrhs), nrhs, s, "k_translate (M2M)");
         }
         prof_end(g, ST_M2M, s);
-        {   // M2L, all levels (precision form: the levels >= lm in FP32)
+        {   // M2L: the coarse (wide-band) levels in FP64, the levels >= lm in FP32
             prof_begin(g, ST_M2L, s);
-            const int n64 = g->m2l_item_level_start[lm];
-            const int r64 = g->m2l_red_level_start[lm];
-            if (lm <= D && mixed_coarse_df(g)) {
-                // precision form: the coarse (wide-band) levels in double-float, the rest in FP32
-                ensure_m2l_part(g, nrhs);
-                mixed_m2l_coarse(g, nrhs, n64, s);
-                launch_m2l_reduce(g, nrhs, r64, s);
-            } else {
-                launch_split(g, nrhs, lm, s);
-            }
-            if (lm <= D) mixed_m2l(g, nrhs, lm, s);
+            launch_split(g, nrhs, lm, s);
+            mixed_m2l(g, nrhs, lm, s);
             prof_end(g, ST_M2L, s);
         }
         prof_begin(g, ST_L2L, s);

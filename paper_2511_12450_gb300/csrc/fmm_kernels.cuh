@@ -218,27 +218,6 @@ __global__ void __launch_bounds__(128) k_basis(const ExpGroup* __restrict__ grou
     }
 }
 
-// Sum the partial results of split (box, chunk)s in part order and write them (the
-// precision form's double-float M2L).
-__global__ void __launch_bounds__(64) k_m2l_reduce(const M2LReduce* __restrict__ reds,
-                      const int* __restrict__ box_level, const int* __restrict__ p_level,
-                      const int64_t* __restrict__ coef_off, const int* __restrict__ slot_of,
-                      const int64_t* __restrict__ slot_coef, int nrhs, int64_t ncoef, int64_t nslotcoef, int nparts,
-                      const cd* __restrict__ part, cd* __restrict__ Lout, cd* __restrict__ Lp) {
-    const M2LReduce r = reds[blockIdx.x];
-    const int p = p_level[box_level[r.box]];
-    const int lane = threadIdx.x % XT_W, k = threadIdx.x / XT_W;   // k < 4; 3 used
-    const int idx = r.chunk * XT_W + lane;
-    if (k >= 3 || idx >= 2 * p + 1) return;
-    const int ts = (k == 0) ? -1 : slot_of[2 * r.box + k - 1];
-    if (k > 0 && ts < 0) return;
-    for (int col = 0; col < nrhs; ++col) {
-        cd t = mk(0, 0);
-        for (int q = 0; q < r.nparts; ++q) t += part[(((int64_t)col * nparts + r.part0 + q) * 3 + k) * XT_W + lane];
-        if (k == 0) Lout[(int64_t)col * ncoef + coef_off[r.box] + idx] = t;
-        else Lp[(int64_t)col * nslotcoef + slot_coef[ts] + idx] = t;
-    }
-}
 // L2P: y_j += sum_n L_n J_n(k rho_j) e^{i n theta_j} over the leaf's cell centre and, for a
 // straddling leaf, its reaction centres.  Per entry, A_n = L_n and B_n = (-1)^n L_{-n} are
 // folded into P_n = A_n + B_n and Q_n = A_n - B_n, so that A_n z^n + B_n conj(z^n) =

@@ -98,8 +98,8 @@ struct M2LItem {
     int part;         // -1: write L directly; else partial-sum slot (always XT_W lanes)
     int w;            // output lanes per row: XT_W (chunks of XT_W coefficients) or 2p+1 (all of them)
 };
-// CTAs a block right-hand side's columns are split over in the translation and double-float
-// M2L kernels (groups of four columns); one column keeps one CTA
+// CTAs a block right-hand side's columns are split over in the translation
+// kernels (groups of four columns); one column keeps one CTA
 inline int col_groups(int nrhs) { return nrhs <= 2 ? 1 : (nrhs + 3) / 4; }
 // Lanes per output row for nco coefficients on a 128-thread CTA: chunks of XT_W
 // lanes (8 slices of the sum), or one lane per coefficient with 128 / nco slices,
@@ -337,8 +337,6 @@ struct lfmm_geometry_s {
     int n_m2l_items = 0, n_m2l_parts = 0;
     std::vector<int> m2l_item_level_start;  // [nlev + 2]: first item of each level (levels > D: the end)
     std::vector<int> m2l_red_level_start;   // same for the reductions
-    cd* d_m2l_part = nullptr;               // partial sums [cols][n_m2l_parts][3][XT_W]
-    int m2l_part_cols = 0;
     // FP64 M2L as split integer products: matrices, pairs, units and destinations, coarse
     // levels first
     std::vector<lfmm::SplitTab> sp_tabs_host;
@@ -526,15 +524,11 @@ void mixed_p2m(lfmm_geometry_s* g, const cd* x_sorted, int nrhs, cudaStream_t s)
 void mixed_m2m(lfmm_geometry_s* g, int parent_level, int nrhs, cudaStream_t s);
 void mixed_m_to64(lfmm_geometry_s* g, int level, int nrhs, cudaStream_t s);   // FP32 multipoles -> FP64
 void mixed_m2l(lfmm_geometry_s* g, int nrhs, int min_level, cudaStream_t s);
-// the M2L work items [0, n_items) (the levels below the first FP32 level) in double-float;
-// writes the FP64 locals and partial sums (the caller adds the reductions)
-bool mixed_coarse_df(lfmm_geometry_s* g);
-// first FP32 level of the precision form, whether its coarser levels' M2L runs in
-// double-float (1), in FP64 (0), or is not set up yet (-1: no precision-form call so far), and
-// the log10 magnitudes that decided it (largest free-space and reaction table component, largest
-// scaled multipole basis value)
+// first FP32 level of the precision form; whether its coarser levels' table magnitudes stay in
+// the FP32 exponent range (1), do not or there are no such levels (0), or are not known yet
+// (-1: no precision-form call so far); and their log10 (largest free-space and reaction table
+// component, largest scaled multipole basis value)
 void mixed_info(lfmm_geometry_s* g, int* lm, int* df, double* range);
-void mixed_m2l_coarse(lfmm_geometry_s* g, int nrhs, int n_items, cudaStream_t s);
 void mixed_l_add(lfmm_geometry_s* g, int level, int nrhs, cudaStream_t s);    // FP64 locals += into FP32
 void mixed_l2l(lfmm_geometry_s* g, int child_level, int nrhs, cudaStream_t s);
 void mixed_l2p(lfmm_geometry_s* g, cd* y_sorted, int nrhs, cudaStream_t s);

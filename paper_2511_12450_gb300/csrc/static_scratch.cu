@@ -64,19 +64,16 @@ static inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 // call and restored when the call ends (also when it throws).
 struct ScratchSwap {
     lfmm_geometry_s* g;
-    cd *xs, *ys, *M, *L, *Mp, *Lp, *part;
-    int nrhs_cap, coef_cols, part_cols;
+    cd *xs, *ys, *M, *L, *Mp, *Lp;
+    int nrhs_cap, coef_cols;
     bool prof;
     explicit ScratchSwap(lfmm_geometry_s* geo)
         : g(geo), xs(geo->d_xs), ys(geo->d_ys), M(geo->d_M), L(geo->d_L), Mp(geo->d_Mp), Lp(geo->d_Lp),
-          part(geo->d_m2l_part), nrhs_cap(geo->nrhs_cap), coef_cols(geo->coef_cols),
-          part_cols(geo->m2l_part_cols), prof(geo->prof.on) {}
+          nrhs_cap(geo->nrhs_cap), coef_cols(geo->coef_cols), prof(geo->prof.on) {}
     ~ScratchSwap() {
         g->d_xs = xs; g->d_ys = ys; g->d_M = M; g->d_L = L; g->d_Mp = Mp; g->d_Lp = Lp;
-        g->d_m2l_part = part;
         g->nrhs_cap = nrhs_cap;
         g->coef_cols = coef_cols;
-        g->m2l_part_cols = part_cols;
         g->prof.on = prof;
     }
 };
@@ -90,8 +87,9 @@ extern "C" lfmm_status lfmm_matvec_static(lfmm_geometry g, const void* x, void* 
         if (!g || !x || !y) throw ArgError{"NULL argument"};
         if (x == y) throw ArgError{"x and y must not overlap"};
         if ((uintptr_t)x % 8 != 0 || (uintptr_t)y % 8 != 0) throw ArgError{"device vectors must be 8-byte aligned"};
-        // work buffers: sorted x and y, multipoles/locals (cell centres and reaction centres), M2L
-        // partial sums, one column
+        // work buffers: sorted x and y, multipoles/locals (cell centres and reaction centres), one
+        // column; the room asked for includes the M2L's split items, so that the sizes this
+        // call takes do not depend on which kernel sums them
         const size_t n = (size_t)g->n;
         const size_t b_xs = align256(sizeof(cd) * n), b_ys = b_xs;
         const size_t b_m = align256(sizeof(cd) * (size_t)(g->ncoef > 0 ? g->ncoef : 1));
@@ -113,10 +111,8 @@ extern "C" lfmm_status lfmm_matvec_static(lfmm_geometry g, const void* x, void* 
         g->d_L = (cd*)(base + o); o += b_m;
         g->d_Mp = (cd*)(base + o); o += b_mp;
         g->d_Lp = (cd*)(base + o); o += b_mp;
-        g->d_m2l_part = (cd*)(base + o); o += b_part;
         g->nrhs_cap = 1;
         g->coef_cols = 1;
-        g->m2l_part_cols = 1;
         cudaStream_t s = (cudaStream_t)stream;
         gather_sorted(g, (const cd*)x, g->d_xs, 1, s);
         apply_operator_sorted(g, g->d_xs, g->d_ys, 1, s);
