@@ -51,8 +51,20 @@ struct xcd {
     int e;
 };
 __host__ __device__ __forceinline__ xcd xnorm(cd m, int e) {
-    const double a = fmax(fabs(m.x), fabs(m.y));
     xcd r;
+#ifdef __CUDA_ARCH__
+    // the larger component's exponent and its power of two from the bits, where both are
+    // normal: two products instead of calls (this is the chain that starts every power run)
+    const int ex = max((__double2hiint(m.x) >> 20) & 0x7ff, (__double2hiint(m.y) >> 20) & 0x7ff);
+    if (ex >= 23 && ex <= 2022) {
+        const double f = __hiloint2double((2045 - ex) << 20, 0);   // 2^(1022 - ex)
+        r.m.x = m.x * f;
+        r.m.y = m.y * f;
+        r.e = e + ex - 1022;
+        return r;
+    }
+#endif
+    const double a = fmax(fabs(m.x), fabs(m.y));
     if (!(a > 0.0) || !(a <= 1.7e308)) { r.m = m; r.e = e; return r; }   // zero or not finite: as is
     int k = 0;
     frexp(a, &k);

@@ -12,6 +12,7 @@
 #include <mutex>
 #include <cmath>
 #include <map>
+#include <numeric>
 #include <stdexcept>
 #include <tuple>
 #include <vector>
@@ -487,6 +488,89 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     *g->wait_err = 0;
 }
 
+// The reaction M2L tables: same-layer components from 4p + 1 moments, the others in runs of
+// entries.  Batches of tables share a scratch array of at most TAB_NODE_MAX nodes (one table's
+// at least), which goes back when the batch is queued.
+#define TAB_NODE_MAX (2ll << 20)
+static void build_react_tables(lfmm_geometry_s* g, const std::vector<ReactKey>& keys) {
+    const int nk = (int)keys.size();
+    for (int k0 = 0, k1; k0 < nk; k0 = k1) {
+        std::vector<TableJob> jobs;
+        std::vector<TableSame> same;
+        std::vector<TableChunk> work;
+        std::vector<TableSum> sums;
+        size_t smem = 0, smem_same = 0;
+        int64_t off = 0, npart = 0;
+        int most = 0, most_same = 0, nd_same = 0;
+        for (k1 = k0; k1 < nk; ++k1) {
+            const ReactKey& K = keys[k1];
+            const Component& C = g->tree.comps[K.comp];
+            double h = 0.0;
+            const int nodes = (table_panels(g->quad, K.X, K.D, &h) * g->quad.tab_panel_mult + K.pS + K.pT) * 8 +
+                              2 * g->quad.tab_nes;
+            if (k1 > k0 && off + nodes > TAB_NODE_MAX) break;
+            const TableJob J{k1, nodes, off};
+            jobs.push_back(J);
+            off += nodes;
+            most = std::max(most, nodes);
+            if (C.ls == C.lt && K.pS == K.pT) {
+                const int parts = (nodes + TAB_SAME_RUN - 1) / TAB_SAME_RUN, nd = 4 * K.pS + 1;
+                same.push_back(TableSame{J, parts, npart});
+                npart += (int64_t)parts * nd;
+                most_same = std::max(most_same, parts);
+                nd_same = std::max(nd_same, nd);
+                smem_same = std::max(smem_same, table_same_smem(K.pS));
+                g->table_cmacs[1] += 2.0 * nd * nodes;   // 4p + 1 moments, two terms per node
+                continue;
+            }
+            const int ncT = 2 * K.pT + 1, ne = ncT * (2 * K.pS + 1);
+            g->table_cmacs[0] += 2.0 * ne * nodes;   // every entry, two terms per node
+            const int nch = (ne + 256 * TAB_KPER - 1) / (256 * TAB_KPER);   // runs of nearly equal length
+            for (int ci = 0; ci < nch; ++ci) {
+                const int e0 = (int)((int64_t)ne * ci / nch), e1 = (int)((int64_t)ne * (ci + 1) / nch);
+                const int np = table_parts(e1 - e0, nodes), step = ((nodes + np - 1) / np + TAB_CH - 1) / TAB_CH * TAB_CH;
+                const int parts = (nodes + step - 1) / step;
+                smem = std::max(smem, table_chunk_smem(ncT, (e1 - 1) / ncT - e0 / ncT + 1));
+                if (parts > 1) sums.push_back(TableSum{k1, e0, e1, parts, npart});
+                for (int n0 = 0; n0 < nodes; n0 += step) {
+                    work.push_back(TableChunk{J, e0, e1, n0, std::min(nodes, n0 + step), parts > 1 ? npart : -1});
+                    if (parts > 1) npart += e1 - e0;
+                }
+            }
+        }
+        // the longest first: the last CTAs to start are the shortest
+        std::stable_sort(work.begin(), work.end(), [](const TableChunk& a, const TableChunk& b) {
+            return (int64_t)(a.e1 - a.e0) * (a.n1 - a.n0) > (int64_t)(b.e1 - b.e0) * (b.n1 - b.n0);
+        });
+        const size_t kept = g->allocs.size();
+        const TableJob* d_jobs = dupload(g, jobs);
+        TableNode* d_nodes = dalloc<TableNode>(g, (size_t)off);
+        cd* d_part = dalloc<cd>(g, (size_t)npart);   // sums over parts of the nodes
+        k_table_nodes<<<dim3((int)jobs.size(), (most + TAB_NODE_THREADS - 1) / TAB_NODE_THREADS), TAB_NODE_THREADS>>>(
+            g->m, g->quad, g->d_rkeys, d_jobs, g->d_comp, d_nodes);
+        cuda_check(cudaGetLastError(), "k_table_nodes");
+        if (!work.empty()) {
+            raise_smem_limit((const void*)k_react_tables, smem, "reaction tables smem");
+            k_react_tables<<<(int)work.size(), 256, smem>>>(g->d_rkeys, dupload(g, work), d_nodes, d_part, g->d_m2lr);
+            cuda_check(cudaGetLastError(), "k_react_tables");
+            if (!sums.empty()) {
+                k_react_sum<<<(int)sums.size(), 256>>>(g->d_rkeys, dupload(g, sums), d_part, g->d_m2lr);
+                cuda_check(cudaGetLastError(), "k_react_sum");
+            }
+        }
+        if (!same.empty()) {
+            raise_smem_limit((const void*)k_react_tables_same, smem_same, "same-layer tables smem");
+            const TableSame* d_same = dupload(g, same);
+            k_react_tables_same<<<dim3((int)same.size(), most_same), 256, smem_same>>>(g->d_rkeys, d_same, d_nodes, d_part);
+            cuda_check(cudaGetLastError(), "k_react_tables_same");
+            k_react_toeplitz<<<(int)same.size(), 256, sizeof(cd) * nd_same>>>(g->d_rkeys, d_same, d_part, g->d_m2lr);
+            cuda_check(cudaGetLastError(), "k_react_toeplitz");
+        }
+        for (size_t i = kept; i < g->allocs.size(); ++i) dev_release(g->allocs[i]);
+        g->allocs.resize(kept);
+    }
+}
+
 void fmm_build(lfmm_geometry_s* g) {
     TreeHost& t = g->tree;
     const int D = t.D, l0 = t.l0;
@@ -862,50 +946,7 @@ void fmm_build(lfmm_geometry_s* g) {
         g->d_m2lr = dalloc<cd>(g, (size_t)std::max<int64_t>(tot, 1));
         g->m2lr_len = tot;
         if (!keys.empty()) {
-            // same-layer components: Toeplitz tables from 4p+1 moments; others in runs of entries
-            std::vector<TableChunk> work;
-            std::vector<int> same;
-            int pmax_same = 0;
-            size_t smem = 0;
-            for (int kk = 0; kk < (int)keys.size(); ++kk) {
-                const Component& C = t.comps[keys[kk].comp];
-                int p = keys[kk].pS;
-                double hq = 0.0;
-                const int P0 = table_panels(g->quad, keys[kk].X, keys[kk].D, &hq) * g->quad.tab_panel_mult;
-                if (C.ls == C.lt && keys[kk].pS == keys[kk].pT) {
-                    same.push_back(kk);
-                    pmax_same = std::max(pmax_same, p);
-                    // 4p + 1 moments, two terms per node
-                    g->table_cmacs[1] += 2.0 * (4 * p + 1) * ((P0 + 2 * p) * 8.0 + 2 * g->quad.tab_nes);
-                    continue;
-                }
-                // (2pT + 1) (2pS + 1) entries, two terms per node
-                const int ncT = 2 * keys[kk].pT + 1, ne = ncT * (2 * keys[kk].pS + 1);
-                g->table_cmacs[0] += 2.0 * ne * ((P0 + keys[kk].pS + keys[kk].pT) * 8.0 + 2 * g->quad.tab_nes);
-                // runs of nearly equal length, at most 256 TAB_KPER entries each
-                const int nch = (ne + 256 * TAB_KPER - 1) / (256 * TAB_KPER);
-                for (int ci = 0; ci < nch; ++ci) {
-                    const int e0 = (int)((int64_t)ne * ci / nch), e1 = (int)((int64_t)ne * (ci + 1) / nch);
-                    work.push_back(TableChunk{kk, e0, e1});
-                    smem = std::max(smem, table_chunk_smem(ncT, (e1 - 1) / ncT - e0 / ncT + 1));
-                }
-            }
-            if (!work.empty()) {
-                TableChunk* d_work = dupload(g, work);
-                raise_smem_limit((const void*)k_react_tables, smem, "reaction tables smem");
-                k_react_tables<<<(int)work.size(), 256, smem>>>(g->m, g->quad, g->d_rkeys, d_work, g->d_comp,
-                                                                g->d_m2lr);
-                cuda_check(cudaGetLastError(), "k_react_tables");
-            }
-            if (!same.empty()) {
-                int* d_same = dupload(g, same);
-                const int nd = 4 * pmax_same + 1;
-                const size_t smem = (size_t)(2 * TAB_SAME_CH * nd + 3 * 256 + nd) * sizeof(cd);   // k_react_tables_same layout
-                raise_smem_limit((const void*)k_react_tables_same, smem, "same-layer tables smem");
-                k_react_tables_same<<<(int)same.size(), 256, smem>>>(g->m, g->quad, g->d_rkeys, d_same, g->d_comp,
-                                                                     g->d_m2lr);
-                cuda_check(cudaGetLastError(), "k_react_tables_same");
-            }
+            build_react_tables(g, keys);
         }
         if (g->sp_ntab > 0) {
             k_split_rexp<<<g->sp_ntab, 128>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_xvec, g->d_sp_dexp,

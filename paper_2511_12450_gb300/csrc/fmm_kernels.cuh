@@ -555,6 +555,44 @@ __global__ void __launch_bounds__(128) k_translate(const XPass P, int nrhs) {
     translate_item(blockIdx.x, P, col0, col1, xsm);
 }
 
+// Nodes of the reaction tables' rule: u = w(k_a), v = w(k_b) and the weights F+- with the
+// spectral density and the height factors, per table once (a node costs some 2,000 FP64
+// operations, as much as 250 of the table entries that it serves; the tables are computed by
+// several CTAs each).  A node whose weights vanish (far along a ray) adds nothing: powers of 1
+// keep its finite-valued rows from meeting an infinite power.
+struct TableNode {
+    cd fp, fm, u, v;
+};
+struct TableJob {   // one reaction table: its key, its nodes' place and number
+    int key, nodes;
+    int64_t off;
+};
+#define TAB_NODE_THREADS 64
+__global__ void __launch_bounds__(TAB_NODE_THREADS) k_table_nodes(MediumDev med, QuadRule q, const ReactKey* __restrict__ keys,
+                                                                  const TableJob* __restrict__ jobs,
+                                                                  const int* __restrict__ comp, TableNode* __restrict__ out) {
+    const TableJob J = jobs[blockIdx.x];
+    const ReactKey K = keys[J.key];
+    const int c = K.comp;
+    const int ls = comp[4 * c], a = comp[4 * c + 1], lt = comp[4 * c + 2], b = comp[4 * c + 3];
+    const double ka = med.k[ls], kb = med.k[lt];
+    double h;
+    const int P = table_panels(q, K.X, K.D, &h) * q.tab_panel_mult + (K.pS + K.pT);
+    const int j = blockIdx.y * TAB_NODE_THREADS + threadIdx.x;
+    if (j >= J.nodes) return;
+    const QuadNode nd = table_contour_node(q, j, P, h, K.X, K.D);
+    const cd S = sigma_comp(med, nd.lam, ls, a, lt, b);
+    const cd kya = ky_of(ka, nd.lam), kyb = ky_of(kb, nd.lam);
+    const cd SE = S * (eikh(kya, K.hS) * eikh(kyb, K.hT));
+    TableNode o;
+    o.fp = SE * nd.fp;
+    o.fm = SE * nd.fm;
+    const bool zero = o.fp.x == 0.0 && o.fp.y == 0.0 && o.fm.x == 0.0 && o.fm.y == 0.0;
+    o.u = zero ? mk(1.0, 0.0) : w_of(kya, nd.lam, ka);
+    o.v = zero ? mk(1.0, 0.0) : w_of(kyb, nd.lam, kb);
+    out[J.off + j] = o;
+}
+
 // Reaction M2L moment tables of components whose source and field layers are the
 // same (k_S = k_T, so u = v on every node): I_{mn} = h_{n-m} with
 // h_d = sum_q (Fp_q u_q^d + Fm_q u_q^-d), d = -2p..2p -- 4p+1 moments per key
@@ -562,42 +600,49 @@ __global__ void __launch_bounds__(128) k_translate(const XPass P, int nrhs) {
 // weights are folded into the power rows, each run of 32 starting from F u^d0 formed
 // with a separate exponent (xpow_times): far along the rays u^d alone leaves the double
 // range (|u| ~ 2 lambda / k) where F u^d does not, and F = 0 there must not meet u^d = inf.
-#define TAB_SAME_CH 8
-__global__ void __launch_bounds__(256) k_react_tables_same(MediumDev med, QuadRule q,
-                                                           const ReactKey* __restrict__ keys,
-                                                           const int* __restrict__ key_list,
-                                                           const int* __restrict__ comp, cd* __restrict__ out) {
+// A run of 32 is a serial chain (about a dozen scaled products for F u^d0, then 31 more), so a
+// chunk holds as many nodes as give 192 threads a run each, and in the sums groups of 4p+1
+// threads share its nodes; a CTA takes TAB_SAME_RUN nodes of a table, so that few tables fill
+// the chip too.  The set-ups above: 0.40 ms (a CTA per table, 8 nodes a chunk: 1.6 ms) and
+// 2.9 ms (5.4); 512 nodes a CTA 0.52 and 3.4 ms.
+#define TAB_SAME_NB 256
+__host__ __device__ inline int table_same_nodes(int p) { return 96 / ((4 * p + 32) / 32) + 1; }
+__host__ __device__ inline size_t table_same_smem(int p) {
+    return (size_t)(2 * table_same_nodes(p) * (4 * p + 1) + 3 * TAB_SAME_NB) * sizeof(cd);
+}
+#define TAB_SAME_RUN 256   // nodes a CTA takes
+struct TableSame {   // a same-layer table: its moments' sums, [parts][4p + 1]
+    TableJob job;
+    int parts;
+    int64_t part;
+};
+__global__ void __launch_bounds__(256) k_react_tables_same(const ReactKey* __restrict__ keys,
+                                                           const TableSame* __restrict__ tabs,
+                                                           const TableNode* __restrict__ nodes, cd* __restrict__ part) {
     extern __shared__ cd sh[];
-    const ReactKey K = keys[key_list[blockIdx.x]];
-    const int c = K.comp;
-    const int ls = comp[4 * c], a = comp[4 * c + 1], lt = comp[4 * c + 2], b = comp[4 * c + 3];
-    const int p = K.pS, nco = 2 * p + 1, nd = 4 * p + 1;
-    const double ka = med.k[ls];
-    // nodes in batches of NB = 256 (all threads evaluate the spectral density, one
-    // node each), then in chunks of CH for the power rows and the moment sums
-    const int CH = TAB_SAME_CH, NB = 256;
+    const TableSame T = tabs[blockIdx.x];
+    if (blockIdx.y >= T.parts) return;
+    const int p = keys[T.job.key].pS, nd = 4 * p + 1;
+    const int n0 = blockIdx.y * TAB_SAME_RUN, n1 = min(T.job.nodes, n0 + TAB_SAME_RUN);
+    const int CH = table_same_nodes(p), NB = TAB_SAME_NB;
     cd* Pp = sh;                 // [CH][nd]  Fp u^(d - 2p)
     cd* Pm = Pp + CH * nd;       // [CH][nd]  Fm u^(2p - d)
     cd* Fp = Pm + CH * nd;       // [NB]
     cd* Fm = Fp + NB;            // [NB]
     cd* uu = Fm + NB;            // [NB]
-    cd* hs = uu + NB;            // [nd] moments
-    double h;
-    const int P = table_panels(q, K.X, K.D, &h) * q.tab_panel_mult + 2 * p;
-    const int ntot = P * 8 + 2 * q.tab_nes;
+    cd* hs = Pp;                 // [G][nd] the groups' moments, when the rows are done with
     const int nseg = (nd + 31) / 32;   // runs of 32 consecutive powers per node and side
-    cd acc[2] = {mk(0, 0), mk(0, 0)};   // d = threadIdx.x and threadIdx.x + 256
-    for (int jb = 0; jb < ntot; jb += NB) {
-        const int cntB = min(NB, ntot - jb);
+    const int G = nd <= 256 ? 256 / nd : 1;   // groups; group gi sums the nodes gi, gi + G, ..
+    const int gi = G > 1 ? threadIdx.x / nd : 0, dt = threadIdx.x - gi * nd;
+    cd accp[2] = {mk(0, 0), mk(0, 0)}, accm[2] = {mk(0, 0), mk(0, 0)};   // d = dt and dt + 256
+    for (int jb = n0; jb < n1; jb += NB) {
+        const int cntB = min(NB, n1 - jb);
         __syncthreads();
         if (threadIdx.x < cntB) {
-            QuadNode nd2 = table_contour_node(q, jb + threadIdx.x, P, h, K.X, K.D);
-            cd S = sigma_comp(med, nd2.lam, ls, a, lt, b);
-            cd kya = ky_of(ka, nd2.lam);
-            cd SE = S * (eikh(kya, K.hS) * eikh(kya, K.hT));
-            Fp[threadIdx.x] = SE * nd2.fp;
-            Fm[threadIdx.x] = SE * nd2.fm;
-            uu[threadIdx.x] = w_of(kya, nd2.lam, ka);
+            const TableNode* n = nodes + T.job.off + jb + threadIdx.x;
+            Fp[threadIdx.x] = n->fp;
+            Fm[threadIdx.x] = n->fm;
+            uu[threadIdx.x] = n->u;
         }
         for (int j0 = 0; j0 < cntB; j0 += CH) {
             const int cnt = min(CH, cntB - j0);
@@ -615,23 +660,41 @@ __global__ void __launch_bounds__(256) k_react_tables_same(MediumDev med, QuadRu
             }
             __syncthreads();
             for (int s2 = 0; s2 < 2; ++s2) {
-                const int di = threadIdx.x + 256 * s2;
-                if (di >= nd) break;
-                cd ac = acc[s2];
-                for (int r = 0; r < cnt; ++r) {
-                    ac += Pp[r * nd + di];   // Fp u^d
-                    ac += Pm[r * nd + di];   // Fm u^-d
+                const int di = dt + 256 * s2;
+                if (di >= nd || gi >= G) break;
+                for (int r = gi; r < cnt; r += G) {
+                    accp[s2] += Pp[r * nd + di];   // Fp u^d
+                    accm[s2] += Pm[r * nd + di];   // Fm u^-d
                 }
-                acc[s2] = ac;
             }
         }
     }
+    __syncthreads();
     for (int s2 = 0; s2 < 2; ++s2) {
-        const int di = threadIdx.x + 256 * s2;
-        if (di < nd) hs[di] = acc[s2];
+        const int di = dt + 256 * s2;
+        if (di < nd && gi < G) hs[gi * nd + di] = accp[s2] + accm[s2];
     }
     __syncthreads();
-    // I_{mn} = h_{n-m}, column-major (m, n) at (n + p) nco + (m + p)
+    for (int d = threadIdx.x; d < nd; d += blockDim.x) {
+        cd v = hs[d];
+        for (int k = 1; k < G; ++k) v += hs[k * nd + d];
+        part[T.part + (int64_t)blockIdx.y * nd + d] = v;
+    }
+}
+// I_{mn} = h_{n-m}, column-major (m, n) at (n + p) nco + (m + p)
+__global__ void __launch_bounds__(256) k_react_toeplitz(const ReactKey* __restrict__ keys,
+                                                        const TableSame* __restrict__ tabs, const cd* __restrict__ part,
+                                                        cd* __restrict__ out) {
+    extern __shared__ cd hs[];   // [4p + 1] moments
+    const TableSame T = tabs[blockIdx.x];
+    const ReactKey K = keys[T.job.key];
+    const int p = K.pS, nco = 2 * p + 1, nd = 4 * p + 1;
+    for (int d = threadIdx.x; d < nd; d += blockDim.x) {
+        cd v = mk(0.0, 0.0);
+        for (int q = 0; q < T.parts; ++q) v += part[T.part + (int64_t)q * nd + d];
+        hs[d] = v;
+    }
+    __syncthreads();
     for (int e = threadIdx.x; e < nco * nco; e += blockDim.x) {
         const int ni = e / nco, mi = e - ni * nco;
         out[K.off + e] = hs[(ni - mi) + 2 * p];
@@ -642,35 +705,47 @@ __global__ void __launch_bounds__(256) k_react_tables_same(MediumDev med, QuadRu
 //     I_mn = sum_q [ F+_q v_q^-m u_q^n + F-_q v_q^m u_q^-n ]
 // over the table rule's nodes q (u = w(k_a), v = w(k_b), F+- the weights with the spectral
 // density and the height factors).  One CTA per run of consecutive entries of one table
-// (column-major, (m, n) at (n + pS) ncT + (m + pT)); each thread keeps up to TAB_KPER of them
-// in registers.  Per chunk of TAB_CH nodes the CTA stores the powers v^k (k = -pT..pT, one
-// table serves both v^-m and v^m) and, for its columns, F+ u^n and F- u^-n (the weights folded
-// in), so each entry costs two complex multiply-adds per node and nothing else: the FP64 pipe,
-// which bounds the kernel, does only the sum itself, apart from the powers and node values
-// (a few per cent).
-#define TAB_KPER 16
-#define TAB_CH 8
+// (column-major, (m, n) at (n + pS) ncT + (m + pT)) and range of its nodes; each thread keeps up
+// to TAB_KPER entries in registers.  Per chunk of TAB_CH nodes the CTA stores the powers v^k
+// (k = -pT..pT, one table serves both v^-m and v^m) and, for its columns, F+ u^n and F- u^-n (the
+// weights folded in), so each entry costs two complex multiply-adds per node and nothing else.
+// The FP64 pipe bounds the kernel (97% busy): what remains above the multiply-adds is the power
+// rows, which is why a table is split over its nodes (each power row is formed once) and not over
+// more runs of entries (every run forms all v^k again: 34 ms instead of 18 at 256 entries a run).
+// TAB_COST entries x nodes per CTA keep the last CTAs short: a set-up of 8,200 points over a half
+// space takes 1.25 ms (4.27 with one CTA per table's 4,096 entries, the nodes evaluated in each),
+// one of 16,400 points and 6,000 targets in three layers 17.7 ms (24.8).  A CTA of 4 times
+// the cost takes 2.6 and 18.5 ms.
+#define TAB_KPER 8
+#define TAB_CH 32
 #define TAB_NB 128
+#define TAB_COST 262144.0
 struct TableChunk {
-    int key;
-    int e0, e1;   // entry range [e0, e1) of the key's table, e1 - e0 <= 256 TAB_KPER
+    TableJob job;
+    int e0, e1;     // entry range [e0, e1) of the key's table, e1 - e0 <= 256 TAB_KPER
+    int n0, n1;     // node range
+    int64_t part;   // place of its sums among the partial ones; -1: all nodes, the table itself
 };
+struct TableSum {   // a run of entries whose nodes were split: its sums, [parts][e1 - e0]
+    int key, e0, e1, parts;
+    int64_t part;
+};
+// node ranges for a run of ne entries
+inline int table_parts(int ne, int nodes) { return (int)((double)ne * nodes / TAB_COST) + 1; }
 // dynamic shared memory of one chunk: TAB_CH x (ncT + 2 ncols) powers + 4 TAB_NB node values
 __host__ __device__ inline size_t table_chunk_smem(int ncT, int ncols) {
     return (size_t)(TAB_CH * (ncT + 2 * ncols) + 4 * TAB_NB) * sizeof(cd);
 }
 
-__global__ void __launch_bounds__(256) k_react_tables(MediumDev med, QuadRule q, const ReactKey* __restrict__ keys,
-                                                      const TableChunk* __restrict__ work,
-                                                      const int* __restrict__ comp, cd* __restrict__ out) {
+__global__ void __launch_bounds__(256, 2) k_react_tables(const ReactKey* __restrict__ keys,
+                                                         const TableChunk* __restrict__ work,
+                                                         const TableNode* __restrict__ nodes, cd* __restrict__ part,
+                                                         cd* __restrict__ out) {
     extern __shared__ cd st[];
     const TableChunk wk = work[blockIdx.x];
-    const ReactKey K = keys[wk.key];
-    const int c = K.comp;
-    const int ls = comp[4 * c], a = comp[4 * c + 1], lt = comp[4 * c + 2], b = comp[4 * c + 3];
+    const ReactKey K = keys[wk.job.key];
     const int pS = K.pS, pT = K.pT;
     const int ncT = 2 * pT + 1;
-    const double ka = med.k[ls], kb = med.k[lt];
     const int nlo = wk.e0 / ncT, nhi = (wk.e1 - 1) / ncT;   // column indices (from -pS) of the run
     const int ncols = nhi - nlo + 1;
     cd* Wv = st;                          // [TAB_CH][ncT]    v^(k - pT)
@@ -681,7 +756,7 @@ __global__ void __launch_bounds__(256) k_react_tables(MediumDev med, QuadRule q,
     cd* uu = Fm + TAB_NB;                 // [TAB_NB] u
     cd* vv = uu + TAB_NB;                 // [TAB_NB] v
     // this thread's entries: e = e0 + threadIdx.x + 256 k; row mi and column j within the run
-    const int kper = (wk.e1 - wk.e0 + 255) / 256;
+    const int kper = max(0, (wk.e1 - wk.e0 - (int)(threadIdx.x & ~31u) + 255) / 256);   // of its warp
     int rowc[TAB_KPER], colc[TAB_KPER];
 #pragma unroll
     for (int k = 0; k < TAB_KPER; ++k) {
@@ -689,29 +764,19 @@ __global__ void __launch_bounds__(256) k_react_tables(MediumDev med, QuadRule q,
         rowc[k] = e % ncT;
         colc[k] = e / ncT - nlo;
     }
-    double h;
-    const int P = table_panels(q, K.X, K.D, &h) * q.tab_panel_mult + (pS + pT);
-    const int ntot = P * 8 + 2 * q.tab_nes;
     cd acc[TAB_KPER];
 #pragma unroll
     for (int k = 0; k < TAB_KPER; ++k) acc[k] = mk(0, 0);
     const int wruns = (ncT + 31) / 32, uruns = (ncols + 31) / 32;
-    for (int jb = 0; jb < ntot; jb += TAB_NB) {
-        const int cntB = min(TAB_NB, ntot - jb);
+    for (int jb = wk.n0; jb < wk.n1; jb += TAB_NB) {
+        const int cntB = min(TAB_NB, wk.n1 - jb);
         __syncthreads();
         if (threadIdx.x < cntB) {
-            QuadNode nd = table_contour_node(q, jb + threadIdx.x, P, h, K.X, K.D);
-            cd S = sigma_comp(med, nd.lam, ls, a, lt, b);
-            cd kya = ky_of(ka, nd.lam), kyb = ky_of(kb, nd.lam);
-            cd SE = S * (eikh(kya, K.hS) * eikh(kyb, K.hT));
-            const cd fp = SE * nd.fp, fm = SE * nd.fm;
-            Fp[threadIdx.x] = fp;
-            Fm[threadIdx.x] = fm;
-            // a node whose weights vanish (far along a ray) adds nothing: powers of 1 keep
-            // its finite-valued rows from meeting an infinite power
-            const bool zero = fp.x == 0.0 && fp.y == 0.0 && fm.x == 0.0 && fm.y == 0.0;
-            uu[threadIdx.x] = zero ? mk(1.0, 0.0) : w_of(kya, nd.lam, ka);
-            vv[threadIdx.x] = zero ? mk(1.0, 0.0) : w_of(kyb, nd.lam, kb);
+            const TableNode* n = nodes + wk.job.off + jb + threadIdx.x;
+            Fp[threadIdx.x] = n->fp;
+            Fm[threadIdx.x] = n->fm;
+            uu[threadIdx.x] = n->u;
+            vv[threadIdx.x] = n->v;
         }
         for (int j0 = 0; j0 < cntB; j0 += TAB_CH) {
             const int cnt = min(TAB_CH, cntB - j0);
@@ -758,7 +823,21 @@ __global__ void __launch_bounds__(256) k_react_tables(MediumDev med, QuadRule q,
 #pragma unroll
     for (int k = 0; k < TAB_KPER; ++k) {
         const int e = wk.e0 + (int)threadIdx.x + 256 * k;
-        if (k < kper && e < wk.e1) out[K.off + e] = acc[k];
+        if (k < kper && e < wk.e1) {
+            if (wk.part < 0) out[K.off + e] = acc[k];
+            else part[wk.part + e - wk.e0] = acc[k];
+        }
+    }
+}
+// the split runs' entries, parts in node order
+__global__ void __launch_bounds__(256) k_react_sum(const ReactKey* __restrict__ keys, const TableSum* __restrict__ sums,
+                                                   const cd* __restrict__ part, cd* __restrict__ out) {
+    const TableSum T = sums[blockIdx.x];
+    const int ne = T.e1 - T.e0;
+    for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+        cd v = mk(0.0, 0.0);
+        for (int q = 0; q < T.parts; ++q) v += part[T.part + (int64_t)q * ne + e];
+        out[keys[T.key].off + T.e0 + e] = v;
     }
 }
 
