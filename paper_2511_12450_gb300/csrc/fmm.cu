@@ -490,10 +490,33 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
 
 // The reaction M2L tables: same-layer components from 4p + 1 moments, the others in runs of
 // entries.  Batches of tables share a scratch array of at most TAB_NODE_MAX nodes (one table's
-// at least), which goes back when the batch is queued.
+// at least), which goes back when the batch is queued.  All of it on the geometry's side stream:
+// the host builds the M2L lists meanwhile.
 #define TAB_NODE_MAX (2ll << 20)
 static void build_react_tables(lfmm_geometry_s* g, const std::vector<ReactKey>& keys) {
     const int nk = (int)keys.size();
+    const cudaStream_t s = g->side;
+    struct Scratch {
+        cudaStream_t s;
+        std::vector<void*> v;
+        void drop() {
+            for (void* p : v) cudaFreeAsync(p, s);
+            v.clear();
+        }
+        ~Scratch() { drop(); }
+    } scratch{s, {}};
+    auto room = [&](size_t bytes) {
+        void* p = nullptr;
+        cuda_check(cudaMallocAsync(&p, std::max<size_t>(bytes, 16), s), "table scratch");
+        scratch.v.push_back(p);
+        return p;
+    };
+    auto upload = [&](const auto& v) {   // (pageable memory: the call returns once it is staged)
+        auto* p = (typename std::decay_t<decltype(v)>::value_type*)room(v.size() * sizeof(typename std::decay_t<decltype(v)>::value_type));
+        if (!v.empty())
+            cuda_check(cudaMemcpyAsync(p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, s), "table jobs");
+        return p;
+    };
     for (int k0 = 0, k1; k0 < nk; k0 = k1) {
         std::vector<TableJob> jobs;
         std::vector<TableSame> same;
@@ -542,32 +565,32 @@ static void build_react_tables(lfmm_geometry_s* g, const std::vector<ReactKey>& 
         std::stable_sort(work.begin(), work.end(), [](const TableChunk& a, const TableChunk& b) {
             return (int64_t)(a.e1 - a.e0) * (a.n1 - a.n0) > (int64_t)(b.e1 - b.e0) * (b.n1 - b.n0);
         });
-        const size_t kept = g->allocs.size();
-        const TableJob* d_jobs = dupload(g, jobs);
-        TableNode* d_nodes = dalloc<TableNode>(g, (size_t)off);
-        cd* d_part = dalloc<cd>(g, (size_t)npart);   // sums over parts of the nodes
-        k_table_nodes<<<dim3((int)jobs.size(), (most + TAB_NODE_THREADS - 1) / TAB_NODE_THREADS), TAB_NODE_THREADS>>>(
+        const TableJob* d_jobs = upload(jobs);   // all uploads before the first kernel: a large one waits for its stream
+        const TableChunk* d_work = upload(work);
+        const TableSum* d_sums = upload(sums);
+        const TableSame* d_same = upload(same);
+        TableNode* d_nodes = (TableNode*)room(sizeof(TableNode) * off);
+        cd* d_part = (cd*)room(sizeof(cd) * npart);   // sums over parts of the nodes
+        k_table_nodes<<<dim3((int)jobs.size(), (most + TAB_NODE_THREADS - 1) / TAB_NODE_THREADS), TAB_NODE_THREADS, 0, s>>>(
             g->m, g->quad, g->d_rkeys, d_jobs, g->d_comp, d_nodes);
         cuda_check(cudaGetLastError(), "k_table_nodes");
         if (!work.empty()) {
             raise_smem_limit((const void*)k_react_tables, smem, "reaction tables smem");
-            k_react_tables<<<(int)work.size(), 256, smem>>>(g->d_rkeys, dupload(g, work), d_nodes, d_part, g->d_m2lr);
+            k_react_tables<<<(int)work.size(), 256, smem, s>>>(g->d_rkeys, d_work, d_nodes, d_part, g->d_m2lr);
             cuda_check(cudaGetLastError(), "k_react_tables");
             if (!sums.empty()) {
-                k_react_sum<<<(int)sums.size(), 256>>>(g->d_rkeys, dupload(g, sums), d_part, g->d_m2lr);
+                k_react_sum<<<(int)sums.size(), 256, 0, s>>>(g->d_rkeys, d_sums, d_part, g->d_m2lr);
                 cuda_check(cudaGetLastError(), "k_react_sum");
             }
         }
         if (!same.empty()) {
             raise_smem_limit((const void*)k_react_tables_same, smem_same, "same-layer tables smem");
-            const TableSame* d_same = dupload(g, same);
-            k_react_tables_same<<<dim3((int)same.size(), most_same), 256, smem_same>>>(g->d_rkeys, d_same, d_nodes, d_part);
+            k_react_tables_same<<<dim3((int)same.size(), most_same), 256, smem_same, s>>>(g->d_rkeys, d_same, d_nodes, d_part);
             cuda_check(cudaGetLastError(), "k_react_tables_same");
-            k_react_toeplitz<<<(int)same.size(), 256, sizeof(cd) * nd_same>>>(g->d_rkeys, d_same, d_part, g->d_m2lr);
+            k_react_toeplitz<<<(int)same.size(), 256, sizeof(cd) * nd_same, s>>>(g->d_rkeys, d_same, d_part, g->d_m2lr);
             cuda_check(cudaGetLastError(), "k_react_toeplitz");
         }
-        for (size_t i = kept; i < g->allocs.size(); ++i) dev_release(g->allocs[i]);
-        g->allocs.resize(kept);
+        scratch.drop();
     }
 }
 
@@ -939,15 +962,22 @@ void fmm_build(lfmm_geometry_s* g) {
         g->d_vr_src = dupload(g, vr_src);
         g->d_vr_key = dupload(g, vr_key);
         g->d_vr_comp = dupload(g, vr_comp);
-        build_m2l_work(g, vr_ptr, vr_src, vr_key, vr_comp, vr_flip, keys);
-        build_split(g, vr_ptr, vr_src, vr_key, vr_comp, vr_flip, keys);
         g->d_rkeys = dupload(g, keys);
         g->rkeys_host = keys;
         g->d_m2lr = dalloc<cd>(g, (size_t)std::max<int64_t>(tot, 1));
         g->m2lr_len = tot;
-        if (!keys.empty()) {
-            build_react_tables(g, keys);
-        }
+        // the reaction tables on the side stream, beside the lists on the host
+        struct SideWork {
+            cudaStream_t s;
+            ~SideWork() { cudaStreamSynchronize(s); }   // a failing build must not free what they read
+        } side{g->side};
+        cuda_check(cudaEventRecord(g->ev_fork, cudaStreamPerThread), "fork record");
+        cuda_check(cudaStreamWaitEvent(g->side, g->ev_fork), "fork wait");
+        build_react_tables(g, keys);
+        cuda_check(cudaEventRecord(g->ev_join, g->side), "join record");
+        build_m2l_work(g, vr_ptr, vr_src, vr_key, vr_comp, vr_flip, keys);
+        build_split(g, vr_ptr, vr_src, vr_key, vr_comp, vr_flip, keys);
+        cuda_check(cudaStreamWaitEvent(cudaStreamPerThread, g->ev_join), "join wait");
         if (g->sp_ntab > 0) {
             k_split_rexp<<<g->sp_ntab, 128>>>(g->d_sp_tab, g->d_m2lf, g->d_m2lr, g->d_xvec, g->d_sp_dexp,
                                               g->d_sp_rexp);
