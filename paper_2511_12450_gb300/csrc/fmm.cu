@@ -612,6 +612,70 @@ void fmm_build(lfmm_geometry_s* g) {
     g->box_coef_off_host = off;
     if (l0 > D) return;   // no far field: everything is in the near field
 
+    // reaction M2L keys, tables and lists; the tables on the side stream, beside what the host
+    // does from here on
+    std::vector<ReactKey> keys;
+    std::vector<int> vr_ptr(t.nbox + 1, 0), vr_src, vr_key, vr_comp, vr_flip;
+    struct SideWork {
+        cudaStream_t s;
+        ~SideWork() { cudaStreamSynchronize(s); }   // a failing build must not free what they read
+    } side{g->side};
+    {
+        std::map<std::tuple<int, int, int, int, int>, int> id;
+        int64_t tot = 0;
+        for (int T = 0; T < t.nbox; ++T) {
+            for (int e = t.vreact_ptr[T]; e < t.vreact_ptr[T + 1]; ++e) {
+                int S = t.vreact_idx[e], c = t.vreact_comp[e];
+                int l = t.box_level[T];
+                // a pair at horizontal offset -X uses the table of +X with both indices
+                // reversed: lambda -> -lambda maps e^{i lambda X} to e^{-i lambda X} and
+                // w(lambda, k) to 1 / w(lambda, k) (k_y is even in lambda), so
+                // I(-X)_{mn} = I(X)_{-m,-n}
+                const int dix = t.box_ix[S] - t.box_ix[T];
+                const int flip = dix < 0 ? 1 : 0;
+                auto key = std::make_tuple(c, l, flip ? -dix : dix, t.box_iy[S], t.box_iy[T]);
+                auto it = id.find(key);
+                int kid;
+                if (it == id.end()) {
+                    kid = (int)keys.size();
+                    id[key] = kid;
+                    const Component& C = t.comps[c];
+                    ReactKey rk;
+                    rk.comp = c; rk.level = l; rk.pS = t.p_level[l]; rk.pT = t.p_level[l];
+                    double w = t.width(l);
+                    rk.X = (flip ? -dix : dix) * w;
+                    double loS = t.y0 + t.box_iy[S] * w, hiS = t.y0 + (t.box_iy[S] + 1) * w;
+                    double loT = t.y0 + t.box_iy[T] * w, hiT = t.y0 + (t.box_iy[T] + 1) * w;
+                    rk.hS = src_height_box(g->m, C.ls, C.a, loS, hiS);
+                    rk.hT = tgt_height_box(g->m, C.lt, C.b, loT, hiT);
+                    rk.D = rk.hS + rk.hT + C.Hc;
+                    rk.off = tot;
+                    g->rkey_lay_s.push_back(t.box_layer[S]);
+                    g->rkey_lay_t.push_back(t.box_layer[T]);
+                    tot += (int64_t)(2 * rk.pT + 1) * (2 * rk.pS + 1);
+                    keys.push_back(rk);
+                } else {
+                    kid = it->second;
+                }
+                vr_src.push_back(S); vr_key.push_back(kid); vr_comp.push_back(c); vr_flip.push_back(flip);
+            }
+            vr_ptr[T + 1] = (int)vr_src.size();
+        }
+        g->n_rkeys = (int)keys.size();
+        g->d_vr_ptr = dupload(g, vr_ptr);
+        g->d_vr_src = dupload(g, vr_src);
+        g->d_vr_key = dupload(g, vr_key);
+        g->d_vr_comp = dupload(g, vr_comp);
+        g->d_rkeys = dupload(g, keys);
+        g->rkeys_host = keys;
+        g->d_m2lr = dalloc<cd>(g, (size_t)std::max<int64_t>(tot, 1));
+        g->m2lr_len = tot;
+        cuda_check(cudaEventRecord(g->ev_fork, cudaStreamPerThread), "fork record");
+        cuda_check(cudaStreamWaitEvent(g->side, g->ev_fork), "fork wait");
+        build_react_tables(g, keys);
+        cuda_check(cudaEventRecord(g->ev_join, g->side), "join record");
+    }
+
     // Reaction centres of cells that straddle their layer's interfaces: the
     // centre of the part of the cell on the layer's side (one slot per
     // (box, side); side 0 = the layer's bottom interface, 1 = its top one).
@@ -913,68 +977,8 @@ void fmm_build(lfmm_geometry_s* g) {
             cuda_check(cudaGetLastError(), "k_m2lf_tables");
         }
     }
-    // reaction M2L keys, tables and lists
+    // M2L work from the lists and tables
     {
-        std::map<std::tuple<int, int, int, int, int>, int> id;
-        std::vector<ReactKey> keys;
-        std::vector<int> vr_ptr(t.nbox + 1, 0), vr_src, vr_key, vr_comp, vr_flip;
-        int64_t tot = 0;
-        for (int T = 0; T < t.nbox; ++T) {
-            for (int e = t.vreact_ptr[T]; e < t.vreact_ptr[T + 1]; ++e) {
-                int S = t.vreact_idx[e], c = t.vreact_comp[e];
-                int l = t.box_level[T];
-                // a pair at horizontal offset -X uses the table of +X with both indices
-                // reversed: lambda -> -lambda maps e^{i lambda X} to e^{-i lambda X} and
-                // w(lambda, k) to 1 / w(lambda, k) (k_y is even in lambda), so
-                // I(-X)_{mn} = I(X)_{-m,-n}
-                const int dix = t.box_ix[S] - t.box_ix[T];
-                const int flip = dix < 0 ? 1 : 0;
-                auto key = std::make_tuple(c, l, flip ? -dix : dix, t.box_iy[S], t.box_iy[T]);
-                auto it = id.find(key);
-                int kid;
-                if (it == id.end()) {
-                    kid = (int)keys.size();
-                    id[key] = kid;
-                    const Component& C = t.comps[c];
-                    ReactKey rk;
-                    rk.comp = c; rk.level = l; rk.pS = t.p_level[l]; rk.pT = t.p_level[l];
-                    double w = t.width(l);
-                    rk.X = (flip ? -dix : dix) * w;
-                    double loS = t.y0 + t.box_iy[S] * w, hiS = t.y0 + (t.box_iy[S] + 1) * w;
-                    double loT = t.y0 + t.box_iy[T] * w, hiT = t.y0 + (t.box_iy[T] + 1) * w;
-                    rk.hS = src_height_box(g->m, C.ls, C.a, loS, hiS);
-                    rk.hT = tgt_height_box(g->m, C.lt, C.b, loT, hiT);
-                    rk.D = rk.hS + rk.hT + C.Hc;
-                    rk.off = tot;
-                    g->rkey_lay_s.push_back(t.box_layer[S]);
-                    g->rkey_lay_t.push_back(t.box_layer[T]);
-                    tot += (int64_t)(2 * rk.pT + 1) * (2 * rk.pS + 1);
-                    keys.push_back(rk);
-                } else {
-                    kid = it->second;
-                }
-                vr_src.push_back(S); vr_key.push_back(kid); vr_comp.push_back(c); vr_flip.push_back(flip);
-            }
-            vr_ptr[T + 1] = (int)vr_src.size();
-        }
-        g->n_rkeys = (int)keys.size();
-        g->d_vr_ptr = dupload(g, vr_ptr);
-        g->d_vr_src = dupload(g, vr_src);
-        g->d_vr_key = dupload(g, vr_key);
-        g->d_vr_comp = dupload(g, vr_comp);
-        g->d_rkeys = dupload(g, keys);
-        g->rkeys_host = keys;
-        g->d_m2lr = dalloc<cd>(g, (size_t)std::max<int64_t>(tot, 1));
-        g->m2lr_len = tot;
-        // the reaction tables on the side stream, beside the lists on the host
-        struct SideWork {
-            cudaStream_t s;
-            ~SideWork() { cudaStreamSynchronize(s); }   // a failing build must not free what they read
-        } side{g->side};
-        cuda_check(cudaEventRecord(g->ev_fork, cudaStreamPerThread), "fork record");
-        cuda_check(cudaStreamWaitEvent(g->side, g->ev_fork), "fork wait");
-        build_react_tables(g, keys);
-        cuda_check(cudaEventRecord(g->ev_join, g->side), "join record");
         build_m2l_work(g, vr_ptr, vr_src, vr_key, vr_comp, vr_flip, keys);
         build_split(g, vr_ptr, vr_src, vr_key, vr_comp, vr_flip, keys);
         cuda_check(cudaStreamWaitEvent(cudaStreamPerThread, g->ev_join), "join wait");
