@@ -170,6 +170,7 @@ static void free_geometry(lfmm_geometry_s* g) {
         cudaStreamDestroy(g->side);
         g->side = nullptr;
     }
+    mixed_wait(g);
     if (g->ev_fork) cudaEventDestroy(g->ev_fork);
     if (g->ev_join) cudaEventDestroy(g->ev_join);
     g->ev_fork = g->ev_join = nullptr;

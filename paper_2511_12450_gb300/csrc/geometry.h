@@ -520,6 +520,9 @@ void apply_operator_batch_sorted(const std::vector<BatchOp>& ops, cudaStream_t s
 void raise_smem_limit(const void* func, size_t bytes, const char* what);
 // precision form: M2L in FP32 on scaled expansions (mixed.cu)
 void mixed_setup(lfmm_geometry_s* g, int nrhs);                       // tables, scales, FP32 buffers
+cudaStream_t mixed_fork(lfmm_geometry_s* g, cudaStream_t s);         // a stream beside s, until mixed_join
+void mixed_join(lfmm_geometry_s* g, cudaStream_t s);
+void mixed_wait(lfmm_geometry_s* g);   // host wait for that stream (before the buffers go)
 void mixed_p2m(lfmm_geometry_s* g, const cd* x_sorted, int nrhs, cudaStream_t s);
 void mixed_m2m(lfmm_geometry_s* g, int parent_level, int nrhs, cudaStream_t s);
 void mixed_m_to64(lfmm_geometry_s* g, int level, int nrhs, cudaStream_t s);   // FP32 multipoles -> FP64

@@ -84,6 +84,8 @@ struct MixedState {
     int tc_p = 0;                       // largest expansion order of the FP32 levels (the coarsest)
     int* tc_err = nullptr;              // set when an mbarrier wait of k_m2l32_tc gave up
     int* tc_err_host = nullptr;         // pinned copy, read at the next call
+    cudaStream_t top = nullptr;         // the coarse levels' FP64 chain, beside the FP32 M2L
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     double range[3] = {0, 0, 0};        // log10: largest free-space, reaction table component of the levels below lm; scaled basis
     bool range_ok = false;              // they stay inside the FP32 exponent range
 };
@@ -736,6 +738,9 @@ void mixed_destroy(lfmm_geometry_s* g) {
     dev_release(ms->q_bwoff);
     dev_release(ms->tc_boxes); dev_release(ms->tc_ent_ptr); dev_release(ms->tc_err);
     if (ms->tc_err_host) cudaFreeHost(ms->tc_err_host);
+    if (ms->top) cudaStreamDestroy(ms->top);
+    if (ms->ev_fork) cudaEventDestroy(ms->ev_fork);
+    if (ms->ev_join) cudaEventDestroy(ms->ev_join);
     delete ms;
     g->mixed = nullptr;
 }
@@ -773,6 +778,11 @@ static void mixed_build(lfmm_geometry_s* g) {
     const int D = t.D, l0 = t.l0, nlev = D + 1, nl = g->m.nl;
     MixedState* ms = new MixedState();
     g->mixed = ms;
+    int least = 0, greatest = 0;
+    cuda_check(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priorities");
+    cuda_check(cudaStreamCreateWithPriority(&ms->top, cudaStreamNonBlocking, greatest), "coarse levels' stream");
+    cuda_check(cudaEventCreateWithFlags(&ms->ev_fork, cudaEventDisableTiming), "event");
+    cuda_check(cudaEventCreateWithFlags(&ms->ev_join, cudaEventDisableTiming), "event");
     ms->scale.assign((size_t)nl * nlev, 1.0);
     for (int lay = 0; lay < nl; ++lay)
         for (int l = l0; l <= D; ++l)
@@ -991,6 +1001,22 @@ void mixed_setup(lfmm_geometry_s* g, int nrhs) {
                                         "M2L partial sums 32");
         ms->cols = nrhs;
     }
+}
+
+// a stream that continues from s beside it, until mixed_join
+cudaStream_t mixed_fork(lfmm_geometry_s* g, cudaStream_t s) {
+    MixedState* ms = g->mixed;
+    cuda_check(cudaEventRecord(ms->ev_fork, s), "coarse levels' fork");
+    cuda_check(cudaStreamWaitEvent(ms->top, ms->ev_fork, 0), "coarse levels' fork");
+    return ms->top;
+}
+void mixed_join(lfmm_geometry_s* g, cudaStream_t s) {
+    MixedState* ms = g->mixed;
+    cuda_check(cudaEventRecord(ms->ev_join, ms->top), "coarse levels' join");
+    cuda_check(cudaStreamWaitEvent(s, ms->ev_join, 0), "coarse levels' join");
+}
+void mixed_wait(lfmm_geometry_s* g) {
+    if (g->mixed && g->mixed->top) cudaStreamSynchronize(g->mixed->top);
 }
 
 void mixed_p2m(lfmm_geometry_s* g, const cd* x_sorted, int nrhs, cudaStream_t s) {
