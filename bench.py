@@ -36,13 +36,14 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 HBM_FALLBACK_GBS = 6800.0
+BF16_FALLBACK_TFLOPS = 1900.0
 # FP64 peak from unit counts and clock: 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz
 # (a DFMA microbenchmark on the same GPU model reached 1.194 TFLOP/s, 95 %)
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # DRAM traffic per launch from the committed ncu captures (profiles/); null once the
 # kernel changes after the capture
-NCU_TRAFFIC_BYTES = {"k_m2l": 85761280.0 + 3519488.0, "k_near_leaf": 67980800.0 + 316160.0,
-                     "k_near_leaf (precision form)": 38071040.0}
+NCU_TRAFFIC_BYTES = {"k_split": 427517440.0 + 29704704.0, "k_near_leaf": 67043072.0 + 274688.0,
+                     "k_near_leaf (precision form)": 40003072.0}
 
 
 def run_combined(lfmm, wl, M, pts, w, nrm, x, flush, stream, args, dist, n):
@@ -730,11 +731,12 @@ def run_ours(args):
     dom = max(("m2l", "near"), key=lambda k: stages[k]["ms"])
     if dom == "m2l":
         avg_s = stages["m2l"]["ms"] / max(stages["m2l"]["count"], 1) * 1e-3
-        achieved = work["m2l_flops"] / avg_s / 1e12
-        roof = {"kernel": "k_m2l", "bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
-                "traffic": NCU_TRAFFIC_BYTES.get("k_m2l"),
-                "peak_source": "FP64 from unit counts x clock (152 SMs x 2 DFMA/clk x 2.07 GHz)"}
+        # the FP64 sums as products of 8-bit digits: 36 digit pairs per real product
+        achieved = 36.0 * work["m2l_flops"] / avg_s / 1e12
+        peak = float(peaks.get("bf16_tflops", BF16_FALLBACK_TFLOPS))
+        roof = {"kernel": "k_split", "bound": "tensor", "achieved": achieved, "peak": peak,
+                "unit": "TFLOP/s", "frac": achieved / peak, "traffic": NCU_TRAFFIC_BYTES.get("k_split"),
+                "fp64_equivalent_tflops": work["m2l_flops"] / avg_s / 1e12, "peak_source": src}
     else:
         avg_s = stages["near"]["ms"] / max(stages["near"]["count"], 1) * 1e-3
         peak = float(peaks.get("hbm_gbs", HBM_FALLBACK_GBS))

@@ -97,3 +97,25 @@ def test_passes_as_products_in_blocks_and_batches(gpu_lib):
     single = [x[0].contiguous() for x in xs]
     for y, ref in zip(lf.matvec_batch(geos, single), own):
         assert torch.equal(y, ref[0])
+
+
+def test_coarse_levels_beside_the_fp32_ones(gpu_lib):
+    """Precision form: the coarse levels' chain on its own stream, beside the FP32 M2L (SIMT and, from
+    16 columns, on the tensor cores), gives the bits of the chain in one stream (stage timers on)."""
+    import torch
+
+    from workloads import layered_wide
+
+    lf = gpu_lib
+    wl = layered_wide()
+    pts, w, _, _ = onys.elements(wl.bodies)
+    M = lf.medium_create(wl.medium.interfaces, wl.medium.k, wl.medium.eta)
+    G, S = (lf.geometry_build(M, pts, w, p=20, leaf_size=8, profile=prof) for prof in (False, True))
+    rng = np.random.default_rng(8)
+    for cols in (1, 5, 20):
+        X = torch.from_numpy(rng.standard_normal((cols, G.n)) + 1j * rng.standard_normal((cols, G.n))).cuda()
+        ref = lf.matvec(S, X, mixed=True)
+        for _ in range(5):
+            assert torch.equal(lf.matvec(G, X, mixed=True), ref)
+    lm = lf.geometry_query(G, "precision_form", np.float64)[0]
+    assert lm > lf.geometry_query(G, "tree_params", np.float64)[4], "coarse levels must be in use"
