@@ -203,14 +203,14 @@ static void build_m2l_work(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, c
 // first FP32 level are a prefix.
 static size_t split_col_bytes(const lfmm_geometry_s* g) {   // workspace of one column
     return sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) +
-           (size_t)g->sp_nvec * (SP_ND * SP_POS * sizeof(uint32_t) + sizeof(int)) + 16;
+           (size_t)g->sp_nvec * (SP_ND * SP_BLK * sizeof(uint32_t) + sizeof(int)) + 16;
 }
 static void split_alloc(lfmm_geometry_s* g, int cols) {   // products, then digits, then exponents
     unsigned char* p = (unsigned char*)dev_alloc_ready(split_col_bytes(g) * cols, "split M2L workspace");
     const size_t rows = sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) * cols;
     g->d_sp_ws = (double*)p;
     g->d_sp_vdig = (uint32_t*)(p + ((rows + 15) & ~(size_t)15));
-    g->d_sp_vexp = (int*)(g->d_sp_vdig + (size_t)g->sp_nvec * cols * SP_ND * SP_POS);
+    g->d_sp_vexp = (int*)(g->d_sp_vdig + (size_t)g->sp_nvec * cols * SP_ND * SP_BLK);
     g->sp_ws_cols = cols;
 }
 // Units: a matrix's (pair, column) columns in groups of up to sp_cap, of nearly equal size, by
@@ -227,8 +227,8 @@ static void make_split_plan(lfmm_geometry_s* g, SplitPlan& P, int ncols) {
             for (int k = 0; k * split_tile(nco) < nco; ++k)
             {
                 const int nr8 = (split_tile(nco) + 7) & ~7;
-                units.push_back(SplitUnit{s.dig + k * split_tile_bytes(s.pS, nr8), s.out0 * ncols + (int64_t)q0 * 2 * nco, s.pT,
-                                          s.pS, s.rexp, s.pair0, q0, q1 - q0, k});
+                units.push_back(SplitUnit{s.dig + k * split_tile_bytes(s.pS, s.z, nr8), s.out0 * ncols + (int64_t)q0 * 2 * nco, s.pT,
+                                          s.pS, s.z, s.rexp, s.pair0, q0, q1 - q0, k});
             }
         }
     }
@@ -295,6 +295,8 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     std::vector<std::vector<int>> by_level(nlev);
     for (int i = 0; i < nF; ++i) if (cnt[i]) by_level[g->ftab_lev[i]].push_back(i);
     for (int i = 0; i < nR; ++i) if (cnt[nF + i]) by_level[keys[i].level].push_back(nF + i);
+    for (std::vector<int>& v : by_level)   // the matrices in fine segments first: their units take longest
+        std::stable_partition(v.begin(), v.end(), [&](int i) { return i >= nF && g->rkey_fine[i - nF] != 0; });
     std::vector<SplitTab> tabs;
     std::vector<int> tab_of(nF + nR, -1);
     int64_t dig = 0;
@@ -309,40 +311,55 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
                 s.base = g->ftab_off_host[i] + 2 * p;
                 s.sr = -1; s.sc = 1; s.react = 0;
                 s.dexp = dexp_off[g->ftab_lay[i] * nlev + l];
+                s.z = split_size(p, false);
             } else {        // column-major
                 s.base = keys[i - nF].off;
                 s.sr = 1; s.sc = nco; s.react = 1;
                 s.dexp = dexp_off[g->rkey_lay_s[i - nF] * nlev + l];
+                s.z = split_size(p, g->rkey_fine[i - nF] != 0);
             }
-            s.rexp = nrexp; nrexp += nco * split_nseg(p);
+            s.rexp = nrexp; nrexp += nco * split_nseg(p, s.z);
             s.pair0 = np; s.npairs = cnt[i]; np += cnt[i];
             s.out0 = rows; rows += (int64_t)cnt[i] * 2 * nco;
             const int tiles = (nco + split_tile(nco) - 1) / split_tile(nco);
-            s.dig = dig; dig += tiles * split_tile_bytes(p, (split_tile(nco) + 7) & ~7);
+            s.dig = dig; dig += tiles * split_tile_bytes(p, s.z, (split_tile(nco) + 7) & ~7);
             g->sp_max_tiles = std::max(g->sp_max_tiles, tiles);
             tab_of[i] = (int)tabs.size();
             s.level = l;
             tabs.push_back(s);
         }
     }
-    // source vectors: every cell's and reaction centre's multipole, by segments
+    // source vectors: every cell's and reaction centre's multipole, by segments; a vector's index
+    // is its first block of digits.  Those of a layer's level with fine matrices a second time, in
+    // fine segments, after the others of their level
     std::vector<SplitVec> vecs;
-    std::vector<int> vec_of(t.nbox, -1), vec_of_slot(g->n_slots, -1);
+    int nblk = 0;
+    std::vector<int> vec_of(t.nbox, -1), vec_of_slot(g->n_slots, -1), fine_of(t.nbox, -1), fine_of_slot(g->n_slots, -1);
+    std::vector<char> fine_used((size_t)nl * nlev, 0);
+    for (int i = 0; i < nR; ++i)
+        if (g->rkey_fine[i]) fine_used[(size_t)g->rkey_lay_s[i] * nlev + keys[i].level] = 1;
     g->sp_vec_start.assign(nlev + 2, 0);
+    g->sp_fine_start.assign(nlev, 0);
     for (int l = 0; l < nlev; ++l) {
         g->sp_vec_start[l] = (int)vecs.size();
+        g->sp_fine_start[l] = (int)vecs.size();
         if (l < l0) continue;
         const int p = t.p_level[l];
-        auto add = [&](int64_t off, int lay, int slot) {
-            const int v = (int)vecs.size();
-            for (int s = 0; s < split_nseg(p); ++s) vecs.push_back(SplitVec{off, p, s, dexp_off[lay * nlev + l], slot});
-            return v;
-        };
-        for (int b = t.level_start[l]; b < t.level_start[l + 1]; ++b) {
-            vec_of[b] = add(g->box_coef_off_host[b], t.box_layer[b], 0);
-            for (int side = 0; side < 2; ++side) {
-                const int q = g->slot_of_host[2 * b + side];
-                if (q >= 0) vec_of_slot[q] = add(g->slot_coef_host[q], t.box_layer[b], 1);
+        for (int fine = 0; fine < 2; ++fine) {
+            if (fine) g->sp_fine_start[l] = (int)vecs.size();
+            auto add = [&](int64_t off, int lay, int slot) {
+                const int v = nblk, z = split_size(p, fine != 0);
+                for (int s = 0; s < split_nseg(p, z); ++s, nblk += split_blocks(z))
+                    vecs.push_back(SplitVec{off, p, z, s, dexp_off[lay * nlev + l], slot, nblk});
+                return v;
+            };
+            for (int b = t.level_start[l]; b < t.level_start[l + 1]; ++b) {
+                if (fine && !fine_used[(size_t)t.box_layer[b] * nlev + l]) continue;
+                (fine ? fine_of : vec_of)[b] = add(g->box_coef_off_host[b], t.box_layer[b], 0);
+                for (int side = 0; side < 2; ++side) {
+                    const int q = g->slot_of_host[2 * b + side];
+                    if (q >= 0) (fine ? fine_of_slot : vec_of_slot)[q] = add(g->slot_coef_host[q], t.box_layer[b], 1);
+                }
             }
         }
     }
@@ -375,7 +392,8 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
                 const int side = (C.b == 0) ? 1 : 0;
                 const int d = (g->slot_of_host[2 * T + side] >= 0) ? 1 + side : 0;
                 const int rout = (C.b ? 0 : 1) ^ vr_flip[e];
-                add(nF + vr_key[e], ssl >= 0 ? vec_of_slot[ssl] : vec_of[S],
+                const bool fine = g->rkey_fine[vr_key[e]] != 0;
+                add(nF + vr_key[e], ssl >= 0 ? (fine ? fine_of_slot : vec_of_slot)[ssl] : (fine ? fine_of : vec_of)[S],
                     react_flags(e), (rout ? SP_REV : 0) | ((C.b ? 0 : 2) << SP_Q_SHIFT), d);
             }
             for (int d = 0; d < 3; ++d) {
@@ -424,11 +442,12 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
                 s.base = g->qvec_host[2 * ((size_t)lay * nlev + l) + down] + 2 * pS;   // element (r, c) at r - c + 2 pS
                 s.sr = 1; s.sc = -1; s.react = 2; s.pT = pT; s.pS = pS;
                 s.dexp = down ? g->sp_ndexp + dexp_off[lay * nlev + l - 1] : dexp_off[lay * nlev + l];
-                s.rexp = nrexp; nrexp += nT * split_nseg(pS);
+                s.z = split_size(pS, false);
+                s.rexp = nrexp; nrexp += nT * split_nseg(pS, s.z);
                 s.pair0 = (int)pairs.size(); s.npairs = nlay[lay];
                 s.out0 = lrows; lrows += (int64_t)nlay[lay] * 2 * nT;
                 const int tiles = (nT + split_tile(nT) - 1) / split_tile(nT);
-                s.dig = dig; dig += tiles * split_tile_bytes(pS, (split_tile(nT) + 7) & ~7);
+                s.dig = dig; dig += tiles * split_tile_bytes(pS, s.z, (split_tile(nT) + 7) & ~7);
                 g->sp_max_tiles = std::max(g->sp_max_tiles, tiles);
                 s.level = (down ? 2 : 1) * nlev + l;
                 lay_tab[lay] = (int)tabs.size();
@@ -469,7 +488,7 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     g->d_xdst_vec = dupload(g, xv);
     g->d_sp_tab = dupload(g, tabs);
     g->d_sp_vec = dupload(g, vecs);
-    g->sp_nvec = (int)vecs.size();
+    g->sp_nvec = nblk;
     g->d_sp_pair = dupload(g, pairs);
     g->d_sp_row = dupload(g, rlist);
     g->d_sp_dst = dupload(g, dst);
@@ -652,6 +671,8 @@ void fmm_build(lfmm_geometry_s* g) {
                     rk.off = tot;
                     g->rkey_lay_s.push_back(t.box_layer[S]);
                     g->rkey_lay_t.push_back(t.box_layer[T]);
+                    g->rkey_fine.push_back(rk.pS >= 24 && split_growth(g->m.k[C.ls], g->m.k[C.lt], g->m.kmax, table_detour_end(g->m),
+                                                                       w, rk.hS, rk.hT, C.Hc) > SP_GROWTH);
                     tot += (int64_t)(2 * rk.pT + 1) * (2 * rk.pS + 1);
                     keys.push_back(rk);
                 } else {
@@ -1200,7 +1221,7 @@ static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
                 launch_pass(g, columns(make_pass(g, l, 0, 0, nc)), nc, s, "k_translate (M2M)");
                 continue;
             }
-            if (!ready[l]) { launch_split_vec(g, a, g->sp_vec_start[l], g->sp_vec_start[l + 1], s); ready[l] = 1; }
+            if (!ready[l]) { launch_split_vec(g, a, g->sp_vec_start[l], g->sp_fine_start[l], s); ready[l] = 1; }
             launch_split_units(g, a, nlev + l, nlev + l + 1, s);
             finish(l, 0);
             ready[l - 1] = 1;
@@ -1208,7 +1229,10 @@ static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
         prof_end(g, ST_M2M, s);
         prof_begin(g, ST_M2L, s);
         for (int l = l0; l <= D; ++l) {   // the levels without digits, whole runs at a time
-            if (ready[l]) continue;
+            if (ready[l]) {               // (the others' fine ones)
+                launch_split_vec(g, a, g->sp_fine_start[l], g->sp_vec_start[l + 1], s);
+                continue;
+            }
             int e = l;
             while (e + 1 <= D && !ready[e + 1]) ++e;
             launch_split_vec(g, a, g->sp_vec_start[l], g->sp_vec_start[e + 1], s);
@@ -1224,7 +1248,7 @@ static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
                 continue;
             }
             if (l == l0 + 1 || !g->sp_dn[l - 1])
-                launch_split_vec(g, local_args(g, a), g->sp_vec_start[l - 1], g->sp_vec_start[l], s);
+                launch_split_vec(g, local_args(g, a), g->sp_vec_start[l - 1], g->sp_fine_start[l - 1], s);
             launch_split_units(g, a, 2 * nlev + l, 2 * nlev + l + 1, s);
             finish(l, 1);
         }
@@ -1547,7 +1571,7 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
                  lfmm_geometry_s* g = op->g;
                  std::vector<char>& r = ready_of(op);
                  if (!r[l])
-                     vj.push_back(SplitJob{split_args(g, 0, op->nrhs), g->sp_vec_start[l], g->sp_vec_start[l + 1] - g->sp_vec_start[l]});
+                     vj.push_back(SplitJob{split_args(g, 0, op->nrhs), g->sp_vec_start[l], g->sp_fine_start[l] - g->sp_vec_start[l]});
                  r[l] = r[l - 1] = 1;
              });
     {   // M2L of every level: the digits still missing, products, each destination's sum
@@ -1557,9 +1581,10 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
             lfmm_geometry_s* g = op->g;
             const int D = g->tree.D;
             std::vector<char>& r = ready_of(op);
-            for (int l = g->tree.l0; l <= D; ++l)
-                if (!r[l])
-                    vj.push_back(SplitJob{split_args(g, 0, op->nrhs), g->sp_vec_start[l], g->sp_vec_start[l + 1] - g->sp_vec_start[l]});
+            for (int l = g->tree.l0; l <= D; ++l) {
+                const int v0 = r[l] ? g->sp_fine_start[l] : g->sp_vec_start[l], nv = g->sp_vec_start[l + 1] - v0;
+                if (nv > 0) vj.push_back(SplitJob{split_args(g, 0, op->nrhs), v0, nv});
+            }
             const int nd = g->sp_dst_start[D + 1], nbig = split_big(g, nd);
             jobs.push_back(SplitJob{split_args(g, 0, op->nrhs), nbig, nd});
             rblocks.push_back(split_red_ctas(nbig, nd - nbig) * op->nrhs);
@@ -1575,7 +1600,7 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
                  lfmm_geometry_s* g = op->g;
                  if (l == g->tree.l0 + 1 || !g->sp_dn[l - 1])
                      vj.push_back(SplitJob{local_args(g, split_args(g, 0, op->nrhs)), g->sp_vec_start[l - 1],
-                                           g->sp_vec_start[l] - g->sp_vec_start[l - 1]});
+                                           g->sp_fine_start[l - 1] - g->sp_vec_start[l - 1]});
              });
     // L2P after the near field, which adds into the same y
     if (before_l2p) cuda_check(cudaStreamWaitEvent(s, before_l2p, 0), "wait for the near field");

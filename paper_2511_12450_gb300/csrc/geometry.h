@@ -147,6 +147,7 @@ struct SplitTab {
     int pT, pS;        // orders of the result and of the source
     int rexp, dexp;    // offsets of its row exponents and of its source scales (by |n|)
     int pair0, npairs;
+    int z;             // values of |n| per segment of the source
     int react;         // 0: free-space Toeplitz vectors, 1: reaction tables, 2: translation vectors
     int level;         // M2L: level l; M2M from level l: nlev + l; L2L into it: 2 nlev + l
 };
@@ -156,12 +157,13 @@ struct SplitTab {
 // directions and mirror images of a reaction pair) are exact in these forms.
 enum { SP_REV = 1, SP_Q_SHIFT = 2 };
 struct SplitPair {
-    int vec;           // source vector (index of its first segment)
+    int vec;           // source vector (its first block)
     int flags;
 };
 struct SplitVec {      // one segment of a source vector
     int64_t src;       // coefficient offset (M, or Mp with slot)
-    int p, seg, dexp, slot;
+    int p, z, seg, dexp, slot;   // z: values of |n| per segment
+    int blk;           // its digits' place (blocks of SP_BLK positions)
 };
 struct SplitRow {
     int64_t row;       // the pair's workspace row (doubles, one column)
@@ -169,7 +171,7 @@ struct SplitRow {
 };
 struct SplitUnit {     // up to SP_COLS (pair, right-hand side) columns of one matrix, one row tile
     int64_t dig, out0;          // the tile's digits; workspace row of the first column
-    int pT, pS, rexp;           // as the matrix's
+    int pT, pS, z, rexp;        // as the matrix's
     int pair0, col0, cnt, tile; // the matrix's first pair; column c is pair c / ncols
 };
 // the units for blocks of ncols right-hand sides, coarse levels first
@@ -360,9 +362,10 @@ struct lfmm_geometry_s {
     lfmm::SplitPlan sp_plan[2];                     // one column; the block width used last
     int sp_cap = 0;                                 // most columns of a unit (LFMM_AUTOTUNE)
     std::vector<int> sp_dst_start, sp_vec_start;    // [nlev + 2]: first destination / vector of each level
+    std::vector<int> sp_fine_start;                 // [nlev]: first of its vectors in fine segments
     uint32_t* d_sp_vdig = nullptr;                  // digits and exponents of the vectors, sp_ws_cols columns
     int* d_sp_vexp = nullptr;
-    int sp_nvec = 0;
+    int sp_nvec = 0;                                // blocks of one column
     int sp_ntab = 0;
     int64_t sp_rows = 0;                            // workspace doubles per column
     double* d_sp_ws = nullptr;
@@ -378,6 +381,7 @@ struct lfmm_geometry_s {
     // host copies kept for the precision form's tables
     std::vector<lfmm::ReactKey> rkeys_host;
     std::vector<int> rkey_lay_s, rkey_lay_t;       // layers of the source / target boxes of each key
+    std::vector<char> rkey_fine;                   // its split product takes fine segments (split_layout.h)
     std::vector<int> ftab_lay, ftab_lev;           // layer and level of each free-space M2L table
     std::vector<int> ftab_p;                       // order and offset of each
     std::vector<int64_t> ftab_off_host;

@@ -12,12 +12,8 @@
 //    multipoles of a cell have about one size (unscaled they span |J_20| ~ 1e-38 to 1);
 //  - every row of A and every source vector is divided by a power of two above its
 //    largest entry and cut to 62 bits after the point: an integer I, |I| <= 2^62.  Orders
-//    from 24 on (the wide-band levels) do this per segment of 12 values of |n|: there the
-//    reaction tables of a layer with k below k_max grow along a row by up to e^16
-//    (evanescent waves) while the multipoles of a cell whose points lie near its centre
-//    fall, and fewer bits are left where both meet.  Against the oracle on a sparse
-//    four-layer case (orders 28 to 64): one segment 1.7e-9, segments of 24 1.4e-10, of 12
-//    2.1e-11 and 3.2e-11, FP64 FMAs 2e-11 and 3e-11;
+//    from 24 on (the wide-band levels) do this per segment of 12 values of |n|, or of 4 where
+//    the matrix grows along its rows (split_layout.h);
 //  - I = sum_j D_j 256^(7-j), eight signed digits |D_j| <= 128 (|D_0| <= 64), exact in FP16;
 //  - y = sum over digit pairs (i, j) of 256^(14-i-j) A_i v_j.  Pairs with i + j <= 7 are
 //    taken (36 of 64).  Pairs of equal i + j share one FP32 accumulator in TMEM: at most
@@ -26,10 +22,12 @@
 //  - the eight accumulators combine to a 64-bit integer and, with the row's and vector's
 //    exponents, to one FP64 value per segment; segments are added in FP64 in order.
 //
-// Errors against the exact product of the stored FP64 values, relative to (largest entry
-// of the scaled row) x (largest entry of the scaled vector): 2^-62 per term for each
-// operand's cut and about 2^-58 in all for the digit pairs left out; an FP64 FMA chain has
-// 2^-53 of the running sum per term.  (Seven digits, 54 bits, cost 6% less and made the
+// The sums of digits are exact, the product is not: against that of the stored FP64 values it
+// is off by 2^-62 per term for each operand's cut and about 2^-58 in all for the digit pairs
+// left out, relative to (largest entry of the scaled row segment) x (largest entry of the scaled
+// vector segment), so entries far below their segment's largest keep fewer than FP64's 53
+// bits.  An FP64 FMA chain has 2^-53 of the running sum per term.  The segments of
+// split_layout.h keep the first below the second.  (Seven digits, 54 bits, cost 6% less and made the
 // worst of 64 sampled rows of a million-point four-layer product 6.0e-7 where FP64 FMAs
 // gave 9.9e-8.)  The sums of digits are exact, so a product does not depend on how pairs
 // are grouped into CTAs, on the columns beside it or on the launch it is part of.
@@ -58,15 +56,11 @@
 
 #include "devmath.cuh"
 #include "geometry.h"
+#include "split_layout.h"
 
 namespace lfmm {
 
-#define SP_ORD 24                   // orders below this are one segment
-#define SP_SEG 12                   // values of |n| per segment of a larger order
-#define SP_POS 48                   // most positions of a segment
-#define SP_MAXSEG 7                 // segments: (LFMM_PMAX + 1) / SP_SEG
 #define SP_COLS 32                  // columns per unit
-#define SP_ND 8                     // digits
 #define SP_PLANE 9216u              // most bytes of one digit of A: 96 rows x 48, 128 x 32
 #define SP_NONE (-100000)           // column exponents: all zero, not finite
 #define SP_INF (1 << 20)
@@ -162,26 +156,6 @@ __device__ __forceinline__ double sp_value(long long hi, long long lo, int x) {
     return __longlong_as_double((long long)(b | ((uint64_t)T & 0x8000000000000000ull)));
 }
 
-// complex rows per tile of a matrix with nT rows, in units of 8 rows, and the positions
-// per staged chunk
-__host__ __device__ inline int split_tile(int nT) { const int k = (nT + 63) >> 6; return (nT + k - 1) / k; }
-__host__ __device__ inline int split_chunk(int nT) { return split_tile(nT) <= 48 ? 24 : 16; }
-// segments of an order-p source, the values of |n| in one, and its half length in positions
-// (a multiple of 4, so that n -> -n is a reversal of whole groups of 4 positions)
-__host__ __device__ inline int split_size(int p) { return p < SP_ORD ? SP_ORD : SP_SEG; }
-__host__ __device__ inline int split_nseg(int p) { return p / split_size(p) + 1; }
-__host__ __device__ inline int split_vals(int p, int seg) {
-    const int z = split_size(p), h = p + 1 - z * seg;
-    return h < z ? h : z;
-}
-__host__ __device__ inline int split_half(int p, int seg) { return (split_vals(p, seg) + 3) & ~3; }
-// positions of all segments, and the digits of one row tile of nr8 rows of each part
-__host__ __device__ inline int split_positions(int p) {
-    int n = 0;
-    for (int seg = 0; seg < split_nseg(p); ++seg) n += 2 * split_half(p, seg);
-    return n;
-}
-__host__ __device__ inline int64_t split_tile_bytes(int p, int nr8) { return (int64_t)split_positions(p) * nr8 * (8 * SP_ND); }
 // |n| less the segment's first at position k of a segment of half length H; n < 0 in the first half
 __device__ __forceinline__ int split_abs(int k, int H) { return k < H ? H - 1 - k : k - H; }
 
@@ -192,12 +166,12 @@ __global__ void __launch_bounds__(128) k_split_rexp(const SplitTab* __restrict__
                                                     const int* __restrict__ dexp, int* __restrict__ rexp) {
     const SplitTab t = tabs[blockIdx.x];
     const cd* a = (t.react == 2 ? tx : t.react ? tr : tf) + t.base + (int64_t)t.pS * t.sc;
-    const int nT = 2 * t.pT + 1, nseg = split_nseg(t.pS);
+    const int nT = 2 * t.pT + 1, nseg = split_nseg(t.pS, t.z);
     for (int i = threadIdx.x; i < nT * nseg; i += blockDim.x) {
         const int seg = i / nT, r = i - seg * nT;
         int e = -4000;
-        for (int j = 0; j < 2 * split_vals(t.pS, seg); ++j) {
-            const int m = split_size(t.pS) * seg + (j >> 1);
+        for (int j = 0; j < 2 * split_vals(t.pS, t.z, seg); ++j) {
+            const int m = t.z * seg + (j >> 1);
             const cd z = a[(int64_t)r * t.sr + (int64_t)((j & 1) ? -m : m) * t.sc];
             const int eb = max(sp_expo(z.x), sp_expo(z.y));
             if (eb > 0) e = max(e, eb - 1022 - dexp[t.dexp + m]);
@@ -233,9 +207,9 @@ __global__ void __launch_bounds__(256) k_split_digits(const SplitTab* __restrict
     if (n0 >= nT) return;
     const int nt = min(per, nT - n0), nr8 = (per + 7) & ~7, KC = split_chunk(nT);
     const cd* A = (t.react == 2 ? tx : t.react ? tr : tf) + t.base + (int64_t)n0 * t.sr + (int64_t)t.pS * t.sc;   // column n = 0
-    unsigned char* out = dig + t.dig + (int64_t)blockIdx.y * split_tile_bytes(t.pS, nr8);
-    for (int seg = 0; seg < split_nseg(t.pS); ++seg) {
-        const int H = split_half(t.pS, seg), h = split_vals(t.pS, seg), n1 = split_size(t.pS) * seg;
+    unsigned char* out = dig + t.dig + (int64_t)blockIdx.y * split_tile_bytes(t.pS, t.z, nr8);
+    for (int seg = 0; seg < split_nseg(t.pS, t.z); ++seg) {
+        const int H = split_half(t.pS, t.z, seg), h = split_vals(t.pS, t.z, seg), n1 = t.z * seg;
         for (int k0 = 0; k0 < 2 * H; k0 += KC) {
             const int ng = min(2 * H - k0, KC) >> 2;
             const uint32_t sbo = (uint32_t)ng * 128u, plane = (uint32_t)(nr8 >> 2) * sbo;
@@ -271,45 +245,47 @@ __global__ void __launch_bounds__(256) k_split_digits(const SplitTab* __restrict
     }
 }
 
-// The source vectors as digits: per (vector, segment) eight planes of SP_POS words (a word is
-// the FP16 pair (re, im) of one coefficient's digit) and the exponent.  One warp per (vector,
-// segment); a vector serves all its pairs (about 7 at one column).
-// One warp writes one segment's digits and exponent: m the vector at n = 0, o its index.
-__device__ __forceinline__ void split_vec_seg(const SplitArgs& S, const cd* m, int p, int seg, int dexp, int64_t o, int lane) {
-    const int H = split_half(p, seg), h = split_vals(p, seg);
-    cd z[2];
+// The source vectors as digits: per (vector, segment) eight planes of words (a word is the FP16
+// pair (re, im) of one coefficient's digit), split_blocks positions' blocks of eight each, and the
+// exponent.  One warp per (vector, segment); a vector serves all its pairs (about 7 at one column).
+// One warp writes one segment's digits and exponent: m the vector at n = 0, o its first block.
+__device__ __forceinline__ void split_vec_seg(const SplitArgs& S, const cd* m, int p, int z, int seg, int dexp, int64_t o,
+                                              int lane) {
+    const int H = split_half(p, z, seg), h = split_vals(p, z, seg);
+    cd c[2];
     int d[2], e = SP_NONE;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        const int k = lane + 32 * i, j = split_abs(k, H), n = split_size(p) * seg + j;
-        z[i] = mk(0, 0);
+        const int k = lane + 32 * i, j = split_abs(k, H), n = z * seg + j;
+        c[i] = mk(0, 0);
         d[i] = 0;
         if (k < 2 * H && j < h) {
-            z[i] = m[k < H ? -n : n];
+            c[i] = m[k < H ? -n : n];
             d[i] = S.dexp[dexp + n];
-            const int eb = max(sp_expo(z[i].x), sp_expo(z[i].y));
+            const int eb = max(sp_expo(c[i].x), sp_expo(c[i].y));
             if (eb == 2047) e = SP_INF;
             else if (eb > 0) e = max(e, eb - 1022 + d[i]);
         }
     }
     e = __reduce_max_sync(0xffffffffu, e);
     if (lane == 0) S.vexp[o] = e;
-    uint32_t* out = S.vdig + o * (SP_ND * SP_POS);
+    uint32_t* out = S.vdig + o * (SP_ND * SP_BLK);
+    const int pos = split_blocks(z) * SP_BLK;
     const bool live = e > SP_NONE && e < SP_INF;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const int k = lane + 32 * i;
-        if (k >= SP_POS) break;
+        if (k >= pos) break;
         const uint2 zero = make_uint2(0x80808080u, 0x80808080u);
-        const uint2 a = live ? sp_digits(z[i].x, 1022 + e - d[i]) : zero, b = live ? sp_digits(z[i].y, 1022 + e - d[i]) : zero;
+        const uint2 a = live ? sp_digits(c[i].x, 1022 + e - d[i]) : zero, b = live ? sp_digits(c[i].y, 1022 + e - d[i]) : zero;
         out[k] = sp_digit<0>(a, b);
-        out[SP_POS + k] = sp_digit<1>(a, b);
-        out[2 * SP_POS + k] = sp_digit<2>(a, b);
-        out[3 * SP_POS + k] = sp_digit<3>(a, b);
-        out[4 * SP_POS + k] = sp_digit<4>(a, b);
-        out[5 * SP_POS + k] = sp_digit<5>(a, b);
-        out[6 * SP_POS + k] = sp_digit<6>(a, b);
-        out[7 * SP_POS + k] = sp_digit<7>(a, b);
+        out[pos + k] = sp_digit<1>(a, b);
+        out[2 * pos + k] = sp_digit<2>(a, b);
+        out[3 * pos + k] = sp_digit<3>(a, b);
+        out[4 * pos + k] = sp_digit<4>(a, b);
+        out[5 * pos + k] = sp_digit<5>(a, b);
+        out[6 * pos + k] = sp_digit<6>(a, b);
+        out[7 * pos + k] = sp_digit<7>(a, b);
     }
 }
 __device__ __forceinline__ void split_vec(const SplitArgs& S, int block, int column, int v0, int nv) {
@@ -319,7 +295,7 @@ __device__ __forceinline__ void split_vec(const SplitArgs& S, int block, int col
     const SplitVec V = S.vec[v0 + w];
     const int col = S.col0 + column;
     const cd* m = (V.slot ? S.Mp + (int64_t)col * S.nslotcoef : S.M + (int64_t)col * S.ncoef) + V.src + V.p;
-    split_vec_seg(S, m, V.p, V.seg, V.dexp, (int64_t)column * S.nvec + v0 + w, lane);
+    split_vec_seg(S, m, V.p, V.z, V.seg, V.dexp, (int64_t)column * S.nvec + V.blk, lane);
 }
 __global__ void __launch_bounds__(128) k_split_vec(const SplitArgs S, int v0, int nv) {
     split_vec(S, blockIdx.x, blockIdx.y, v0, nv);
@@ -351,7 +327,7 @@ struct SplitSlot {   // a unit's descriptor; u.cnt = 0: no more
     SplitUnit u;
     const SplitArgs* args;
     int flag[SP_COLS];
-    int64_t vec[SP_COLS];   // the columns' vectors (index of their first segment)
+    int64_t vec[SP_COLS];   // the columns' vectors (their first block)
 };
 struct SplitShared {
     SplitSlot ring[SP_RING];
@@ -410,11 +386,13 @@ __device__ __forceinline__ void sp_chunk(uint32_t d, uint64_t da, uint64_t db, u
 
 // geometry of a unit
 struct SplitGeo {
-    int nT, pS, nseg, n0, nt, nr8, KC, lc, C;
+    int nT, pS, z, nseg, blk, n0, nt, nr8, KC, lc, C;
     __device__ __forceinline__ explicit SplitGeo(const SplitUnit& U) {
         nT = 2 * U.pT + 1;
         pS = U.pS;
-        nseg = split_nseg(pS);
+        z = U.z;
+        nseg = split_nseg(pS, z);
+        blk = split_blocks(z);
         const int per = split_tile(nT);
         n0 = U.tile * per;
         nt = min(per, nT - n0);
@@ -437,13 +415,13 @@ __device__ __forceinline__ uint4 sp_turned(uint4 w, const uint32_t (&sel)[4], co
 // B: the digits of 4 positions at k (group g of the chunk, 8-row groups sbo apart) of column bc
 // (the words are loaded beforehand by split_load_b)
 __device__ __forceinline__ void split_load_b(uint4 (&w)[SP_ND], const SplitArgs& S, const SplitSlot& sl, int bc, int k, int seg,
-                                             int H) {
+                                             int H, int blocks) {
     if (bc >= sl.u.cnt) return;
     const int P = k >> 2;
-    const uint4* src = (const uint4*)(S.vdig + (sl.vec[bc] + seg) * (SP_ND * SP_POS)) +
+    const uint4* src = (const uint4*)(S.vdig + (sl.vec[bc] + seg * blocks) * (SP_ND * SP_BLK)) +
                        ((sl.flag[bc] & SP_REV) ? (H >> 1) - 1 - P : P);
 #pragma unroll
-    for (int j = 0; j < SP_ND; ++j) w[j] = src[j * (SP_POS / 4)];
+    for (int j = 0; j < SP_ND; ++j) w[j] = src[j * blocks * (SP_BLK / 4)];
 }
 __device__ __forceinline__ void split_stage_b(const uint4 (&w)[SP_ND], const SplitSlot& sl, int C, uint32_t sbo, unsigned char* sB,
                                               int bc, int g, int k, int seg, int H, int n1) {
@@ -552,13 +530,13 @@ __device__ __forceinline__ void split_units(const JOBS& jobs) {
             const SplitArgs& S = *sl.args;
             const SplitGeo G(sl.u);
             for (int seg = 0; seg < G.nseg && ok; ++seg) {
-                const int H = split_half(G.pS, seg), n1 = split_size(G.pS) * seg;
+                const int H = split_half(G.pS, G.z, seg), n1 = G.z * seg;
                 for (int k0 = 0; k0 < 2 * H; k0 += G.KC, ++chunk) {
                     if ((chunk & 1) != grp) continue;
                     const int ng = min(2 * H - k0, G.KC) >> 2;   // groups of 4 positions (an even number)
                     const int nq = ng << G.lc, bc = t & (G.C - 1);
                     uint4 w[SP_ND];
-                    if (t < nq) split_load_b(w, S, sl, bc, k0 + 4 * (t >> G.lc), seg, H);
+                    if (t < nq) split_load_b(w, S, sl, bc, k0 + 4 * (t >> G.lc), seg, H, G.blk);
                     if (chunk >= 2) {   // the MMAs that read this buffer
                         ok = sp_wait_warp(sh, &sh.empty[grp], ((chunk >> 1) - 1) & 1);
                         if (!ok) break;
@@ -566,7 +544,7 @@ __device__ __forceinline__ void split_units(const JOBS& jobs) {
 #pragma unroll 1
                     for (int q = t; q < nq; q += 128) {
                         const int g = q >> G.lc;
-                        if (q != t) split_load_b(w, S, sl, bc, k0 + 4 * g, seg, H);
+                        if (q != t) split_load_b(w, S, sl, bc, k0 + 4 * g, seg, H, G.blk);
                         split_stage_b(w, sl, G.C, (uint32_t)ng * 128u, sB, bc, g, k0 + 4 * g, seg, H, n1);
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -594,7 +572,7 @@ __device__ __forceinline__ void split_units(const JOBS& jobs) {
             const int64_t vec = sl.vec[min(lane, cnt - 1)];
             double* out = S.ws + sl.u.out0 + part * G.nT + G.n0 + r0;   // this row's result, column 0
             for (int seg = 0; seg < G.nseg; ++seg, ++sgc) {
-                const int xv = S.vexp[vec + seg];   // lane's column
+                const int xv = S.vexp[vec + seg * G.blk];   // lane's column
                 const int xe = S.rexp[sl.u.rexp + seg * G.nT + G.n0 + r0] - 68;
                 ok = sp_wait_warp(sh, &sh.accfull[sgc & 1], (sgc >> 1) & 1);
                 if (!ok) break;
@@ -653,7 +631,7 @@ __device__ __forceinline__ void split_units(const JOBS& jobs) {
             if (!ok || sh.ring[k & (SP_RING - 1)].u.cnt == 0) break;
             const SplitGeo G(sh.ring[k & (SP_RING - 1)].u);
             for (int seg = 0; seg < G.nseg && ok; ++seg, ++sgc) {
-                const int len = 2 * split_half(G.pS, seg);
+                const int len = 2 * split_half(G.pS, G.z, seg);
                 const uint32_t acc = tb + (uint32_t)(sgc & 1) * (SP_ND * SP_COLS);
                 if (sgc >= 2) {
                     ok = sp_wait_warp(sh, &sh.accempty[sgc & 1], ((sgc >> 1) - 1) & 1);
@@ -701,7 +679,7 @@ __device__ __forceinline__ void split_units(const JOBS& jobs) {
             const SplitGeo G(sh.ring[k & (SP_RING - 1)].u);
             const unsigned char* src = sh.ring[k & (SP_RING - 1)].args->dig + sh.ring[k & (SP_RING - 1)].u.dig;
             for (int seg = 0; seg < G.nseg && ok; ++seg) {
-                const int len = 2 * split_half(G.pS, seg);
+                const int len = 2 * split_half(G.pS, G.z, seg);
                 for (int k0 = 0; k0 < len; k0 += G.KC, ++chunk) {
                     const int b = chunk & 1;
                     const uint32_t bytes = (uint32_t)min(len - k0, G.KC) * (uint32_t)G.nr8 * (8 * SP_ND);
@@ -898,6 +876,11 @@ struct FinArgs {
 #define SP_XSTAGE 4            // sources of an XDst staged together
 inline size_t fin_smem(int pS, int pD) { return sizeof(cd) * SP_XSTAGE * (size_t)(2 * pS + 1 + 2 * (pS + pD) + 1); }
 __host__ __device__ inline int fin_ctas(const FinArgs& F) { return F.nd + split_red_ctas(F.big ? F.ncell : 0, F.big ? 0 : F.ncell); }
+// one segment of a cell's digits, o the first block of them all
+__device__ __forceinline__ void fin_digits(const SplitArgs& S, const cd* m, int p, int seg, int dexp, int64_t o, int lane) {
+    const int z = split_size(p, false);
+    split_vec_seg(S, m, p, z, seg, dexp, o + seg * split_blocks(z), lane);
+}
 __device__ __forceinline__ void split_fin(const FinArgs& F, int b, int column) {
     extern __shared__ __align__(16) cd fin_sm[];   // XDst: sources, then their translation vectors
     __shared__ cd red[192], z[SP_RED_WARPS * 64 > 2 * LFMM_PMAX + 1 ? SP_RED_WARPS * 64 : 2 * LFMM_PMAX + 1];
@@ -923,8 +906,8 @@ __device__ __forceinline__ void split_fin(const FinArgs& F, int b, int column) {
         }
         if (!F.digits) return;
         __syncwarp();
-        for (int seg = 0; seg < split_nseg(f.p); ++seg)
-            split_vec_seg(S, z + w * 64 + f.p, f.p, seg, f.dexp, (int64_t)column * S.nvec + f.vec + seg, lane);
+        for (int seg = 0; seg < split_nseg(f.p, split_size(f.p, false)); ++seg)
+            fin_digits(S, z + w * 64 + f.p, f.p, seg, f.dexp, (int64_t)column * S.nvec + f.vec, lane);
         return;
     }
     cd* out;
@@ -973,8 +956,8 @@ __device__ __forceinline__ void split_fin(const FinArgs& F, int b, int column) {
     }
     if (!F.digits) return;
     __syncthreads();
-    for (int seg = tid >> 5; seg < split_nseg(p); seg += 6)
-        split_vec_seg(S, z + p, p, seg, dexp, (int64_t)column * S.nvec + vec + seg, lane);
+    for (int seg = tid >> 5; seg < split_nseg(p, split_size(p, false)); seg += 6)
+        fin_digits(S, z + p, p, seg, dexp, (int64_t)column * S.nvec + vec, lane);
 }
 __global__ void __launch_bounds__(192) k_split_fin(const FinArgs F) { split_fin(F, blockIdx.x, blockIdx.y); }
 
