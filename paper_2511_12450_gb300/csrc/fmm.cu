@@ -215,7 +215,8 @@ static void split_alloc(lfmm_geometry_s* g, int cols) {   // products, then digi
 }
 // Units: a matrix's (pair, column) columns in groups of up to sp_cap, of nearly equal size, by
 // row tiles of up to 64 complex rows.
-static void make_split_plan(lfmm_geometry_s* g, SplitPlan& P, int ncols) {
+static SplitPlan make_split_plan(lfmm_geometry_s* g, int ncols) {
+    SplitPlan P;
     std::vector<SplitUnit> units;
     const int nst = 3 * (g->tree.D + 1), cap = g->sp_cap;
     P.start.assign(nst + 1, -1);
@@ -236,19 +237,18 @@ static void make_split_plan(lfmm_geometry_s* g, SplitPlan& P, int ncols) {
         if (P.start[l] < 0) P.start[l] = next;
         next = P.start[l];
     }
-    if (P.d_unit) {   // units being replaced; work queued on any stream may still read them
-        g->allocs.erase(std::find(g->allocs.begin(), g->allocs.end(), (void*)P.d_unit));
-        dev_release_now(P.d_unit);
-        P.d_unit = nullptr;
-    }
     P.d_unit = dupload(g, units);
     cuda_check(cudaStreamSynchronize(cudaStreamPerThread), "split M2L units");
-    P.ncols = ncols;
-}
-static const SplitPlan& split_plan(lfmm_geometry_s* g, int ncols) {
-    SplitPlan& P = g->sp_plan[ncols == 1 ? 0 : 1];
-    if (P.ncols != ncols) make_split_plan(g, P, ncols);
     return P;
+}
+// The plan of a block width, made on its first use and kept while the geometry lives: callers
+// alternate widths, a block wider than its workspace runs in rounds of two widths, and a captured
+// product holds its plan's units.  56 bytes per unit of up to 32 columns, where the workspace of
+// that width holds 2 (2p + 1) doubles per column: less than half a per cent of it.
+static const SplitPlan& split_plan(lfmm_geometry_s* g, int ncols) {
+    auto it = g->sp_plan.find(ncols);
+    if (it == g->sp_plan.end()) it = g->sp_plan.emplace(ncols, make_split_plan(g, ncols)).first;
+    return it->second;
 }
 static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, const std::vector<int>& vr_src,
                         const std::vector<int>& vr_key, const std::vector<int>& vr_comp,
@@ -500,7 +500,7 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     g->d_sp_dig = dalloc<unsigned char>(g, (size_t)dig);
     g->d_sp_ctr = dalloc<int>(g, 1);
     g->sp_cap = SP_COLS;
-    make_split_plan(g, g->sp_plan[0], 1);
+    split_plan(g, 1);
     g->sp_rows = rows;
     split_alloc(g, 1);
     cuda_check(cudaHostAlloc((void**)&g->wait_err, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable), "wait status");
@@ -1053,14 +1053,17 @@ void fmm_free(lfmm_geometry_s* g) {
 }
 
 // The split M2L's workspace: one row of products per (pair, column), for as many columns
-// at once as fit SP_WS_BYTES (at least one); a wider block takes several rounds.
+// at once as fit SP_WS_BYTES (at least one); a wider block takes several rounds, of widths that
+// differ by one at most (32 columns where 31 fit: 16 + 16, not 31 and a round for one).
 #define SP_WS_BYTES (2ll << 30)
 #define SP_SMS 152   // persistent CTAs of k_split: one per SM
-static int split_round(const lfmm_geometry_s* g, int nrhs) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(nrhs, 2048), SP_WS_BYTES / (int64_t)split_col_bytes(g)));
+static int split_rounds(const lfmm_geometry_s* g, int nrhs) {
+    const int cap = (int)std::max<int64_t>(1, std::min<int64_t>(2048, SP_WS_BYTES / (int64_t)split_col_bytes(g)));
+    return (nrhs + cap - 1) / cap;
 }
+static int round_start(int nrhs, int rounds, int r) { return (int)((int64_t)nrhs * r / rounds); }   // first column
 static void ensure_split(lfmm_geometry_s* g, int nrhs) {
-    const int want = split_round(g, nrhs);
+    const int rounds = split_rounds(g, nrhs), want = (nrhs + rounds - 1) / rounds;
     if (g->sp_ws_cols >= want) return;
     dev_release_now(g->d_sp_ws);
     g->d_sp_ws = nullptr;
@@ -1112,8 +1115,9 @@ static void launch_split_reduce(lfmm_geometry_s* g, const SplitArgs& a, int nd, 
 static void launch_split(lfmm_geometry_s* g, int nrhs, int lm, cudaStream_t s) {
     split_check_waits(g);
     ensure_split(g, nrhs);
-    for (int c0 = 0; c0 < nrhs; c0 += g->sp_ws_cols) {
-        const SplitArgs a = split_args(g, c0, std::min(nrhs - c0, g->sp_ws_cols));
+    for (int r = 0, n = split_rounds(g, nrhs); r < n; ++r) {
+        const int c0 = round_start(nrhs, n, r);
+        const SplitArgs a = split_args(g, c0, round_start(nrhs, n, r + 1) - c0);
         launch_split_vec(g, a, 0, g->sp_vec_start[lm], s);
         launch_split_units(g, a, 0, lm, s);
         launch_split_reduce(g, a, g->sp_dst_start[lm], s);
@@ -1198,8 +1202,8 @@ static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
     const int D = t.D, l0 = t.l0, nlev = D + 1;
     split_check_waits(g);
     ensure_split(g, nrhs);
-    for (int c0 = 0; c0 < nrhs; c0 += g->sp_ws_cols) {
-        const int nc = std::min(nrhs - c0, g->sp_ws_cols);
+    for (int r = 0, n = split_rounds(g, nrhs); r < n; ++r) {
+        const int c0 = round_start(nrhs, n, r), nc = round_start(nrhs, n, r + 1) - c0;
         const SplitArgs a = split_args(g, c0, nc);
         auto columns = [&](XPass P) {
             P.X += (int64_t)c0 * g->ncoef;
@@ -1494,7 +1498,7 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
     // a block too wide for its workspace: its own rounds; the others share every launch
     std::vector<const BatchOp*> sh;
     for (const BatchOp* op : far) {
-        if (op->nrhs > op->g->sp_ws_cols) far_fp64(op->g, op->nrhs, s);
+        if (split_rounds(op->g, op->nrhs) > 1) far_fp64(op->g, op->nrhs, s);
         else sh.push_back(op);
     }
     auto vec_jobs = [&](const std::vector<SplitJob>& jobs) {
@@ -1632,11 +1636,20 @@ void fmm_autotune(lfmm_geometry_s* g) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cuda_check(cudaEventCreate(&e0), "event");
     cuda_check(cudaEventCreate(&e1), "event");
+    auto replan = [&]() {   // the one plan of a geometry being built; its work is done
+        cuda_check(cudaStreamSynchronize(s), "tune sync");
+        for (auto& e : g->sp_plan) {
+            g->allocs.erase(std::find(g->allocs.begin(), g->allocs.end(), (void*)e.second.d_unit));
+            dev_release(e.second.d_unit);
+        }
+        g->sp_plan.clear();
+        split_plan(g, 1);
+    };
     int best_work = M2L_ITEM_WORK;
     double best = 1e300, dflt = 0.0;
     for (int work : {1024, M2L_ITEM_WORK}) {   // 16 and 32 pairs
         g->sp_cap = std::min(SP_COLS, work / 64);
-        make_split_plan(g, g->sp_plan[0], 1);
+        replan();
         for (int r = 0; r < 2; ++r) launch_split(g, 1, t.D + 1, s);
         cuda_check(cudaEventRecord(e0, s), "event");
         for (int r = 0; r < 3; ++r) launch_split(g, 1, t.D + 1, s);
@@ -1651,7 +1664,7 @@ void fmm_autotune(lfmm_geometry_s* g) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     g->sp_cap = std::min(SP_COLS, best_work / 64);
-    make_split_plan(g, g->sp_plan[0], 1);
+    replan();
     make_m2l_items(g, best_work, 1);
     cuda_check(cudaStreamSynchronize(s), "tune");
     g->n_launches = launches;

@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cstring>
 #include <functional>
+#include <map>
 #include <mutex>
 #include <cstdint>
 #include <string>
@@ -176,7 +177,6 @@ struct SplitUnit {     // up to SP_COLS (pair, right-hand side) columns of one m
 };
 // the units for blocks of ncols right-hand sides, coarse levels first
 struct SplitPlan {
-    int ncols = 0;
     SplitUnit* d_unit = nullptr;
     std::vector<int> start;     // [3 nlev + 1]: first unit of each SplitTab::level
 };
@@ -359,7 +359,7 @@ struct lfmm_geometry_s {
     int64_t sp_dig_bytes = 0;
     int* d_sp_ctr = nullptr;
     int sp_max_tiles = 1;
-    lfmm::SplitPlan sp_plan[2];                     // one column; the block width used last
+    std::map<int, lfmm::SplitPlan> sp_plan;         // by block width
     int sp_cap = 0;                                 // most columns of a unit (LFMM_AUTOTUNE)
     std::vector<int> sp_dst_start, sp_vec_start;    // [nlev + 2]: first destination / vector of each level
     std::vector<int> sp_fine_start;                 // [nlev]: first of its vectors in fine segments

@@ -1,0 +1,78 @@
+"""Block right-hand sides: more columns than the products' workspace holds at once (rounds), and widths
+that alternate between calls, also inside captured graphs."""
+
+import numpy as np
+import pytest
+
+from oracle import nystrom as onys
+from workloads import config_c2, layered_small
+
+pytestmark = pytest.mark.gpu
+
+
+def geometry(lf, wl, leaf):
+    pts, w, _, _ = onys.elements(wl.bodies)
+    M = lf.medium_create(wl.medium.interfaces, wl.medium.k, wl.medium.eta)
+    return lf.geometry_build(M, pts, w, p=20, leaf_size=leaf)
+
+
+def columns(n, cols, seed):
+    import torch
+
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.view_as_complex(torch.randn((cols, n, 2), dtype=torch.float64, device="cuda", generator=g))
+
+
+def launches(lf, G):
+    return int(lf.geometry_query(G, "launch_count", np.float64)[0])
+
+
+def test_rounds_equal_single_products(gpu_lib):
+    """45 columns of 65,536 points: 66 MB of workspace each, so 2 GiB takes them in two rounds (23 + 22)."""
+    import torch
+
+    lf = gpu_lib
+    G = geometry(lf, config_c2(), 64)
+    X = columns(G.n, 45, 1)
+    count = []
+    for cols in (5, 45):
+        l0 = launches(lf, G)
+        Y = lf.matvec(G, X[:cols].contiguous())
+        count.append(launches(lf, G) - l0)
+    assert count[1] > count[0], "more than one round must be in use"
+    for c in (0, 1, 21, 22, 23, 44):
+        assert torch.equal(Y[c], lf.matvec(G, X[c].contiguous()))
+    small = geometry(lf, layered_small(n_bodies=3, nodes=150, seed=7), 16)
+    xs = columns(small.n, 2, 2)
+    yb, ys = lf.matvec_batch([G, small], [X, xs])
+    assert torch.equal(yb, Y) and torch.equal(ys, lf.matvec(small, xs))
+
+
+def test_captured_products_outlive_other_widths(gpu_lib):
+    """A warmed-up width can be captured whatever width ran last, and its graph stays valid while
+    narrower products run."""
+    import torch
+
+    lf = gpu_lib
+    G = geometry(lf, layered_small(n_bodies=3, nodes=150, seed=7), 16)
+    X, Y = columns(G.n, 5, 3), columns(G.n, 5, 4)
+    narrow = columns(G.n, 3, 5)
+    ref5, ref3 = lf.matvec(G, X), lf.matvec(G, narrow)
+    new = columns(G.n, 5, 6)
+    ref_new = lf.matvec(G, new)
+    assert torch.equal(lf.matvec(G, narrow), ref3)   # the width used last is not the captured one
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        lf.matvec(G, X, Y)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Y, ref5)
+    for _ in range(3):
+        assert torch.equal(lf.matvec(G, narrow), ref3)
+        assert torch.equal(lf.matvec(G, X[:2].contiguous()), ref5[:2])
+    X.copy_(new)
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Y, ref_new)
