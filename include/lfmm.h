@@ -277,8 +277,12 @@ lfmm_status lfmm_precond_apply(lfmm_geometry g, int32_t nrhs, const void *x, voi
  *     vectors and for geometries whose work buffers do not fit (y is then left
  *     untouched); LFMM_ERR_CUDA for a failed launch.
  *   - Geometries whose work buffers (sorted x and y, multipole and local
- *     coefficients, M2L partial sums) exceed the array are rejected with LFMM_ERR_INVALID_ARG
- *     before any device work (C2-sized problems, N = 65536, need about 16 MiB).
+ *     coefficients, and the room of one partial sum per M2L item) exceed the array are rejected
+ *     with LFMM_ERR_INVALID_ARG before any device work (C2-sized problems, N = 65536, need about
+ *     16 MiB).  The M2L's products go to the geometry's own workspace of one column, made by
+ *     lfmm_geometry_build and kept until the geometry is destroyed.
+ *   - After the first call, a call can be captured into a graph; the graph stays valid while the
+ *     geometry lives, whatever other calls run on it meanwhile.
  *   - The stage profiler is not run by this call; the operator is the FP64 one.
  */
 lfmm_status lfmm_matvec_static(lfmm_geometry g, const void *x, void *y, void *stream);

@@ -205,14 +205,6 @@ static size_t split_col_bytes(const lfmm_geometry_s* g) {   // workspace of one 
     return sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) +
            (size_t)g->sp_nvec * (SP_ND * SP_BLK * sizeof(uint32_t) + sizeof(int)) + 16;
 }
-static void split_alloc(lfmm_geometry_s* g, int cols) {   // products, then digits, then exponents
-    unsigned char* p = (unsigned char*)dev_alloc_ready(split_col_bytes(g) * cols, "split M2L workspace");
-    const size_t rows = sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) * cols;
-    g->d_sp_ws = (double*)p;
-    g->d_sp_vdig = (uint32_t*)(p + ((rows + 15) & ~(size_t)15));
-    g->d_sp_vexp = (int*)(g->d_sp_vdig + (size_t)g->sp_nvec * cols * SP_ND * SP_BLK);
-    g->sp_ws_cols = cols;
-}
 // Units: a matrix's (pair, column) columns in groups of up to sp_cap, of nearly equal size, by
 // row tiles of up to 64 complex rows.
 static SplitPlan make_split_plan(lfmm_geometry_s* g, int ncols) {
@@ -502,7 +494,7 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     g->sp_cap = SP_COLS;
     split_plan(g, 1);
     g->sp_rows = rows;
-    split_alloc(g, 1);
+    g->d_sp_ws1 = dalloc<unsigned char>(g, split_col_bytes(g));
     cuda_check(cudaHostAlloc((void**)&g->wait_err, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable), "wait status");
     *g->wait_err = 0;
 }
@@ -1043,7 +1035,7 @@ static void ensure_coef(lfmm_geometry_s* g, int nrhs) {
 void fmm_free(lfmm_geometry_s* g) {
     dev_release(g->d_sp_ws);
     g->d_sp_ws = nullptr;
-    g->sp_ws_cols = 0;
+    g->sp_ws_bytes = 0;
     if (g->wait_err) cudaFreeHost(g->wait_err);
     g->wait_err = nullptr;
     dev_release(g->d_M); dev_release(g->d_L);
@@ -1054,7 +1046,9 @@ void fmm_free(lfmm_geometry_s* g) {
 
 // The split M2L's workspace: one row of products per (pair, column), for as many columns
 // at once as fit SP_WS_BYTES (at least one); a wider block takes several rounds, of widths that
-// differ by one at most (32 columns where 31 fit: 16 + 16, not 31 and a round for one).
+// differ by one at most (32 columns where 31 fit: 16 + 16, not 31 and a round for one).  One column's
+// is made with the geometry and stays: a call that may not allocate has it, and a captured product
+// keeps what it points to when a block makes the other one grow.
 #define SP_WS_BYTES (2ll << 30)
 #define SP_SMS 152   // persistent CTAs of k_split: one per SM
 static int split_rounds(const lfmm_geometry_s* g, int nrhs) {
@@ -1063,12 +1057,14 @@ static int split_rounds(const lfmm_geometry_s* g, int nrhs) {
 }
 static int round_start(int nrhs, int rounds, int r) { return (int)((int64_t)nrhs * r / rounds); }   // first column
 static void ensure_split(lfmm_geometry_s* g, int nrhs) {
-    const int rounds = split_rounds(g, nrhs), want = (nrhs + rounds - 1) / rounds;
-    if (g->sp_ws_cols >= want) return;
+    const int rounds = split_rounds(g, nrhs), cols = (nrhs + rounds - 1) / rounds;
+    const size_t want = split_col_bytes(g) * cols;
+    if (cols == 1 || g->sp_ws_bytes >= want) return;
     dev_release_now(g->d_sp_ws);
     g->d_sp_ws = nullptr;
-    g->sp_ws_cols = 0;
-    split_alloc(g, want);
+    g->sp_ws_bytes = 0;
+    g->d_sp_ws = (unsigned char*)dev_alloc_ready(want, "split M2L workspace");
+    g->sp_ws_bytes = want;
 }
 void split_check_waits(lfmm_geometry_s* g) {
     if (!g->wait_err || *(volatile int*)g->wait_err == 0) return;
@@ -1077,9 +1073,14 @@ void split_check_waits(lfmm_geometry_s* g) {
 }
 static SplitArgs split_args(lfmm_geometry_s* g, int col0, int ncols) {
     const SplitPlan& P = split_plan(g, ncols);
+    // products, then digits, then exponents
+    unsigned char* ws = ncols == 1 ? g->d_sp_ws1 : g->d_sp_ws;
+    const size_t rows = sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) * ncols;
+    uint32_t* vdig = (uint32_t*)(ws + ((rows + 15) & ~(size_t)15));
+    int* vexp = (int*)(vdig + (size_t)g->sp_nvec * ncols * SP_ND * SP_BLK);
     return SplitArgs{g->d_sp_vec, g->d_sp_pair, P.d_unit, g->d_sp_ctr, g->d_sp_row, g->d_sp_dst, g->d_sp_rexp, g->d_sp_dexp,
                      g->d_sp_dig, g->d_M, g->d_Mp, g->d_L, g->d_Lp, g->ncoef, g->nslotcoef,
-                     g->d_sp_vdig, g->d_sp_vexp, g->sp_nvec, g->d_sp_ws, col0, ncols, g->wait_err};
+                     vdig, vexp, g->sp_nvec, (double*)ws, col0, ncols, g->wait_err};
 }
 static void launch_split_vec(lfmm_geometry_s* g, const SplitArgs& a, int v0, int v1, cudaStream_t s) {
     if (v1 <= v0) return;

@@ -363,13 +363,11 @@ struct lfmm_geometry_s {
     int sp_cap = 0;                                 // most columns of a unit (LFMM_AUTOTUNE)
     std::vector<int> sp_dst_start, sp_vec_start;    // [nlev + 2]: first destination / vector of each level
     std::vector<int> sp_fine_start;                 // [nlev]: first of its vectors in fine segments
-    uint32_t* d_sp_vdig = nullptr;                  // digits and exponents of the vectors, sp_ws_cols columns
-    int* d_sp_vexp = nullptr;
     int sp_nvec = 0;                                // blocks of one column
     int sp_ntab = 0;
     int64_t sp_rows = 0;                            // workspace doubles per column
-    double* d_sp_ws = nullptr;
-    int sp_ws_cols = 0;                             // columns it holds
+    unsigned char *d_sp_ws1 = nullptr, *d_sp_ws = nullptr;   // workspace of one column, of a block
+    size_t sp_ws_bytes = 0;                                  // the block's
     int* wait_err = nullptr;                        // pinned, written by the device: a bounded wait gave up
     std::vector<int> vf_ptr_host, vf_src_host, vf_tab_host, slot_of_host;
     std::vector<int> m2l_ent_ptr_host;      // entry range per target box

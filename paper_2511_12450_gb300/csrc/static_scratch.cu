@@ -19,7 +19,9 @@
 //    it has to start at zero: the sorted output is cleared by the call itself and
 //    every coefficient is written before it is read.  Calls that overlap on the GPU
 //    (other streams, other threads) race on the array and must be serialised;
-//  * geometries whose work buffers do not fit are rejected before any device work;
+//  * geometries whose work buffers do not fit are rejected before any device work; the M2L's
+//    products go to the geometry's one-column workspace, which is made with the geometry and stays
+//    at its place while it lives, so that a captured call stays valid;
 //  * for the length of the call the geometry's work-buffer fields point into the
 //    array, under the geometry's call lock, which every other entry point that
 //    applies the operator also takes: a concurrent lfmm_matvec, lfmm_gmres_solve,

@@ -48,6 +48,32 @@ def test_rounds_equal_single_products(gpu_lib):
     assert torch.equal(yb, Y) and torch.equal(ys, lf.matvec(small, xs))
 
 
+def test_captured_static_product_outlives_wider_blocks(gpu_lib):
+    """A captured allocation-free product keeps its workspace when blocks make the geometry's grow."""
+    import torch
+
+    lf = gpu_lib
+    G = geometry(lf, layered_small(n_bodies=3, nodes=150, seed=7), 16)
+    x, y = columns(G.n, 1, 7)[0], torch.empty(G.n, dtype=torch.complex128, device="cuda")
+    lf.matvec_static(G, x, y)
+    torch.cuda.synchronize()
+    ref = y.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        lf.matvec_static(G, x, y)
+    other = []
+    for cols in (2, 9, 40):
+        X = columns(G.n, cols, 10 + cols)
+        other.append((X, lf.matvec(G, X)))
+        y.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, ref)
+        for X, Y in other:   # nothing of theirs was written by the replay
+            assert torch.equal(lf.matvec(G, X), Y)
+
+
 def test_captured_products_outlive_other_widths(gpu_lib):
     """A warmed-up width can be captured whatever width ran last, and its graph stays valid while
     narrower products run."""
