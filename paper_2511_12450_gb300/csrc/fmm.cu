@@ -201,18 +201,23 @@ static void build_m2l_work(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, c
 // The split M2L's matrices, pairs and destinations (split.cuh).  Matrices, and with them
 // units and workspace rows, in level order, so that the levels above the precision form's
 // first FP32 level are a prefix.
-static size_t split_col_bytes(const lfmm_geometry_s* g) {   // workspace of one column
-    return sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) +
-           (size_t)g->sp_nvec * (SP_ND * SP_BLK * sizeof(uint32_t) + sizeof(int)) + 16;
+// The M2L of the levels below lm alone (the precision form's FP64 part), or with lm = D + 1 all of
+// the FP64 form: workspace rows and blocks of vector digits, and bytes, of one column.
+static int64_t split_rows(const lfmm_geometry_s* g, int lm) { return lm > g->tree.D ? g->sp_rows : g->sp_row_start[lm]; }
+static int64_t split_nblk(const lfmm_geometry_s* g, int lm) { return lm > g->tree.D ? g->sp_nvec : g->sp_blk_start[lm]; }
+static size_t split_col_bytes(const lfmm_geometry_s* g, int lm) {
+    return sizeof(double) * (size_t)std::max<int64_t>(split_rows(g, lm), 1) +
+           (size_t)split_nblk(g, lm) * (SP_ND * SP_BLK * sizeof(uint32_t) + sizeof(int)) + 16;
 }
 // Units: a matrix's (pair, column) columns in groups of up to sp_cap, of nearly equal size, by
 // row tiles of up to 64 complex rows.
-static SplitPlan make_split_plan(lfmm_geometry_s* g, int ncols) {
+static SplitPlan make_split_plan(lfmm_geometry_s* g, int ncols, int lm) {
     SplitPlan P;
     std::vector<SplitUnit> units;
     const int nst = 3 * (g->tree.D + 1), cap = g->sp_cap;
     P.start.assign(nst + 1, -1);
     for (const SplitTab& s : g->sp_tabs_host) {
+        if (lm <= g->tree.D && s.level >= lm) continue;
         if (P.start[s.level] < 0) P.start[s.level] = (int)units.size();
         const int nco = 2 * s.pT + 1, Q = s.npairs * ncols, nu = (Q + cap - 1) / cap;
         for (int u = 0; u < nu; ++u) {
@@ -236,10 +241,13 @@ static SplitPlan make_split_plan(lfmm_geometry_s* g, int ncols) {
 // The plan of a block width, made on its first use and kept while the geometry lives: callers
 // alternate widths, a block wider than its workspace runs in rounds of two widths, and a captured
 // product holds its plan's units.  56 bytes per unit of up to 32 columns, where the workspace of
-// that width holds 2 (2p + 1) doubles per column: less than half a per cent of it.
-static const SplitPlan& split_plan(lfmm_geometry_s* g, int ncols) {
-    auto it = g->sp_plan.find(ncols);
-    if (it == g->sp_plan.end()) it = g->sp_plan.emplace(ncols, make_split_plan(g, ncols)).first;
+// that width holds 2 (2p + 1) doubles per column: less than half a per cent of it.  The levels below
+// lm come first in a plan of all levels, which serves them too.
+static const SplitPlan& split_plan(lfmm_geometry_s* g, int ncols, int lm) {
+    const int all = g->tree.D + 1;
+    auto it = g->sp_plan.find({ncols, all});
+    if (it == g->sp_plan.end() && lm < all) it = g->sp_plan.find({ncols, lm});
+    if (it == g->sp_plan.end()) it = g->sp_plan.emplace(std::make_pair(ncols, lm), make_split_plan(g, ncols, lm)).first;
     return it->second;
 }
 static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, const std::vector<int>& vr_src,
@@ -294,7 +302,9 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     int64_t dig = 0;
     int np = 0, nrexp = 0;
     int64_t rows = 0;
+    g->sp_row_start.assign(nlev, 0);
     for (int l = 0; l < nlev; ++l) {
+        g->sp_row_start[l] = rows;
         for (int i : by_level[l]) {
             SplitTab s{};
             const int p = t.p_level[l], nco = 2 * p + 1;
@@ -332,8 +342,10 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
         if (g->rkey_fine[i]) fine_used[(size_t)g->rkey_lay_s[i] * nlev + keys[i].level] = 1;
     g->sp_vec_start.assign(nlev + 2, 0);
     g->sp_fine_start.assign(nlev, 0);
+    g->sp_blk_start.assign(nlev, 0);
     for (int l = 0; l < nlev; ++l) {
         g->sp_vec_start[l] = (int)vecs.size();
+        g->sp_blk_start[l] = nblk;
         g->sp_fine_start[l] = (int)vecs.size();
         if (l < l0) continue;
         const int p = t.p_level[l];
@@ -492,9 +504,9 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     g->d_sp_dig = dalloc<unsigned char>(g, (size_t)dig);
     g->d_sp_ctr = dalloc<int>(g, 1);
     g->sp_cap = SP_COLS;
-    split_plan(g, 1);
+    split_plan(g, 1, nlev);
     g->sp_rows = rows;
-    g->d_sp_ws1 = dalloc<unsigned char>(g, split_col_bytes(g));
+    g->d_sp_ws1 = dalloc<unsigned char>(g, split_col_bytes(g, nlev));
     cuda_check(cudaHostAlloc((void**)&g->wait_err, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable), "wait status");
     *g->wait_err = 0;
 }
@@ -1051,14 +1063,14 @@ void fmm_free(lfmm_geometry_s* g) {
 // keeps what it points to when a block makes the other one grow.
 #define SP_WS_BYTES (2ll << 30)
 #define SP_SMS 152   // persistent CTAs of k_split: one per SM
-static int split_rounds(const lfmm_geometry_s* g, int nrhs) {
-    const int cap = (int)std::max<int64_t>(1, std::min<int64_t>(2048, SP_WS_BYTES / (int64_t)split_col_bytes(g)));
+static int split_rounds(const lfmm_geometry_s* g, int nrhs, int lm) {
+    const int cap = (int)std::max<int64_t>(1, std::min<int64_t>(2048, SP_WS_BYTES / (int64_t)split_col_bytes(g, lm)));
     return (nrhs + cap - 1) / cap;
 }
 static int round_start(int nrhs, int rounds, int r) { return (int)((int64_t)nrhs * r / rounds); }   // first column
-static void ensure_split(lfmm_geometry_s* g, int nrhs) {
-    const int rounds = split_rounds(g, nrhs), cols = (nrhs + rounds - 1) / rounds;
-    const size_t want = split_col_bytes(g) * cols;
+static void ensure_split(lfmm_geometry_s* g, int nrhs, int lm) {
+    const int rounds = split_rounds(g, nrhs, lm), cols = (nrhs + rounds - 1) / rounds;
+    const size_t want = split_col_bytes(g, lm) * cols;
     if (cols == 1 || g->sp_ws_bytes >= want) return;
     dev_release_now(g->d_sp_ws);
     g->d_sp_ws = nullptr;
@@ -1071,16 +1083,16 @@ void split_check_waits(lfmm_geometry_s* g) {
     *(volatile int*)g->wait_err = 0;
     throw TimeoutError{"split M2L: an mbarrier wait gave up; that product's M2L contributions were zeroed"};
 }
-static SplitArgs split_args(lfmm_geometry_s* g, int col0, int ncols) {
-    const SplitPlan& P = split_plan(g, ncols);
+static SplitArgs split_args(lfmm_geometry_s* g, int col0, int ncols, int lm) {
+    const SplitPlan& P = split_plan(g, ncols, lm);
     // products, then digits, then exponents
     unsigned char* ws = ncols == 1 ? g->d_sp_ws1 : g->d_sp_ws;
-    const size_t rows = sizeof(double) * (size_t)std::max<int64_t>(g->sp_rows, 1) * ncols;
+    const size_t rows = sizeof(double) * (size_t)std::max<int64_t>(split_rows(g, lm), 1) * ncols;
     uint32_t* vdig = (uint32_t*)(ws + ((rows + 15) & ~(size_t)15));
-    int* vexp = (int*)(vdig + (size_t)g->sp_nvec * ncols * SP_ND * SP_BLK);
+    int* vexp = (int*)(vdig + (size_t)split_nblk(g, lm) * ncols * SP_ND * SP_BLK);
     return SplitArgs{g->d_sp_vec, g->d_sp_pair, P.d_unit, g->d_sp_ctr, g->d_sp_row, g->d_sp_dst, g->d_sp_rexp, g->d_sp_dexp,
                      g->d_sp_dig, g->d_M, g->d_Mp, g->d_L, g->d_Lp, g->ncoef, g->nslotcoef,
-                     vdig, vexp, g->sp_nvec, (double*)ws, col0, ncols, g->wait_err};
+                     vdig, vexp, split_nblk(g, lm), (double*)ws, col0, ncols, g->wait_err};
 }
 static void launch_split_vec(lfmm_geometry_s* g, const SplitArgs& a, int v0, int v1, cudaStream_t s) {
     if (v1 <= v0) return;
@@ -1089,8 +1101,8 @@ static void launch_split_vec(lfmm_geometry_s* g, const SplitArgs& a, int v0, int
     ++g->n_launches;
 }
 // the products of the stages [st0, st1)
-static void launch_split_units(lfmm_geometry_s* g, SplitArgs a, int st0, int st1, cudaStream_t s) {
-    const SplitPlan& P = split_plan(g, a.ncols);
+static void launch_split_units(lfmm_geometry_s* g, SplitArgs a, int lm, int st0, int st1, cudaStream_t s) {
+    const SplitPlan& P = split_plan(g, a.ncols, lm);
     const int n = P.start[st1] - P.start[st0];
     if (n <= 0) return;
     raise_smem_limit((const void*)k_split, SP_SMEM, "split M2L smem");
@@ -1115,12 +1127,12 @@ static void launch_split_reduce(lfmm_geometry_s* g, const SplitArgs& a, int nd, 
 // FP64 M2L of the levels below lm, digits included
 static void launch_split(lfmm_geometry_s* g, int nrhs, int lm, cudaStream_t s) {
     split_check_waits(g);
-    ensure_split(g, nrhs);
-    for (int r = 0, n = split_rounds(g, nrhs); r < n; ++r) {
+    ensure_split(g, nrhs, lm);
+    for (int r = 0, n = split_rounds(g, nrhs, lm); r < n; ++r) {
         const int c0 = round_start(nrhs, n, r);
-        const SplitArgs a = split_args(g, c0, round_start(nrhs, n, r + 1) - c0);
+        const SplitArgs a = split_args(g, c0, round_start(nrhs, n, r + 1) - c0, lm);
         launch_split_vec(g, a, 0, g->sp_vec_start[lm], s);
-        launch_split_units(g, a, 0, lm, s);
+        launch_split_units(g, a, lm, 0, lm, s);
         launch_split_reduce(g, a, g->sp_dst_start[lm], s);
     }
 }
@@ -1202,10 +1214,10 @@ static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
     const TreeHost& t = g->tree;
     const int D = t.D, l0 = t.l0, nlev = D + 1;
     split_check_waits(g);
-    ensure_split(g, nrhs);
-    for (int r = 0, n = split_rounds(g, nrhs); r < n; ++r) {
+    ensure_split(g, nrhs, nlev);
+    for (int r = 0, n = split_rounds(g, nrhs, nlev); r < n; ++r) {
         const int c0 = round_start(nrhs, n, r), nc = round_start(nrhs, n, r + 1) - c0;
-        const SplitArgs a = split_args(g, c0, nc);
+        const SplitArgs a = split_args(g, c0, nc, nlev);
         auto columns = [&](XPass P) {
             P.X += (int64_t)c0 * g->ncoef;
             P.Xp += (int64_t)c0 * g->nslotcoef;
@@ -1227,7 +1239,7 @@ static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
                 continue;
             }
             if (!ready[l]) { launch_split_vec(g, a, g->sp_vec_start[l], g->sp_fine_start[l], s); ready[l] = 1; }
-            launch_split_units(g, a, nlev + l, nlev + l + 1, s);
+            launch_split_units(g, a, nlev, nlev + l, nlev + l + 1, s);
             finish(l, 0);
             ready[l - 1] = 1;
         }
@@ -1243,7 +1255,7 @@ static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
             launch_split_vec(g, a, g->sp_vec_start[l], g->sp_vec_start[e + 1], s);
             l = e;
         }
-        launch_split_units(g, a, 0, nlev, s);
+        launch_split_units(g, a, nlev, 0, nlev, s);
         launch_split_reduce(g, a, g->sp_dst_start[nlev], s);
         prof_end(g, ST_M2L, s);
         prof_begin(g, ST_L2L, s);
@@ -1254,7 +1266,7 @@ static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
             }
             if (l == l0 + 1 || !g->sp_dn[l - 1])
                 launch_split_vec(g, local_args(g, a), g->sp_vec_start[l - 1], g->sp_fine_start[l - 1], s);
-            launch_split_units(g, a, 2 * nlev + l, 2 * nlev + l + 1, s);
+            launch_split_units(g, a, nlev, 2 * nlev + l, 2 * nlev + l + 1, s);
             finish(l, 1);
         }
         prof_end(g, ST_L2L, s);
@@ -1471,7 +1483,7 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
         far.push_back(&op);
         ensure_coef(g, op.nrhs);
         split_check_waits(g);
-        ensure_split(g, op.nrhs);
+        ensure_split(g, op.nrhs, t.D + 1);
         max_nrhs = std::max(max_nrhs, op.nrhs);
         cb_l2p = std::min(cb_l2p, t.p_level[t.D] <= 40 ? 4 : 1);
         max_up = std::max(max_up, t.D - t.l0);
@@ -1499,7 +1511,7 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
     // a block too wide for its workspace: its own rounds; the others share every launch
     std::vector<const BatchOp*> sh;
     for (const BatchOp* op : far) {
-        if (split_rounds(op->g, op->nrhs) > 1) far_fp64(op->g, op->nrhs, s);
+        if (split_rounds(op->g, op->nrhs, op->g->tree.D + 1) > 1) far_fp64(op->g, op->nrhs, s);
         else sh.push_back(op);
     }
     auto vec_jobs = [&](const std::vector<SplitJob>& jobs) {
@@ -1512,9 +1524,9 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
         std::vector<SplitArgs> args;
         std::vector<int> prefix(1, 0);
         for (const BatchOp* op : ops2) {
-            const SplitPlan& P = split_plan(op->g, op->nrhs);
+            const SplitPlan& P = split_plan(op->g, op->nrhs, op->g->tree.D + 1);
             const std::pair<int, int> st = range(op->g);
-            args.push_back(split_args(op->g, 0, op->nrhs));
+            args.push_back(split_args(op->g, 0, op->nrhs, op->g->tree.D + 1));
             args.back().unit += P.start[st.first];
             prefix.push_back(prefix.back() + P.start[st.second] - P.start[st.first]);
         }
@@ -1552,7 +1564,7 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
             }
             sp.push_back(op);
             vec_of_level(op, l, vj);
-            fj.push_back(FinJob{fin_args(g, split_args(g, 0, op->nrhs), l, down)});
+            fj.push_back(FinJob{fin_args(g, split_args(g, 0, op->nrhs, g->tree.D + 1), l, down)});
             fb.push_back(fin_ctas(fj.back().F) * op->nrhs);
             fs = std::max(fs, fin_smem_of(g, l, down));
         }
@@ -1576,7 +1588,7 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
                  lfmm_geometry_s* g = op->g;
                  std::vector<char>& r = ready_of(op);
                  if (!r[l])
-                     vj.push_back(SplitJob{split_args(g, 0, op->nrhs), g->sp_vec_start[l], g->sp_fine_start[l] - g->sp_vec_start[l]});
+                     vj.push_back(SplitJob{split_args(g, 0, op->nrhs, g->tree.D + 1), g->sp_vec_start[l], g->sp_fine_start[l] - g->sp_vec_start[l]});
                  r[l] = r[l - 1] = 1;
              });
     {   // M2L of every level: the digits still missing, products, each destination's sum
@@ -1588,10 +1600,10 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
             std::vector<char>& r = ready_of(op);
             for (int l = g->tree.l0; l <= D; ++l) {
                 const int v0 = r[l] ? g->sp_fine_start[l] : g->sp_vec_start[l], nv = g->sp_vec_start[l + 1] - v0;
-                if (nv > 0) vj.push_back(SplitJob{split_args(g, 0, op->nrhs), v0, nv});
+                if (nv > 0) vj.push_back(SplitJob{split_args(g, 0, op->nrhs, g->tree.D + 1), v0, nv});
             }
             const int nd = g->sp_dst_start[D + 1], nbig = split_big(g, nd);
-            jobs.push_back(SplitJob{split_args(g, 0, op->nrhs), nbig, nd});
+            jobs.push_back(SplitJob{split_args(g, 0, op->nrhs, g->tree.D + 1), nbig, nd});
             rblocks.push_back(split_red_ctas(nbig, nd - nbig) * op->nrhs);
         }
         vec_jobs(vj);
@@ -1604,7 +1616,7 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
              [&](const BatchOp* op, int l, std::vector<SplitJob>& vj) {
                  lfmm_geometry_s* g = op->g;
                  if (l == g->tree.l0 + 1 || !g->sp_dn[l - 1])
-                     vj.push_back(SplitJob{local_args(g, split_args(g, 0, op->nrhs)), g->sp_vec_start[l - 1],
+                     vj.push_back(SplitJob{local_args(g, split_args(g, 0, op->nrhs, g->tree.D + 1)), g->sp_vec_start[l - 1],
                                            g->sp_fine_start[l - 1] - g->sp_vec_start[l - 1]});
              });
     // L2P after the near field, which adds into the same y
@@ -1644,7 +1656,7 @@ void fmm_autotune(lfmm_geometry_s* g) {
             dev_release(e.second.d_unit);
         }
         g->sp_plan.clear();
-        split_plan(g, 1);
+        split_plan(g, 1, t.D + 1);
     };
     int best_work = M2L_ITEM_WORK;
     double best = 1e300, dflt = 0.0;

@@ -359,10 +359,11 @@ struct lfmm_geometry_s {
     int64_t sp_dig_bytes = 0;
     int* d_sp_ctr = nullptr;
     int sp_max_tiles = 1;
-    std::map<int, lfmm::SplitPlan> sp_plan;         // by block width
+    std::map<std::pair<int, int>, lfmm::SplitPlan> sp_plan;   // by block width and levels (below it)
     int sp_cap = 0;                                 // most columns of a unit (LFMM_AUTOTUNE)
     std::vector<int> sp_dst_start, sp_vec_start;    // [nlev + 2]: first destination / vector of each level
-    std::vector<int> sp_fine_start;                 // [nlev]: first of its vectors in fine segments
+    std::vector<int> sp_fine_start, sp_blk_start;   // [nlev]: first of its vectors in fine segments; first block
+    std::vector<int64_t> sp_row_start;              // [nlev]: first workspace row of its M2L
     int sp_nvec = 0;                                // blocks of one column
     int sp_ntab = 0;
     int64_t sp_rows = 0;                            // workspace doubles per column

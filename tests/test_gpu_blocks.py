@@ -102,3 +102,30 @@ def test_captured_products_outlive_other_widths(gpu_lib):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(Y, ref_new)
+
+
+def test_precision_form_holds_its_own_levels_only(gpu_lib):
+    """The precision form's FP64 products are those of the levels above its FP32 ones: 3 MB of workspace
+    per column at 65,536 points, where all levels take 66 MB.  Beside it a column holds its FP64 and
+    FP32 expansions (18 MB), sorted vectors and partial sums (some 8 MB): below 50 MB in all.  The
+    result is that of a geometry whose blocks have products of all levels already."""
+    import torch
+
+    lf = gpu_lib
+    cols = 32
+    G = geometry(lf, config_c2(), 64)
+    X = columns(G.n, cols, 1)
+    Y = torch.empty_like(X)
+    lf.matvec(G, X[0].contiguous(), mixed=True)   # the form's tables
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    lf.matvec(G, X, Y, mixed=True)
+    torch.cuda.synchronize()
+    assert free0 - torch.cuda.mem_get_info()[0] <= cols * (50 << 20)
+    S = geometry(lf, config_c2(), 64)
+    lf.matvec(S, X)
+    assert torch.equal(lf.matvec(S, X, mixed=True), Y)
+    five = X[:5].contiguous()
+    ref = lf.matvec(G, five, mixed=True)
+    lf.matvec(S, five)
+    assert torch.equal(lf.matvec(S, five, mixed=True), ref)
