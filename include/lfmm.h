@@ -429,6 +429,9 @@ lfmm_status lfmm_server_destroy(lfmm_server s);
  * "launch_count" (double[1]: kernels launched so far by this geometry's
  * matvec path -- gather, P2M, M2M, M2L, L2L, L2P, near field, scatter --
  * counted on the host as they are enqueued),
+ * "wait_word" (int64[1]: host address of the int32 that a kernel sets when one of the FP64
+ * products' bounded waits gives up, 0 without a far field; a test that sets it stands in for
+ * the kernel -- see LFMM_ERR_TIMEOUT),
  * "tuning" (double[4]: M2L item work cap, one row per narrow box (1/0), and
  * with LFMM_AUTOTUNE the milliseconds of one FP64 M2L with the default and the
  * chosen schedule, else 0, 0),

@@ -752,6 +752,7 @@ lfmm_status lfmm_geometry_query(lfmm_geometry g, const char* name, void* host_ou
         TreeHost& t = g->tree;
         std::vector<int> tmp;
         std::vector<double> dtmp;
+        int64_t word = 0;
         const void* src = nullptr;
         int64_t bytes = 0;
         std::string nm(name);
@@ -815,6 +816,10 @@ lfmm_status lfmm_geometry_query(lfmm_geometry g, const char* name, void* host_ou
             dtmp = {(double)g->n_launches};
             src = dtmp.data();
             bytes = (int64_t)sizeof(double);
+        } else if (nm == "wait_word") {
+            word = (int64_t)(uintptr_t)g->wait_err;
+            src = &word;
+            bytes = (int64_t)sizeof(word);
         } else if (nm == "tuning") {
             dtmp = {(double)g->m2l_item_work, (double)g->m2l_wide, g->tune_ms_default, g->tune_ms_best};
             src = dtmp.data();

@@ -1068,15 +1068,18 @@ static int split_rounds(const lfmm_geometry_s* g, int nrhs, int lm) {
     return (nrhs + cap - 1) / cap;
 }
 static int round_start(int nrhs, int rounds, int r) { return (int)((int64_t)nrhs * r / rounds); }   // first column
-static void ensure_split(lfmm_geometry_s* g, int nrhs, int lm) {
+static void ensure_split(lfmm_geometry_s* g, int nrhs, int lm) {   // workspace and plans of the rounds' widths
     const int rounds = split_rounds(g, nrhs, lm), cols = (nrhs + rounds - 1) / rounds;
     const size_t want = split_col_bytes(g, lm) * cols;
-    if (cols == 1 || g->sp_ws_bytes >= want) return;
-    dev_release_now(g->d_sp_ws);
-    g->d_sp_ws = nullptr;
-    g->sp_ws_bytes = 0;
-    g->d_sp_ws = (unsigned char*)dev_alloc_ready(want, "split M2L workspace");
-    g->sp_ws_bytes = want;
+    if (cols > 1 && g->sp_ws_bytes < want) {
+        dev_release_now(g->d_sp_ws);
+        g->d_sp_ws = nullptr;
+        g->sp_ws_bytes = 0;
+        g->d_sp_ws = (unsigned char*)dev_alloc_ready(want, "split M2L workspace");
+        g->sp_ws_bytes = want;
+    }
+    split_plan(g, cols, lm);
+    split_plan(g, nrhs / rounds, lm);
 }
 void split_check_waits(lfmm_geometry_s* g) {
     if (!g->wait_err || *(volatile int*)g->wait_err == 0) return;
@@ -1126,8 +1129,6 @@ static void launch_split_reduce(lfmm_geometry_s* g, const SplitArgs& a, int nd, 
 }
 // FP64 M2L of the levels below lm, digits included
 static void launch_split(lfmm_geometry_s* g, int nrhs, int lm, cudaStream_t s) {
-    split_check_waits(g);
-    ensure_split(g, nrhs, lm);
     for (int r = 0, n = split_rounds(g, nrhs, lm); r < n; ++r) {
         const int c0 = round_start(nrhs, n, r);
         const SplitArgs a = split_args(g, c0, round_start(nrhs, n, r + 1) - c0, lm);
@@ -1213,8 +1214,6 @@ static void launch_pass(lfmm_geometry_s* g, const XPass& P, int nrhs, cudaStream
 static void far_fp64(lfmm_geometry_s* g, int nrhs, cudaStream_t s) {
     const TreeHost& t = g->tree;
     const int D = t.D, l0 = t.l0, nlev = D + 1;
-    split_check_waits(g);
-    ensure_split(g, nrhs, nlev);
     for (int r = 0, n = split_rounds(g, nrhs, nlev); r < n; ++r) {
         const int c0 = round_start(nrhs, n, r), nc = round_start(nrhs, n, r + 1) - c0;
         const SplitArgs a = split_args(g, c0, nc, nlev);
@@ -1284,15 +1283,30 @@ static L2PArgs l2p_args(lfmm_geometry_s* g, cd* y, int nrhs) {
 // right-hand sides per CTA of the L2P: four where their P, Q fit beside the basis rows
 static int l2p_cols(const lfmm_geometry_s* g, int nrhs) { return nrhs > 1 && g->tree.p_level[g->tree.D] <= 40 ? 4 : 1; }
 
+// precision form: the levels >= lm run in FP32 on scaled expansions (lm > D: none)
+static int first_fp32(lfmm_geometry_s* g, bool mixed) {
+    const int D = g->tree.D;
+    return mixed ? std::max(g->tree.l0, std::min(mixed_level(g), D + 1)) : D + 1;
+}
+void fmm_prepare(lfmm_geometry_s* g, int nrhs, bool mixed) {
+    const int l0 = g->tree.l0;
+    if (l0 > g->tree.D) return;
+    ensure_coef(g, nrhs);
+    const int lm = first_fp32(g, mixed);
+    if (lm <= g->tree.D) mixed_setup(g, nrhs);
+    if (lm > l0) ensure_split(g, nrhs, lm);
+}
+void fmm_check_waits(lfmm_geometry_s* g) {
+    split_check_waits(g);
+    mixed_check_waits(g);
+}
+
 void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s, bool mixed,
                cudaEvent_t before_l2p) {
     TreeHost& t = g->tree;
     const int D = t.D, l0 = t.l0;
     if (l0 > D) return;
-    ensure_coef(g, nrhs);
-    // precision form: the levels >= lm run in FP32 on scaled expansions (lm > D: none)
-    const int lm = mixed ? std::max(l0, std::min(mixed_level(g), D + 1)) : D + 1;
-    if (lm <= D) mixed_setup(g, nrhs);
+    const int lm = first_fp32(g, mixed);
     {   // P2M: leaves about cell centres, straddling leaves about reaction centres
         prof_begin(g, ST_P2M, s);
         if (lm <= D) {
@@ -1332,13 +1346,19 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
         prof_end(g, ST_M2M, s);
         prof_begin(g, ST_M2L, s);
         if (coarse && !beside) launch_split(g, nrhs, lm, s);
-        cudaStream_t q = beside ? mixed_fork(g, s) : s;
-        mixed_m2l(g, nrhs, lm, s);
         if (beside) {
+            const cudaStream_t q = mixed_fork(g, s);
+            struct Join {   // also when a launch fails: what the chain writes, later calls write on s
+                lfmm_geometry_s* g;
+                cudaStream_t s;
+                ~Join() { mixed_join(g, s); }
+            } join{g, s};
+            mixed_m2l(g, nrhs, lm, s);
             coarse_up(q);
             launch_split(g, nrhs, lm, q);
             coarse_down(q);
-            mixed_join(g, s);
+        } else {
+            mixed_m2l(g, nrhs, lm, s);
         }
         prof_end(g, ST_M2L, s);
         prof_begin(g, ST_L2L, s);
@@ -1481,9 +1501,6 @@ void fmm_apply_batch(const std::vector<BatchOp>& ops, cudaStream_t s, cudaEvent_
         const TreeHost& t = g->tree;
         if (t.l0 > t.D) continue;
         far.push_back(&op);
-        ensure_coef(g, op.nrhs);
-        split_check_waits(g);
-        ensure_split(g, op.nrhs, t.D + 1);
         max_nrhs = std::max(max_nrhs, op.nrhs);
         cb_l2p = std::min(cb_l2p, t.p_level[t.D] <= 40 ? 4 : 1);
         max_up = std::max(max_up, t.D - t.l0);

@@ -486,6 +486,11 @@ void near_build(lfmm_geometry_s* g);
 void near_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s, bool mixed = false);
 // FMM far field (fmm.cu)
 void fmm_build(lfmm_geometry_s* g);
+// work buffers, tables and plans of a product of nrhs columns: what can run out of memory, before
+// anything of the product is queued
+void fmm_prepare(lfmm_geometry_s* g, int nrhs, bool mixed);
+// throws TimeoutError, once, if a bounded wait of a product that has run by now gave up
+void fmm_check_waits(lfmm_geometry_s* g);
 void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s, bool mixed = false,
                cudaEvent_t before_l2p = nullptr);
 void fmm_autotune(lfmm_geometry_s* g);

@@ -1010,10 +1010,9 @@ cudaStream_t mixed_fork(lfmm_geometry_s* g, cudaStream_t s) {
     cuda_check(cudaStreamWaitEvent(ms->top, ms->ev_fork, 0), "coarse levels' fork");
     return ms->top;
 }
-void mixed_join(lfmm_geometry_s* g, cudaStream_t s) {
+void mixed_join(lfmm_geometry_s* g, cudaStream_t s) {   // throws nothing: a failure is the thread's last CUDA error
     MixedState* ms = g->mixed;
-    cuda_check(cudaEventRecord(ms->ev_join, ms->top), "coarse levels' join");
-    cuda_check(cudaStreamWaitEvent(s, ms->ev_join, 0), "coarse levels' join");
+    if (cudaEventRecord(ms->ev_join, ms->top) == cudaSuccess) cudaStreamWaitEvent(s, ms->ev_join, 0);
 }
 void mixed_wait(lfmm_geometry_s* g) {
     if (g->mixed && g->mixed->top) cudaStreamSynchronize(g->mixed->top);
@@ -1148,7 +1147,6 @@ static bool m2l_tc(lfmm_geometry_s* g, int nrhs, int min_level, cudaStream_t s) 
     const int nco = 2 * ms->tc_p + 1;
     if (nrhs < TC_MIN_COLS || g->m2l_simt || ms->n_tc_boxes == 0 || 2 * nco > 128 || min_level != ms->lm)
         return false;
-    mixed_check_waits(g);
     // K: real part at 0, imaginary part at kh = nco rounded up to 4 (16-byte stores), padded to 8
     const int kp = (2 * ((nco + 3) / 4 * 4) + 7) / 8 * 8;
     for (int c0 = 0; c0 < nrhs; c0 += TC_MAXN) {

@@ -75,17 +75,42 @@ void round_to_c64(const cd* in, float2* out, int64_t n, cudaStream_t s) {
     cuda_check(cudaGetLastError(), "k_round_c64");
 }
 
-void apply_operator_sorted(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s,
-                           bool mixed) {
+// A geometry's side stream between a fork from s and its join; joined also when something in
+// between throws, so that the next call's work on s does not run beside what is still queued there.
+struct SideFork {
+    lfmm_geometry_s* g;
+    cudaStream_t s;
+    bool joined = false;
+    SideFork(lfmm_geometry_s* g_, cudaStream_t s_) : g(g_), s(s_) {
+        cuda_check(cudaEventRecord(g->ev_fork, s), "fork");
+        cuda_check(cudaStreamWaitEvent(g->side, g->ev_fork, 0), "fork");
+    }
+    void join() {
+        joined = true;
+        cuda_check(cudaStreamWaitEvent(s, g->ev_join, 0), "join");
+    }
+    ~SideFork() {
+        if (!joined && cudaEventRecord(g->ev_join, g->side) == cudaSuccess) cudaStreamWaitEvent(s, g->ev_join, 0);
+    }
+};
+
+// Work buffers and plans are there (fmm_prepare): nothing below allocates but a first
+// precision-form call's near field.
+static void queue_operator(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s, bool mixed) {
     cuda_check(cudaMemsetAsync(y_sorted, 0, sizeof(cd) * g->n * nrhs, s), "memset y");
     // the stored near field (bound by HBM) on the geometry's side stream, beside the far
     // field (bound by the FP64 pipe); both add into y, the leaf evaluations after it
-    cuda_check(cudaEventRecord(g->ev_fork, s), "fork");
-    cuda_check(cudaStreamWaitEvent(g->side, g->ev_fork, 0), "fork");
+    SideFork side(g, s);
     near_apply(g, x_sorted, y_sorted, nrhs, g->side, mixed);
     cuda_check(cudaEventRecord(g->ev_join, g->side), "join");
     fmm_apply(g, x_sorted, y_sorted, nrhs, s, mixed, g->ev_join);
-    cuda_check(cudaStreamWaitEvent(s, g->ev_join, 0), "join");   // also when there is no far field
+    side.join();   // also when there is no far field
+}
+void apply_operator_sorted(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s,
+                           bool mixed) {
+    fmm_check_waits(g);
+    fmm_prepare(g, nrhs, mixed);
+    queue_operator(g, x_sorted, y_sorted, nrhs, s, mixed);
 }
 
 // Several geometries' FP64 operators in shared launches (one launch per stage for all of
@@ -93,15 +118,16 @@ void apply_operator_sorted(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted,
 // near fields run on the first geometry's side stream beside the far fields.
 void apply_operator_batch_sorted(const std::vector<BatchOp>& ops, cudaStream_t s) {
     if (ops.empty()) return;
+    for (const BatchOp& op : ops) fmm_check_waits(op.g);
+    for (const BatchOp& op : ops) fmm_prepare(op.g, op.nrhs, false);
     for (const BatchOp& op : ops)
         cuda_check(cudaMemsetAsync(op.y, 0, sizeof(cd) * op.g->n * op.nrhs, s), "memset y");
     lfmm_geometry_s* g0 = ops[0].g;
-    cuda_check(cudaEventRecord(g0->ev_fork, s), "fork");
-    cuda_check(cudaStreamWaitEvent(g0->side, g0->ev_fork, 0), "fork");
+    SideFork side(g0, s);
     near_apply_batch(ops, g0->side);
     cuda_check(cudaEventRecord(g0->ev_join, g0->side), "join");
     fmm_apply_batch(ops, s, g0->ev_join);
-    cuda_check(cudaStreamWaitEvent(s, g0->ev_join, 0), "join");
+    side.join();
 }
 
 // ------------------------------------------------------------------ BLAS-2 helpers for GMRES
@@ -255,7 +281,7 @@ struct OpGraph {
         bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
         if (ok) {
             try {
-                apply_operator_sorted(g, z, w, 1, cs, mixed);
+                queue_operator(g, z, w, 1, cs, mixed);   // (a time-out stays for the check after the step)
             } catch (...) {
                 ok = false;
             }
