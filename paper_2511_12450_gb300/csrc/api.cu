@@ -487,8 +487,7 @@ lfmm_status lfmm_matvec(lfmm_geometry g, int32_t nrhs, const void* x, void* y, i
         if (!dev) {
             cuda_check(cudaMemcpyAsync(y, g->d_hostbuf_y, esz * elems, cudaMemcpyDeviceToHost, s), "y d2h");
             cuda_check(cudaStreamSynchronize(s), "matvec sync");
-            split_check_waits(g);
-            mixed_check_waits(g);
+            fmm_check_waits(g);
         }
         return LFMM_OK;
     });
@@ -713,6 +712,7 @@ lfmm_status lfmm_eval_field(lfmm_geometry g, int32_t nrhs, const void* density, 
         field_unpack(d_xy, d_ie, n, m, nrhs, c64, d_u, s);
         cuda_check(cudaMemcpyAsync(u, d_u, esz * m * nrhs, cudaMemcpyDefault, s), "u copy");
         cuda_check(cudaStreamSynchronize(s), "field sync");
+        fmm_check_waits(F);
         return LFMM_OK;
     });
 }

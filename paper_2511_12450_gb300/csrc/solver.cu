@@ -7,6 +7,7 @@
 #include <cmath>
 #include <complex>
 #include <stdexcept>
+#include <string>
 #include <vector>
 
 #include "geometry.h"
@@ -246,6 +247,7 @@ struct Blas {
         vh(w, 1, n, w, n, dres + 2 * cap);
         cuda_check(cudaMemcpyAsync(host.data(), dres + 2 * cap, sizeof(cd), cudaMemcpyDeviceToHost, s), "norm d2h");
         cuda_check(cudaStreamSynchronize(s), "norm sync");
+        fmm_check_waits(g);   // of the products that this is the norm of
         return std::sqrt(std::max(host[0].x, 0.0));
     }
 };
@@ -342,6 +344,7 @@ static int gmres_one(lfmm_geometry_s* g, const cd* b, cd* x, double tol, int max
         cuda_check(cudaMemcpyAsync(bl.host.data(), bl.dres, sizeof(cd) * (2 * bl.cap + 1), cudaMemcpyDeviceToHost, s),
                    "arnoldi d2h");
         cuda_check(cudaStreamSynchronize(s), "arnoldi sync");
+        fmm_check_waits(g);   // of this step's product (a replayed graph's too)
         for (int c = 0; c <= j; ++c)
             h[c] = C(bl.host[c].x, bl.host[c].y) + C(bl.host[bl.cap + c].x, bl.host[bl.cap + c].y);
         const double hn = std::sqrt(std::max(bl.host[2 * bl.cap].x, 0.0));
@@ -458,6 +461,7 @@ static int gmres_simul(lfmm_geometry_s* g, const cd* B, cd* X, int nrhs, double 
         }
         cuda_check(cudaMemcpyAsync(hres.data(), dres, sizeof(cd) * per * nrhs, cudaMemcpyDeviceToHost, s), "arnoldi d2h");
         cuda_check(cudaStreamSynchronize(s), "arnoldi sync");
+        fmm_check_waits(g);   // of this step's product (a replayed graph's too)
         for (int c = 0; c < nrhs; ++c) {
             if (!active[c]) continue;
             const cd* hr = hres.data() + (size_t)c * per;
@@ -726,6 +730,7 @@ struct BatchSolve {
     cd *b = nullptr, *x = nullptr;   // sorted order, owned
     // the driver (gmres_sorted)
     bool done = false;
+    std::string timeout;     // a product's bounded wait gave up: what batch_solve_finish reports
     int ok = 0, outer = 0, total = 0, f64 = 0, it = 0;
     double bn = 0, rn = 0, eps = 0, below = 0, res_est = 0;
     cd *r = nullptr, *d = nullptr, *y2 = nullptr;
@@ -978,7 +983,18 @@ void batch_solve_round(const std::vector<BatchSolve*>& all, cudaStream_t s) {
                    "arnoldi d2h");
     }
     for (BatchSolve* S : act) cuda_check(cudaStreamSynchronize(S->st), "round sync");
+    auto timed_out = [](BatchSolve* S, const TimeoutError& e) {   // ends this solve, not the others'
+        S->timeout = e.msg;
+        S->done = true;
+        S->in_pass = false;
+    };
     for (BatchSolve* S : act) {
+        try {
+            fmm_check_waits(S->g);
+        } catch (const TimeoutError& e) {
+            timed_out(S, e);
+            continue;
+        }
         const int j = (int)S->H.size();
         const int capb = S->bl->cap;
         const cd* hh = S->hpin;
@@ -1004,7 +1020,11 @@ void batch_solve_round(const std::vector<BatchSolve*>& all, cudaStream_t s) {
         S->gg[j] = cj * S->gg[j];
         S->H.push_back(h);
         S->res = std::abs(S->gg[j + 1]) / S->beta;
-        if (S->res <= S->tol_in || hn == 0.0 || (int)S->H.size() >= S->cap) bs_pass_end(*S, S->st);
+        try {
+            if (S->res <= S->tol_in || hn == 0.0 || (int)S->H.size() >= S->cap) bs_pass_end(*S, S->st);
+        } catch (const TimeoutError& e) {
+            timed_out(S, e);
+        }
     }
 }
 
@@ -1012,6 +1032,7 @@ bool batch_solve_done(const BatchSolve* S) { return S->done; }
 
 void batch_solve_finish(BatchSolve* S, cd* x_out, lfmm_gmres_info* info, cudaStream_t s) {
     if (S->st) cuda_check(cudaStreamSynchronize(S->st), "solve stream");
+    if (!S->timeout.empty()) throw TimeoutError{S->timeout};
     scatter_sorted(S->g, S->x, x_out, 1, s);
     if (info) {
         info->iterations = S->it;

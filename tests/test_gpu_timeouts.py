@@ -2,6 +2,8 @@
 that a kernel would set, in host memory, and looks at what the calls do with it."""
 
 import ctypes
+import threading
+import time
 
 import numpy as np
 import pytest
@@ -50,3 +52,34 @@ def test_a_call_that_reports_a_time_out_queues_nothing(gpu_lib, mixed):
         # the gather into the sorted order is queued by the call itself
         assert lf.geometry_query(G, "launch_count", np.float64)[0] <= n0 + 1
         assert torch.equal(lf.matvec(G, x, mixed=mixed), ref)
+
+
+@pytest.mark.parametrize("cols", [1, 3])
+def test_a_solve_looks_at_every_step(gpu_lib, cols):
+    """A time-out of one step's product (a replayed graph, a block) ends the solve there, instead of
+    after its last step or not at all."""
+    lf = gpu_lib
+    G = geometry(lf, layered_wide(), 8)
+    rng = np.random.default_rng(2)
+    b = np.asfortranarray(rng.standard_normal((G.n, cols)) + 1j * rng.standard_normal((G.n, cols)))
+    b = b[:, 0].copy() if cols == 1 else b
+
+    def solve():   # never reaches its tolerance
+        t0 = time.perf_counter()
+        try:
+            return lf.gmres_solve(G, b, tol=1e-30, max_iter=300, precond=False), time.perf_counter() - t0
+        except lf.LfmmError as e:
+            return e, time.perf_counter() - t0
+
+    solve()
+    (x, info), full = solve()
+    assert info["iterations"] >= 100
+    w = word(lf, G)
+    timer = threading.Timer(0.2 * full, lambda: setattr(w, "value", 1))
+    timer.start()
+    err, took = solve()
+    timer.join()
+    assert isinstance(err, lf.LfmmError) and err.status == lf.LFMM_ERR_TIMEOUT
+    assert took <= 0.7 * full, (took, full)
+    again, _ = solve()
+    assert np.array_equal(again[0], x)
