@@ -57,13 +57,18 @@ typedef enum {
                                          translation table came out non-finite (checked at the
                                          end of every build); the quadrature rules are fixed, so
                                          this marks a medium or order beyond their range */
-    LFMM_ERR_TIMEOUT = -6,            /* a bounded device wait gave up: the tensor-core
-                                         M2L of LFMM_MIXED (16+ columns) waits on its own
-                                         MMAs.  The affected products were computed with
-                                         those M2L contributions zeroed.  A call with host
-                                         vectors reports it itself; with device vectors the
-                                         next lfmm_matvec on the geometry does.  Reported
-                                         once, after which the geometry is usable again */
+    LFMM_ERR_TIMEOUT = -6,            /* a bounded device wait gave up: the tensor-core products
+                                         of the FP64 form (and of the precision form's coarse
+                                         levels) wait on their own copies and MMAs, the
+                                         tensor-core M2L of LFMM_MIXED (16+ columns) on its MMAs.
+                                         The product concerned is not valid (the latter's M2L
+                                         contributions are zeroed, the former's undefined; in a
+                                         batch any of its products).  Calls that synchronise --
+                                         host vectors, lfmm_gmres_solve, lfmm_eval_field, served
+                                         requests -- report it themselves; with device vectors the
+                                         next call that multiplies on the geometry does, before it
+                                         queues anything.  Reported once, after which the
+                                         geometry is usable again */
     LFMM_ERR_HBM_BUDGET = -7
 } lfmm_status;
 

@@ -1084,7 +1084,7 @@ static void ensure_split(lfmm_geometry_s* g, int nrhs, int lm) {   // workspace 
 void split_check_waits(lfmm_geometry_s* g) {
     if (!g->wait_err || *(volatile int*)g->wait_err == 0) return;
     *(volatile int*)g->wait_err = 0;
-    throw TimeoutError{"split M2L: an mbarrier wait gave up; that product's M2L contributions were zeroed"};
+    throw TimeoutError{"split M2L: an mbarrier wait gave up; that product's result is not valid"};
 }
 static SplitArgs split_args(lfmm_geometry_s* g, int col0, int ncols, int lm) {
     const SplitPlan& P = split_plan(g, ncols, lm);

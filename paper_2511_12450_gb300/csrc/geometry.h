@@ -549,7 +549,7 @@ void mixed_destroy(lfmm_geometry_s* g);
 // this geometry's host copy of the status has seen (copied after every launch; current
 // once the launching stream has been synchronised).  Clears the status.
 void mixed_check_waits(lfmm_geometry_s* g);
-// the same for the FP64 form's split M2L
+// the same for the FP64 products (split.cuh), whose kernels set the host's word themselves
 void split_check_waits(lfmm_geometry_s* g);
 void fmm_free(lfmm_geometry_s* g);   // per-nrhs coefficient buffers
 // permutation helpers and the full operator (solver.cu)

@@ -471,6 +471,7 @@ struct SplitOne {
     const SplitArgs* a;
     int n;
     __device__ __forceinline__ int count() const { return n; }
+    __device__ __forceinline__ int njob() const { return 1; }
     __device__ __forceinline__ const SplitArgs* at(int t, int* u) const { *u = t; return a; }
 };
 struct SplitMany {
@@ -478,6 +479,7 @@ struct SplitMany {
     const int* prefix;
     int njobs;
     __device__ __forceinline__ int count() const { return prefix[njobs]; }
+    __device__ __forceinline__ int njob() const { return njobs; }
     __device__ __forceinline__ const SplitArgs* at(int t, int* u) const {
         int lo = 0, hi = njobs - 1;   // the last job whose first unit is <= t
         while (lo < hi) {
@@ -772,7 +774,10 @@ __device__ __forceinline__ void split_units(const JOBS& jobs) {
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (sh.dead && tid == 0) { *(volatile int*)jobs.a->err = 1; __threadfence_system(); }
+    if (sh.dead && tid == 0) {   // any geometry's units may have been left
+        for (int j = 0; j < jobs.njob(); ++j) *(volatile int*)jobs.a[j].err = 1;
+        __threadfence_system();
+    }
     if (warp == SP_MMA_WARP)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tb), "r"(SP_TMEM));
 }

@@ -83,3 +83,24 @@ def test_a_solve_looks_at_every_step(gpu_lib, cols):
     assert took <= 0.7 * full, (took, full)
     again, _ = solve()
     assert np.array_equal(again[0], x)
+
+
+def test_each_geometry_of_a_batch_has_its_own_word(gpu_lib):
+    """A time-out of one geometry's product is not taken for another's, alone or in a batch."""
+    import torch
+
+    lf = gpu_lib
+    geos = [geometry(lf, layered_wide(), leaf) for leaf in (8, 16, 12)]
+    xs = [vector(G, i) for i, G in enumerate(geos)]
+    ref = lf.matvec_batch(geos, xs)
+    assert len({int(lf.geometry_query(G, "wait_word", np.int64)[0]) for G in geos}) == 3
+    for late in range(3):
+        word(lf, geos[late]).value = 1
+        for i in range(3):
+            if i != late:
+                assert torch.equal(lf.matvec(geos[i], xs[i]), ref[i])
+        with pytest.raises(lf.LfmmError) as err:
+            lf.matvec_batch(geos, xs)
+        assert err.value.status == lf.LFMM_ERR_TIMEOUT
+        for y, r in zip(lf.matvec_batch(geos, xs), ref):
+            assert torch.equal(y, r)
