@@ -625,7 +625,7 @@ __device__ __forceinline__ void split_units(const JOBS& jobs) {
         // ---------------------------------------------------------------- MMAs
         // The issuing lane is elected inside the warp's uniform flow (sp_chunk); from a lane-index
         // branch with descriptors built in the loop an MMA took 180 cycles to issue whatever its N.
-        int chunk = 0, sgc = 0, k = 0;
+        int chunk = 0, sgc = 0, k = 0, told = 0;   // told: segments whose accfull is committed
         bool ok = true;
         const uint32_t sm0 = sp_saddr(sp_sm);
         for (; ok; ++k) {
@@ -660,14 +660,18 @@ __device__ __forceinline__ void split_units(const JOBS& jobs) {
                         if (k0 + G.KC >= len) sp_commit(&sh.accfull[sgc & 1]);
                     }
                     __syncwarp();
+                    if (k0 + G.KC >= len) ++told;
                 }
             }
             if (lane == 0) sp_arrive(&sh.slotfree[k & (SP_RING - 1)]);
         }
-        // the last MMAs are done before the TMEM is freed (bounded, also after a wait gave up)
+        // the last MMAs are done before the TMEM is freed, and after a wait gave up, when the epilogue
+        // may not take them any more, their arrivals have come before the CTA's shared memory goes
+        // (all bounded)
         if (chunk > 0 && lane == 0) {
             sp_wait(sp_saddr(&sh.empty[(chunk - 1) & 1]), ((chunk - 1) >> 1) & 1);
             if (chunk > 1) sp_wait(sp_saddr(&sh.empty[chunk & 1]), ((chunk - 2) >> 1) & 1);
+            for (int i = ok ? told : max(0, told - 2); i < told; ++i) sp_wait(sp_saddr(&sh.accfull[i & 1]), (i >> 1) & 1);
         }
         __syncwarp();
     } else if (warp == SP_MMA_WARP + 1) {
