@@ -198,6 +198,50 @@ static void build_m2l_work(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, c
     make_m2l_items(g, M2L_ITEM_WORK, 1);
 }
 
+// Host-mapped words that kernels set when a bounded wait gives up, one per geometry.  Pinning and
+// unpinning host memory blocks the calls of every thread, which a served request and a field
+// evaluation, each with a geometry of its own, would otherwise pay twice; so the words of up to 1,024
+// live geometries come from one page, pinned on first use and kept.
+#define WAIT_WORDS 1024
+struct WaitWords {
+    std::mutex mu;
+    int* page = nullptr;
+    std::vector<int> unused;
+};
+static WaitWords& wait_words() {
+    static WaitWords* w = new WaitWords();   // (never destroyed: geometries may be released at exit)
+    return *w;
+}
+static int* pin_words(size_t count) {
+    int* p = nullptr;
+    cuda_check(cudaHostAlloc((void**)&p, sizeof(int) * count, cudaHostAllocMapped | cudaHostAllocPortable), "wait status");
+    return p;
+}
+static int* take_wait_word() {
+    WaitWords& W = wait_words();
+    std::lock_guard<std::mutex> lock(W.mu);
+    if (!W.page) {
+        W.unused.reserve(WAIT_WORDS);   // returning a word never allocates
+        W.page = pin_words(WAIT_WORDS);
+        for (int i = WAIT_WORDS - 1; i >= 0; --i) W.unused.push_back(i);
+    }
+    int* p = nullptr;
+    if (W.unused.empty()) {
+        p = pin_words(1);
+    } else {
+        p = W.page + W.unused.back();
+        W.unused.pop_back();
+    }
+    *p = 0;
+    return p;
+}
+static void give_wait_word(int* p) {
+    WaitWords& W = wait_words();
+    std::lock_guard<std::mutex> lock(W.mu);
+    if (p >= W.page && p < W.page + WAIT_WORDS) W.unused.push_back((int)(p - W.page));
+    else cudaFreeHost(p);
+}
+
 // The split M2L's matrices, pairs and destinations (split.cuh).  Matrices, and with them
 // units and workspace rows, in level order, so that the levels above the precision form's
 // first FP32 level are a prefix.
@@ -507,8 +551,7 @@ static void build_split(lfmm_geometry_s* g, const std::vector<int>& vr_ptr, cons
     split_plan(g, 1, nlev);
     g->sp_rows = rows;
     g->d_sp_ws1 = dalloc<unsigned char>(g, split_col_bytes(g, nlev));
-    cuda_check(cudaHostAlloc((void**)&g->wait_err, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable), "wait status");
-    *g->wait_err = 0;
+    g->wait_err = take_wait_word();
 }
 
 // The reaction M2L tables: same-layer components from 4p + 1 moments, the others in runs of
@@ -1048,7 +1091,7 @@ void fmm_free(lfmm_geometry_s* g) {
     dev_release(g->d_sp_ws);
     g->d_sp_ws = nullptr;
     g->sp_ws_bytes = 0;
-    if (g->wait_err) cudaFreeHost(g->wait_err);
+    if (g->wait_err) give_wait_word(g->wait_err);
     g->wait_err = nullptr;
     dev_release(g->d_M); dev_release(g->d_L);
     dev_release(g->d_Mp); dev_release(g->d_Lp);

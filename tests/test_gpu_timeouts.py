@@ -104,3 +104,19 @@ def test_each_geometry_of_a_batch_has_its_own_word(gpu_lib):
         assert err.value.status == lf.LFMM_ERR_TIMEOUT
         for y, r in zip(lf.matvec_batch(geos, xs), ref):
             assert torch.equal(y, r)
+
+
+def test_words_come_from_one_page(gpu_lib):
+    """Builds and releases pin no memory of their own: live geometries have words of one page, and a
+    released word comes back cleared."""
+    lf = gpu_lib
+    geos = [geometry(lf, layered_wide(), 16) for _ in range(4)]
+    at = [int(lf.geometry_query(G, "wait_word", np.int64)[0]) for G in geos]
+    assert len(set(at)) == 4 and max(at) - min(at) < 4096
+    for _ in range(3):
+        word(lf, geos[-1]).value = 1
+        last = int(lf.geometry_query(geos[-1], "wait_word", np.int64)[0])
+        geos.pop().destroy()
+        geos.append(geometry(lf, layered_wide(), 16))
+        assert int(lf.geometry_query(geos[-1], "wait_word", np.int64)[0]) == last
+        assert word(lf, geos[-1]).value == 0
