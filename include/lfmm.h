@@ -355,7 +355,14 @@ lfmm_status lfmm_polygon_elements(int32_t n_poly, const int32_t *counts, const d
  * same alone and in the mix.
  *   footprint estimate (bytes): 16 n (max_iter + 1) for the Krylov basis, plus
  *   about 16 n (120 (1 + leaf/64) + 24) for near field, preconditioner and work
- *   vectors, 4 n (2p + 1) for expansions, and 256 MiB for tables and scratch.
+ *   vectors, 4 n (2p + 1) for expansions, and 256 MiB for tables and scratch (a
+ *   request for which these are above the budget is refused), or where they are
+ *   more the reaction tables, their digits and the products' workspace, from the
+ *   number of layers, n, p and the width of the region times the largest
+ *   wavenumber.  That part can be several times what the geometry turns out to
+ *   need; once it is built, the request is counted with what it holds (queries
+ *   "device_bytes"), at least the first part.  A request whose estimate is above
+ *   the budget although the first part is not runs by itself.
  */
 typedef struct lfmm_server_s *lfmm_server;
 typedef struct {
@@ -392,8 +399,8 @@ typedef struct {
 
 /* Errors: LFMM_ERR_INVALID_ARG; LFMM_ERR_CUDA if no device is current. */
 lfmm_status lfmm_server_create(const lfmm_server_params *prm, lfmm_server *out);
-/* Queue a request; *ticket identifies it.  LFMM_ERR_HBM_BUDGET if its footprint
- * estimate alone exceeds the budget (it could never be admitted). */
+/* Queue a request; *ticket identifies it.  LFMM_ERR_HBM_BUDGET if the first part of its
+ * footprint estimate alone exceeds the budget. */
 lfmm_status lfmm_server_submit(lfmm_server s, const lfmm_request *req, int64_t *ticket);
 /* Block until the request is done; x (host, n complex) receives the solution Phi,
  * info and times (either may be NULL) its GMRES record and timings.  Returns the
@@ -434,6 +441,8 @@ lfmm_status lfmm_server_destroy(lfmm_server s);
  * "launch_count" (double[1]: kernels launched so far by this geometry's
  * matvec path -- gather, P2M, M2M, M2L, L2L, L2P, near field, scatter --
  * counted on the host as they are enqueued),
+ * "device_bytes" (double[3]: device memory that the geometry holds now; of it the FP64 products'
+ * matrices as digits, and their workspace of one column),
  * "wait_word" (int64[1]: host address of the int32 that a kernel sets when one of the FP64
  * products' bounded waits gives up, 0 without a far field; a test that sets it stands in for
  * the kernel -- see LFMM_ERR_TIMEOUT),

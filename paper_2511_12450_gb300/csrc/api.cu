@@ -816,6 +816,11 @@ lfmm_status lfmm_geometry_query(lfmm_geometry g, const char* name, void* host_ou
             dtmp = {(double)g->n_launches};
             src = dtmp.data();
             bytes = (int64_t)sizeof(double);
+        } else if (nm == "device_bytes") {
+            dtmp.assign(3, 0.0);
+            geometry_bytes(g, dtmp.data());
+            src = dtmp.data();
+            bytes = (int64_t)(dtmp.size() * sizeof(double));
         } else if (nm == "wait_word") {
             word = (int64_t)(uintptr_t)g->wait_err;
             src = &word;

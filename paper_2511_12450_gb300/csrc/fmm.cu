@@ -1339,6 +1339,13 @@ void fmm_prepare(lfmm_geometry_s* g, int nrhs, bool mixed) {
     if (lm <= g->tree.D) mixed_setup(g, nrhs);
     if (lm > l0) ensure_split(g, nrhs, lm);
 }
+void geometry_bytes(const lfmm_geometry_s* g, double out[3]) {
+    const size_t cols = 2 * sizeof(cd) * ((size_t)g->n * g->nrhs_cap + (size_t)(g->ncoef + g->nslotcoef) * g->coef_cols);
+    out[0] = (double)(g->alloc_bytes + cols + 2 * sizeof(cd) * g->hostbuf_cap + g->sp_ws_bytes +
+                      sizeof(float2) * (size_t)g->near_x32_cap + mixed_bytes(g));
+    out[1] = (double)g->sp_dig_bytes;
+    out[2] = g->d_sp_ws1 ? (double)split_col_bytes(g, g->tree.D + 1) : 0.0;
+}
 void fmm_check_waits(lfmm_geometry_s* g) {
     split_check_waits(g);
     mixed_check_waits(g);

@@ -412,6 +412,7 @@ struct lfmm_geometry_s {
     double table_cmacs[2] = {0.0, 0.0};        // complex multiply-adds of the moment tables: cross-layer, same-layer
     int64_t m2lr_len = 0, pc_w_len = 0;         // entries of the reaction tables and of the preconditioner's W
     std::vector<void*> allocs;        // everything cudaMalloc'ed for this geometry
+    size_t alloc_bytes = 0;           // in all
     // held by every call that applies the operator or the preconditioner to vectors
     // (matvec, the allocation-free matvec, precondition, solve, right-hand side, field):
     // calls on one geometry run one after another even if a caller does not serialise them
@@ -469,6 +470,7 @@ T* dalloc(lfmm_geometry_s* g, size_t count) {
     // running while this one is built (the build synchronises its own stream at the end)
     cuda_check(cudaMallocAsync(&p, count * sizeof(T), cudaStreamPerThread), "cudaMallocAsync");
     g->allocs.push_back(p);
+    g->alloc_bytes += count * sizeof(T);
     return (T*)p;
 }
 template <class T>
@@ -489,6 +491,9 @@ void fmm_build(lfmm_geometry_s* g);
 // work buffers, tables and plans of a product of nrhs columns: what can run out of memory, before
 // anything of the product is queued
 void fmm_prepare(lfmm_geometry_s* g, int nrhs, bool mixed);
+// device memory the geometry holds now: in all, the products' matrices as digits, the products'
+// workspace of one column (bytes)
+void geometry_bytes(const lfmm_geometry_s* g, double out[3]);
 // throws TimeoutError, once, if a bounded wait of a product that has run by now gave up
 void fmm_check_waits(lfmm_geometry_s* g);
 void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, cudaStream_t s, bool mixed = false,
@@ -544,6 +549,7 @@ void mixed_l_add(lfmm_geometry_s* g, int level, int nrhs, cudaStream_t s);    //
 void mixed_l2l(lfmm_geometry_s* g, int child_level, int nrhs, cudaStream_t s);
 void mixed_l2p(lfmm_geometry_s* g, cd* y_sorted, int nrhs, cudaStream_t s);
 int mixed_level(lfmm_geometry_s* g);   // first level whose M2L runs in FP32
+size_t mixed_bytes(const lfmm_geometry_s* g);
 void mixed_destroy(lfmm_geometry_s* g);
 // Throws TimeoutError, once, if a bounded wait of the tensor-core M2L gave up in work
 // this geometry's host copy of the status has seen (copied after every launch; current

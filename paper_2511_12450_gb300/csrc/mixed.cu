@@ -727,6 +727,12 @@ static void mixed_free_buffers(MixedState* ms, bool in_flight) {
     ms->M = ms->L = ms->Mp = ms->Lp = ms->part = nullptr;
     ms->cols = 0;
 }
+size_t mixed_bytes(const lfmm_geometry_s* g) {
+    const MixedState* ms = g->mixed;
+    if (!ms) return 0;
+    const size_t col = 2 * (size_t)(g->ncoef + g->nslotcoef) + (size_t)std::max(g->n_m2l_parts, 1) * 3 * XT_W;
+    return ms->bytes + sizeof(cf) * col * ms->cols;
+}
 void mixed_destroy(lfmm_geometry_s* g) {
     if (!g->mixed) return;
     MixedState* ms = g->mixed;

@@ -20,6 +20,7 @@
 // (solver.cu), so a result is the same alone and in the mix.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
@@ -50,7 +51,8 @@ struct Request {
     int32_t flags = 0;
     double angle = 0.0, tol = 1e-8;
     int32_t precision = 0, p = 20, leaf = 64, max_iter = 1000, precond = 1;
-    int64_t footprint = 0;
+    int64_t footprint = 0, least = 0;   // the estimate that admits it; the part that must fit the budget
+    int64_t reserved = 0;               // of the budget, while it runs
     // results
     std::vector<double> x;   // 2n (re, im)
     lfmm_gmres_info info{};
@@ -88,16 +90,37 @@ struct lfmm_server_s {
 
 namespace {
 
-// Device bytes one request holds while it runs: the Krylov basis (max_iter + 1
-// vectors), the stored near field and preconditioner (~62 and ~50 complex entries
-// per point at leaf size 64), the leaf expansion basis (p + 2 complex values per
-// point), multipoles/locals and work vectors, and the reaction tables and set-up
-// scratch (a fixed allowance).
-int64_t footprint_estimate(int64_t n, int p, int leaf, int max_iter) {
+// Device bytes one request holds while it runs, from its sizes: the Krylov basis (max_iter + 1
+// vectors), the stored near field and preconditioner (~62 and ~50 complex entries per point at leaf
+// size 64), the leaf expansion basis (p + 2 complex values per point), multipoles/locals and work
+// vectors, and 256 MiB of tables and set-up scratch.  A request for which this alone is above the
+// budget is refused.
+int64_t least_footprint(int64_t n, int p, int leaf, int max_iter) {
     const double per_point = 16.0 * (max_iter + 1) + 16.0 * (1.0 + leaf / 64.0) * 120.0 + 16.0 * 24.0 +
                              16.0 * (p + 2.0);
     const double expansions = 16.0 * (2.0 * p + 1.0) * (double)n / 4.0;
     return (int64_t)(per_point * (double)n + expansions) + ((int64_t)256 << 20);
+}
+// The same with the reaction tables, their digits for the products (5.5 times the tables) and the
+// products' workspace, where those take more than the 256 MiB.  Their number and orders follow the
+// layers and the region's width in wavelengths more than n: 60 geometries of 256 to 262,144 points
+// in 2 to 6 layers had at most 0.62 n and 1,460 tables per interface, 5.5 x 16 (2p + 1)^2 + 1,400 kmax
+// width bytes of digits per table and 1.2 KB per point and 20 KB per table of workspace.  (6,656
+// points in four layers, 26 wide, kmax 8.3: 1.13 GB held, 300 MB by the estimate above alone.)
+int64_t footprint_estimate(int64_t n, int p, int leaf, int max_iter, int n_layers, double kmax, double width, int precision) {
+    const double tables = std::min(0.7 * (double)n, 1500.0 * (n_layers - 1));
+    const double digits = tables * (5.5 * 16.0 * (2.0 * p + 1.0) * (2.0 * p + 1.0) + 1400.0 * kmax * width);
+    double more = 1.2 * digits + 1200.0 * (double)n + 20e3 * tables;
+    if (precision == 1) more += 0.15 * digits + 1200.0 * (double)n;   // the FP32 tables and near field beside them
+    return least_footprint(n, p, leaf, max_iter) + std::max<int64_t>((int64_t)more - ((int64_t)256 << 20), 0);
+}
+// What a request that has been set up holds until it is done: what its geometry holds now, its
+// products' expansions and the solve's vectors, the precision form's tables.
+int64_t held_bytes(const Request& r) {
+    double b[3];
+    lfmm::geometry_bytes(r.geo, b);
+    const double cols = 32.0 * (double)(r.geo->ncoef + r.geo->nslotcoef) + 16.0 * (double)r.n * (r.max_iter + 12.0);
+    return (int64_t)(b[0] * (r.precision == 1 ? 1.2 : 1.0) + cols);
 }
 
 // set-up of a request on its worker's stream: medium, geometry, right-hand side, and the
@@ -182,15 +205,18 @@ void worker_main(lfmm_server_s* S) {
         std::shared_ptr<Request> r;
         {
             std::unique_lock<std::mutex> lk(S->mu);
-            // admission: the head of the queue, once its footprint fits beside the running ones
+            // admission: the head of the queue, once its footprint fits beside the running ones, or
+            // by itself
             S->cv_work.wait(lk, [&] {
                 return (S->stop && S->queue.empty()) ||
-                       (!S->queue.empty() && S->in_use + S->queue.front()->footprint <= S->budget);
+                       (!S->queue.empty() &&
+                        (S->running == 0 || S->in_use + S->queue.front()->footprint <= S->budget));
             });
             if (S->queue.empty()) break;   // stopping, nothing left
             r = S->queue.front();
             S->queue.pop_front();
-            S->in_use += r->footprint;
+            r->reserved = r->footprint;
+            S->in_use += r->reserved;
             S->peak_in_use = std::max(S->peak_in_use, S->in_use);
             S->running += 1;
             S->peak_running = std::max(S->peak_running, S->running);
@@ -198,8 +224,13 @@ void worker_main(lfmm_server_s* S) {
         }
         try {
             if (setup_request(*r, s)) {
-                // hand the solve to the engine and wait for it
+                // what it holds is known now; then hand the solve to the engine and wait for it
+                const int64_t held = std::max(r->least, held_bytes(*r));
                 std::unique_lock<std::mutex> lk(S->mu);
+                S->in_use += held - r->reserved;
+                r->reserved = held;
+                S->peak_in_use = std::max(S->peak_in_use, S->in_use);
+                S->cv_work.notify_all();
                 S->pending.push_back(r);
                 S->cv_engine.notify_all();
                 S->cv_solved.wait(lk, [&] { return r->solved; });
@@ -213,7 +244,7 @@ void worker_main(lfmm_server_s* S) {
             std::lock_guard<std::mutex> lk(S->mu);
             r->t_done = now_s();
             r->done = true;
-            S->in_use -= r->footprint;
+            S->in_use -= r->reserved;
             S->running -= 1;
         }
         S->cv_done.notify_all();
@@ -336,11 +367,19 @@ static lfmm_status server_submit(lfmm_server S, const lfmm_request* q, int64_t* 
     r->leaf = q->leaf_size > 0 ? q->leaf_size : 64;
     r->max_iter = q->max_iter;
     r->precond = q->precond;
-    r->footprint = footprint_estimate(r->n, r->p, r->leaf, r->max_iter);
+    double kmax = 0.0, lo[2] = {r->pts[0], r->pts[1]}, hi[2] = {lo[0], lo[1]};
+    for (int32_t l = 0; l < r->n_layers; ++l) kmax = std::max(kmax, r->k[2 * l]);
+    for (int64_t i = 0; i < 2 * r->n; ++i) {
+        lo[i & 1] = std::min(lo[i & 1], r->pts[i]);
+        hi[i & 1] = std::max(hi[i & 1], r->pts[i]);
+    }
+    r->least = least_footprint(r->n, r->p, r->leaf, r->max_iter);
+    r->footprint = footprint_estimate(r->n, r->p, r->leaf, r->max_iter, r->n_layers, kmax,
+                                      std::max(hi[0] - lo[0], hi[1] - lo[1]), r->precision);
     {
         std::lock_guard<std::mutex> lk(S->mu);
         if (S->stop) return LFMM_ERR_INVALID_ARG;
-        if (r->footprint > S->budget) return LFMM_ERR_HBM_BUDGET;   // would never be admitted
+        if (r->least > S->budget) return LFMM_ERR_HBM_BUDGET;
         r->ticket = S->next_ticket++;
         r->t_submit = now_s();
         S->queue.push_back(r);
