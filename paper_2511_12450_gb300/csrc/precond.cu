@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "geometry.h"
+#include "precond_layout.h"
 
 namespace lfmm {
 
@@ -31,16 +32,17 @@ namespace lfmm {
 // cluster barrier hands the block over, and every CTA updates its own columns.  The E columns
 // need no exchange backwards.  8,199 points: 5.6 ms; one CTA a leaf with column-by-column
 // elimination in global memory took 19.3 ms.
-#define PC_NB 16
 struct PcLeaf {
     int leaf, q, s;          // leaf, points of the neighbourhood, own points
-    int64_t aoff;            // (q + s) q scratch values
+    int64_t aoff;            // (q + s) q scratch values, then the CTAs' panels if those are global
 };
 __device__ __forceinline__ void pc_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ double pc_abs2(cd v) { return v.x * v.x + v.y * v.y; }
 
+// GLOBAL: the panel of a CTA in global memory, after its leaf's [A | E] (pc_panel_columns)
+template <bool GLOBAL>
 __global__ void __launch_bounds__(256) k_pc_setup(MediumDev m, const int* __restrict__ pc_ptr,
                                                   const int* __restrict__ pc_idx, const int* __restrict__ own_pos,
                                                   const PcLeaf* __restrict__ leaves, int cs, int nb,
@@ -61,7 +63,7 @@ __global__ void __launch_bounds__(256) k_pc_setup(MediumDev m, const int* __rest
     const double k = m.k[layer_of_leaf[B]];
     cd* A = Ascr + lf.aoff;
     int* piv = pivscr + jb;
-    cd* P = pc_sm;
+    cd* P = GLOBAL ? A + (int64_t)q * (q + s) + (int64_t)rank * nb * q : pc_sm;
     const int nA = (q + nb - 1) / nb, nR = (s + nb - 1) / nb;   // column blocks of A and of E
     // A[a][b] = P[b][a]: P[i][j] = w_j G(c_j, c_i) (i != j), I^s_i (i == j); own columns only
     const bool cf = nx != nullptr;
@@ -270,7 +272,7 @@ void precond_build(lfmm_geometry_s* g) {
     std::vector<int64_t> woff(nleaf);
     std::vector<PcLeaf> leaves;
     double flops = 0.0, flops_max = 0.0;
-    int64_t at = 0, wt = 0;
+    int64_t wt = 0;
     for (int li = 0; li < nleaf; ++li) {
         const int B = g->leaf0 + li;
         int q = 0;
@@ -284,8 +286,7 @@ void precond_build(lfmm_geometry_s* g) {
         own_cnt[li] = t.box_end[B] - t.box_begin[B];
         own_first[li] = t.box_begin[B];
         lay[li] = t.box_layer[B];
-        leaves.push_back(PcLeaf{li, q, own_cnt[li], at});
-        at += (int64_t)q * (q + own_cnt[li]);
+        leaves.push_back(PcLeaf{li, q, own_cnt[li], 0});
         const double fl = 8.0 / 3.0 * q * (double)q * q + 8.0 * q * (double)q * own_cnt[li];
         flops += fl;
         flops_max = std::max(flops_max, fl);
@@ -311,10 +312,17 @@ void precond_build(lfmm_geometry_s* g) {
     std::stable_sort(leaves.begin(), leaves.end(), [](const PcLeaf& a, const PcLeaf& b) { return a.q > b.q; });
     int cs = 1;
     while (cs < 8 && flops_max / cs > flops / 152.0) cs *= 2;
-    // columns per block: the panel (nb q values) stays within 200 KB
-    const int nb = std::max(1, std::min<int>(PC_NB, (int)(200 * 1024 / (sizeof(cd) * std::max(qmax, 1)))));
-    const size_t smem_setup = sizeof(cd) * (size_t)nb * qmax;
-    raise_smem_limit((const void*)k_pc_setup, smem_setup, "pc set-up smem");
+    const int shared_nb = pc_panel_columns(qmax);
+    const bool global = shared_nb == 0;
+    const int nb = global ? PC_NB : shared_nb;
+    const size_t smem_setup = global ? 0 : sizeof(cd) * (size_t)nb * qmax;
+    auto kern = global ? k_pc_setup<true> : k_pc_setup<false>;
+    raise_smem_limit((const void*)kern, smem_setup, "pc set-up smem");
+    int64_t at = 0;
+    for (PcLeaf& f : leaves) {
+        f.aoff = at;
+        at += (int64_t)f.q * (f.q + f.s) + (global ? (int64_t)cs * nb * f.q : 0);
+    }
     PcLeaf* d_leaves = dupload(g, leaves);
     g->d_pc_W = dalloc<cd>(g, (size_t)wt);
     g->pc_w_len = wt;
@@ -335,7 +343,7 @@ void precond_build(lfmm_geometry_s* g) {
     att.val.clusterDim.y = att.val.clusterDim.z = 1;
     cfg.attrs = &att;
     cfg.numAttrs = 1;
-    cudaError_t e1 = cudaLaunchKernelEx(&cfg, k_pc_setup, g->m, (const int*)g->d_pc_ptr, (const int*)g->d_pc_idx,
+    cudaError_t e1 = cudaLaunchKernelEx(&cfg, kern, g->m, (const int*)g->d_pc_ptr, (const int*)g->d_pc_idx,
                                         (const int*)d_own_pos, (const PcLeaf*)d_leaves, cs, nb,
                                         (const int64_t*)g->d_pc_woff, (const int*)d_lay, (const double*)g->d_x,
                                         (const double*)g->d_y, (const double*)g->d_w, (const double*)g->d_nx,
