@@ -1362,12 +1362,17 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
         if (lm <= D) {
             mixed_p2m(g, x_sorted, nrhs, s);
         } else {
-            const P2MArgs a = p2m_args(g, x_sorted, nrhs);
             const int nb = g->n_leaf_groups + g->n_slot_groups;
-            if (nrhs > 1) k_p2m<4><<<dim3(nb, (nrhs + 3) / 4), 128, 0, s>>>(a);
-            else k_p2m<1><<<nb, 128, 0, s>>>(a);
-            cuda_check(cudaGetLastError(), "k_p2m");
-            ++g->n_launches;
+            for (int c0 = 0; c0 < nrhs; c0 += 4 * MAX_GRID_Y) {
+                const int nc = std::min(nrhs - c0, 4 * MAX_GRID_Y);
+                P2MArgs a = p2m_args(g, x_sorted + (int64_t)c0 * g->n, nc);
+                a.M += (int64_t)c0 * g->ncoef;
+                a.Mp += (int64_t)c0 * g->nslotcoef;
+                if (nrhs > 1) k_p2m<4><<<dim3(nb, (nc + 3) / 4), 128, 0, s>>>(a);
+                else k_p2m<1><<<nb, 128, 0, s>>>(a);
+                cuda_check(cudaGetLastError(), "k_p2m");
+                ++g->n_launches;
+            }
         }
         prof_end(g, ST_P2M, s);
     }
@@ -1424,14 +1429,19 @@ void fmm_apply(lfmm_geometry_s* g, const cd* x_sorted, cd* y_sorted, int nrhs, c
         if (lm <= D) {
             mixed_l2p(g, y_sorted, nrhs, s);
         } else {
-            const L2PArgs a = l2p_args(g, y_sorted, nrhs);
             const int cb = l2p_cols(g, nrhs);
             const size_t smem = l2p_smem(cb, g->group_max_ent, t.p_level[D]);
             raise_smem_limit(cb > 1 ? (const void*)k_l2p<4> : (const void*)k_l2p<1>, smem, "l2p smem");
-            if (cb > 1) k_l2p<4><<<dim3(g->n_leaf_groups, (nrhs + 3) / 4), 128, smem, s>>>(a);
-            else k_l2p<1><<<dim3(g->n_leaf_groups, nrhs), 128, smem, s>>>(a);
-            cuda_check(cudaGetLastError(), "k_l2p");
-            ++g->n_launches;
+            for (int c0 = 0; c0 < nrhs; c0 += cb * MAX_GRID_Y) {
+                const int nc = std::min(nrhs - c0, cb * MAX_GRID_Y);
+                L2PArgs a = l2p_args(g, y_sorted + (int64_t)c0 * g->n, nc);
+                a.L += (int64_t)c0 * g->ncoef;
+                a.Lp += (int64_t)c0 * g->nslotcoef;
+                if (cb > 1) k_l2p<4><<<dim3(g->n_leaf_groups, (nc + 3) / 4), 128, smem, s>>>(a);
+                else k_l2p<1><<<dim3(g->n_leaf_groups, nc), 128, smem, s>>>(a);
+                cuda_check(cudaGetLastError(), "k_l2p");
+                ++g->n_launches;
+            }
         }
         prof_end(g, ST_L2P, s);
     }

@@ -99,6 +99,8 @@ struct M2LItem {
     int part;         // -1: write L directly; else partial-sum slot (always XT_W lanes)
     int w;            // output lanes per row: XT_W (chunks of XT_W coefficients) or 2p+1 (all of them)
 };
+// column groups of one launch: CUDA's limit of a grid's y extent; wider blocks take several launches
+constexpr int MAX_GRID_Y = 65535;
 // CTAs a block right-hand side's columns are split over in the translation
 // kernels (groups of four columns); one column keeps one CTA
 inline int col_groups(int nrhs) { return nrhs <= 2 ? 1 : (nrhs + 3) / 4; }

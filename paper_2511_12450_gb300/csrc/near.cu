@@ -313,17 +313,25 @@ static void launch_near(lfmm_geometry_s* g, const NearRowPart& p64, const cd* v6
                         const float2* v32, const cd* diag, const cd* x, const float2* x32, cd* y, int nrhs,
                         cudaStream_t s) {
     const int T = near_threads(g);
-    const dim3 grid(g->nleaf, (nrhs + CB - 1) / CB, (g->max_leaf + NEAR_ROWS - 1) / NEAR_ROWS);
-    if (T == 32)
+    if (T == 32) {
         k_near_leaf_w<MIX, CB><<<(g->nleaf + 3) / 4, 128, 0, s>>>(g->nleaf, g->leaf0, g->d_box_begin, g->d_box_end, p64, v64,
                                                                  p32, v32, diag, x, x32, y, g->n, nrhs);
-    else if (T == 128)
-        k_near_leaf<MIX, 128, CB><<<grid, 128, 0, s>>>(g->leaf0, g->d_box_begin, g->d_box_end, p64, v64, p32, v32, diag, x,
-                                                      x32, y, g->n, nrhs);
-    else
-        k_near_leaf<MIX, 256, CB><<<grid, 256, 0, s>>>(g->leaf0, g->d_box_begin, g->d_box_end, p64, v64, p32, v32, diag, x,
-                                                      x32, y, g->n, nrhs);
-    cuda_check(cudaGetLastError(), "k_near_leaf");
+        cuda_check(cudaGetLastError(), "k_near_leaf");
+        return;
+    }
+    for (int c0 = 0; c0 < nrhs; c0 += MAX_GRID_Y * CB) {
+        const int nc = std::min(nrhs - c0, MAX_GRID_Y * CB);
+        const int64_t at = (int64_t)c0 * g->n;
+        const float2* xs = MIX ? x32 + at : nullptr;
+        const dim3 grid(g->nleaf, (nc + CB - 1) / CB, (g->max_leaf + NEAR_ROWS - 1) / NEAR_ROWS);
+        if (T == 128)
+            k_near_leaf<MIX, 128, CB><<<grid, 128, 0, s>>>(g->leaf0, g->d_box_begin, g->d_box_end, p64, v64, p32, v32, diag,
+                                                          x + at, xs, y + at, g->n, nc);
+        else
+            k_near_leaf<MIX, 256, CB><<<grid, 256, 0, s>>>(g->leaf0, g->d_box_begin, g->d_box_end, p64, v64, p32, v32, diag,
+                                                          x + at, xs, y + at, g->n, nc);
+        cuda_check(cudaGetLastError(), "k_near_leaf");
+    }
 }
 // x rounded to complex64 (the precision form's FP32 near-field products)
 __global__ void k_round_x32(const cd* __restrict__ x, float2* __restrict__ x32, int64_t tot) {

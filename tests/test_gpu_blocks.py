@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from oracle import nystrom as onys
-from workloads import config_c2, layered_small
+from workloads import Medium, circle, config_c2, layered_small
 
 pytestmark = pytest.mark.gpu
 
@@ -129,3 +129,28 @@ def test_precision_form_holds_its_own_levels_only(gpu_lib):
     ref = lf.matvec(G, five, mixed=True)
     lf.matvec(S, five)
     assert torch.equal(lf.matvec(S, five, mixed=True), ref)
+
+
+@pytest.mark.parametrize("far", [False, True])
+def test_blocks_wider_than_a_grid(gpu_lib, far):
+    """More columns than a launch's grid holds: 65,535 groups of four in the near field, of one in the
+    evaluation of locals of order 41 and more."""
+    import torch
+
+    lf = gpu_lib
+    med = Medium(interfaces=[], k=[3.0], eta=[1.0])
+    bodies = [circle(-1.0, 0.2, 0.3, 12), circle(1.1, -0.1, 0.3, 12)]
+    pts, w, _, _ = onys.elements(bodies)
+    G = lf.geometry_build(lf.medium_create(med.interfaces, med.k, med.eta), pts, w, p=41 if far else 20,
+                          leaf_size=4 if far else 64)
+    tp = lf.geometry_query(G, "tree_params", np.float64)
+    assert (tp[4] <= tp[3]) == far
+    cols = 66000 if far else 262145
+    X = columns(G.n, cols, 9)
+    K = torch.from_numpy(onys.dense_matrix(med, pts, w, reaction=False)).cuda()
+    ref = X @ K.T
+    Y = lf.matvec(G, X)
+    # truncation far below (0.547^42), rounding of 24 terms with a margin
+    assert float((Y - ref).abs().max()) <= 1e-9 * float(ref.abs().max())
+    for c in (0, cols - 1):
+        assert torch.equal(Y[c], lf.matvec(G, X[c].contiguous()))
