@@ -42,7 +42,7 @@ BF16_FALLBACK_TFLOPS = 1900.0
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # DRAM traffic per launch from the committed ncu captures (profiles/); null once the
 # kernel changes after the capture
-NCU_TRAFFIC_BYTES = {"k_split": 427517440.0 + 29704704.0, "k_near_leaf": 67043072.0 + 274688.0,
+NCU_TRAFFIC_BYTES = {"k_split": 428668672.0 + 30697216.0, "k_near_leaf": 67043072.0 + 274688.0,
                      "k_near_leaf (precision form)": 40003072.0}
 
 

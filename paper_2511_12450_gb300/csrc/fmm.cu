@@ -147,7 +147,6 @@ static void make_m2l_items(lfmm_geometry_s* g, int item_work, int wide) {
     g->d_m2l_reds = dupload(g, reds);
     g->m2l_item_work = item_work;
     g->m2l_wide = wide;
-    // the partial-sum buffer is sized for the parts: make the next matvec size it again
 }
 
 // M2L entry descriptors and work items.  Every list entry of a target box
@@ -1023,7 +1022,6 @@ void fmm_build(lfmm_geometry_s* g) {
             g->ftab_turn[i] = (q & 3) | (mir << 2);
         }
         g->ftab_off_host = toff;
-        g->ftab_p = tp;
         g->d_m2lf = dalloc<cd>(g, (size_t)std::max<int64_t>(tot, 1));
         g->m2lf_len = tot;
         g->d_m2lf_off = dupload(g, toff);

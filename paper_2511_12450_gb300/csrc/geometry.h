@@ -384,8 +384,7 @@ struct lfmm_geometry_s {
     std::vector<int> rkey_lay_s, rkey_lay_t;       // layers of the source / target boxes of each key
     std::vector<char> rkey_fine;                   // its split product takes fine segments (split_layout.h)
     std::vector<int> ftab_lay, ftab_lev;           // layer and level of each free-space M2L table
-    std::vector<int> ftab_p;                       // order and offset of each
-    std::vector<int64_t> ftab_off_host;
+    std::vector<int64_t> ftab_off_host;            // offset of each
     std::vector<int> ftab_canon, ftab_turn;        // per listed offset: its first-octant table; quarter turns | mirrored << 2
     std::vector<int> slot_box_host;
     std::vector<int64_t> box_coef_off_host;

@@ -1,4 +1,4 @@
-// split.cuh -- FP64 translations as exact integer products on the tensor cores.
+// split.cuh -- FP64 translations as integer products on the tensor cores.
 //
 // A translation (free-space or reaction M2L) is a dense complex product y = A v of one
 // of few matrices A with many source vectors v: a reaction table serves about 13 box
@@ -32,7 +32,8 @@
 // gave 9.9e-8.)  The sums of digits are exact, so a product does not depend on how pairs
 // are grouped into CTAs, on the columns beside it or on the launch it is part of.
 //
-// k_split_digits writes every matrix's digits once per geometry (5 times its FP64 size),
+// k_split_digits writes every matrix's digits once per geometry (5.5 times its FP64 size
+// at order 20: 48 positions by 48 rows of sixteen FP16 digits for 41 by 41 entries),
 // k_split_vec every source vector's once per product (a vector serves about 7 pairs).
 // k_split: a unit is up to 32 (pair, right-hand side) columns of one matrix and up to 64 of its
 // complex rows: one MMA tile of 128 rows, K index 2 position + part.  Positions run over a
@@ -48,8 +49,8 @@
 // column); k_split_reduce adds every target's rows in list order.
 //
 // Measured at N = 65,536, three layers (72,000 pairs, 2,000 matrices, orders 57 to 20): k_split
-// 172 us, k_split_vec 9, k_split_reduce 34, where the FP64 FMA kernel took 1,040 us at 97% of
-// the FP64 pipe; at N = 262,144 1.0 ms against 5.7.  About equally bound by the MMAs' issue (112 us
+// 181 us (168 with segments of 12 for every table), k_split_vec 5, k_split_reduce 42, where the
+// FP64 FMA kernel took 1,040 us at 97% of the FP64 pipe; at N = 262,144 1.0 ms against 5.7.  About equally bound by the MMAs' issue (112 us
 // with nothing else left in the kernel), the gathering of the columns and the combination of
 // the accumulators.
 #pragma once
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(128) k_split_rexp(const SplitTab* __restrict__
 //   [Re y; Im y] = [zr, -zi; zi, zr] [vr; vi].
 // A chunk is one contiguous block, so a bulk copy stages it.  Converting the FP64 tables in
 // every product instead took a third of the instructions of the product kernel (256 us at N =
-// 65,536, where copies of the 330 MB of digits take about 50).  One CTA per (matrix, tile).
+// 65,536, where copies of the 410 MB of digits take about 60).  One CTA per (matrix, tile).
 __device__ __forceinline__ void split_load(cd (&z)[4], const cd* __restrict__ A, int sr, int sc, int r, int k, int H,
                                            int h, int n1) {
     // row r's entries at positions k..k+3 of a segment (A at column n = 0); the positions past
