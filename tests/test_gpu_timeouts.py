@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 from oracle import nystrom as onys
-from workloads import layered_wide
+from workloads import config_c2, layered_wide
 
 pytestmark = pytest.mark.gpu
 
@@ -59,7 +59,7 @@ def test_a_solve_looks_at_every_step(gpu_lib, cols):
     """A time-out of one step's product (a replayed graph, a block) ends the solve there, instead of
     after its last step or not at all."""
     lf = gpu_lib
-    G = geometry(lf, layered_wide(), 8)
+    G = geometry(lf, config_c2(), 64)   # 300 steps take a third of a second
     rng = np.random.default_rng(2)
     b = np.asfortranarray(rng.standard_normal((G.n, cols)) + 1j * rng.standard_normal((G.n, cols)))
     b = b[:, 0].copy() if cols == 1 else b
